@@ -6,7 +6,7 @@
 // hop (A_ee on the aux term, A_oo^-1 on the result) run in the hop epilogue
 // (hr_hop_dev.cuh), so every hop kernel variant carries them.
 //
-// Build (native FP64: a precomputation, not the hot path).  Per site x:
+// Build (fundamental: fixed point, k_clover_build_fx; else native FP64).  Per site x:
 //   Q_mn   the four leaves of the (mu, nu) plane from x, mu-first,
 //   F_mn = (Q_mn - Q_mn^+) / 8, B_l = e_jkl F_jk / 2 (B_1 = F_23, B_2 = F_31, B_3 = F_12),
 //   in the chiral basis s_0k = diag(-s_k, s_k) and s_jk = -e_jkl diag(s_l, s_l), so
@@ -23,6 +23,7 @@
 #include "hr_clover.cuh"
 #include "hr_clover_leaf.cuh"
 #include "hr_eigh.cuh"
+#include "hr_fix_dev.cuh"
 #include "hr_host.h"
 
 using namespace hr;
@@ -258,17 +259,16 @@ struct BuildArgs {
     double m0, csw;
     int kind;
     void *half[4]; // A even, A odd, A^-1 even, A^-1 odd
-    unsigned *bad; // set when an A is singular
+    unsigned *bad; // kBuildSingular, kBuildOutside
 };
+// an A is singular; a site lies outside the fixed-point range (the whole field is then built in native FP64)
+constexpr unsigned kBuildSingular = 1u, kBuildOutside = 2u;
 
-// one thread per lexicographic site
-template <int NC, int CP> __global__ void __launch_bounds__(64) k_clover_build(BuildArgs B)
+// one lexicographic site in native FP64
+template <int NC, int CP> __device__ void build_site(const BuildArgs &B, long long t)
 {
     constexpr int N = 2 * NC;
     const Geom &g = B.g;
-    const long long V = 2LL * g.vh;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= V) return;
     int x[4];
     long long r = t;
     for (int k = 3; k >= 0; --k) {
@@ -332,13 +332,309 @@ template <int NC, int CP> __global__ void __launch_bounds__(64) k_clover_build(B
             for (int rr = 0; rr < N; ++rr)
                 for (int cc = 0; cc < N; ++cc)
                     A.m[rr][cc] = zadd(zscale(B.csw, C.m[rr][cc]), {rr == cc ? a : 0.0, 0.0});
-            if (!inverse(A, Ai)) atomicExch(B.bad, 1u);
+            if (!inverse(A, Ai)) atomicOr(B.bad, kBuildSingular);
         }
         block_reals(A, &reals[0][b * N * N]);
         block_reals(Ai, &reals[1][b * N * N]);
     }
     store_site<NC, CP>(B.half[p], i, reals[0]);
     store_site<NC, CP>(B.half[2 + p], i, reals[1]);
+}
+
+// native FP64, one thread per lexicographic site: the adjoint field, and a
+// fundamental one outside the fixed-point range
+template <int NC, int CP> __global__ void __launch_bounds__(64) k_clover_build(BuildArgs B)
+{
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < 2LL * B.g.vh) build_site<NC, CP>(B, t);
+}
+
+// ---------------------------------------------------------------- fundamental build in fixed point
+//
+// For SU(2) fundamental links F_mn = (i/4) f_mn.s with f_mn the vector part of
+// the sum of the four leaves (quaternions), so each chiral block is
+//   C_b = sum_lk M_lk s_l (x) s_k,  M_lk = (f_0l + b_l)_k / 8 (upper), -(f_0l - b_l)_k / 8 (lower),
+// real coefficients, and the whole site term lives in the four-dimensional
+// algebra of 1, X, X^2, X^3, X = sum N_lk s_l (x) s_k, N = c_sw M / a, a = 4 + m0:
+//   X^2 = t - 2 K,  X^3 = 3 t X - 6 d - 2 L,  X^4 = 2 t X^2 - 8 d X - q,
+//   t = |N|^2, d = det N, K = cof N, L = N N^T N, q = t^2 - 4 |K|^2
+// (matrices K, L read as K_lk s_l (x) s_k).  Clover: A = a (1 + X) and
+//   A^-1 = [(1 - t - 2 d) - ((1 + t) N + 2 K - 2 L)] / (a D),  D = det(1 + X) = 1 - 2 t - 8 d + q;
+// exponential: the Taylor series of exp(+-X) to degree 18 (|X| <= 1: remainder
+// 8e-18) by Horner's rule on the four coefficients, three products a step
+// where a 4 x 4 complex matrix product has 256.  All of it in two-digit fixed
+// point (hr_fix.cuh).  A site with links off unit length, |N| too large, D near
+// 0 or a factor out of range sets kBuildOutside, and the call, which reads its
+// status word in any case, builds the field again in native FP64 (a call to
+// the native code inside this kernel would hold it at 255 registers).
+// Measured: the clover solve of 24^4 (build, FP32-inner CG to 1e-10, links and
+// source in, solution out) 9.75 ms with the native build, 3.36 ms of it the
+// build, 7.03 ms with this one; solution error against 64 bits unchanged.
+
+struct FxMat {
+    fx m[3][3];
+};
+
+// vector part of the sum of the four leaves of the (mu, nu) plane at x, in units of 2^-56
+template <bool VEC>
+__device__ __forceinline__ void leaf_sum(const Geom &g, const double *can, const LexSite &x, int mu, int nu,
+                                         long long (&f)[3], bool &ok)
+{
+    int um, dm, un, dn;
+    lex_steps(g, x, mu, um, dm);
+    lex_steps(g, x, nu, un, dn);
+    const size_t V = 2 * (size_t)g.vh, bm = (size_t)mu * V + x.t, bn = (size_t)nu * V + x.t;
+    auto U = [&](size_t at) { return load_fxq<VEC>(can, at, ok); };
+    fxa s[3] = {};
+    const fxq a = U(bm), b = U(bn);
+    // U_mu(x) U_nu(x+mu) [U_nu(x) U_mu(x+nu)]^+
+    fxq l = fxq_mul(a, U(bn + um)), r = fxq_mul(b, U(bm + un));
+    fxq_mac_vec(s, l, fxq_conj(r));
+    // U_nu(x) U_mu(x-mu+nu)^+ U_nu(x-mu)^+ U_mu(x-mu)
+    const fxq am = U(bm + dm);
+    l = fxq_mul(b, fxq_conj(U(bm + dm + un)));
+    r = fxq_mul(fxq_conj(U(bn + dm)), am);
+    fxq_mac_vec(s, l, r);
+    // [U_nu(x-mu-nu) U_mu(x-mu)]^+ U_mu(x-mu-nu) U_nu(x-nu)
+    const fxq bd = U(bn + dn);
+    l = fxq_conj(fxq_mul(U(bn + dm + dn), am));
+    r = fxq_mul(U(bm + dm + dn), bd);
+    fxq_mac_vec(s, l, r);
+    // U_nu(x-nu)^+ U_mu(x-nu) [U_mu(x) U_nu(x-nu+mu)^+]^+
+    l = fxq_mul(fxq_conj(bd), U(bm + dn));
+    r = fxq_conj(fxq_mul(a, fxq_conj(U(bn + dn + um))));
+    fxq_mac_vec(s, l, r);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) f[k] = fx_round(s[k]);
+}
+
+// the 16 reals of a block u + sum P_lk s_l (x) s_k (units of 2^-56), each times
+// the digits `sc` and 2^ksc, as pairs
+__device__ __forceinline__ void block_pairs(long long u, const FxMat &P, fx sc, float ksc, float2 (&out)[16])
+{
+    auto pair = [&](long long t) {
+        fxa s = {0, 0};
+        fx_mac(s, fx_split(t), sc);
+        float2 v;
+        fx_to_pair(fx_round(s), v.x, v.y);
+        return make_float2(v.x * ksc, v.y * ksc);
+    };
+    auto T = [](fx v) { return fx_units64(v); };
+    auto neg = [](float2 v) { return make_float2(-v.x, -v.y); };
+    const float2 dp = pair(u + T(P.m[2][2])), dm = pair(u - T(P.m[2][2]));
+    out[0] = dp; out[1] = dm; out[2] = dm; out[3] = dp;
+    const float2 p31 = pair(T(P.m[2][0])), p32 = pair(T(P.m[2][1])), p13 = pair(T(P.m[0][2])), p23 = pair(T(P.m[1][2]));
+    out[4] = p31; out[5] = neg(p32);                 // (0, 1)
+    out[6] = p13; out[7] = neg(p23);                 // (0, 2)
+    out[8] = pair(T(P.m[0][0]) - T(P.m[1][1]));      // (0, 3)
+    out[9] = neg(pair(T(P.m[1][0]) + T(P.m[0][1])));
+    out[10] = pair(T(P.m[0][0]) + T(P.m[1][1]));     // (1, 2)
+    out[11] = pair(T(P.m[0][1]) - T(P.m[1][0]));
+    out[12] = neg(p13); out[13] = p23;               // (1, 3)
+    out[14] = neg(p31); out[15] = p32;               // (2, 3)
+}
+template <int CP> __device__ __forceinline__ void store_block(void *half, int i, int b, const float2 (&r)[16])
+{
+    using L = CloverLayout<2, CP>;
+    float4 *base = (float4 *)half + (size_t)(i >> 5) * L::NVEC * 32 + (i & 31);
+    if constexpr (CP == kF64) {
+#pragma unroll
+        for (int v = 0; v < 8; ++v) base[(8 * b + v) * 32] = make_float4(r[2 * v].x, r[2 * v].y, r[2 * v + 1].x, r[2 * v + 1].y);
+    } else {
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            base[(4 * b + v) * 32] = make_float4(r[4 * v].x, r[4 * v + 1].x, r[4 * v + 2].x, r[4 * v + 3].x);
+    }
+}
+
+struct BuildFx {
+    fx kappa;    // c_sw / a
+    fx am;       // a = am 2^ka, am in [1, 2)
+    float ka;    // 2^ka
+    double inva; // 1 / a
+};
+
+template <int CP, bool EXP, bool VEC> __global__ void __launch_bounds__(64) k_clover_build_fx(BuildArgs B, BuildFx X)
+{
+    const Geom &g = B.g;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 2 * g.vh) return;
+    const LexSite x = lex_site(g, t);
+    const int p = (x.x0 + x.x1 + x.x2 + x.x3) & 1, i = t >> 1;
+    bool ok = true;
+    FxMat N[2];
+#pragma unroll 1
+    for (int l = 0; l < 3; ++l) {
+        long long e[3], f[3];
+        leaf_sum<VEC>(g, B.can, x, 0, l + 1, e, ok);
+        // B_1 = F_23, B_2 = F_31 = -F_13, B_3 = F_12
+        leaf_sum<VEC>(g, B.can, x, l == 0 ? 2 : 1, l == 2 ? 2 : 3, f, ok);
+        fx row[2][3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const long long bk = l == 1 ? -f[k] : f[k];
+            fxa u = {0, 0}, d = {0, 0};
+            fx_mac(u, fx_split((e[k] + bk) >> 3), X.kappa);
+            fx_mac(d, fx_split((bk - e[k]) >> 3), X.kappa);
+            row[0][k] = fx_of(u);
+            row[1][k] = fx_of(d);
+        }
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                if (l == 0) N[b].m[0][k] = row[b][k];
+                else if (l == 1) N[b].m[1][k] = row[b][k];
+                else N[b].m[2][k] = row[b][k];
+            }
+    }
+    const long long one = 1LL << 56;
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+        const FxMat &n = N[b];
+        fxa ta = {0, 0}, da = {0, 0}, ka = {0, 0};
+        FxMat K, L;
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                fx_mac(ta, n.m[r][c], n.m[r][c]);
+                const int r1 = (r + 1) % 3, r2 = (r + 2) % 3, c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+                fxa s = {0, 0};
+                fx_mac(s, n.m[r1][c1], n.m[r2][c2]);
+                fx_mac(s, fx_neg(n.m[r1][c2]), n.m[r2][c1]);
+                K.m[r][c] = fx_of(s);
+            }
+        const long long tt = fx_round(ta);
+        if (tt > (EXP ? one / 3 : one)) ok = false;
+        fx S[3][3]; // N N^T (symmetric)
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int c = r; c < 3; ++c) {
+                fxa s = {0, 0};
+#pragma unroll
+                for (int k = 0; k < 3; ++k) fx_mac(s, n.m[r][k], n.m[c][k]);
+                S[r][c] = S[c][r] = fx_of(s);
+            }
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                fxa s = {0, 0};
+#pragma unroll
+                for (int k = 0; k < 3; ++k) fx_mac(s, S[r][k], n.m[k][c]);
+                L.m[r][c] = fx_of(s);
+                fx_mac(ka, K.m[r][c], K.m[r][c]);
+            }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) fx_mac(da, n.m[0][c], K.m[0][c]);
+        const fx td = fx_split(tt);
+        const long long dt = fx_round(da);
+        fxa qa = {-4 * ka.a, -4 * ka.b};
+        fx_mac(qa, td, td);
+        const long long qt = fx_round(qa);
+        // coefficients of 1, X, X^2, X^3 of A / a and A^-1 a (clover: times D)
+        FxMat P, Q;
+        long long u, v;
+        fx sc_inv;
+        float ks_inv = 1.f;
+        if constexpr (EXP) {
+            const fx q = fx_split(-qt), d8 = fx_split(-8 * dt), t2 = fx_split(2 * tt);
+#pragma unroll
+            for (int inv = 0; inv < 2; ++inv) {
+                // 1/k! 2^56 for k = 18 .. 0
+                constexpr double rf[19] = {1.0 / 6402373705728000.0, 1.0 / 355687428096000.0, 1.0 / 20922789888000.0,
+                                           1.0 / 1307674368000.0, 1.0 / 87178291200.0, 1.0 / 6227020800.0,
+                                           1.0 / 479001600.0, 1.0 / 39916800.0, 1.0 / 3628800.0, 1.0 / 362880.0,
+                                           1.0 / 40320.0, 1.0 / 5040.0, 1.0 / 720.0, 1.0 / 120.0, 1.0 / 24.0,
+                                           1.0 / 6.0, 0.5, 1.0, 1.0};
+                fx c0 = fx_split((long long)(rf[0] * 0x1p56)), c1 = {0, 0}, c2 = {0, 0}, c3 = {0, 0};
+#pragma unroll 1
+                for (int k = 1; k < 19; ++k) {
+                    const long long f = (long long)(rf[k] * 0x1p56);
+                    fxa s0 = {inv && (k & 1) ? -f : f, 0}, s1 = {fx_units64(c0), 0}, s2 = {fx_units64(c1), 0};
+                    fx_mac(s0, q, c3);
+                    fx_mac(s1, d8, c3);
+                    fx_mac(s2, t2, c3);
+                    c3 = c2;
+                    c0 = fx_of(s0);
+                    c1 = fx_of(s1);
+                    c2 = fx_of(s2);
+                }
+                // c0 + c2 t - 6 d c3,  c1 + 3 t c3,  -2 c2,  -2 c3
+                fxa w = {fx_units64(c0), 0}, e1 = {fx_units64(c1), 0};
+                fx_mac(w, c2, td);
+                fx_mac(w, c3, fx_split(-6 * dt));
+                fx_mac(e1, c3, fx_split(3 * tt));
+                const fx k1 = fx_of(e1), k2 = {-2 * c2.h, -2 * c2.l}, k3 = {-2 * c3.h, -2 * c3.l};
+                FxMat &O = inv ? Q : P;
+#pragma unroll
+                for (int r = 0; r < 3; ++r)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        fxa s = {0, 0};
+                        fx_mac(s, k1, n.m[r][c]);
+                        fx_mac(s, k2, K.m[r][c]);
+                        fx_mac(s, k3, L.m[r][c]);
+                        O.m[r][c] = fx_of(s);
+                    }
+                if (inv) v = fx_round(w);
+                else u = fx_round(w);
+            }
+        } else {
+            u = one;
+            P = n;
+            v = one - tt - 2 * dt;
+            const fx t1 = fx_split(-one - tt);
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    fxa s = {2 * (fx_units64(L.m[r][c]) - fx_units64(K.m[r][c])), 0};
+                    fx_mac(s, t1, n.m[r][c]);
+                    Q.m[r][c] = fx_of(s);
+                }
+        }
+        double inv = X.inva;
+        if constexpr (!EXP) {
+            const long long D = one - 2 * tt - 8 * dt + qt;
+            if (D < one / 16) ok = false;
+            inv = inv / fx_to_double(D);
+        }
+        {
+            // 1 / a (clover: 1 / (a D)) = m 2^k, m in [1, 2)
+            const unsigned long long ib = fx_dbits(inv);
+            const int k = (int)(ib >> 52) - 1023;
+            if (k < -60 || k > 60) ok = false;
+            sc_inv = fx_from_double(fx_double((ib & 0xfffffffffffffULL) | 0x3ff0000000000000ULL));
+            ks_inv = fx_float((unsigned)(127 + min(max(k, -60), 60)) << 23);
+        }
+        float2 out[16];
+        block_pairs(u, P, X.am, X.ka, out);
+        store_block<CP>(B.half[p], i, b, out);
+        block_pairs(v, Q, sc_inv, ks_inv, out);
+        store_block<CP>(B.half[2 + p], i, b, out);
+    }
+    if (!ok) atomicOr(B.bad, kBuildOutside);
+}
+
+template <int CP>
+void launch_build_fx(const BuildArgs &B, double a, cudaStream_t s)
+{
+    BuildFx X;
+    int k;
+    const double am = 2.0 * std::frexp(a, &k); // [1, 2)
+    X.kappa = fx_from_double(B.csw / a);
+    X.am = fx_from_double(am);
+    X.ka = std::ldexp(1.f, k - 1);
+    X.inva = 1.0 / a;
+    const int bs = 64, grid = (int)((2LL * B.g.vh + bs - 1) / bs);
+    const bool vec = ((uintptr_t)B.can & 15u) == 0, ex = B.kind == HR_CLOVER_EXP;
+    if (ex && vec) k_clover_build_fx<CP, true, true><<<grid, bs, 0, s>>>(B, X);
+    else if (ex) k_clover_build_fx<CP, true, false><<<grid, bs, 0, s>>>(B, X);
+    else if (vec) k_clover_build_fx<CP, false, true><<<grid, bs, 0, s>>>(B, X);
+    else k_clover_build_fx<CP, false, false><<<grid, bs, 0, s>>>(B, X);
 }
 
 // FP64 -> FP32 field, one thread per FP32 vector
@@ -456,25 +752,34 @@ hr_status hr_clover_build(hr_ctx *ctx, hr_lattice lat, hr_rep rep, hr_prec prec,
     B.kind = kind;
     for (int h = 0; h < 4; ++h) B.half[h] = (void *)clover_half(clover, g, rep, prec, h >= 2, h & 1);
     B.bad = ctx->d_counters + C_STATUS;
-    cudaError_t e = cudaMemsetAsync(B.bad, 0, sizeof(unsigned), s);
-    if (e != cudaSuccess) return set_error(ctx, HR_ERR_CUDA, "status reset: %s", cudaGetErrorString(e));
     const long long V = 2LL * g.vh;
     const int bs = 64, grid = (int)((V + bs - 1) / bs);
     const bool three = rep_nc(rep) == 3;
-    if (prec == kF64) {
-        if (three) k_clover_build<3, kF64><<<grid, bs, 0, s>>>(B);
-        else k_clover_build<2, kF64><<<grid, bs, 0, s>>>(B);
-    } else {
-        if (three) k_clover_build<3, kF32><<<grid, bs, 0, s>>>(B);
-        else k_clover_build<2, kF32><<<grid, bs, 0, s>>>(B);
-    }
-    st = check_launch(ctx, "clover build");
-    if (st) return st;
+    // fixed point: fundamental links, 0 < a and |c_sw / a| within the digits' range
+    const double a = 4.0 + m0;
+    bool fixed = !three && a > 0x1p-20 && a < 0x1p20 && std::fabs(c_sw) < 2.0 * a;
     unsigned bad = 0;
-    e = cudaMemcpyAsync(&bad, B.bad, sizeof bad, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return set_error(ctx, HR_ERR_CUDA, "clover build status: %s", cudaGetErrorString(e));
-    if (bad) return set_error(ctx, HR_ERR_NUMERIC, "a clover site block is singular (no inverse)");
+    for (;;) {
+        cudaError_t e = cudaMemsetAsync(B.bad, 0, sizeof(unsigned), s);
+        if (e != cudaSuccess) return set_error(ctx, HR_ERR_CUDA, "status reset: %s", cudaGetErrorString(e));
+        if (prec == kF64) {
+            if (fixed) launch_build_fx<kF64>(B, a, s);
+            else if (three) k_clover_build<3, kF64><<<grid, bs, 0, s>>>(B);
+            else k_clover_build<2, kF64><<<grid, bs, 0, s>>>(B);
+        } else {
+            if (fixed) launch_build_fx<kF32>(B, a, s);
+            else if (three) k_clover_build<3, kF32><<<grid, bs, 0, s>>>(B);
+            else k_clover_build<2, kF32><<<grid, bs, 0, s>>>(B);
+        }
+        st = check_launch(ctx, "clover build");
+        if (st) return st;
+        e = cudaMemcpyAsync(&bad, B.bad, sizeof bad, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return set_error(ctx, HR_ERR_CUDA, "clover build status: %s", cudaGetErrorString(e));
+        if (!(bad & kBuildOutside)) break;
+        fixed = false;
+    }
+    if (bad & kBuildSingular) return set_error(ctx, HR_ERR_NUMERIC, "a clover site block is singular (no inverse)");
     return HR_OK;
 }
 

@@ -1,0 +1,58 @@
+// hr_fix_dev.cuh -- lexicographic site steps and canonical links as digits, shared
+// by the fixed-point kernels (gauge force, clover build, clover force).
+#pragma once
+
+#include "hr_fix.cuh"
+#include "hr_internal.cuh"
+
+namespace hr {
+
+// a site by its lexicographic index, with 32-bit steps to its neighbours
+struct LexSite {
+    int t, x0, x1, x2, x3;
+};
+__device__ __forceinline__ LexSite lex_site(const Geom &g, int t)
+{
+    LexSite s;
+    const int row = fdiv(t >> 1, g.div_h3), r1 = fdiv(row, g.div_d2);
+    s.t = t;
+    s.x3 = t - row * g.d[3];
+    s.x2 = row - r1 * g.d[2];
+    s.x0 = fdiv(r1, g.div_d1);
+    s.x1 = r1 - s.x0 * g.d[1];
+    return s;
+}
+// index steps from the site to x + mu and x - mu (periodic)
+__device__ __forceinline__ void lex_steps(const Geom &g, const LexSite &s, int mu, int &up, int &down)
+{
+    const int x = mu == 0 ? s.x0 : mu == 1 ? s.x1 : mu == 2 ? s.x2 : s.x3;
+    const int d = mu == 0 ? g.d[0] : mu == 1 ? g.d[1] : mu == 2 ? g.d[2] : g.d[3];
+    const int st = mu == 3 ? 1 : mu == 2 ? g.d[3] : mu == 1 ? g.d[3] * g.d[2] : g.d[3] * g.d[2] * g.d[1];
+    up = x == d - 1 ? -(d - 1) * st : st;
+    down = x == 0 ? (d - 1) * st : -st;
+}
+// a canonical link as digits; ok stays true only for links of unit length to 1 %
+// (VEC: the field is 16-byte aligned)
+template <bool VEC> __device__ __forceinline__ void load_link4(const double *q, size_t link, double (&c)[4])
+{
+    if constexpr (VEC) {
+        const double2 *p = (const double2 *)q + 2 * link;
+        const double2 a = p[0], b = p[1];
+        c[0] = a.x; c[1] = a.y; c[2] = b.x; c[3] = b.y;
+    } else {
+        const double *p = q + 4 * link;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) c[k] = p[k];
+    }
+}
+template <bool VEC> __device__ __forceinline__ fxq load_fxq(const double *q, size_t link, bool &ok)
+{
+    double c[4];
+    load_link4<VEC>(q, link, c);
+    const unsigned m = max(max(fx_abs_high(c[0]), fx_abs_high(c[1])), max(fx_abs_high(c[2]), fx_abs_high(c[3])));
+    const fxq r = {{fx_from_double(c[0]), fx_from_double(c[1]), fx_from_double(c[2]), fx_from_double(c[3])}};
+    ok = ok && m < kFxHigh2 && fxq_near_unit(r);
+    return r;
+}
+
+} // namespace hr
