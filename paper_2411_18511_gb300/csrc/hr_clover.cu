@@ -454,7 +454,7 @@ struct BuildFx {
     double inva; // 1 / a
 };
 
-template <int CP, bool EXP, bool VEC> __global__ void __launch_bounds__(64) k_clover_build_fx(BuildArgs B, BuildFx X)
+template <int CP, bool EXP, bool VEC> __global__ void __launch_bounds__(64, 6) k_clover_build_fx(BuildArgs B, BuildFx X)
 {
     const Geom &g = B.g;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -867,7 +867,8 @@ hr_status hr_dirac_eo_clover(hr_ctx *ctx, hr_lattice lat, hr_rep rep, hr_prec pr
 // and in the chiral blocks (C+ on spins 0, 1, C- on 2, 3, as in the build), with
 // P_l^b = sum_{s,t} (s_l)_st Lam[(2b+t, .), (2b+s, .)] (colour 2x2),
 //   K_0l = P_l^1 - P_l^0,  K_23 = -(P_1^0 + P_1^1),  K_13 = P_2^0 + P_2^1,  K_12 = -(P_3^0 + P_3^1).
-// K field: double [V][6][2][2][2] (lexicographic site, planes 01 02 03 12 13 23).
+// Only kappa_k = Re tr(s_k K) of a plane enters f (F_mn is (i/4) f.s with real f),
+// so the field kept is double [6][3][V] (planes 01 02 03 12 13 23, lexicographic site).
 // The link derivative of f: each link lies on two plaquettes of each of the
 // three planes that contain its direction, and each plaquette enters the
 // leaves of its four corners; hr_clover_leaf.cuh sums the four corner
@@ -908,26 +909,29 @@ template <class Lam> __device__ void add_blocks(zc (&P)[2][3][2][2], double coef
                 }
 }
 
-__device__ void store_k(double *K, long long x, const zc (&P)[2][3][2][2])
+// kappa_k = Re tr(s_k K) of the six planes, double [6][3][V]; with Pi^b_lk =
+// Re tr_c(s_k P_l^b): kappa_0l = Pi^1_l - Pi^0_l, kappa_23 = -(Pi^0_1 + Pi^1_1),
+// kappa_13 = Pi^0_2 + Pi^1_2, kappa_12 = -(Pi^0_3 + Pi^1_3)
+__device__ __forceinline__ void store_kappa(double *K, long long V, long long x, int l, int k, double lower, double upper)
 {
-    for (int d = 0; d < 2; ++d)
-        for (int c = 0; c < 2; ++c) {
-            zc k[6];
-            k[0] = zsub(P[1][0][d][c], P[0][0][d][c]);
-            k[1] = zsub(P[1][1][d][c], P[0][1][d][c]);
-            k[2] = zsub(P[1][2][d][c], P[0][2][d][c]);
-            k[3] = zscale(-1.0, zadd(P[0][2][d][c], P[1][2][d][c])); // 12: -(P_3^0 + P_3^1)
-            k[4] = zadd(P[0][1][d][c], P[1][1][d][c]);               // 13: P_2^0 + P_2^1
-            k[5] = zscale(-1.0, zadd(P[0][0][d][c], P[1][0][d][c])); // 23: -(P_1^0 + P_1^1)
-            for (int pl = 0; pl < 6; ++pl) {
-                double *o = K + ((x * 6 + pl) * 4 + d * 2 + c) * 2;
-                o[0] = k[pl].re;
-                o[1] = k[pl].im;
-            }
+    K[((long long)l * 3 + k) * V + x] = upper - lower;
+    const int pl = l == 0 ? 5 : l == 1 ? 4 : 3;
+    K[((long long)pl * 3 + k) * V + x] = l == 1 ? lower + upper : -(lower + upper);
+}
+__device__ void store_k(double *K, long long V, long long x, const zc (&P)[2][3][2][2])
+{
+    for (int l = 0; l < 3; ++l) {
+        double pi[2][3];
+        for (int b = 0; b < 2; ++b) {
+            pi[b][0] = P[b][l][0][1].re + P[b][l][1][0].re;
+            pi[b][1] = P[b][l][1][0].im - P[b][l][0][1].im;
+            pi[b][2] = P[b][l][0][0].re - P[b][l][1][1].re;
         }
+        for (int k = 0; k < 3; ++k) store_kappa(K, V, x, l, k, pi[0][k], pi[1][k]);
+    }
 }
 
-// K from a canonical insertion Lam: complex [V][8][8], index spin * 2 + colour
+// kappa from a canonical insertion Lam: complex [V][8][8], index spin * 2 + colour
 __global__ void k_clover_k_from_lam(long long V, const double *lam, double *K)
 {
     const long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -938,7 +942,7 @@ __global__ void k_clover_k_from_lam(long long V, const double *lam, double *K)
         const int r = t * 2 + d, q = s * 2 + c;
         return zc{L[(r * 8 + q) * 2], L[(r * 8 + q) * 2 + 1]};
     });
-    store_k(K, x, P);
+    store_k(K, V, x, P);
 }
 
 struct KFieldArgs {
@@ -1004,20 +1008,11 @@ __device__ void read_blocks(const void *half, int i, zd (&M)[2][4][4])
     }
 }
 
-// K of the two-flavour clover pseudofermion (and det A_oo) insertion
-__global__ void k_clover_k_from_fields(KFieldArgs A)
+// kappa of the two-flavour clover pseudofermion (and det A_oo) insertion at one site, native FP64
+__device__ void kappa_site(const KFieldArgs &A, long long x, int p)
 {
     const Geom &g = A.g;
     const long long V = 2LL * g.vh;
-    const long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= V) return;
-    int c4[4];
-    long long r = x;
-    for (int k = 3; k >= 0; --k) {
-        c4[k] = (int)(r % g.d[k]);
-        r /= g.d[k];
-    }
-    const int p = (c4[0] + c4[1] + c4[2] + c4[3]) & 1;
     const int i = (int)(x >> 1);
     zc P[2][3][2][2] = {};
     cpx<double> u[4][2], v[4][2];
@@ -1041,7 +1036,7 @@ __global__ void k_clover_k_from_fields(KFieldArgs A)
             const zd z = Lb[t >> 1][(t & 1) * 2 + d][(s & 1) * 2 + c];
             return zc{z.re, z.im};
         });
-        store_k(A.K, x, P);
+        store_k(A.K, V, x, P);
         return;
     }
     add_blocks(P, coef, [&](int t, int d, int s, int c) {
@@ -1067,32 +1062,215 @@ __global__ void k_clover_k_from_fields(KFieldArgs A)
             return M[b][(t & 1) * 2 + d][(s & 1) * 2 + c];
         });
     }
-    store_k(A.K, x, P);
+    store_k(A.K, V, x, P);
+}
+__device__ __forceinline__ int site_parity(const LexSite &x) { return (x.x0 + x.x1 + x.x2 + x.x3) & 1; }
+
+// the exponential form: the insertion goes through the eigenbasis of A
+__global__ void k_clover_kappa_exp(KFieldArgs A)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < 2 * A.g.vh) kappa_site(A, t, site_parity(lex_site(A.g, t)));
 }
 
-// F[rho][z][a] += scale * d/dw_a Re sum_y tr[C Lam], one thread per link (rho, z):
-// the two plaquettes of each of the three planes that hold rho, each with its
-// four corner insertions around one staple (hr_clover_leaf.cuh)
-__global__ void __launch_bounds__(128) k_clover_leaf_force(Geom g, const double *can, const double *K, double scale,
-                                                           double *F)
+__device__ __noinline__ void kappa_site_native(const KFieldArgs &A, long long x, int p) { kappa_site(A, x, p); }
+
+// Re v^+ (s_l (x) s_k) u of one chiral block, u and v [4 spin + 2 colour + (re, im)]
+__device__ __forceinline__ long long sigma_sigma(const fx *u, const fx *v, int l, int k)
 {
+    fxa s = {0, 0};
+#pragma unroll
+    for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            // row (sp, c) of s_l (x) s_k has one entry, i^n at column (sc, cc)
+            const int sc = l < 2 ? 1 - sp : sp, cc = k < 2 ? 1 - c : c;
+            const int n = ((l == 1 ? (sp ? 1 : 3) : l == 2 && sp ? 2 : 0) + (k == 1 ? (c ? 1 : 3) : k == 2 && c ? 2 : 0)) & 3;
+            const fx vr = v[4 * sp + 2 * c], vi = v[4 * sp + 2 * c + 1];
+            const fx ur = u[4 * sc + 2 * cc], ui = u[4 * sc + 2 * cc + 1];
+            // Re(conj(v) i^n u)
+            if (n == 0) { fx_mac(s, vr, ur); fx_mac(s, vi, ui); }
+            else if (n == 1) { fx_mac(s, fx_neg(vr), ui); fx_mac(s, vi, ur); }
+            else if (n == 2) { fx_mac(s, fx_neg(vr), ur); fx_mac(s, fx_neg(vi), ui); }
+            else { fx_mac(s, vr, ui); fx_mac(s, fx_neg(vi), ur); }
+        }
+    return fx_round(s);
+}
+
+// Clover form, one thread per lexicographic site, in fixed point (hr_fix.cuh):
+// Pi^b_lk = coef Re v^+ (s_l (x) s_k) u needs the real parts of 9 x 8 products
+// a block instead of the complex outer product u v^+; on odd sites the
+// determinant adds -8 (A^-1)_lk, the coefficient of s_l (x) s_k in A^-1.
+__global__ void __launch_bounds__(128, 3) k_clover_kappa(KFieldArgs A)
+{
+    const Geom &g = A.g;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 2 * g.vh) return;
     const long long V = 2LL * g.vh;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 4 * V) return;
-    const int rho = (int)(t / V);
-    const long long z = t - (long long)rho * V;
-    int x[4];
-    long long r = z;
-    for (int k = 3; k >= 0; --k) {
-        x[k] = (int)(r % g.d[k]);
-        r /= g.d[k];
+    const int p = site_parity(lex_site(g, t)), i = t >> 1;
+    fx u[16], v[16];
+    int eu, ev;
+    bool ok = load_fx(p == 0 ? A.X : A.Z, i, u, eu);
+    ok = load_fx(p == 0 ? A.Y : A.W, i, v, ev) && ok;
+    if (!ok) {
+        kappa_site_native(A, t, p);
+        return;
     }
+    const double f = (p == 0 ? -2.0 : -0.5) * fx_pow2(eu + ev - 2 * kFxPairBias - 56);
+    const bool det = p == 1 && A.ainv;
+    double pi[2][9];
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+#pragma unroll
+        for (int e = 0; e < 9; ++e) pi[b][e] = f * (double)sigma_sigma(u + 8 * b, v + 8 * b, e / 3, e % 3);
+        if (det) {
+            // block reals 0-3: diagonal; 4-15: (0,1) (0,2) (0,3) (1,2) (1,3) (2,3) as (re, im)
+            const float4 *q = (const float4 *)A.ainv + ((size_t)(i >> 5) * 16 + 8 * b) * 32 + (i & 31);
+            float4 w[8];
+            unsigned m = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                w[k] = __ldg(q + k * 32);
+                m = max(m, max(__float_as_uint(w[k].x) & 0x7fffffffu, __float_as_uint(w[k].z) & 0x7fffffffu));
+            }
+            const int E = min(max((int)(m >> 23), kFxMinExp), 254);
+            const float sc = fx_pair_scale(E);
+            long long R[16];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                R[2 * k] = fx_units64(fx_from_pair(w[k].x, w[k].y, sc));
+                R[2 * k + 1] = fx_units64(fx_from_pair(w[k].z, w[k].w, sc));
+            }
+            // 4 N_lk
+            const long long n[9] = {2 * (R[10] + R[8]), 2 * (R[11] - R[9]), 2 * (R[6] - R[12]),
+                                    -2 * (R[9] + R[11]), 2 * (R[10] - R[8]), 2 * (R[13] - R[7]),
+                                    2 * (R[4] - R[14]), 2 * (R[15] - R[5]), (R[0] - R[1]) - (R[2] - R[3])};
+            const double h = -2.0 * fx_pow2(E - kFxPairBias - 56);
+#pragma unroll
+            for (int e = 0; e < 9; ++e) pi[b][e] += h * (double)n[e];
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 9; ++e) store_kappa(A.K, V, t, e / 3, e % 3, pi[0][e], pi[1][e]);
+}
+
+// one link in native FP64: links off unit length, NaN or Inf
+__device__ __noinline__ void leaf_force_native(const Geom &g, const double *can, const double *K, double scale, int rho,
+                                               int t, double *o)
+{
     LeafLattice L;
     for (int k = 0; k < 4; ++k) L.d[k] = g.d[k];
+    const LexSite s = lex_site(g, t);
+    const int x[4] = {s.x0, s.x1, s.x2, s.x3};
     double out[3];
-    leaf_force_link(L, can, K, rho, x, out);
-    double *o = F + ((long long)rho * V + z) * 3;
+    leaf_force_link(L, can, KappaField{K, 2LL * g.vh}, rho, x, out);
     for (int a = 0; a < 3; ++a) o[a] += scale * out[a];
+}
+
+// F[rho][z][a] += scale * d/dw_a Re sum_y tr[C Lam], one thread per link (rho =
+// blockIdx.y, z): the two plaquettes of each of the three planes that hold rho,
+// each as the loop V e1 e2 e3 from z (V = U_rho(z)) with the four corner
+// vectors k0 .. k3 (pure quaternions) inserted around one staple S = e1 e2 e3,
+//   F = -/+ vec(V B) / 16,  B = k1 S + e1 (k2 e2 + e2 k3) e3 + S k0
+// (- where the loop runs mu-first in the plane's orientation), V taken out of
+// the sum of the six B.  Fixed point (hr_fix.cuh): about 110 products a
+// plaquette, where the 2 x 2 complex matrices of hr_clover_leaf.cuh take 700.
+// The kappa of a plaquette are read in units of their largest component, and
+// the running sum of the B follows the largest unit met so far.  20 x 14 x 18 x 22:
+// 4.99 ms in native FP64, 0.286 ms here (128 registers: 0.298); the whole
+// clover force (hops, link derivatives, kappa, this) 5.77 -> 0.48 ms, error
+// against 64 bits unchanged (7.8e-15, the hops').
+template <bool VEC>
+__global__ void __launch_bounds__(128, 3) k_clover_leaf_force(Geom g, const double *__restrict__ can,
+                                                              const double *__restrict__ K, double scale,
+                                                              double *__restrict__ F)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, rho = blockIdx.y;
+    const int V = 2 * g.vh;
+    if (t >= V) return;
+    const LexSite x = lex_site(g, t);
+    int ur, unused;
+    lex_steps(g, x, rho, ur, unused);
+    bool ok = true;
+    const size_t br = (size_t)rho * V + t;
+    long long B[4] = {0, 0, 0, 0};
+    int eB = -4096; // B in units of 2^(eB - 56)
+#pragma unroll 1
+    for (int k = 2; k < 8; ++k) {
+        const int sig = (rho + (k >> 1)) & 3;
+        const bool down = k & 1;
+        int us, ds;
+        lex_steps(g, x, sig, us, ds);
+        const int off = down ? ds : us, s0 = down ? ds : 0;
+        const size_t bs = (size_t)sig * V + t;
+        fxq e1 = load_fxq<VEC>(can, bs + ur + s0, ok), e3 = load_fxq<VEC>(can, bs + s0, ok);
+        const fxq e2 = fxq_conj(load_fxq<VEC>(can, br + off, ok));
+        if (down) e1 = fxq_conj(e1);
+        else e3 = fxq_conj(e3);
+        const int lo = min(rho, sig), hi = max(rho, sig);
+        const int pl = lo == 0 ? hi - 1 : lo == 1 ? hi + 1 : 5; // 01 02 03 12 13 23
+        const double *kp = K + (size_t)pl * 3 * V + t;
+        double kd[4][3];
+        unsigned m = 0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const double *q = kp + (size_t)a * V;
+            kd[0][a] = __ldg(q);
+            kd[1][a] = __ldg(q + ur);
+            kd[2][a] = __ldg(q + ur + off);
+            kd[3][a] = __ldg(q + off);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) m = max(m, fx_abs_high(kd[c][a]));
+        }
+        const int E = (int)(m >> 20);
+        ok = ok && E < 2047;
+        fx kq[4][3];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) kq[c][a] = fx_from_double(kd[c][a], E);
+        const fxq S = fxq_mul(e1, fxq_mul(e2, e3));
+        fxa ya[4] = {}, ta[4] = {};
+        fxq_mac_pure_l(ya, kq[2], e2);
+        fxq_mac_pure_r(ya, e2, kq[3]);
+        fxq_mac(ta, fxq_mul(e1, fxq_of(ya)), e3);
+        fxq_mac_pure_l(ta, kq[1], S);
+        fxq_mac_pure_r(ta, S, kq[0]);
+        if (E == 0) continue; // all zero (or subnormal)
+        const int e = E - 1022, dn = min(max(eB - e, 0), 63), db = min(max(e - eB, 0), 63);
+        const bool minus = (rho < sig) != down;
+        eB = max(eB, e);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const long long v = fx_round(ta[c]) >> dn;
+            B[c] = (B[c] >> db) + (minus ? -v : v);
+        }
+    }
+    const fxq U = load_fxq<VEC>(can, br, ok);
+    double *o = F + br * 3;
+    if (!ok) {
+        leaf_force_native(g, can, K, scale, rho, t, o);
+        return;
+    }
+    if (eB == -4096) return;
+    // |B| < 42 units: down to digits below 2^30
+    unsigned long long used = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) used |= (unsigned long long)(B[c] ^ (B[c] >> 63));
+    const int r = max(0, 6 - fx_clz(used | 1u));
+    fxq Bq;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) Bq.c[c] = fx_split(B[c] >> r);
+    fxa w[3] = {};
+    fxq_mac_vec(w, U, Bq);
+    const int ex = eB + r - 60; // 2^-56 and the 1/16
+    if (ex > -1000 && ex < 900) {
+        const double f = scale * fx_pow2(ex);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) o[a] += f * (double)fx_round(w[a]);
+    } else {
+        leaf_force_native(g, can, K, scale, rho, t, o);
+    }
 }
 
 // block sums of sum_{odd sites} log det A (both blocks, Cholesky), one partial per block
@@ -1143,13 +1321,14 @@ template <int NC> __global__ void __launch_bounds__(128) k_clover_logdet(Geom g,
 
 constexpr int kLogdetBlocks = 256;
 
-size_t k_field_bytes(const Geom &g) { return ((size_t)2 * g.vh * 48 * sizeof(double) + 255) & ~(size_t)255; }
+size_t k_field_bytes(const Geom &g) { return ((size_t)2 * g.vh * 18 * sizeof(double) + 255) & ~(size_t)255; }
 
 hr_status leaf_force(hr_ctx *ctx, const Geom &g, const double *can, const double *K, double scale, double *F,
                      cudaStream_t s)
 {
-    const long long n = 8LL * g.vh;
-    k_clover_leaf_force<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(g, can, K, scale, F);
+    const dim3 grid((unsigned)((2LL * g.vh + 127) / 128), 4);
+    if (((uintptr_t)can & 15u) == 0) k_clover_leaf_force<true><<<grid, 128, 0, s>>>(g, can, K, scale, F);
+    else k_clover_leaf_force<false><<<grid, 128, 0, s>>>(g, can, K, scale, F);
     return check_launch(ctx, "clover force");
 }
 
@@ -1253,7 +1432,9 @@ hr_status hr_clover_fermion_force(hr_ctx *ctx, hr_lattice lat, hr_clover_kind ki
     A.a = 4.0 + m0;
     A.K = K;
     const long long V = 2LL * g.vh;
-    k_clover_k_from_fields<<<(unsigned)((V + 127) / 128), 128, 0, s>>>(A);
+    const unsigned kgrid = (unsigned)((V + 127) / 128);
+    if (A.exp_kind) k_clover_kappa_exp<<<kgrid, 128, 0, s>>>(A);
+    else k_clover_kappa<<<kgrid, 128, 0, s>>>(A);
     st = check_launch(ctx, "clover insertion");
     if (!st) st = leaf_force(ctx, g, gauge, K, coeff * c_sw, force, s);
     return st;

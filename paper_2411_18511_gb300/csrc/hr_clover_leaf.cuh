@@ -100,9 +100,29 @@ HR_HD inline M2 leaf_k(const double *K, long long x, int pl, bool dag)
     return dag ? m2_dag(M) : M;
 }
 
+// The same sums need only kappa_k = Re tr(s_k K): (R - R^+) = 2 i vec(R).s, so
+// K and (kappa . s) / 2 give the same f.  KappaField: double [6][3][V].
+struct KappaField {
+    const double *k;
+    long long V;
+};
+HR_HD inline M2 leaf_k(const KappaField &K, long long x, int pl, bool dag)
+{
+    (void)dag; // Hermitian
+    const double *k = K.k + (long long)pl * 3 * K.V + x;
+    const double a = 0.5 * k[0], b = 0.5 * k[K.V], c = 0.5 * k[2 * K.V];
+    M2 M;
+    M.m[0][0] = {c, 0.0};
+    M.m[0][1] = {a, -b};
+    M.m[1][0] = {a, b};
+    M.m[1][1] = {-c, 0.0};
+    return M;
+}
+
 // G of one plaquette of the (mu, nu) plane (mu < nu, plane index pl) with
 // lower corner w, for the varied link `which` (0: a, 1: b, 2: c, 3: d)
-HR_HD inline M2 plaquette_g(const LeafLattice &L, const double *can, const double *K, int mu, int nu, int pl,
+template <class KF>
+HR_HD inline M2 plaquette_g(const LeafLattice &L, const double *can, const KF &K, int mu, int nu, int pl,
                             const int (&w)[4], int which)
 {
     const long long V = (long long)L.d[0] * L.d[1] * L.d[2] * L.d[3];
@@ -151,7 +171,8 @@ HR_HD inline M2 plaquette_g(const LeafLattice &L, const double *can, const doubl
 }
 
 // out[a] = d f / d w_a for the link U_rho(z) (coordinates x of z)
-HR_HD inline void leaf_force_link(const LeafLattice &L, const double *can, const double *K, int rho,
+template <class KF>
+HR_HD inline void leaf_force_link(const LeafLattice &L, const double *can, const KF &K, int rho,
                                   const int (&x)[4], double (&out)[3])
 {
     out[0] = out[1] = out[2] = 0.0;

@@ -157,6 +157,23 @@ HR_HD inline fx fx_from_double(double x)
     const long long sg = (long long)u >> 63;
     return fx_split((long long)(t ^ (unsigned long long)sg) - sg);
 }
+// Digits of x / 2^(E - 1022) for |x| < 2^(E - 1022), E the biased exponent of the
+// largest number of a block
+HR_HD inline fx fx_from_double(double x, int E)
+{
+    const unsigned long long u = fx_dbits(x);
+    const int e = (int)(u >> 52) & 0x7ff;
+    const unsigned long long m = ((u & 0xfffffffffffffULL) | (e ? 0x10000000000000ULL : 0)) << 10;
+    const int s = E - (e ? e : 1) + 7;
+#ifdef __CUDA_ARCH__
+    unsigned long long t;
+    asm("shr.u64 %0, %1, %2;" : "=l"(t) : "l"(m), "r"(s));
+#else
+    const unsigned long long t = s > 63 ? 0 : m >> s;
+#endif
+    const long long sg = (long long)u >> 63;
+    return fx_split((long long)(t ^ (unsigned long long)sg) - sg);
+}
 // |x| as the high word of its bits, for range tests: below fx_high(2^k) = (1023 + k) << 20
 HR_HD inline unsigned fx_abs_high(double x) { return (unsigned)(fx_dbits(x) >> 32) & 0x7fffffffu; }
 constexpr unsigned kFxHigh1 = 0x3ff00000u, kFxHigh2 = 0x40000000u;
@@ -259,6 +276,33 @@ HR_HD inline void fxq_mac_scalar(fxa &s, const fxq &a, const fxq &b)
     fx_mac(s, fx_neg(a.c[2]), b.c[2]);
     fx_mac(s, fx_neg(a.c[3]), b.c[3]);
 }
+// s += k q or q k, k = (0, k1, k2, k3) a pure vector
+HR_HD inline void fxq_mac_pure_l(fxa (&s)[4], const fx (&k)[3], const fxq &q)
+{
+    const fx n0 = fx_neg(k[0]), n1 = fx_neg(k[1]), n2 = fx_neg(k[2]);
+    fx_mac(s[0], n0, q.c[1]); fx_mac(s[0], n1, q.c[2]); fx_mac(s[0], n2, q.c[3]);
+    fx_mac(s[1], k[0], q.c[0]); fx_mac(s[1], n1, q.c[3]); fx_mac(s[1], k[2], q.c[2]);
+    fx_mac(s[2], k[1], q.c[0]); fx_mac(s[2], n2, q.c[1]); fx_mac(s[2], k[0], q.c[3]);
+    fx_mac(s[3], k[2], q.c[0]); fx_mac(s[3], n0, q.c[2]); fx_mac(s[3], k[1], q.c[1]);
+}
+HR_HD inline void fxq_mac_pure_r(fxa (&s)[4], const fxq &q, const fx (&k)[3])
+{
+    const fx n0 = fx_neg(k[0]), n1 = fx_neg(k[1]), n2 = fx_neg(k[2]);
+    fx_mac(s[0], n0, q.c[1]); fx_mac(s[0], n1, q.c[2]); fx_mac(s[0], n2, q.c[3]);
+    fx_mac(s[1], k[0], q.c[0]); fx_mac(s[1], k[1], q.c[3]); fx_mac(s[1], n2, q.c[2]);
+    fx_mac(s[2], k[1], q.c[0]); fx_mac(s[2], k[2], q.c[1]); fx_mac(s[2], n0, q.c[3]);
+    fx_mac(s[3], k[2], q.c[0]); fx_mac(s[3], k[0], q.c[2]); fx_mac(s[3], n1, q.c[1]);
+}
+HR_HD inline void fxq_mac(fxa (&s)[4], const fxq &a, const fxq &b)
+{
+    fxa v[3] = {s[1], s[2], s[3]};
+    fxq_mac_scalar(s[0], a, b);
+    fxq_mac_vec(v, a, b);
+    s[1] = v[0];
+    s[2] = v[1];
+    s[3] = v[2];
+}
+HR_HD inline fxq fxq_of(const fxa (&s)[4]) { return {{fx_of(s[0]), fx_of(s[1]), fx_of(s[2]), fx_of(s[3])}}; }
 HR_HD inline fxq fxq_mul(const fxq &a, const fxq &b)
 {
     fxa s0 = {0, 0}, s[3] = {{0, 0}, {0, 0}, {0, 0}};

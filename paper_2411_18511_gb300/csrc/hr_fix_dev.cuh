@@ -55,4 +55,35 @@ template <bool VEC> __device__ __forceinline__ fxq load_fxq(const double *q, siz
     return r;
 }
 
+// the 16 reals of a packed FP64 spinor as digits, [2 (2 spin + colour) + (0 re, 1 im)],
+// in units of 2^(E - kFxPairBias); E = biased exponent of the largest |hi|.  false: out
+// of range (a nonzero spinor below 2^-105, Inf or NaN)
+__device__ __forceinline__ bool load_fx(const void *base, int j, fx (&v)[16], int &E)
+{
+    const float4 *p = (const float4 *)base;
+    float4 w[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w[k] = __ldg(p + vec_index(j, k, 8));
+    unsigned m = 0;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const float4 h = w[2 * s];
+        m = max(max(m, max(__float_as_uint(h.x) & 0x7fffffffu, __float_as_uint(h.y) & 0x7fffffffu)),
+                max(__float_as_uint(h.z) & 0x7fffffffu, __float_as_uint(h.w) & 0x7fffffffu));
+    }
+    E = (int)(m >> 23);
+    const bool ok = m == 0 || (E >= kFxMinExp && E < 255);
+    E = ok ? max(E, kFxMinExp) : 127;
+    const float sc = fx_pair_scale(E);
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const float4 h = w[2 * s], l = w[2 * s + 1];
+        v[4 * s + 0] = fx_from_pair(h.x, l.x, sc);
+        v[4 * s + 1] = fx_from_pair(h.z, l.z, sc);
+        v[4 * s + 2] = fx_from_pair(h.y, l.y, sc);
+        v[4 * s + 3] = fx_from_pair(h.w, l.w, sc);
+    }
+    return ok;
+}
+
 } // namespace hr

@@ -29,7 +29,7 @@
 // range (link_terms).
 #include <cmath>
 
-#include "hr_fix.cuh"
+#include "hr_fix_dev.cuh"
 #include "hr_host.h"
 
 using namespace hr;
@@ -166,37 +166,6 @@ __device__ __noinline__ void link_terms_native(const ForceArgs &A, int p, int i,
     link_terms<MU>(A, p, i, ifw, lex, sg, false);
 }
 
-// the 16 reals of a packed FP64 spinor as digits, [2 (2 spin + colour) + (0 re, 1 im)],
-// in units of 2^(E - kFxPairBias); E = biased exponent of the largest |hi|.  false: out
-// of range (a nonzero spinor below 2^-105, Inf or NaN)
-__device__ __forceinline__ bool load_fx(const void *base, int j, fx (&v)[16], int &E)
-{
-    const float4 *p = (const float4 *)base;
-    float4 w[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) w[k] = __ldg(p + vec_index(j, k, 8));
-    unsigned m = 0;
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const float4 h = w[2 * s];
-        m = max(max(m, max(__float_as_uint(h.x) & 0x7fffffffu, __float_as_uint(h.y) & 0x7fffffffu)),
-                max(__float_as_uint(h.z) & 0x7fffffffu, __float_as_uint(h.w) & 0x7fffffffu));
-    }
-    E = (int)(m >> 23);
-    const bool ok = m == 0 || (E >= kFxMinExp && E < 255);
-    E = ok ? max(E, kFxMinExp) : 127;
-    const float sc = fx_pair_scale(E);
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const float4 h = w[2 * s], l = w[2 * s + 1];
-        v[4 * s + 0] = fx_from_pair(h.x, l.x, sc);
-        v[4 * s + 1] = fx_from_pair(h.z, l.z, sc);
-        v[4 * s + 2] = fx_from_pair(h.y, l.y, sc);
-        v[4 * s + 3] = fx_from_pair(h.w, l.w, sc);
-    }
-    return ok;
-}
-
 // h[t][c] = s_t + sgn i^c s_pi of (1 - g_mu) (sgn = 1) or (1 + g_mu) (sgn = -1):
 // mu = 0: (0, 2) -1, (1, 3) -1;  1: (0, 3) i, (1, 2) i;  2: (0, 3) 1, (1, 2) -1;  3: (0, 2) i, (1, 3) -i
 __device__ __forceinline__ void project_fx(int mu, bool minus, const fx (&s)[16], fx (&h)[8])
@@ -244,14 +213,15 @@ template <bool DAG> __device__ __forceinline__ void mac_links(fxa (&g)[4], const
 // Measured: hr_fermion_force at 32^4 (four hops and this kernel) 4.39 ms with the
 // native kernel, of it 3.97 ms in the kernel (bound by the FP64 pipe: about 700
 // conversions and 1400 operations a site), 0.905 ms with this one; error
-// against a 64-bit evaluation 7.2e-15 with both (the hops').
+// against a 64-bit evaluation 7.2e-15 with both (the hops').  The kernel alone:
+// 0.479 ms at the compiler's 216 registers, 0.399 at 168, 0.438 at 128 (spills).
 // One thread per site in lexicographic order (so that a warp's outputs are
 // contiguous), a run-time loop over the four directions around one copy of the
 // conversion and product code: unrolled, the kernel would not fit the
 // instruction cache.  Ranges: |h| <= 2^27 per component, 2^28 projected, 8 terms
 // of 2^56 per sum.  Each of the two terms of a link is brought to 56 bits below
 // its own largest component and the two are aligned before they are added.
-template <int MODE> __global__ void __launch_bounds__(128) k_link_deriv_fx(ForceArgs A)
+template <int MODE> __global__ void __launch_bounds__(128, 3) k_link_deriv_fx(ForceArgs A)
 {
     const Geom &g = A.g;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;

@@ -113,3 +113,30 @@ def test_clover_build(dims, m0, csw, kind, prec):
             cond = np.linalg.cond(A).max() if inverse else 1.0
             assert np.abs(got - want).max() <= tol * size * cond
     ctx.close()
+
+
+@pytest.mark.parametrize("links", ["unit", "mixed"])
+@pytest.mark.parametrize("kind", ["gauss", "range", "zeros"])
+@pytest.mark.parametrize("dims", DIMS)
+def test_clover_insertion_force(dims, kind, links):
+    """Insertions of very different magnitude from site to site: each link within
+    the rounding of the corners of its own plaquettes."""
+    ctx = hr.Context(0)
+    V = int(np.prod(dims))
+    q = _links(dims, links, 88)
+    rng = np.random.default_rng(89)
+    lam = rng.normal(size=(V, 8, 8)) + 1j * rng.normal(size=(V, 8, 8))
+    if kind == "range":
+        lam *= (2.0 ** rng.integers(-40, 41, V))[:, None, None]
+    elif kind == "zeros":
+        lam[rng.random(V) < 0.7] = 0.0
+    F = torch.zeros((4, V, 3), dtype=torch.float64, device="cuda")
+    work = fields.empty_bytes(hr.hr_clover_force_workspace_bytes(dims))
+    hr.hr_clover_insertion_force(ctx, dims, 1.3, _dev(q), torch.tensor(lam, device="cuda"), 0.7, F, work)
+    want = 0.91 * ocl.clover_derivative(dims, oracle.expand_links(dims, 2, q), lam)
+    n = np.linalg.norm(lam, axis=(1, 2)).reshape(dims)
+    for rho in range(4):
+        near = sum(np.roll(m, s, sig) for m in (n, np.roll(n, -1, rho)) for sig in range(4) for s in (-1, 0, 1))
+        # about 150 products per plaquette of unit links (1.25^4 with the mixed ones)
+        assert np.all(np.abs(F[rho].cpu().numpy() - want[rho]) <= 2.0 ** -45 * near.reshape(V, 1) + 1e-300)
+    ctx.close()
