@@ -171,10 +171,9 @@ __device__ __forceinline__ void x2t_term(const HopArgs &a, const K2 &k, int site
     float4 w[8];
 #pragma unroll
     for (int v = 0; v < 8; ++v) w[v] = __ldg(sp + vec_index(j_nb, v, 8));
-    const size_t slot = (size_t)(link_par * 4 + MU) * a.g.nblk_g + (site_link >> 5);
-    const float4 *qp = (const float4 *)a.gauge;
-    const float4 qh = __ldg(qp + (slot * 2 + 0) * 32 + (site_link & 31));
-    const float4 ql = __ldg(qp + (slot * 2 + 1) * 32 + (site_link & 31));
+    const float4 *qp = link_base<float4>(a.gauge, a.g.nblk_g, link_par, MU, 2);
+    const float4 qh = __ldg(qp + vec_index(site_link, 0, 2));
+    const float4 ql = __ldg(qp + vec_index(site_link, 1, 2));
     cdd2 sv[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {

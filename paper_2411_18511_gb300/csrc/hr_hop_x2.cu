@@ -561,8 +561,7 @@ __device__ __forceinline__ void x2a_link(const HopArgs &a, const K2 &k, int link
                                          dd (&R)[3][3])
 {
     if constexpr (REP == kRepAdj) {
-        const size_t slot = (size_t)(link_par * 4 + mu) * a.g.nblk_g + (site_link >> 5);
-        const float4 *q = (const float4 *)a.gauge + slot * 64 + (site_link & 31);
+        const float4 *q = link_base<float4>(a.gauge, a.g.nblk_g, link_par, mu, 2) + vec_index(site_link, 0, 2);
         quat_to_adj_x2(k, __ldg(q), __ldg(q + 32), R);
     } else {
         load_mat<kF64>(a.gauge, a.g.nblk_g, link_par, mu, site_link, R);
