@@ -4,12 +4,12 @@
 // overheads dominate there (Sec. 3); on one GB300 a small lattice leaves most
 // of the 152 SMs idle and a solve is bound by launch latency.  This solver runs
 // every lattice of a batch inside the same launches: each CG phase (the four
-// hops of Mhat^+ Mhat, the x/r update, the p update) is one persistent launch
-// whose blocks walk a work list of (lattice, 128-site tile) entries.  Each
-// lattice keeps its own device scalars (alpha, beta, |r|^2, convergence flag);
-// reductions finish per lattice in its last tile (deterministic tile order);
-// converged lattices drop out of the work.  The iteration loop runs on the
-// device as one CUDA graph: a conditional WHILE node over passes of 8
+// hops of Mhat^+ Mhat, the last with the x/r update, and the p update) is one
+// launch with a block per (lattice, 128-site tile).  Each lattice keeps its own
+// device scalars (alpha, beta, |r|^2, convergence flag); a reducing phase leaves
+// one sum per tile, which a launch of one block per lattice adds in a fixed
+// order; converged lattices drop out of the work.  The iteration loop runs on
+// the device as one CUDA graph: a conditional WHILE node over passes of 8
 // iterations, its condition set from the lattices' done flags.
 #include <cmath>
 #include <cstring>
@@ -23,7 +23,7 @@ namespace {
 
 constexpr int kTile = 128; // sites per tile = threads per block
 constexpr int kMaxLattices = 64;
-constexpr int kBatchCounters = 4;
+constexpr int kFinThreads = 256;
 
 struct BatchLat {
     Geom g;
@@ -32,7 +32,6 @@ struct BatchLat {
     void *x, *r, *p, *q, *u, *t;
     double *scal;       // S_NSLOTS x kMaxRhsSlots doubles
     double *partials;   // one per tile
-    unsigned *counters; // kBatchCounters
     int tile0, ntiles;
     coef2 A, negc;      // 4 + m0 and -1/(4(4+m0))
 };
@@ -46,149 +45,117 @@ struct BatchArgs {
     float unit, nil; // 1 and 0 at run time (the paired arithmetic's multipliers)
 };
 
+// the lattice of a tile: a warp compares all (at most 64) first tiles at once
 __device__ __forceinline__ int find_lat(const BatchLat *L, int n, int tile)
 {
-    int l = 0;
-    while (l + 1 < n && tile >= L[l + 1].tile0) ++l;
-    return l;
+    static_assert(kMaxLattices <= 64, "two lattices a lane");
+    const int a = threadIdx.x & 31, b = a + 32;
+    const unsigned m0 = __ballot_sync(0xffffffffu, a < n && L[a].tile0 <= tile);
+    const unsigned m1 = n > 32 ? __ballot_sync(0xffffffffu, b < n && L[b].tile0 <= tile) : 0u;
+    return __popc(m0) + __popc(m1) - 1;
 }
 
-// Block sum of v; the last tile of the lattice adds the tile partials in order
-// and runs the scalar update `fin` (and `fin2` after it, if nonzero).
-__device__ void tile_reduce(double v, const BatchLat &L, int tile, int counter, int fin, int fin2)
+// the tile's sum (a block's threads are one tile)
+template <class V> __device__ __forceinline__ void tile_partial(const V &red, const BatchLat &L, int tile)
 {
-    __shared__ double wsum[kTile]; // >= 32 per warp for sum_partials
-    __shared__ bool last;
-    __shared__ double sums[32];
-    v = warp_sum_strided(v, 1);
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = v;
+    __shared__ double w[kTile / 32];
+    const double v = warp_total(red, 1);
+    if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
         double s = 0;
-        for (int w = 0; w < kTile / 32; ++w) s += wsum[w];
+        for (int k = 0; k < kTile / 32; ++k) s += w[k];
         L.partials[tile - L.tile0] = s;
-        __threadfence();
-        unsigned prev = atomicAdd(L.counters + counter, 1u);
-        last = (prev == (unsigned)L.ntiles - 1);
     }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    sum_partials(L.partials, (unsigned)L.ntiles, 1, sums, wsum);
-    if (threadIdx.x == 0) L.counters[counter] = 0u;
-    finish_reduction(fin, sums, 1, L.scal);
+}
+
+// One block per lattice adds its tiles' sums and runs the scalar update `fin`
+// (and `fin2` after it, if nonzero).
+__global__ void __launch_bounds__(kFinThreads) k_batch_finish(BatchArgs B, int fin, int fin2)
+{
+    __shared__ double sums[kFinThreads];
+    const BatchLat &L = B.lat[blockIdx.x];
+    if (!B.ignore_done && sc(L.scal, S_FLAGS, F_DONE) != 0.0) return;
+    const FinIn in = load_fin(L.scal, 1);
+    sum_partials(L.partials, L.ntiles, 1, sums);
+    finish_reduction(fin, sums, 1, L.scal, in);
     if (fin2) {
         __syncthreads();
-        finish_reduction(fin2, sums, 1, L.scal);
+        finish_reduction(fin2, sums, 1, L.scal, load_fin(L.scal, 1));
     }
-    __syncthreads();
 }
 
 // PHASE 0: t = H_oe v            1: u = A v - c H_eo t, |u|^2 -> alpha
 //       2: t = H_oe g5 u         3: q = A u - c g5 H_eo t        (v = p, or x)
+// In the recurrence phase 3 updates x += alpha p, r -= alpha q with q in
+// registers and reduces |r|^2: a separate pass took 95 us for the 530 k sites of
+// twelve lattices (8^4 .. 24^4).
 template <int REP, int PHASE>
 __global__ void __launch_bounds__(kTile) k_batch_hop(BatchArgs B)
 {
     using T = dd;
-    for (int tile = blockIdx.x; tile < B.total_tiles; tile += gridDim.x) {
-        const int l = find_lat(B.lat, B.nlat, tile);
-        const BatchLat &L = B.lat[l];
-        if (!B.ignore_done && sc(L.scal, S_FLAGS, F_DONE) != 0.0) continue;
-        const void *v = B.use_x ? (const void *)L.x : (const void *)L.p;
-        HopArgs a{};
-        a.g = L.g;
-        a.gauge = L.gauge;
-        a.red = RedSlot{nullptr, nullptr};
-        a.scal = L.scal;
-        a.fin = (PHASE == 1) ? kFinAlpha : kFinNone;
-        coef2 zero = {0.f, 0.f}, one = {1.f, 0.f};
-        if (PHASE == 0) { a.p = 1; a.in = v; a.out = L.t; a.alpha = zero; a.beta = one; a.beta_pow2 = 1; }
-        if (PHASE == 1) { a.p = 0; a.in = L.t; a.aux = v; a.out = L.u; a.alpha = L.A; a.beta = L.negc; }
-        if (PHASE == 2) { a.p = 1; a.in = L.u; a.out = L.t; a.alpha = zero; a.beta = one; a.beta_pow2 = 1; a.g5_in = 1; }
-        if (PHASE == 3) { a.p = 0; a.in = L.t; a.aux = L.u; a.out = L.q; a.alpha = L.A; a.beta = L.negc; a.g5_out = 1; }
-        const T be = Real<T>::from_coef(a.beta);
-        const T bu = a.g5_out ? -be : be;
-        const T al = Real<T>::from_coef(a.alpha);
-        SqAcc<T> red;
-        const int j = (tile - L.tile0) * kTile + threadIdx.x;
-        if (j < L.g.vh) {
-            if constexpr (REP == kRepFund) {
-                // the paired (f32x2) double-float arithmetic of the single-lattice
-                // hop: the same sums in the same order, half the instructions
-                constexpr bool NEG = PHASE == 2;
-                const K2 k = make_k2(B.unit, B.nil);
-                SiteNb nb;
-                site_neighbours(a.g, j, a.p, nb);
-                cdd2 acc[4];
-                x2_dir<0, true, NEG>(a, k, j, 0, nb, acc);
-                x2_dir<1, false, NEG>(a, k, j, 0, nb, acc);
-                x2_dir<2, false, NEG>(a, k, j, 0, nb, acc);
-                x2_dir<3, false, NEG>(a, k, j, 0, nb, acc);
-                x2_epilogue(a, j, acc, al, be, bu, red);
-            } else {
-                hop_site<REP, kF64>(a, j, al, be, bu, red);
-            }
+    const int tile = blockIdx.x;
+    const BatchLat &L = B.lat[find_lat(B.lat, B.nlat, tile)];
+    if (!B.ignore_done && sc(L.scal, S_FLAGS, F_DONE) != 0.0) return;
+    const bool fused = PHASE == 3 && !B.use_x;
+    const void *v = B.use_x ? (const void *)L.x : (const void *)L.p;
+    HopArgs a{};
+    a.g = L.g;
+    a.gauge = L.gauge;
+    a.scal = L.scal;
+    a.fin = (PHASE == 1) ? kFinAlpha : kFinNone;
+    coef2 zero = {0.f, 0.f}, one = {1.f, 0.f};
+    if (PHASE == 0) { a.p = 1; a.in = v; a.out = L.t; a.alpha = zero; a.beta = one; a.beta_pow2 = 1; }
+    if (PHASE == 1) { a.p = 0; a.in = L.t; a.aux = v; a.out = L.u; a.alpha = L.A; a.beta = L.negc; }
+    if (PHASE == 2) { a.p = 1; a.in = L.u; a.out = L.t; a.alpha = zero; a.beta = one; a.beta_pow2 = 1; a.g5_in = 1; }
+    if (PHASE == 3) { a.p = 0; a.in = L.t; a.aux = L.u; a.out = L.q; a.alpha = L.A; a.beta = L.negc; a.g5_out = 1; }
+    if (fused) { a.cg_x = L.x; a.cg_p = L.p; a.cg_r = L.r; }
+    const T be = Real<T>::from_coef(a.beta);
+    const T bu = a.g5_out ? -be : be;
+    const T al = Real<T>::from_coef(a.alpha);
+    SqAcc<T> red;
+    const int j = (tile - L.tile0) * kTile + threadIdx.x;
+    if (j < L.g.vh) {
+        if constexpr (REP == kRepFund) {
+            // the paired (f32x2) double-float arithmetic of the single-lattice
+            // hop: the same sums in the same order, half the instructions
+            constexpr bool NEG = PHASE == 2;
+            const K2 k = make_k2(B.unit, B.nil);
+            SiteNb nb;
+            site_neighbours(a.g, j, a.p, nb);
+            epilogue_prefetch<2, kF64>(a, j);
+            cdd2 acc[4];
+            x2_dir<0, true, NEG>(a, k, j, 0, nb, acc);
+            x2_dir<1, false, NEG>(a, k, j, 0, nb, acc);
+            x2_dir<2, false, NEG>(a, k, j, 0, nb, acc);
+            x2_dir<3, false, NEG>(a, k, j, 0, nb, acc);
+            x2_epilogue(a, j, acc, al, be, bu, red);
+        } else {
+            hop_site<REP, kF64>(a, j, al, be, bu, red);
         }
-        if (PHASE == 1) tile_reduce(red.get(), L, tile, 0, kFinAlpha, 0);
     }
-}
-
-template <int NC>
-__global__ void __launch_bounds__(kTile) k_batch_xr(BatchArgs B)
-{
-    using T = dd;
-    for (int tile = blockIdx.x; tile < B.total_tiles; tile += gridDim.x) {
-        const int l = find_lat(B.lat, B.nlat, tile);
-        const BatchLat &L = B.lat[l];
-        if (sc(L.scal, S_FLAGS, F_DONE) != 0.0) continue;
-        const T al = Real<T>::from_double(sc(L.scal, S_ALPHA, 0));
-        SqAcc<T> red;
-        const int j = (tile - L.tile0) * kTile + threadIdx.x;
-        if (j < L.g.vh) {
-            cpx<T> xv[4][NC], pv[4][NC], rv[4][NC], qv[4][NC];
-            load_spinor<NC, kF64>(L.x, L.g.nblk_s, j, xv);
-            load_spinor<NC, kF64>(L.p, L.g.nblk_s, j, pv);
-            load_spinor<NC, kF64>(L.r, L.g.nblk_s, j, rv);
-            load_spinor<NC, kF64>(L.q, L.g.nblk_s, j, qv);
-#pragma unroll
-            for (int s = 0; s < 4; ++s)
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    xv[s][c].re += al * pv[s][c].re;
-                    xv[s][c].im += al * pv[s][c].im;
-                    rv[s][c].re -= al * qv[s][c].re;
-                    rv[s][c].im -= al * qv[s][c].im;
-                    red.add(rv[s][c].re);
-                    red.add(rv[s][c].im);
-                }
-            store_spinor<NC, kF64>(L.x, L.g.nblk_s, j, xv);
-            store_spinor<NC, kF64>(L.r, L.g.nblk_s, j, rv);
-        }
-        tile_reduce(red.get(), L, tile, 1, kFinBeta, 0);
-    }
+    if (PHASE == 1 || fused) tile_partial(red, L, tile);
 }
 
 template <int NC>
 __global__ void __launch_bounds__(kTile) k_batch_p(BatchArgs B)
 {
     using T = dd;
-    for (int tile = blockIdx.x; tile < B.total_tiles; tile += gridDim.x) {
-        const int l = find_lat(B.lat, B.nlat, tile);
-        const BatchLat &L = B.lat[l];
-        if (sc(L.scal, S_FLAGS, F_DONE) != 0.0) continue;
-        const T be = Real<T>::from_double(sc(L.scal, S_BETA, 0));
-        const int j = (tile - L.tile0) * kTile + threadIdx.x;
-        if (j < L.g.vh) {
-            cpx<T> pv[4][NC], rv[4][NC];
-            load_spinor<NC, kF64>(L.p, L.g.nblk_s, j, pv);
-            load_spinor<NC, kF64>(L.r, L.g.nblk_s, j, rv);
+    const int tile = blockIdx.x;
+    const BatchLat &L = B.lat[find_lat(B.lat, B.nlat, tile)];
+    if (sc(L.scal, S_FLAGS, F_DONE) != 0.0) return;
+    const T be = Real<T>::from_double(sc(L.scal, S_BETA, 0));
+    const int j = (tile - L.tile0) * kTile + threadIdx.x;
+    if (j < L.g.vh) {
+        cpx<T> pv[4][NC], rv[4][NC];
+        load_spinor<NC, kF64>(L.p, L.g.nblk_s, j, pv);
+        load_spinor<NC, kF64>(L.r, L.g.nblk_s, j, rv);
 #pragma unroll
-            for (int s = 0; s < 4; ++s)
+        for (int s = 0; s < 4; ++s)
 #pragma unroll
-                for (int c = 0; c < NC; ++c)
-                    pv[s][c] = {rv[s][c].re + be * pv[s][c].re, rv[s][c].im + be * pv[s][c].im};
-            store_spinor<NC, kF64>(L.p, L.g.nblk_s, j, pv);
-        }
+            for (int c = 0; c < NC; ++c)
+                pv[s][c] = {rv[s][c].re + be * pv[s][c].re, rv[s][c].im + be * pv[s][c].im};
+        store_spinor<NC, kF64>(L.p, L.g.nblk_s, j, pv);
     }
 }
 
@@ -197,28 +164,26 @@ template <int NC>
 __global__ void __launch_bounds__(kTile) k_batch_start(BatchArgs B)
 {
     using T = dd;
-    for (int tile = blockIdx.x; tile < B.total_tiles; tile += gridDim.x) {
-        const int l = find_lat(B.lat, B.nlat, tile);
-        const BatchLat &L = B.lat[l];
-        SqAcc<T> red;
-        const int j = (tile - L.tile0) * kTile + threadIdx.x;
-        if (j < L.g.vh) {
-            cpx<T> bv[4][NC], z[4][NC];
-            load_spinor<NC, kF64>(L.b, L.g.nblk_s, j, bv);
+    const int tile = blockIdx.x;
+    const BatchLat &L = B.lat[find_lat(B.lat, B.nlat, tile)];
+    SqAcc<T> red;
+    const int j = (tile - L.tile0) * kTile + threadIdx.x;
+    if (j < L.g.vh) {
+        cpx<T> bv[4][NC], z[4][NC];
+        load_spinor<NC, kF64>(L.b, L.g.nblk_s, j, bv);
 #pragma unroll
-            for (int s = 0; s < 4; ++s)
+        for (int s = 0; s < 4; ++s)
 #pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    z[s][c] = {T(0.f), T(0.f)};
-                    red.add(bv[s][c].re);
-                    red.add(bv[s][c].im);
-                }
-            store_spinor<NC, kF64>(L.x, L.g.nblk_s, j, z);
-            store_spinor<NC, kF64>(L.r, L.g.nblk_s, j, bv);
-            store_spinor<NC, kF64>(L.p, L.g.nblk_s, j, bv);
-        }
-        tile_reduce(red.get(), L, tile, 2, kFinBB, kFinInit);
+            for (int c = 0; c < NC; ++c) {
+                z[s][c] = {T(0.f), T(0.f)};
+                red.add(bv[s][c].re);
+                red.add(bv[s][c].im);
+            }
+        store_spinor<NC, kF64>(L.x, L.g.nblk_s, j, z);
+        store_spinor<NC, kF64>(L.r, L.g.nblk_s, j, bv);
+        store_spinor<NC, kF64>(L.p, L.g.nblk_s, j, bv);
     }
+    tile_partial(red, L, tile);
 }
 
 // r = b - q (q = A x), |r|^2 -> S_OUT
@@ -226,26 +191,24 @@ template <int NC>
 __global__ void __launch_bounds__(kTile) k_batch_residual(BatchArgs B)
 {
     using T = dd;
-    for (int tile = blockIdx.x; tile < B.total_tiles; tile += gridDim.x) {
-        const int l = find_lat(B.lat, B.nlat, tile);
-        const BatchLat &L = B.lat[l];
-        SqAcc<T> red;
-        const int j = (tile - L.tile0) * kTile + threadIdx.x;
-        if (j < L.g.vh) {
-            cpx<T> bv[4][NC], qv[4][NC];
-            load_spinor<NC, kF64>(L.b, L.g.nblk_s, j, bv);
-            load_spinor<NC, kF64>(L.q, L.g.nblk_s, j, qv);
+    const int tile = blockIdx.x;
+    const BatchLat &L = B.lat[find_lat(B.lat, B.nlat, tile)];
+    SqAcc<T> red;
+    const int j = (tile - L.tile0) * kTile + threadIdx.x;
+    if (j < L.g.vh) {
+        cpx<T> bv[4][NC], qv[4][NC];
+        load_spinor<NC, kF64>(L.b, L.g.nblk_s, j, bv);
+        load_spinor<NC, kF64>(L.q, L.g.nblk_s, j, qv);
 #pragma unroll
-            for (int s = 0; s < 4; ++s)
+        for (int s = 0; s < 4; ++s)
 #pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    cpx<T> d = csub(bv[s][c], qv[s][c]);
-                    red.add(d.re);
-                    red.add(d.im);
-                }
-        }
-        tile_reduce(red.get(), L, tile, 3, kFinStore, 0);
+            for (int c = 0; c < NC; ++c) {
+                cpx<T> d = csub(bv[s][c], qv[s][c]);
+                red.add(d.re);
+                red.add(d.im);
+            }
     }
+    tile_partial(red, L, tile);
 }
 
 struct GraphExec {
@@ -260,7 +223,7 @@ struct GraphExec {
 
 struct BatchPlan {
     size_t bytes = 0;
-    std::vector<size_t> vec_off, scal_off, part_off, cnt_off;
+    std::vector<size_t> vec_off, scal_off, part_off;
     size_t desc_off = 0;
     std::vector<Geom> geoms;
     int total_tiles = 0;
@@ -284,7 +247,6 @@ BatchPlan plan_batch(int n, const hr_lattice *lats, int rep)
         P.scal_off.push_back(take(sizeof(double) * S_NSLOTS * kMaxRhsSlots));
         int nt = (g.vh + kTile - 1) / kTile;
         P.part_off.push_back(take(sizeof(double) * nt));
-        P.cnt_off.push_back(take(sizeof(unsigned) * kBatchCounters));
         P.total_tiles += nt;
     }
     P.bytes = off;
@@ -297,9 +259,10 @@ hr_status batch_launch_iteration(hr_ctx *ctx, const BatchArgs &B, int grid, cuda
     constexpr int NC = RepTraits<REP>::NC;
     k_batch_hop<REP, 0><<<grid, kTile, 0, s>>>(B);
     k_batch_hop<REP, 1><<<grid, kTile, 0, s>>>(B);
+    k_batch_finish<<<B.nlat, kFinThreads, 0, s>>>(B, kFinAlpha, 0);
     k_batch_hop<REP, 2><<<grid, kTile, 0, s>>>(B);
     k_batch_hop<REP, 3><<<grid, kTile, 0, s>>>(B);
-    k_batch_xr<NC><<<grid, kTile, 0, s>>>(B);
+    k_batch_finish<<<B.nlat, kFinThreads, 0, s>>>(B, kFinBeta, 0);
     k_batch_p<NC><<<grid, kTile, 0, s>>>(B);
     return check_launch(ctx, "batched CG iteration");
 }
@@ -380,6 +343,7 @@ hr_status batch_true_residual(hr_ctx *ctx, BatchArgs B, int grid, cudaStream_t s
     k_batch_hop<REP, 2><<<grid, kTile, 0, s>>>(B);
     k_batch_hop<REP, 3><<<grid, kTile, 0, s>>>(B);
     k_batch_residual<NC><<<grid, kTile, 0, s>>>(B);
+    k_batch_finish<<<B.nlat, kFinThreads, 0, s>>>(B, kFinStore, 0);
     return check_launch(ctx, "batched true residual");
 }
 
@@ -452,14 +416,12 @@ hr_status hr_cg_solve_batch(hr_ctx *ctx, int n_lat, const hr_lattice *lats, doub
         L.t = v + 4 * h;
         L.scal = (double *)(w + P.scal_off[l]);
         L.partials = (double *)(w + P.part_off[l]);
-        L.counters = (unsigned *)(w + P.cnt_off[l]);
         L.ntiles = (L.g.vh + kTile - 1) / kTile;
         L.tile0 = tile0;
         tile0 += L.ntiles;
         L.A = make_coef(A);
         L.negc = make_coef(-1.0 / (4.0 * A));
         if (e == cudaSuccess) e = cudaMemcpyAsync(L.scal, scal0.data(), sizeof(double) * scal0.size(), cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(L.counters, 0, sizeof(unsigned) * kBatchCounters, s);
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(w + P.desc_off, desc.data(), sizeof(BatchLat) * n_lat, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaEventRecord(ctx->ev0, s);
@@ -473,11 +435,11 @@ hr_status hr_cg_solve_batch(hr_ctx *ctx, int n_lat, const hr_lattice *lats, doub
     B.ignore_done = 0;
     B.unit = 1.f;
     B.nil = 0.f;
-    int grid = ctx->sm_count > 0 ? ctx->sm_count * 8 : 1024;
-    if (grid > P.total_tiles) grid = P.total_tiles;
+    const int grid = P.total_tiles; // one block per tile
 
     if (rep == HR_FUND) k_batch_start<2><<<grid, kTile, 0, s>>>(B);
     else k_batch_start<3><<<grid, kTile, 0, s>>>(B);
+    k_batch_finish<<<n_lat, kFinThreads, 0, s>>>(B, kFinBB, kFinInit);
     hr_status st = check_launch(ctx, "batch start");
     if (st) return st;
 

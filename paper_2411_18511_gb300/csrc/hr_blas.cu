@@ -9,8 +9,8 @@
 //   accum   : x_hi += x_lo, x_lo = 0              (mixed precision)
 //   convert : precision change between packed layouts
 // Per-RHS scalars (alpha, beta, ...) are read from the context's device scalar
-// block, so a solver iteration needs no host round trip.  Reductions are FP64,
-// deterministic (warp shuffle, block, then last-block sum in block order).
+// block, so a solver iteration needs no host round trip.  Reductions are FP64 and
+// deterministic: warp shuffle, a row of sums per block, then k_finish in a fixed order.
 #include <vector>
 
 #include "hr_host.h"
@@ -44,7 +44,7 @@ __device__ __forceinline__ void acc_site(SqAcc<T> &acc, const cpx<T> (&v)[4][NC]
 __device__ __forceinline__ int thread_rhs(const Geom &g) { return (blockIdx.x * blockDim.x + threadIdx.x) & (g.nrhs - 1); }
 
 template <int NC, int P>
-__global__ void __launch_bounds__(kBS) k_norm2(Geom g, const void *v, RedSlot red, double *scal, int fin)
+__global__ void __launch_bounds__(kBS) k_norm2(Geom g, const void *v, double *partials)
 {
     using T = RT<P>;
     const int nv = g.vh << g.lrhs;
@@ -54,9 +54,47 @@ __global__ void __launch_bounds__(kBS) k_norm2(Geom g, const void *v, RedSlot re
         load_spinor<NC, P>(v, g.nblk_s, j, a);
         acc_site<NC>(acc, a);
     }
-    __shared__ double smem[32 * 32];
-    __shared__ double sums[32];
-    if (grid_reduce(acc, g.nrhs, red, sums, smem)) finish_reduction(fin, sums, g.nrhs, scal);
+    block_partials(acc, g.nrhs, partials);
+}
+
+// The finishing launch of a reduction: adds `nparts` rows of nrhs partial sums and
+// runs the scalar update on the result.  Latency bound (a trip to L2 for the
+// scalars and the rows, the sum's tree, the update).  One block adds up to 2048
+// sums; beyond that the rows are split over blocks, whose own sums the last of
+// them adds: 2048 additions take the FP64 pipe about as long as that second
+// stage's two round trips.  The order depends on nparts and nrhs only.
+constexpr int kFinThreads = 256, kFinPerBlock = 2048;
+__global__ void __launch_bounds__(kFinThreads) k_finish(const double *partials, int nparts, int nrhs, int rows,
+                                                        double *block_sums, unsigned *counter, double *scal, int fin,
+                                                        const double *gate, const double *done, FinCond cond)
+{
+    __shared__ double sums[kFinThreads];
+    if ((gate && *gate == 0.0) || (done && *done != 0.0)) {
+        // the update may be due from an earlier iteration of the pass
+        if (cond.set && blockIdx.x == 0 && threadIdx.x == 0)
+            cudaGraphSetConditional(cond.handle,
+                                    sc(scal, S_FLAGS, F_GATE) != 0.0 && sc(scal, S_FLAGS, F_DONE) == 0.0 ? 1u : 0u);
+        return;
+    }
+    const FinIn in = load_fin(scal, nrhs);
+    const int first = blockIdx.x * rows;
+    sum_partials(partials + (size_t)first * nrhs, min(rows, nparts - first), nrhs, sums);
+    if (gridDim.x > 1) {
+        __shared__ bool last;
+        if (threadIdx.x < nrhs) {
+            block_sums[blockIdx.x * nrhs + threadIdx.x] = sums[threadIdx.x];
+            __threadfence();
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        sum_partials(block_sums, gridDim.x, nrhs, sums);
+        if (threadIdx.x == 0) *counter = 0u;
+    }
+    const bool update = finish_reduction(fin, sums, nrhs, scal, in);
+    if (cond.set && threadIdx.x == 0) cudaGraphSetConditional(cond.handle, update ? 1u : 0u);
 }
 
 // p = r + beta p
@@ -64,7 +102,7 @@ template <int NC, int PP, int PR>
 __global__ void __launch_bounds__(kBS) k_p(Geom g, void *p, const void *r, const double *scal)
 {
     using T = typename Wider<RT<PP>, RT<PR>>::T;
-    if (sc((double *)scal, S_FLAGS, F_DONE) != 0.0) return;
+    if (sc((double *)scal, S_FLAGS, F_SKIP) != 0.0) return;
     const int nv = g.vh << g.lrhs;
     const T be = Real<T>::from_double(scal[S_BETA * kMaxRhsSlots + thread_rhs(g)]);
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nv; j += gridDim.x * blockDim.x) {
@@ -96,8 +134,8 @@ __global__ void __launch_bounds__(kBS) k_convert(Geom g, const void *src, void *
 // r = b - ax in FP64 (b FP64, ax FP64 or FP32; r nullable: not stored), |r|^2 -> fin,
 // and r_lo = r in the inner precision PL
 template <int NC, int PL, int PA>
-__global__ void __launch_bounds__(kBS) k_residual(Geom g, const void *b, const void *ax, void *r, RedSlot red,
-                                                  double *scal, int fin, const double *gate, void *r_lo)
+__global__ void __launch_bounds__(kBS) k_residual(Geom g, const void *b, const void *ax, void *r, double *partials,
+                                                  const double *gate, void *r_lo)
 {
     using T = RT<kF64>;
     if (gate && *gate == 0.0) return;
@@ -115,9 +153,7 @@ __global__ void __launch_bounds__(kBS) k_residual(Geom g, const void *b, const v
         if (PL != kF64 && r_lo) store_spinor<NC, PL>(r_lo, g.nblk_s, j, bv);
         acc_site<NC>(acc, bv);
     }
-    __shared__ double smem[32 * 32];
-    __shared__ double sums[32];
-    if (grid_reduce(acc, g.nrhs, red, sums, smem)) finish_reduction(fin, sums, g.nrhs, scal);
+    block_partials(acc, g.nrhs, partials);
 }
 
 // x_hi += x_lo ; x_lo = 0  (x_hi FP64 or FP32)
@@ -310,12 +346,22 @@ inline int grid_cap(hr_ctx *ctx, const Geom &g)
 
 namespace hr {
 
+hr_status finish_sums(hr_ctx *ctx, int nparts, int nrhs, int fin, const double *gate, const double *done,
+                      cudaStream_t s, FinCond cond)
+{
+    const int want = grid_for((long long)nparts * nrhs, kFinPerBlock, kFinBlocks);
+    const int rows = (nparts + want - 1) / want, grid = (nparts + rows - 1) / rows;
+    k_finish<<<grid, kFinThreads, 0, s>>>(ctx->d_partials, nparts, nrhs, rows, ctx->d_partials + kMaxPartials,
+                                          ctx->d_counters + C_FIN, ctx->d_scal, fin, gate, done, cond);
+    return check_launch(ctx, "reduction finish");
+}
+
 hr_status blas_norm2(hr_ctx *ctx, const Geom &g, int rep, int prec, const void *v, int fin, cudaStream_t s)
 {
     int grid = grid_cap(ctx, g);
-    RedSlot red = red_slot(ctx, C_NORM);
-    HR_DISPATCH_NC(rep, HR_DISPATCH_P(prec, P, (k_norm2<NC, P><<<grid, kBS, 0, s>>>(g, v, red, ctx->d_scal, fin))));
-    return check_launch(ctx, "norm2");
+    HR_DISPATCH_NC(rep, HR_DISPATCH_P(prec, P, (k_norm2<NC, P><<<grid, kBS, 0, s>>>(g, v, ctx->d_partials))));
+    hr_status st = check_launch(ctx, "norm2");
+    return st ? st : finish_sums(ctx, grid, g.nrhs, fin, nullptr, nullptr, s);
 }
 
 hr_status blas_p(hr_ctx *ctx, const Geom &g, int rep, int pp, int pr, void *p, const void *r, cudaStream_t s)
@@ -344,16 +390,16 @@ hr_status blas_residual(hr_ctx *ctx, const Geom &g, int rep, const void *b, cons
                         const double *gate, int plo, void *r_lo, cudaStream_t s, int pax)
 {
     int grid = grid_cap(ctx, g);
-    RedSlot red = red_slot(ctx, C_RES);
     if (!r_lo) plo = kF64;
     if (pax == kF64) {
-        HR_DISPATCH_NC(rep, HR_DISPATCH_P(plo, P, (k_residual<NC, P, kF64><<<grid, kBS, 0, s>>>(g, b, ax, r, red, ctx->d_scal, fin, gate, r_lo))));
+        HR_DISPATCH_NC(rep, HR_DISPATCH_P(plo, P, (k_residual<NC, P, kF64><<<grid, kBS, 0, s>>>(g, b, ax, r, ctx->d_partials, gate, r_lo))));
     } else if (pax == kF32 && plo == kF16) {
-        HR_DISPATCH_NC(rep, (k_residual<NC, kF16, kF32><<<grid, kBS, 0, s>>>(g, b, ax, r, red, ctx->d_scal, fin, gate, r_lo)));
+        HR_DISPATCH_NC(rep, (k_residual<NC, kF16, kF32><<<grid, kBS, 0, s>>>(g, b, ax, r, ctx->d_partials, gate, r_lo)));
     } else {
         return set_error(ctx, HR_ERR_UNSUPPORTED, "residual precision combination");
     }
-    return check_launch(ctx, "residual");
+    hr_status st = check_launch(ctx, "residual");
+    return st ? st : finish_sums(ctx, grid, g.nrhs, fin, gate, nullptr, s);
 }
 
 hr_status blas_accum(hr_ctx *ctx, const Geom &g, int rep, int plo, void *xhi, void *xlo, const double *gate,

@@ -17,8 +17,8 @@
 //   target), a device-gated block adds the increment into the FP64 solution,
 //   recomputes r = b - A x in FP64 and restarts the low-precision residual from
 //   it, keeping the search direction.  Convergence is only declared on an FP64
-//   residual.  In the one-graph solve the update is a conditional IF node, so
-//   iterations without one launch nothing for it.
+//   residual.  In the one-graph solve the update is a conditional IF node after
+//   every few iterations, so iterations without one launch nothing for it.
 // * n_rhs independent right-hand sides run as one "virtual site" field: every
 //   link load serves all of them, and alpha, beta and convergence are per RHS.
 #include <cmath>
@@ -95,26 +95,23 @@ hr_status read_scalars(hr_ctx *ctx, int first, int n, cudaStream_t s)
 
 inline const double *flag_ptr(hr_ctx *ctx, int f) { return ctx->d_scal + S_FLAGS * kMaxRhsSlots + f; }
 
-enum CtlWhat { kCtlGate = 0, kCtlLoop = 1 };
-constexpr int kIterPerPass = 8; // iterations per pass of the device loop body
+// Iterations per pass of the device loop body, and per conditional reliable
+// update (IF node) within it.  A skipped IF costs about 9 us, a taken one and a
+// pass of the WHILE body 25 us, a launch that skips on its flag about 1.3 us: when
+// an update becomes due, the iterations before the next IF node skip (7 launches
+// each), 1.5 of them on average with an IF every 4.
+constexpr int kIterPerPass = 8, kIterPerUpdate = 4;
 
-// Device-side control of the solve graph.  kCtlGate: run the reliable update
-// (IF node) this iteration?  kCtlLoop: run another pass of the loop body (WHILE
-// node)?  The loop stops when the done flag is up (every RHS stopped, maxiter
-// reached or a NaN seen) and, as a backstop, after 2 maxiter + 64 passes.
-__global__ void k_cg_ctl(double *scal, cudaGraphConditionalHandle h, int what, int maxiter)
+// Device-side control of the solve graph: run another pass of the loop body
+// (WHILE node)?  The loop stops when the done flag is up (every RHS stopped,
+// maxiter reached or a NaN seen) and, as a backstop, after 2 maxiter + 64 passes.
+__global__ void k_cg_ctl(double *scal, cudaGraphConditionalHandle h, int maxiter)
 {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     double *f = scal + S_FLAGS * kMaxRhsSlots;
-    const bool done = f[F_DONE] != 0.0;
-    unsigned v;
-    if (what == kCtlGate) {
-        v = (!done && f[F_GATE] != 0.0) ? 1u : 0u;
-    } else {
-        f[F_BODY] += 1.0;
-        v = (!done && f[F_ITERS] < (double)maxiter && f[F_BODY] < 2.0 * maxiter + 64.0) ? 1u : 0u;
-    }
-    cudaGraphSetConditional(h, v);
+    f[F_BODY] += 1.0;
+    const bool more = f[F_DONE] == 0.0 && f[F_ITERS] < (double)maxiter && f[F_BODY] < 2.0 * maxiter + 64.0;
+    cudaGraphSetConditional(h, more ? 1u : 0u);
 }
 
 struct Solver {
@@ -196,19 +193,21 @@ struct Solver {
 
     // One iteration = part_a (q = A p with <p,q> -> alpha; x, r update with
     // |r|^2 -> beta), then for the mixed solver the reliable update, then
-    // part_b (p = r + beta p).
-    hr_status part_a()
+    // part_b (p = r + beta p).  Both parts skip when the solve is done or a
+    // reliable update is due; the update ends with part_b.  `cond`: the last
+    // reduction also sets the condition of the IF node that follows.
+    hr_status part_a(FinCond cond = {0, 0})
     {
-        const double *done = flag_ptr(ctx, F_DONE);
+        const double *done = flag_ptr(ctx, F_SKIP);
         if (!mixed()) {
             // q = A p with the x/r update and |r|^2 fused into the last hop
-            const CgFuse fz{x, p64, r64, kFinBeta};
+            const CgFuse fz{x, p64, r64, kFinBeta, cond};
             return apply_eo_op(ctx, g, m0, rep, kF64, HR_OP_NORMAL, gauge, p64, q64, t64, u64, kFinAlpha, nullptr,
                                done, s, &fz, clov64);
         }
         // p, r in the inner precision, x_lo in FP32: fused as above (the
         // last hop's epilogue updates x_lo and r from q in registers)
-        const CgFuse fz{x_lo, p_lo, r_lo, kFinBetaMixed};
+        const CgFuse fz{x_lo, p_lo, r_lo, kFinBetaMixed, cond};
         return apply_eo_op(ctx, g, m0, rep, o.inner_prec, HR_OP_NORMAL, gauge_lo, p_lo, q_lo, t_lo, u_lo, kFinAlpha,
                            nullptr, done, s, &fz, clov_lo);
     }
@@ -331,12 +330,10 @@ struct Solver {
 };
 
 // The whole solve loop as one graph: a WHILE node whose body is `per_pass`
-// iterations, with the reliable update of the mixed solver in an IF node per
-// iteration.  Kernels set every condition on the device (k_cg_ctl), so a solve
-// is one graph launch.  A pass of a WHILE body and a taken IF node each cost
-// about 25 us of scheduling on this hardware (a skipped IF about 9 us), so the
-// body holds several iterations; those after convergence skip their work on
-// the done flag.
+// iterations, with the reliable update of the mixed solver in an IF node after
+// every kIterPerUpdate of them (and after the last).  Kernels set every condition
+// on the device (k_finish, k_cg_ctl), so a solve is one graph launch; iterations
+// after convergence skip their work on the done flag.
 hr_status capture_while_graph(Solver &sv, int per_pass, cudaGraph_t *out)
 {
     hr_ctx *ctx = sv.ctx;
@@ -392,14 +389,18 @@ hr_status capture_while_graph(Solver &sv, int per_pass, cudaGraph_t *out)
     sv.s = cs;
     if (!begin(body, nullptr, 0)) return fail("begin capture");
     for (int k = 0; k < per_pass; ++k) {
-        if ((st = sv.part_a())) return fail("iteration");
-        if (sv.mixed()) {
-            // each IF node has its own condition handle
+        const bool update = sv.mixed() && ((k + 1) % kIterPerUpdate == 0 || k + 1 == per_pass);
+        // each IF node has its own condition handle
+        FinCond cond = {0, 0};
+        if (update) {
             cudaGraphConditionalHandle hgate;
             if ((e = cudaGraphConditionalHandleCreate(&hgate, body, 0, cudaGraphCondAssignDefault)) != cudaSuccess)
                 return fail("gate condition");
-            k_cg_ctl<<<1, 32, 0, cs>>>(ctx->d_scal, hgate, kCtlGate, maxiter);
-            if ((st = check_launch(ctx, "cg control"))) return fail("cg control");
+            cond = FinCond{1, hgate};
+        }
+        if ((st = sv.part_a(cond))) return fail("iteration");
+        if ((st = sv.part_b())) return fail("iteration");
+        if (update) {
             cudaStreamCaptureStatus cst;
             const cudaGraphNode_t *d = nullptr;
             size_t nd = 0;
@@ -409,16 +410,16 @@ hr_status capture_while_graph(Solver &sv, int per_pass, cudaGraph_t *out)
             if (!end()) return fail("end capture");
             cudaGraphNode_t inode;
             cudaGraph_t ifbody = nullptr;
-            if (!cond_node(body, hgate, cudaGraphCondTypeIf, deps.data(), deps.size(), &inode, &ifbody))
+            if (!cond_node(body, cond.handle, cudaGraphCondTypeIf, deps.data(), deps.size(), &inode, &ifbody))
                 return fail("if node");
             if (!begin(ifbody, nullptr, 0)) return fail("begin capture");
             if ((st = sv.reliable_update(nullptr))) return fail("reliable update");
+            if ((st = sv.part_b())) return fail("reliable update");
             if (!end()) return fail("end capture");
             if (!begin(body, &inode, 1)) return fail("begin capture");
         }
-        if ((st = sv.part_b())) return fail("iteration");
     }
-    k_cg_ctl<<<1, 32, 0, cs>>>(ctx->d_scal, hloop, kCtlLoop, maxiter);
+    k_cg_ctl<<<1, 32, 0, cs>>>(ctx->d_scal, hloop, maxiter);
     if ((st = check_launch(ctx, "cg control"))) return fail("cg control");
     if (!end()) return fail("end capture");
     cudaStreamDestroy(cs);

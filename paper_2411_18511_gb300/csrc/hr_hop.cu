@@ -45,11 +45,7 @@ __device__ __forceinline__ void hop_body(const HopArgs &a)
     SqAcc<T> red;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nv; j += stride)
         hop_site<REP, PREC, G5IN, CLOV>(a, j, al, be, bu, red);
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 // The unrolled kernel: registers as the compiler likes (about 100 for
@@ -94,12 +90,12 @@ template <int REP, int PREC> struct PlainLaunch {
         if (c.variant == kVarSimpleR96) {
             if (a.g5_in) k_hop_r96<REP, PREC, 1><<<grid, c.block, 0, s>>>(a);
             else k_hop_r96<REP, PREC, 0><<<grid, c.block, 0, s>>>(a);
-            st = check_launch(ctx, "hop kernel (96 registers)");
+            st = hop_launched(ctx, a, grid, s, "hop kernel (96 registers)");
             return true;
         }
         if (a.g5_in) k_hop<REP, PREC, 1><<<grid, c.block, 0, s>>>(a);
         else k_hop<REP, PREC, 0><<<grid, c.block, 0, s>>>(a);
-        st = check_launch(ctx, "hop kernel");
+        st = hop_launched(ctx, a, grid, s, "hop kernel");
         return true;
     }
 };
@@ -109,7 +105,7 @@ template <int REP, int PREC> struct ClovLaunch {
     {
         if (a.g5_in) k_hop_clov<REP, PREC, 1><<<grid, block, 0, s>>>(a);
         else k_hop_clov<REP, PREC, 0><<<grid, block, 0, s>>>(a);
-        st = check_launch(ctx, "hop kernel (clover epilogue)");
+        st = hop_launched(ctx, a, grid, s, "hop kernel (clover epilogue)");
         return true;
     }
 };
@@ -128,7 +124,7 @@ hr_status dispatch(hr_ctx *ctx, const Geom &g, int rep, int prec, const HopArgs 
         // the clover instantiations: paired staged for fundamental FP64, else unrolled
         const bool paired = rep == HR_FUND && prec == kF64;
         const int block = paired ? 256 : 128;
-        const int grid = grid_for(nv, block, a.fin ? kMaxBlocks : (1 << 30));
+        const int grid = hop_grid(a, nv, block);
         hr_status st = HR_OK;
         if (paired) launch_hop_clover_paired(ctx, a, grid, block, s, st);
         else for_config<ClovLaunch>(rep, prec, ctx, a, grid, block, s, st);
@@ -136,7 +132,7 @@ hr_status dispatch(hr_ctx *ctx, const Geom &g, int rep, int prec, const HopArgs 
     }
     // non-reducing launches cover all sites; reducing ones are capped so the
     // per-block partials fit the context's scratch
-    const int grid = grid_for(nv, c.block, a.fin ? kMaxBlocks : (1 << 30));
+    const int grid = hop_grid(a, nv, c.block);
     hr_status st = HR_OK;
     bool done = false;
     switch (c.variant) {
@@ -192,7 +188,7 @@ HopArgs make_args(hr_ctx *ctx, const Geom &g, const HopLaunch &L)
     a.g5_in = L.g5_in;
     a.g5_out = L.g5_out;
     a.fin = L.fin;
-    a.red = red_slot(ctx, C_HOP);
+    a.partials = ctx->d_partials;
     a.scal = ctx->d_scal;
     a.gate = L.gate;
     a.done = L.done;
@@ -205,6 +201,7 @@ HopArgs make_args(hr_ctx *ctx, const Geom &g, const HopLaunch &L)
     a.wait_cycles = ctx->inject_tile_no_copy ? (1LL << 20) : (1LL << 31); // ~0.5 ms / ~1 s
     a.clov = L.clov;
     a.clov_mode = L.clov ? L.clov_mode : kClovNone;
+    a.cond = L.cond;
     return a;
 }
 
@@ -332,6 +329,7 @@ hr_status apply_eo_op(hr_ctx *ctx, const Geom &g, double m0, int rep, int prec, 
             h2.cg_x = fz->x;
             h2.cg_p = fz->p;
             h2.cg_r = fz->r;
+            h2.cond = fz->cond;
         }
         return launch_hop(ctx, g, rep, prec, h2, s);
     };

@@ -101,8 +101,6 @@ __device__ __forceinline__ void chunk_body(const HopArgs &a)
         }
     }
     if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
         __shared__ double vals[256 * 4];
         const int t = threadIdx.x, n = g.nrhs;
         // site slot t >> lm of the block, right-hand side tp + k 2^lm
@@ -114,7 +112,7 @@ __device__ __forceinline__ void chunk_body(const HopArgs &a)
         const int per = blockDim.x >> l;
 #pragma unroll
         for (int s = 0; s < C; ++s) v += vals[((t >> l) + s * per) * n + (t & (n - 1))];
-        if (grid_reduce(v, n, a.red, sums, smem)) finish_reduction(a.fin, sums, n, a.scal);
+        block_partials(v, n, a.partials);
     }
 }
 
@@ -143,10 +141,10 @@ bool launch_hop_chunk(hr_ctx *ctx, const Geom &g, int rep, int prec, const HopAr
     // vals[] of the reduction holds blockDim x C doubles; whole warps
     if (c.block > 256 || c.block < 32 || (c.block & 31)) return false;
     const long long nt = (long long)g.vh << (g.lrhs - lc);
-    const int grid = grid_for(nt, c.block, a.fin ? kMaxBlocks : (1 << 30));
+    const int grid = hop_grid(a, nt, c.block);
     if (prec == kF32) launch_chunk<kF32>(a, lc, grid, c.block, s);
     else launch_chunk<kF16>(a, lc, grid, c.block, s);
-    st = check_launch(ctx, "right-hand-side chunk hop kernel");
+    st = hop_launched(ctx, a, grid, s, "right-hand-side chunk hop kernel");
     return true;
 }
 

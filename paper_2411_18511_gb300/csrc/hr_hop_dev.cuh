@@ -20,7 +20,7 @@ struct HopArgs {
     int beta_pow2; // beta is a power of two and there is no aux: exact scaling
     int g5_in, g5_out;
     int fin;
-    RedSlot red;
+    double *partials; // a row of per-RHS sums per block when fin is set
     double *scal;
     const double *gate;
     const double *done; // skip all work when *done != 0 (solver converged)
@@ -34,7 +34,22 @@ struct HopArgs {
                            // kernels' copies but never queue them
     const void *clov;      // clover half-field of the output parity (kClovAux / kClovOut), or nullptr
     int clov_mode;
+    FinCond cond;          // host side: condition handle the finishing launch sets
 };
+
+// the grid of a hop kernel of one thread per item: a reducing launch is capped
+// so that its rows of partial sums fit the context's scratch
+inline int hop_grid(const HopArgs &a, long long n, int block)
+{
+    return grid_for(n, block, a.fin ? kMaxPartials / a.g.nrhs : (1 << 30));
+}
+// after a hop kernel's launch: its error, and the finishing launch of a reducing one
+inline hr_status hop_launched(hr_ctx *ctx, const HopArgs &a, int grid, cudaStream_t s, const char *what)
+{
+    hr_status st = check_launch(ctx, what);
+    if (!st && a.fin) st = finish_sums(ctx, grid, a.g.nrhs, a.fin, a.gate, a.done, s, a.cond);
+    return st;
+}
 
 
 

@@ -76,11 +76,7 @@ __device__ __forceinline__ void h16_body(const HopArgs &a)
         h16_dir<3, false, NEG>(a, nrm, i, rr, nb, acc);
         hop_epilogue<kF16>(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 // Register-prefetch form: direction K+1's two spinor words, scale and link
@@ -153,11 +149,7 @@ __device__ __forceinline__ void h16p_body(const HopArgs &a)
         h16p_step<7, D, NEG>(a, nrm, i, rr, nb, buf, acc);
         hop_epilogue<kF16>(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 // Staged form: direction K+1's two spinor words, link and scale are copied by
@@ -221,11 +213,7 @@ __device__ __forceinline__ void h16s_body(const HopArgs &a)
         h16_stage_step<7, NEG>(a, i, rr, nb, b0, b1, bd, acc);
         hop_epilogue<kF16>(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 template <int G5IN> __global__ void __launch_bounds__(256) k_hop_h16(HopArgs a) { h16_body<G5IN>(a); }
@@ -264,7 +252,7 @@ bool launch_hop_half(hr_ctx *ctx, const Geom &, int rep, int prec, const HopArgs
     } else {
         (g5 ? k_hop_h16<1> : k_hop_h16<0>)<<<grid, c.block, 0, s>>>(a);
     }
-    st = check_launch(ctx, "binary16 hop kernel (half2 projection)");
+    st = hop_launched(ctx, a, grid, s, "binary16 hop kernel (half2 projection)");
     return true;
 }
 

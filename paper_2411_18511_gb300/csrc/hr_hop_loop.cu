@@ -190,11 +190,7 @@ __global__ void __launch_bounds__(256) k_hop_loop(HopArgs a)
         }
         hop_epilogue<PREC>(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 // ---------------------------------------------------------------- switched variants
@@ -321,11 +317,7 @@ __global__ void __launch_bounds__(256) k_hop_sw(HopArgs a)
         }
         hop_epilogue<PREC>(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 template <int REP, int PREC> struct Launch {
@@ -337,7 +329,7 @@ template <int REP, int PREC> struct Launch {
             const int sm_max = (int)Stage<REP, PREC>::smem_bytes(256);
             if (c.variant == kVarLoop) {
                 k_hop_loop<REP, PREC, false><<<grid, c.block, 0, s>>>(a);
-                st = check_launch(ctx, "looped hop kernel");
+                st = hop_launched(ctx, a, grid, s, "looped hop kernel");
                 return true;
             }
             if (c.variant == kVarLoopStaged) {
@@ -348,12 +340,12 @@ template <int REP, int PREC> struct Launch {
                     attr_set = true;
                 }
                 k_hop_loop<REP, PREC, true><<<grid, c.block, sm, s>>>(a);
-                st = check_launch(ctx, "looped staged hop kernel");
+                st = hop_launched(ctx, a, grid, s, "looped staged hop kernel");
                 return true;
             }
             if (c.variant == kVarSwitch) {
                 k_hop_sw<REP, PREC, false><<<grid, c.block, 0, s>>>(a);
-                st = check_launch(ctx, "switched hop kernel");
+                st = hop_launched(ctx, a, grid, s, "switched hop kernel");
                 return true;
             }
             if (c.variant == kVarSwitchStaged) {
@@ -364,7 +356,7 @@ template <int REP, int PREC> struct Launch {
                     attr_set2 = true;
                 }
                 k_hop_sw<REP, PREC, true><<<grid, c.block, sm, s>>>(a);
-                st = check_launch(ctx, "switched staged hop kernel");
+                st = hop_launched(ctx, a, grid, s, "switched staged hop kernel");
                 return true;
             }
         }

@@ -207,11 +207,7 @@ __device__ __forceinline__ void p2_body(const HopArgs &a)
         hop_epilogue<PREC>(a, j1, o1, al, be, bu, red);
         if (two) hop_epilogue<PREC>(a, j2, o2, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 template <int PREC, int G5IN> __global__ void __launch_bounds__(256) k_hop_p2(HopArgs a) { p2_body<PREC, G5IN>(a); }
@@ -236,10 +232,10 @@ bool launch_hop_pair_sites(hr_ctx *ctx, const Geom &g, int rep, int prec, const 
     // one thread per pair of virtual sites
     const long long nv = (long long)g.vh << g.lrhs;
     const long long npairs = ((nv + 63) >> 6) << 5;
-    const int grid = grid_for(npairs, c.block, a.fin ? kMaxBlocks : (1 << 30));
+    const int grid = hop_grid(a, npairs, c.block);
     if (prec == kF32) launch_p2<kF32>(a, c, grid, s);
     else launch_p2<kF16>(a, c, grid, s);
-    st = check_launch(ctx, "two-site hop kernel");
+    st = hop_launched(ctx, a, grid, s, "two-site hop kernel");
     return true;
 }
 

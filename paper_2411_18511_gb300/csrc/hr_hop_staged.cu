@@ -97,11 +97,7 @@ __global__ void __launch_bounds__(256) k_hop_staged(HopArgs a)
         stage_step<7, REP, PREC>(a, i, rr, nb, b0, b1, bd, acc);
         hop_epilogue<PREC>(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 // ---------------------------------------------------------------- prefetching variant
@@ -187,11 +183,7 @@ __global__ void __launch_bounds__(256) k_hop_pf(HopArgs a)
         pf_compute<7, REP, PREC>(a, sB, qB, cB, acc);
         hop_epilogue<PREC>(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 template <int REP, int PREC> struct Launch {
@@ -208,12 +200,12 @@ template <int REP, int PREC> struct Launch {
                     attr_set = true;
                 }
                 k_hop_staged<REP, PREC><<<grid, c.block, sm, s>>>(a);
-                st = check_launch(ctx, "staged hop kernel");
+                st = hop_launched(ctx, a, grid, s, "staged hop kernel");
                 return true;
             }
             if (c.variant == kVarPrefetch) {
                 k_hop_pf<REP, PREC><<<grid, c.block, 0, s>>>(a);
-                st = check_launch(ctx, "prefetching hop kernel");
+                st = hop_launched(ctx, a, grid, s, "prefetching hop kernel");
                 return true;
             }
         }

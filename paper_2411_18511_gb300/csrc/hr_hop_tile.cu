@@ -139,11 +139,7 @@ __device__ __forceinline__ void hop_tile_body(const HopArgs &a)
         }
         phase ^= 1u;
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 template <int REP, int PREC, int G5IN>
@@ -180,7 +176,7 @@ template <int REP, int PREC> struct Launch {
             // one tile per block; a reducing launch loops over tiles within the partials' cap
             const long long nv = (long long)g.vh << g.lrhs;
             const long long ntiles = (nv + c.block - 1) / c.block;
-            const int tgrid = (int)std::min<long long>(ntiles, a.fin ? kMaxBlocks : (1LL << 30));
+            const int tgrid = hop_grid(a, ntiles, 1);
             if (c.variant == kVarTile) {
                 if (a.g5_in) k_hop_tile<REP, PREC, 1><<<tgrid, c.block, sm, s>>>(a);
                 else k_hop_tile<REP, PREC, 0><<<tgrid, c.block, sm, s>>>(a);
@@ -188,7 +184,7 @@ template <int REP, int PREC> struct Launch {
                 if (a.g5_in) k_hop_tile_r96<REP, PREC, 1><<<tgrid, c.block, sm, s>>>(a);
                 else k_hop_tile_r96<REP, PREC, 0><<<tgrid, c.block, sm, s>>>(a);
             }
-            st = check_launch(ctx, "tiled hop kernel");
+            st = hop_launched(ctx, a, tgrid, s, "tiled hop kernel");
             return true;
         }
         return false;

@@ -136,11 +136,7 @@ __global__ void __launch_bounds__(128) k_hop_twist(HopArgs a)
         twisted_dir<3, REP, PREC, false>(a, i, rr, nb, x, acc);
         hop_epilogue<PREC, CLOV>(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 // ---- fundamental FP64: the paired double-float arithmetic of the tuned
@@ -236,11 +232,7 @@ __device__ __forceinline__ void x2t_body(const HopArgs &a)
         x2t_dir<3, false, NEG>(a, k, i, rr, nb, x, acc);
         x2_epilogue<CLOV>(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 template <int G5IN, bool CLOV> __global__ void __maxnreg__(128) k_hop_x2t(HopArgs a) { x2t_body<G5IN, CLOV>(a); }
@@ -252,12 +244,12 @@ template <int REP, int PREC> struct TwistLaunch {
             const bool g5 = a.g5_in != 0, clov = a.clov_mode != kClovNone;
             if (clov) (g5 ? k_hop_x2t<1, true> : k_hop_x2t<0, true>)<<<grid, kTwistBlock, 0, s>>>(a);
             else (g5 ? k_hop_x2t<1, false> : k_hop_x2t<0, false>)<<<grid, kTwistBlock, 0, s>>>(a);
-            st = check_launch(ctx, "paired hop kernel (twisted boundaries)");
+            st = hop_launched(ctx, a, grid, s, "paired hop kernel (twisted boundaries)");
             return true;
         }
         if (a.clov_mode != kClovNone) k_hop_twist<REP, PREC, true><<<grid, kTwistBlock, 0, s>>>(a);
         else k_hop_twist<REP, PREC, false><<<grid, kTwistBlock, 0, s>>>(a);
-        st = check_launch(ctx, "hop kernel (twisted boundaries)");
+        st = hop_launched(ctx, a, grid, s, "hop kernel (twisted boundaries)");
         return true;
     }
 };
@@ -269,7 +261,7 @@ namespace hr {
 void launch_hop_twisted(hr_ctx *ctx, int rep, int prec, const HopArgs &a, cudaStream_t s, hr_status &st)
 {
     const long long nv = (long long)a.g.vh << a.g.lrhs;
-    const int grid = grid_for(nv, kTwistBlock, a.fin ? kMaxBlocks : (1 << 30));
+    const int grid = hop_grid(a, nv, kTwistBlock);
     if (!for_config<TwistLaunch>(rep, prec, ctx, a, grid, s, st))
         st = set_error(ctx, HR_ERR_INVALID_ARG, "bad rep/prec");
 }

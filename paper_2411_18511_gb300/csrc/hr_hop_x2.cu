@@ -74,11 +74,7 @@ __device__ __forceinline__ void x2s_body(const HopArgs &a)
         x2_stage_step<7, NEG>(a, k, i, rr, nb, b0, b1, bd, acc);
         x2_epilogue<CLOV>(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 template <int G5IN>
@@ -107,11 +103,7 @@ __device__ __forceinline__ void x2_body(const HopArgs &a)
         x2_dir<3, false, NEG>(a, k, i, rr, nb, acc);
         x2_epilogue(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 // registers as the compiler likes (about 100 / 128), or capped at 96: five
@@ -303,11 +295,7 @@ __device__ __forceinline__ void f2_body(const HopArgs &a)
         }
         hop_epilogue<PREC>(a, j, o, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 // staged form: direction K+1's operands copied by cp.async while K is computed
@@ -395,11 +383,7 @@ __device__ __forceinline__ void f2s_body(const HopArgs &a)
         }
         hop_epilogue<PREC>(a, j, o, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 template <int PREC, int G5IN> __global__ void __launch_bounds__(256) k_hop_f2(HopArgs a) { f2_body<PREC, G5IN>(a); }
@@ -621,11 +605,7 @@ __device__ __forceinline__ void x2a_body(const HopArgs &a)
         x2a_term<3, false, false, NEG, REP>(a, k, nb.bwd[3], 1 - a.p, (nb.bwd[3] << l) + rr, acc);
         x2a_epilogue(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 // staged form (quaternion links): direction K+1's operands copied by cp.async while K is computed
@@ -688,11 +668,7 @@ __device__ __forceinline__ void x2as_body(const HopArgs &a)
         x2a_stage_step<7, NEG>(a, k, i, rr, nb, b0, b1, bd, acc);
         x2a_epilogue(a, j, acc, al, be, bu, red);
     }
-    if (a.fin) {
-        __shared__ double smem[32 * 32];
-        __shared__ double sums[32];
-        if (grid_reduce(red, g.nrhs, a.red, sums, smem)) finish_reduction(a.fin, sums, g.nrhs, a.scal);
-    }
+    if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
 template <int REP, int G5IN> __global__ void __maxnreg__(128) k_hop_x2a(HopArgs a) { x2a_body<REP, G5IN>(a); }
@@ -722,7 +698,7 @@ template <int REP, int PREC> struct Launch {
             case kVarPairedR96: (g5 ? k_hop_x2_r96<1> : k_hop_x2_r96<0>)<<<grid, c.block, 0, s>>>(a); break;
             default: (g5 ? k_hop_x2<1> : k_hop_x2<0>)<<<grid, c.block, 0, s>>>(a); break;
             }
-            st = check_launch(ctx, "paired hop kernel");
+            st = hop_launched(ctx, a, grid, s, "paired hop kernel");
             return true;
         } else if constexpr (PREC == kF64) {
             // adjoint (quaternion or stored 3x3 links): (re, im) lanes
@@ -731,7 +707,7 @@ template <int REP, int PREC> struct Launch {
             if (c.variant == kVarPairedR96) {
                 // for the adjoint: the form with 168 registers
                 (g5 ? k_hop_x2a_big<REP, 1> : k_hop_x2a_big<REP, 0>)<<<grid, c.block, 0, s>>>(a);
-                st = check_launch(ctx, "paired adjoint hop kernel (168 registers)");
+                st = hop_launched(ctx, a, grid, s, "paired adjoint hop kernel (168 registers)");
                 return true;
             }
             if constexpr (REP == kRepAdj) {
@@ -745,12 +721,12 @@ template <int REP, int PREC> struct Launch {
                         attr_set = true;
                     }
                     (g5 ? k_hop_x2as<1> : k_hop_x2as<0>)<<<grid, c.block, S::smem_bytes(c.block), s>>>(a);
-                    st = check_launch(ctx, "paired adjoint hop kernel");
+                    st = hop_launched(ctx, a, grid, s, "paired adjoint hop kernel");
                     return true;
                 }
             }
             (g5 ? k_hop_x2a<REP, 1> : k_hop_x2a<REP, 0>)<<<grid, c.block, 0, s>>>(a);
-            st = check_launch(ctx, "paired adjoint hop kernel");
+            st = hop_launched(ctx, a, grid, s, "paired adjoint hop kernel");
             return true;
         } else if constexpr (REP == kRepFund) {
             // FP32 arithmetic: the register-capped forms are not built (the
@@ -768,7 +744,7 @@ template <int REP, int PREC> struct Launch {
                 (g5 ? k_hop_f2s<PREC, 1> : k_hop_f2s<PREC, 0>)<<<grid, c.block, S::smem_bytes(c.block), s>>>(a);
             else
                 (g5 ? k_hop_f2<PREC, 1> : k_hop_f2<PREC, 0>)<<<grid, c.block, 0, s>>>(a);
-            st = check_launch(ctx, "paired hop kernel");
+            st = hop_launched(ctx, a, grid, s, "paired hop kernel");
             return true;
         }
         return false;
@@ -789,7 +765,7 @@ void launch_hop_clover_paired(hr_ctx *ctx, const HopArgs &a, int grid, int block
         attr_set = true;
     }
     (a.g5_in ? k_hop_x2s_clov<1> : k_hop_x2s_clov<0>)<<<grid, block, S::smem_bytes(block), s>>>(a);
-    st = check_launch(ctx, "paired hop kernel (clover epilogue)");
+    st = hop_launched(ctx, a, grid, s, "paired hop kernel (clover epilogue)");
 }
 
 bool launch_hop_paired(hr_ctx *ctx, const Geom &g, int rep, int prec, const HopArgs &a, HopChoice c, int grid,

@@ -18,8 +18,10 @@
 
 // Device scratch owned by a context (allocated once in hr_ctx_create).
 namespace hr {
-constexpr int kMaxBlocks = 4096;      // cap on blocks of any reducing launch
+constexpr int kMaxBlocks = 4096;      // cap on blocks of the vector kernels and of 32-RHS reducing launches
 constexpr int kMaxRhs = 32;
+constexpr int kMaxPartials = kMaxBlocks * kMaxRhs; // partial sums of one reducing launch
+constexpr int kFinBlocks = 64;       // blocks of a finishing launch, at most
 constexpr int kNumCounters = 64;
 constexpr int kScalDoubles = 64 * kMaxRhs;
 
@@ -35,9 +37,8 @@ struct hr_ctx {
     int device = 0;
     int sm_count = 0;
     std::string err;
-    double *d_partials = nullptr;  // kMaxBlocks * kMaxRhs, then kRedMaxGroups * kMaxRhs group sums
+    double *d_partials = nullptr;  // kMaxPartials, then kFinBlocks * kMaxRhs sums of a finishing launch's blocks
     unsigned *d_counters = nullptr;
-    unsigned *d_group_counters = nullptr; // kNumCounters * kRedMaxGroups (two-level reductions)
     double *d_scal = nullptr;      // kScalDoubles
     double *h_scal = nullptr;      // pinned mirror
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -74,17 +75,6 @@ inline int rep_nc(int rep) { return rep == HR_FUND ? 2 : 3; }
 size_t spinor_half_bytes(const Geom &g, int rep, int prec);
 size_t gauge_bytes(const Geom &g, int rep, int prec);
 
-inline RedSlot red_slot(hr_ctx *ctx, int counter)
-{
-    RedSlot s;
-    s.partials = ctx->d_partials;
-    s.counter = ctx->d_counters + counter;
-    s.group_counters = ctx->d_group_counters + (size_t)counter * kRedMaxGroups;
-    s.group_partials = ctx->d_partials + (size_t)kMaxBlocks * kMaxRhs;
-    return s;
-}
-static_assert(kMaxBlocks <= kRedGroup * kRedMaxGroups, "two-level reductions cover every grid");
-
 inline int grid_for(long long n, int block, int cap)
 {
     long long b = (n + block - 1) / block;
@@ -93,15 +83,26 @@ inline int grid_for(long long n, int block, int cap)
     return (int)b;
 }
 
-// counters used by the reducing kernels (each reduction site has its own)
+// device counters: blocks of a finishing launch, native-path requests
 // (C_PACK: the pack status word, kPack* flags of the values packed since the
 // last check, read and cleared by consume_pack_status)
-enum Counter { C_HOP = 0, C_XR = 1, C_RES = 2, C_NORM = 3, C_DOT = 4, C_MISC = 5, C_BATCH = 16, C_PACK = 62,
-               C_STATUS = 63 };
+enum Counter { C_FIN = 0, C_PACK = 62, C_STATUS = 63 };
 
 // clover site term in a hop epilogue (hr_clover.cuh): none, A(x) on the aux
 // term (out = alpha A aux + beta acc), or A(x) on the result (out = A (alpha aux + beta acc))
 enum ClovMode { kClovNone = 0, kClovAux = 1, kClovOut = 2 };
+
+// A condition of the solve graph that a finishing launch sets: 1 when a reliable
+// update is due, else 0 (set == 0: none).
+struct FinCond {
+    int set;
+    unsigned long long handle;
+};
+// Add the `nparts` rows of nrhs partial sums in the context's scratch and run the
+// scalar update `fin` on them (hr_blas.cu); skipped like the launch that wrote
+// them when *gate == 0 or *done != 0.
+hr_status finish_sums(hr_ctx *ctx, int nparts, int nrhs, int fin, const double *gate, const double *done,
+                      cudaStream_t s, FinCond cond = {0, 0});
 
 // ---- hop launches (hr_hop.cu) ----
 struct HopLaunch {
@@ -124,6 +125,7 @@ struct HopLaunch {
     // (clover_half) and how the epilogue applies it (ClovMode)
     const void *clov;
     int clov_mode;
+    FinCond cond;
 };
 // a CG x/r update fused into the last hop of an operator (the operator's
 // precision; x in FP32 when the operator runs in binary16)
@@ -132,6 +134,7 @@ struct CgFuse {
     const void *p;
     void *r;
     int fin; // kFinBeta or kFinBetaMixed
+    FinCond cond;
 };
 hr_status launch_hop(hr_ctx *ctx, const Geom &g, int rep, int prec, const HopLaunch &L, cudaStream_t s);
 hr_status launch_hop_with(hr_ctx *ctx, const Geom &g, int rep, int prec, const HopLaunch &L, HopChoice c,

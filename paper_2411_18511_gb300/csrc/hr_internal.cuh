@@ -901,23 +901,14 @@ __device__ __forceinline__ void spin_accumulate(cpx<T> (&acc)[4][NC], const cpx<
 }
 
 // ---------------------------------------------------------------- reductions
-
-// Deterministic grid reduction of up to 32 per-RHS sums.  Every thread passes
-// its value for right-hand side (j & (nrhs-1)); the block's per-RHS sums go to
-// partials[blockIdx.x*nrhs + r]; the last block to finish adds the partials in
-// block order into sums[r] and returns true (only in that block).
-struct RedSlot {
-    double *partials;  // >= gridDim.x * nrhs doubles
-    unsigned *counter; // zero before the launch; reset by the last block
-    // two-level form (nullable): kRedGroup consecutive blocks form a group;
-    // the last block of a group to finish sums the group's partials into
-    // group_partials[group * nrhs + r] (counted in group_counters[group],
-    // zero before the launch, reset), and the last group summer adds the
-    // groups.  No block then sums more than kRedGroup blocks' partials.
-    unsigned *group_counters; // >= kRedMaxGroups
-    double *group_partials;   // >= kRedMaxGroups * nrhs doubles
-};
-constexpr int kRedGroup = 64, kRedMaxGroups = 64;
+//
+// A reducing kernel leaves one row of per-RHS sums per block (block_partials);
+// a second, small launch adds the rows in a fixed order and runs the solver's
+// scalar update on the result (finish_sums).  The reducing kernel then holds no
+// block back: when each block counted itself on an atomic (its stores fenced
+// first) so that the last one could add the rows, every block stayed resident
+// for those two round trips, and a reducing binary16 hop at 32^4 took 35 us
+// against 21 us for the plain one.
 
 __device__ __forceinline__ double warp_sum_strided(double v, int nrhs)
 {
@@ -925,45 +916,33 @@ __device__ __forceinline__ double warp_sum_strided(double v, int nrhs)
     return v;
 }
 
-// sums[r] = sum over b < nparts of partials[b*nrhs + r], by the whole block.
-// Thread t takes right-hand side t % nrhs and every (blockDim/nrhs)-th partial;
-// the per-thread sums meet in a fixed tree, so the result does not depend on
-// which block runs this.  The partials are read through L2 (ld.cg): other
-// blocks wrote them.  Ends with a block barrier; smem >= 32 doubles per warp.
-__device__ inline void sum_partials(const double *partials, unsigned nparts, int nrhs, double *sums, double *smem)
+// smem[r] = sum over b < nparts of partials[b*nrhs + r], by the whole block (a
+// power of two of threads, one double of smem each).  Thread t takes right-hand
+// side t % nrhs and every (blockDim/nrhs)-th row, eight loads in flight (other
+// blocks wrote the rows: ld.cg), and the threads' sums meet in a tree, so the
+// result depends on nparts, nrhs and blockDim only.  The FP64 pipe runs 1.7
+// additions a clock on this GPU, so it counts them: a tree in shared memory
+// halves its lanes at each step, a shuffle tree would add on all 32.
+// Ends with a block barrier.
+__device__ inline void sum_partials(const double *partials, int nparts, int nrhs, double *smem)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int r = threadIdx.x & (nrhs - 1);
-    const unsigned step = blockDim.x / nrhs;
-    // sixteen independent accumulators keep sixteen L2 loads in flight per
-    // thread (a single running sum leaves this one block latency-bound when
-    // there are many partials, e.g. 4096 blocks x 32 right-hand sides);
-    // combined in a fixed order
-    constexpr int K = 16;
-    double acc[K];
+    const int t = threadIdx.x, r = t & (nrhs - 1), step = blockDim.x / nrhs;
+    constexpr int K = 8;
+    double acc = 0.0;
+    for (int b = t / nrhs; b < nparts; b += K * step) {
+        double v[K];
 #pragma unroll
-    for (int k = 0; k < K; ++k) acc[k] = 0.0;
-    unsigned b = threadIdx.x / nrhs;
-    for (; b + (K - 1) * step < nparts; b += K * step) {
+        for (int k = 0; k < K; ++k) v[k] = b + k * step < nparts ? __ldcg(partials + (size_t)(b + k * step) * nrhs + r) : 0.0;
 #pragma unroll
-        for (int k = 0; k < K; ++k) acc[k] += __ldcg(partials + (size_t)(b + k * step) * nrhs + r);
+        for (int k = 0; k < K; ++k)
+            if (b + k * step < nparts) acc += v[k];
     }
-    for (int k = 0; b < nparts; b += step, ++k) acc[k & (K - 1)] += __ldcg(partials + (size_t)b * nrhs + r);
-#pragma unroll
-    for (int w = K / 2; w > 0; w >>= 1)
-#pragma unroll
-        for (int k = 0; k < w; ++k) acc[k] += acc[k + w];
-    double s = acc[0];
-    s = warp_sum_strided(s, nrhs);
+    smem[t] = acc;
     __syncthreads();
-    if (lane < nrhs) smem[warp * 32 + lane] = s;
-    __syncthreads();
-    if (threadIdx.x < nrhs) {
-        double t = 0;
-        for (int w = 0; w < nwarps; ++w) t += smem[w * 32 + threadIdx.x];
-        sums[threadIdx.x] = t;
+    for (int n = blockDim.x >> 1; n >= nrhs; n >>= 1) {
+        if (t < n) smem[t] += smem[t + n];
+        __syncthreads();
     }
-    __syncthreads();
 }
 
 // The warp stage of a grid reduction in the accumulator's own arithmetic:
@@ -990,69 +969,26 @@ __device__ __forceinline__ double warp_total(const SqAcc<double> &a, int nrhs)
     return warp_sum_strided(a.s, nrhs);
 }
 
-// grid_reduce from per-warp totals (lanes r < nrhs hold right-hand side r's)
-__device__ inline bool grid_reduce_warped(double v, int nrhs, RedSlot slot, double *sums, double *smem)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    if (lane < nrhs) smem[warp * 32 + lane] = v;
-    __syncthreads();
-    if (threadIdx.x < nrhs) {
-        double s = 0;
-        for (int w = 0; w < nwarps; ++w) s += smem[w * 32 + threadIdx.x];
-        slot.partials[(size_t)blockIdx.x * nrhs + threadIdx.x] = s;
-        // only the writers of the partials order them before the block's
-        // count: a fence on every thread would hold each block until its
-        // output stores had drained
-        __threadfence();
-    }
-    __shared__ bool last;
-    __syncthreads();
-    unsigned nparts = gridDim.x;
-    const double *parts = slot.partials;
-    if (slot.group_counters && gridDim.x > (unsigned)kRedGroup) {
-        // first level: the last block of this group sums the group's partials
-        const unsigned grp = blockIdx.x / kRedGroup;
-        const unsigned first = grp * kRedGroup;
-        const unsigned gsize = min((unsigned)kRedGroup, gridDim.x - first);
-        if (threadIdx.x == 0) {
-            unsigned t = atomicAdd(slot.group_counters + grp, 1u);
-            last = (t == gsize - 1);
-        }
-        __syncthreads();
-        if (!last) return false;
-        __threadfence();
-        sum_partials(slot.partials + (size_t)first * nrhs, gsize, nrhs, sums, smem);
-        if (threadIdx.x < nrhs) {
-            slot.group_partials[(size_t)grp * nrhs + threadIdx.x] = sums[threadIdx.x];
-            __threadfence();
-        }
-        if (threadIdx.x == 0) slot.group_counters[grp] = 0u;
-        __syncthreads();
-        nparts = (gridDim.x + kRedGroup - 1) / kRedGroup;
-        parts = slot.group_partials;
-    }
-    if (threadIdx.x == 0) {
-        unsigned t = atomicAdd(slot.counter, 1u);
-        last = (t == nparts - 1);
-    }
-    __syncthreads();
-    if (!last) return false;
-    __threadfence();
-    sum_partials(parts, nparts, nrhs, sums, smem);
-    if (threadIdx.x == 0) *slot.counter = 0u;
-    return true;
-}
+__device__ __forceinline__ double warp_total(double v, int nrhs) { return warp_sum_strided(v, nrhs); }
 
-// Deterministic grid reduction of a value per thread (see RedSlot)
-__device__ inline bool grid_reduce(double v, int nrhs, RedSlot slot, double *sums, double *smem /* >= 32*32 */)
+// The block's per-RHS sums into partials[blockIdx.x * nrhs + r]; every thread
+// passes its accumulator for right-hand side (thread & (nrhs - 1)).
+constexpr int kRedWarps = 8;
+template <class V> __device__ __forceinline__ void block_partials(const V &acc, int nrhs, double *partials)
 {
-    return grid_reduce_warped(warp_sum_strided(v, nrhs), nrhs, slot, sums, smem);
-}
-// ... and of a sum-of-squares accumulator per thread, warp stage in its own arithmetic
-template <class T>
-__device__ inline bool grid_reduce(const SqAcc<T> &acc, int nrhs, RedSlot slot, double *sums, double *smem)
-{
-    return grid_reduce_warped(warp_total(acc, nrhs), nrhs, slot, sums, smem);
+    __shared__ double w[kRedWarps * 32];
+    const double v = warp_total(acc, nrhs);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    double s = 0;
+    for (int w0 = 0; w0 < nwarps; w0 += kRedWarps) { // once, up to 256 threads a block
+        const int nw = min(kRedWarps, nwarps - w0);
+        if (w0) __syncthreads();
+        if (lane < nrhs && warp >= w0 && warp < w0 + nw) w[(warp - w0) * nrhs + lane] = v;
+        __syncthreads();
+        if (threadIdx.x < nrhs)
+            for (int k = 0; k < nw; ++k) s += w[k * nrhs + threadIdx.x];
+    }
+    if (threadIdx.x < nrhs) partials[(size_t)blockIdx.x * nrhs + threadIdx.x] = s;
 }
 
 // ---------------------------------------------------------------- solver scalars
@@ -1075,7 +1011,8 @@ enum ScalSlot {
                    // bulk copy that did not land in time), [7] source out of range,
                    // [8] S_OUT holds the true FP64 residuals of the current x (the
                    // last scalar update was a reliable update's), [9] / [10] the
-                   // open reliable update is of the FP32 / FP64 tier
+                   // open reliable update is of the FP32 / FP64 tier, [11] the recurrence's
+                   // launches skip: all done, or a reliable update is due first
     S_DELTA2 = 11, // [0] reliable-update threshold delta^2, [1] tol^2, [2] maxiter (<= 0: none),
                    // [3] FP32-tier threshold delta_mid^2 (0: every update is an FP64 one)
     S_SCALE = 12,  // per-RHS power of two that brings the source's largest component into [0.5, 1)
@@ -1084,7 +1021,7 @@ enum ScalSlot {
     S_NSLOTS = 15
 };
 constexpr int F_DONE = 0, F_GATE = 1, F_NUMERIC = 2, F_ITERS = 3, F_NRELIABLE = 4, F_BODY = 5, F_DEVERR = 6,
-              F_RANGE = 7, F_TRUERES = 8, F_TIER1 = 9, F_TIER2 = 10;
+              F_RANGE = 7, F_TRUERES = 8, F_TIER1 = 9, F_TIER2 = 10, F_SKIP = 11;
 
 enum FinishMode {
     kFinNone = 0,
@@ -1100,42 +1037,68 @@ enum FinishMode {
 
 __device__ __forceinline__ double &sc(double *scal, int slot, int r) { return scal[slot * kMaxRhsSlots + r]; }
 
-// Scalar updates run by the last block of a grid reduction (threads 0..nrhs-1
-// hold one right-hand side each); afterwards thread 0 refreshes the flags.
-__device__ inline void finish_reduction(int mode, const double *sums, int nrhs, double *scal)
+// The scalars one right-hand side's update reads, loaded together (and, by the
+// finishing kernel, before the sums are there): one round trip instead of a chain.
+struct FinIn {
+    double active, rr, rrold, stop, rmax, rref, d2, tol2, cap, dmid, iters, gate, tier2;
+};
+__device__ __forceinline__ FinIn load_fin(double *scal, int nrhs)
+{
+    const int r = threadIdx.x < nrhs ? threadIdx.x : 0;
+    FinIn f;
+    f.active = sc(scal, S_ACTIVE, r);
+    f.rr = sc(scal, S_RR, r);
+    f.rrold = sc(scal, S_RROLD, r);
+    f.stop = sc(scal, S_STOP, r);
+    f.rmax = sc(scal, S_RMAX, r);
+    f.rref = sc(scal, S_RREF, r);
+    f.d2 = sc(scal, S_DELTA2, 0);
+    f.tol2 = sc(scal, S_DELTA2, 1);
+    f.cap = sc(scal, S_DELTA2, 2);
+    f.dmid = sc(scal, S_DELTA2, 3);
+    f.iters = sc(scal, S_FLAGS, F_ITERS);
+    f.gate = sc(scal, S_FLAGS, F_GATE);
+    f.tier2 = sc(scal, S_FLAGS, F_TIER2);
+    return f;
+}
+
+// Scalar updates run by one block on the finished sums (threads 0..nrhs-1 hold
+// one right-hand side each); thread 0 then refreshes the flags.  Returns, in
+// every thread, whether a reliable update is due (the gate is open and the
+// solve goes on).
+__device__ inline bool finish_reduction(int mode, const double *sums, int nrhs, double *scal, const FinIn &f)
 {
     const int r = threadIdx.x;
+    bool act = false, bad = false, open = false, open2 = false;
     if (r < nrhs) {
-        double v = sums[r];
-        bool bad = !isfinite(v);
-        bool act = sc(scal, S_ACTIVE, r) != 0.0;
+        const double v = sums[r];
+        act = f.active != 0.0;
+        bad = !isfinite(v) && mode != kFinStore;
         switch (mode) {
         case kFinStore:
             sc(scal, S_OUT, r) = v;
             break;
         case kFinAlpha:
             sc(scal, S_PAP, r) = v;
-            sc(scal, S_ALPHA, r) = (act && v > 0.0) ? sc(scal, S_RR, r) / v : 0.0;
+            sc(scal, S_ALPHA, r) = (act && v > 0.0) ? f.rr / v : 0.0;
             break;
         case kFinBeta:
         case kFinBetaMixed: {
-            double rr = sc(scal, S_RR, r);
-            sc(scal, S_RROLD, r) = rr;
+            sc(scal, S_RROLD, r) = f.rr;
             if (act) {
-                sc(scal, S_BETA, r) = v / rr;
+                sc(scal, S_BETA, r) = v / f.rr;
                 sc(scal, S_RR, r) = v;
                 if (mode == kFinBeta) {
-                    if (v <= sc(scal, S_STOP, r)) sc(scal, S_ACTIVE, r) = 0.0;
+                    if (v <= f.stop) act = false;
                 } else {
-                    double rmax = fmax(sc(scal, S_RMAX, r), v);
+                    const double rmax = fmax(f.rmax, v);
                     sc(scal, S_RMAX, r) = rmax;
-                    const bool conv = v <= sc(scal, S_STOP, r);
-                    if (conv || v < sc(scal, S_DELTA2, 0) * rmax) {
-                        sc(scal, S_FLAGS, F_GATE) = 1.0;
+                    const bool conv = v <= f.stop;
+                    if (conv || v < f.d2 * rmax) {
+                        open = true;
                         // the FP64 tier when the FP32 tier is off, at convergence, or
                         // once |r| fell by delta_mid since the last FP64 residual
-                        const double dm = sc(scal, S_DELTA2, 3);
-                        if (dm == 0.0 || conv || v < dm * sc(scal, S_RREF, r)) sc(scal, S_FLAGS, F_TIER2) = 1.0;
+                        open2 = f.dmid == 0.0 || conv || v < f.dmid * f.rref;
                     }
                 }
             } else {
@@ -1148,18 +1111,18 @@ __device__ inline void finish_reduction(int mode, const double *sums, int nrhs, 
             sc(scal, S_RMAX, r) = v;
             sc(scal, S_RROLD, r) = v;
             sc(scal, S_RREF, r) = v;
-            sc(scal, S_ACTIVE, r) = (v > sc(scal, S_STOP, r)) ? 1.0 : 0.0;
+            act = v > f.stop;
             break;
         case kFinBB:
             sc(scal, S_BB, r) = v;
-            sc(scal, S_STOP, r) = sc(scal, S_DELTA2, 1) * v;
+            sc(scal, S_STOP, r) = f.tol2 * v;
             break;
         case kFinResidual:
             if (act) {
-                sc(scal, S_BETA, r) = v / sc(scal, S_RROLD, r);
+                sc(scal, S_BETA, r) = v / f.rrold;
                 sc(scal, S_RR, r) = v;
                 sc(scal, S_RMAX, r) = v;
-                if (v <= sc(scal, S_STOP, r)) sc(scal, S_ACTIVE, r) = 0.0;
+                if (v <= f.stop) act = false;
             } else {
                 sc(scal, S_BETA, r) = 0.0;
             }
@@ -1170,7 +1133,7 @@ __device__ inline void finish_reduction(int mode, const double *sums, int nrhs, 
             // r = r_ref - A_32 dx is accurate to FP32 relative to r_ref only: it
             // restarts the recurrence but stops no right-hand side
             if (act) {
-                sc(scal, S_BETA, r) = v / sc(scal, S_RROLD, r);
+                sc(scal, S_BETA, r) = v / f.rrold;
                 sc(scal, S_RR, r) = v;
                 sc(scal, S_RMAX, r) = v;
             } else {
@@ -1180,39 +1143,48 @@ __device__ inline void finish_reduction(int mode, const double *sums, int nrhs, 
         default:
             break;
         }
-        if (bad && mode != kFinStore) sc(scal, S_FLAGS, F_NUMERIC) = 1.0;
+        if (mode == kFinBeta || mode == kFinResidual || mode == kFinInit) sc(scal, S_ACTIVE, r) = act ? 1.0 : 0.0;
     }
-    __syncthreads();
-    if (threadIdx.x == 0 && mode != kFinStore && mode != kFinBB) {
-        bool all_done = true;
-        for (int k = 0; k < nrhs; ++k) all_done = all_done && (sc(scal, S_ACTIVE, k) == 0.0);
-        if (sc(scal, S_FLAGS, F_NUMERIC) != 0.0) all_done = true;
-        if (mode == kFinBeta || mode == kFinBetaMixed) {
-            // the iteration cap also stops the recurrence (work already queued skips)
-            const double it = sc(scal, S_FLAGS, F_ITERS) + 1.0, cap = sc(scal, S_DELTA2, 2);
-            sc(scal, S_FLAGS, F_ITERS) = it;
-            if (cap > 0.0 && it >= cap) all_done = true;
-        }
-        sc(scal, S_FLAGS, F_DONE) = all_done ? 1.0 : 0.0;
-        if (mode == kFinResidual) {
-            sc(scal, S_FLAGS, F_GATE) = 0.0;
-            sc(scal, S_FLAGS, F_TIER1) = 0.0;
-            sc(scal, S_FLAGS, F_TIER2) = 0.0;
-            sc(scal, S_FLAGS, F_NRELIABLE) += 1.0;
-            // x_lo was folded into x and S_OUT = |b - A x|^2: a loop that stops
-            // here needs no further true-residual computation
-            sc(scal, S_FLAGS, F_TRUERES) = 1.0;
-        } else if (mode == kFinMid) {
-            sc(scal, S_FLAGS, F_GATE) = 0.0;
-            sc(scal, S_FLAGS, F_TIER1) = 0.0;
-            sc(scal, S_FLAGS, F_TRUERES) = 0.0;
-        } else if (mode == kFinBeta || mode == kFinBetaMixed || mode == kFinInit) {
-            sc(scal, S_FLAGS, F_TRUERES) = 0.0; // x (or x_lo) moved since
-        }
+    const bool any_bad = __syncthreads_or(bad), any_act = __syncthreads_or(act);
+    const bool any_open = __syncthreads_or(open), any_open2 = __syncthreads_or(open2);
+    if (mode == kFinStore) return false;
+    bool done = !any_act, gate = f.gate != 0.0;
+    if (threadIdx.x == 0 && any_bad) sc(scal, S_FLAGS, F_NUMERIC) = 1.0;
+    if (mode == kFinBB) return false;
+    done = done || any_bad || sc(scal, S_FLAGS, F_NUMERIC) != 0.0;
+    if (mode == kFinBeta || mode == kFinBetaMixed) {
+        // the iteration cap also stops the recurrence (work already queued skips)
+        done = done || (f.cap > 0.0 && f.iters + 1.0 >= f.cap);
+    }
+    bool tier1 = false, tier2 = f.tier2 != 0.0;
+    if (mode == kFinBetaMixed) {
         // an open gate is of exactly one tier
-        if (mode == kFinBetaMixed && sc(scal, S_FLAGS, F_GATE) != 0.0)
-            sc(scal, S_FLAGS, F_TIER1) = sc(scal, S_FLAGS, F_TIER2) != 0.0 ? 0.0 : 1.0;
+        gate = gate || any_open;
+        tier2 = tier2 || any_open2;
+        tier1 = gate && !tier2;
+    } else if (mode == kFinResidual || mode == kFinInit) {
+        gate = tier2 = false;
+    } else if (mode == kFinMid) {
+        gate = false;
     }
+    if (threadIdx.x == 0) {
+        double *fl = scal + S_FLAGS * kMaxRhsSlots;
+        if (mode == kFinBeta || mode == kFinBetaMixed) fl[F_ITERS] = f.iters + 1.0;
+        if (mode == kFinBetaMixed) fl[F_TIER1] = tier1 ? 1.0 : 0.0;
+        if (mode == kFinResidual || mode == kFinMid || mode == kFinInit) fl[F_TIER1] = 0.0;
+        if (mode != kFinAlpha) {
+            fl[F_GATE] = gate ? 1.0 : 0.0;
+            fl[F_TIER2] = tier2 ? 1.0 : 0.0;
+            // x_lo was folded into x and S_OUT = |b - A x|^2: a loop that stops
+            // after a kFinResidual needs no further true-residual computation;
+            // after the others x (or x_lo) moved
+            fl[F_TRUERES] = mode == kFinResidual ? 1.0 : 0.0;
+        }
+        if (mode == kFinResidual) fl[F_NRELIABLE] += 1.0;
+        fl[F_DONE] = done ? 1.0 : 0.0;
+        fl[F_SKIP] = done || gate ? 1.0 : 0.0;
+    }
+    return gate && !done;
 }
 
 } // namespace hr

@@ -53,16 +53,18 @@ __global__ void __launch_bounds__(256) k_norm2_noalloc(Geom g, const void *v, No
                 acc.add(a[s][c].im);
             }
     }
-    __shared__ double smem[32 * 32];
-    __shared__ double sums[32];
-    RedSlot slot;
-    slot.partials = scr->partials;
-    slot.counter = &scr->counter;
-    slot.group_counters = nullptr; // one level: the fixed scratch has no group slots
-    slot.group_partials = nullptr;
-    if (grid_reduce(acc, g.nrhs, slot, sums, smem)) {
-        if (threadIdx.x < g.nrhs) result[threadIdx.x] = sums[threadIdx.x];
-    }
+    // no second launch here: the last block to finish adds the rows
+    block_partials(acc, g.nrhs, scr->partials);
+    if (threadIdx.x < g.nrhs) __threadfence();
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&scr->counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    __shared__ double sums[256];
+    sum_partials(scr->partials, gridDim.x, g.nrhs, sums);
+    if (threadIdx.x < g.nrhs) result[threadIdx.x] = sums[threadIdx.x];
 }
 
 } // namespace
