@@ -74,6 +74,7 @@ template <class V> __device__ __forceinline__ void tile_partial(const V &red, co
 __global__ void __launch_bounds__(kFinThreads) k_batch_finish(BatchArgs B, int fin, int fin2)
 {
     __shared__ double sums[kFinThreads];
+    after_previous();
     const BatchLat &L = B.lat[blockIdx.x];
     if (!B.ignore_done && sc(L.scal, S_FLAGS, F_DONE) != 0.0) return;
     const FinIn in = load_fin(L.scal, 1);
@@ -94,6 +95,7 @@ template <int REP, int PHASE>
 __global__ void __launch_bounds__(kTile) k_batch_hop(BatchArgs B)
 {
     using T = dd;
+    after_previous();
     const int tile = blockIdx.x;
     const BatchLat &L = B.lat[find_lat(B.lat, B.nlat, tile)];
     if (!B.ignore_done && sc(L.scal, S_FLAGS, F_DONE) != 0.0) return;
@@ -141,6 +143,7 @@ template <int NC>
 __global__ void __launch_bounds__(kTile) k_batch_p(BatchArgs B)
 {
     using T = dd;
+    after_previous();
     const int tile = blockIdx.x;
     const BatchLat &L = B.lat[find_lat(B.lat, B.nlat, tile)];
     if (sc(L.scal, S_FLAGS, F_DONE) != 0.0) return;
@@ -164,6 +167,7 @@ template <int NC>
 __global__ void __launch_bounds__(kTile) k_batch_start(BatchArgs B)
 {
     using T = dd;
+    after_previous();
     const int tile = blockIdx.x;
     const BatchLat &L = B.lat[find_lat(B.lat, B.nlat, tile)];
     SqAcc<T> red;
@@ -191,6 +195,7 @@ template <int NC>
 __global__ void __launch_bounds__(kTile) k_batch_residual(BatchArgs B)
 {
     using T = dd;
+    after_previous();
     const int tile = blockIdx.x;
     const BatchLat &L = B.lat[find_lat(B.lat, B.nlat, tile)];
     SqAcc<T> red;
@@ -257,13 +262,13 @@ template <int REP>
 hr_status batch_launch_iteration(hr_ctx *ctx, const BatchArgs &B, int grid, cudaStream_t s)
 {
     constexpr int NC = RepTraits<REP>::NC;
-    k_batch_hop<REP, 0><<<grid, kTile, 0, s>>>(B);
-    k_batch_hop<REP, 1><<<grid, kTile, 0, s>>>(B);
-    k_batch_finish<<<B.nlat, kFinThreads, 0, s>>>(B, kFinAlpha, 0);
-    k_batch_hop<REP, 2><<<grid, kTile, 0, s>>>(B);
-    k_batch_hop<REP, 3><<<grid, kTile, 0, s>>>(B);
-    k_batch_finish<<<B.nlat, kFinThreads, 0, s>>>(B, kFinBeta, 0);
-    k_batch_p<NC><<<grid, kTile, 0, s>>>(B);
+    launch_after(k_batch_hop<REP, 0>, true, grid, kTile, 0, s, B);
+    launch_after(k_batch_hop<REP, 1>, true, grid, kTile, 0, s, B);
+    launch_after(k_batch_finish, true, B.nlat, kFinThreads, 0, s, B, kFinAlpha, 0);
+    launch_after(k_batch_hop<REP, 2>, true, grid, kTile, 0, s, B);
+    launch_after(k_batch_hop<REP, 3>, true, grid, kTile, 0, s, B);
+    launch_after(k_batch_finish, true, B.nlat, kFinThreads, 0, s, B, kFinBeta, 0);
+    launch_after(k_batch_p<NC>, true, grid, kTile, 0, s, B);
     return check_launch(ctx, "batched CG iteration");
 }
 
@@ -338,12 +343,12 @@ hr_status batch_true_residual(hr_ctx *ctx, BatchArgs B, int grid, cudaStream_t s
     constexpr int NC = RepTraits<REP>::NC;
     B.use_x = 1;
     B.ignore_done = 1;
-    k_batch_hop<REP, 0><<<grid, kTile, 0, s>>>(B);
-    k_batch_hop<REP, 1><<<grid, kTile, 0, s>>>(B);
-    k_batch_hop<REP, 2><<<grid, kTile, 0, s>>>(B);
-    k_batch_hop<REP, 3><<<grid, kTile, 0, s>>>(B);
-    k_batch_residual<NC><<<grid, kTile, 0, s>>>(B);
-    k_batch_finish<<<B.nlat, kFinThreads, 0, s>>>(B, kFinStore, 0);
+    launch_after(k_batch_hop<REP, 0>, true, grid, kTile, 0, s, B);
+    launch_after(k_batch_hop<REP, 1>, true, grid, kTile, 0, s, B);
+    launch_after(k_batch_hop<REP, 2>, true, grid, kTile, 0, s, B);
+    launch_after(k_batch_hop<REP, 3>, true, grid, kTile, 0, s, B);
+    launch_after(k_batch_residual<NC>, true, grid, kTile, 0, s, B);
+    launch_after(k_batch_finish, true, B.nlat, kFinThreads, 0, s, B, kFinStore, 0);
     return check_launch(ctx, "batched true residual");
 }
 
@@ -439,7 +444,7 @@ hr_status hr_cg_solve_batch(hr_ctx *ctx, int n_lat, const hr_lattice *lats, doub
 
     if (rep == HR_FUND) k_batch_start<2><<<grid, kTile, 0, s>>>(B);
     else k_batch_start<3><<<grid, kTile, 0, s>>>(B);
-    k_batch_finish<<<n_lat, kFinThreads, 0, s>>>(B, kFinBB, kFinInit);
+    launch_after(k_batch_finish, true, n_lat, kFinThreads, 0, s, B, kFinBB, kFinInit);
     hr_status st = check_launch(ctx, "batch start");
     if (st) return st;
 

@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finish(const double *partials, 
                                                         const double *gate, const double *done, FinCond cond)
 {
     __shared__ double sums[kFinThreads];
+    after_previous();
     if ((gate && *gate == 0.0) || (done && *done != 0.0)) {
         // the update may be due from an earlier iteration of the pass
         if (cond.set && blockIdx.x == 0 && threadIdx.x == 0)
@@ -102,6 +103,7 @@ template <int NC, int PP, int PR>
 __global__ void __launch_bounds__(kBS) k_p(Geom g, void *p, const void *r, const double *scal)
 {
     using T = typename Wider<RT<PP>, RT<PR>>::T;
+    after_previous();
     if (sc((double *)scal, S_FLAGS, F_SKIP) != 0.0) return;
     const int nv = g.vh << g.lrhs;
     const T be = Real<T>::from_double(scal[S_BETA * kMaxRhsSlots + thread_rhs(g)]);
@@ -121,6 +123,7 @@ template <int NC, int PS, int PD>
 __global__ void __launch_bounds__(kBS) k_convert(Geom g, const void *src, void *dst, const double *gate)
 {
     using T = typename Wider<RT<PS>, RT<PD>>::T;
+    after_previous();
     if (gate && *gate == 0.0) return;
     const int nv = g.vh << g.lrhs;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nv; j += gridDim.x * blockDim.x) {
@@ -138,6 +141,7 @@ __global__ void __launch_bounds__(kBS) k_residual(Geom g, const void *b, const v
                                                   const double *gate, void *r_lo)
 {
     using T = RT<kF64>;
+    after_previous();
     if (gate && *gate == 0.0) return;
     const int nv = g.vh << g.lrhs;
     SqAcc<T> acc;
@@ -161,6 +165,7 @@ template <int NC, int PH, int PL>
 __global__ void __launch_bounds__(kBS) k_accum(Geom g, void *xhi, void *xlo, const double *gate)
 {
     using T = RT<PH>;
+    after_previous();
     if (gate && *gate == 0.0) return;
     const int nv = g.vh << g.lrhs;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nv; j += gridDim.x * blockDim.x) {
@@ -351,7 +356,7 @@ hr_status finish_sums(hr_ctx *ctx, int nparts, int nrhs, int fin, const double *
 {
     const int want = grid_for((long long)nparts * nrhs, kFinPerBlock, kFinBlocks);
     const int rows = (nparts + want - 1) / want, grid = (nparts + rows - 1) / rows;
-    k_finish<<<grid, kFinThreads, 0, s>>>(ctx->d_partials, nparts, nrhs, rows, ctx->d_partials + kMaxPartials,
+    launch_after(k_finish, (long long)nparts * nrhs <= kEarlySites / 64, grid, kFinThreads, 0, s, ctx->d_partials, nparts, nrhs, rows, ctx->d_partials + kMaxPartials,
                                           ctx->d_counters + C_FIN, ctx->d_scal, fin, gate, done, cond);
     return check_launch(ctx, "reduction finish");
 }
@@ -368,7 +373,7 @@ hr_status blas_p(hr_ctx *ctx, const Geom &g, int rep, int pp, int pr, void *p, c
 {
     int grid = grid_cap(ctx, g);
     if (pp != pr) return set_error(ctx, HR_ERR_UNSUPPORTED, "p update precision combination");
-    HR_DISPATCH_NC(rep, HR_DISPATCH_P(pp, P, (k_p<NC, P, P><<<grid, kBS, 0, s>>>(g, p, r, ctx->d_scal))));
+    HR_DISPATCH_NC(rep, HR_DISPATCH_P(pp, P, launch_after(k_p<NC, P, P>, early_start(g), grid, kBS, 0, s, g, p, r, ctx->d_scal)));
     return check_launch(ctx, "p update");
 }
 
@@ -392,9 +397,9 @@ hr_status blas_residual(hr_ctx *ctx, const Geom &g, int rep, const void *b, cons
     int grid = grid_cap(ctx, g);
     if (!r_lo) plo = kF64;
     if (pax == kF64) {
-        HR_DISPATCH_NC(rep, HR_DISPATCH_P(plo, P, (k_residual<NC, P, kF64><<<grid, kBS, 0, s>>>(g, b, ax, r, ctx->d_partials, gate, r_lo))));
+        HR_DISPATCH_NC(rep, HR_DISPATCH_P(plo, P, launch_after(k_residual<NC, P, kF64>, early_start(g), grid, kBS, 0, s, g, b, ax, r, ctx->d_partials, gate, r_lo)));
     } else if (pax == kF32 && plo == kF16) {
-        HR_DISPATCH_NC(rep, (k_residual<NC, kF16, kF32><<<grid, kBS, 0, s>>>(g, b, ax, r, ctx->d_partials, gate, r_lo)));
+        HR_DISPATCH_NC(rep, launch_after(k_residual<NC, kF16, kF32>, early_start(g), grid, kBS, 0, s, g, b, ax, r, ctx->d_partials, gate, r_lo));
     } else {
         return set_error(ctx, HR_ERR_UNSUPPORTED, "residual precision combination");
     }
@@ -407,9 +412,9 @@ hr_status blas_accum(hr_ctx *ctx, const Geom &g, int rep, int plo, void *xhi, vo
 {
     int grid = grid_cap(ctx, g);
     if (plo == kF32 && phi == kF64) {
-        HR_DISPATCH_NC(rep, (k_accum<NC, kF64, kF32><<<grid, kBS, 0, s>>>(g, xhi, xlo, gate)));
+        HR_DISPATCH_NC(rep, launch_after(k_accum<NC, kF64, kF32>, early_start(g), grid, kBS, 0, s, g, xhi, xlo, gate));
     } else if (plo == kF32 && phi == kF32) {
-        HR_DISPATCH_NC(rep, (k_accum<NC, kF32, kF32><<<grid, kBS, 0, s>>>(g, xhi, xlo, gate)));
+        HR_DISPATCH_NC(rep, launch_after(k_accum<NC, kF32, kF32>, early_start(g), grid, kBS, 0, s, g, xhi, xlo, gate));
     } else {
         return set_error(ctx, HR_ERR_UNSUPPORTED, "accumulate precision");
     }

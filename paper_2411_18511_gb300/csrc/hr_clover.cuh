@@ -45,7 +45,7 @@ template <int NC, int CP, class T> struct CloverReader {
     {
         const int v = r / L::PER_VEC, e = r % L::PER_VEC;
         if (v != loaded) {
-            w = __ldg(base + ((size_t)(i >> 5) * L::NVEC + v) * 32 + (i & 31));
+            w = ld_field(base + ((size_t)(i >> 5) * L::NVEC + v) * 32 + (i & 31));
             loaded = v;
         }
         if constexpr (CP == kF64) {

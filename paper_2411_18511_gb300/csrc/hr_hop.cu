@@ -35,7 +35,7 @@ __device__ __forceinline__ void hop_body(const HopArgs &a)
     using T = typename PrecTraits<PREC>::T;
     // nothing to do (gated off, or the solver converged); a reducing launch
     // leaves its counter clean because no block reaches the reduction
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
     const int stride = gridDim.x * blockDim.x;
@@ -88,13 +88,13 @@ template <int REP, int PREC> struct PlainLaunch {
     static bool run(hr_ctx *ctx, const HopArgs &a, HopChoice c, int grid, cudaStream_t s, hr_status &st)
     {
         if (c.variant == kVarSimpleR96) {
-            if (a.g5_in) k_hop_r96<REP, PREC, 1><<<grid, c.block, 0, s>>>(a);
-            else k_hop_r96<REP, PREC, 0><<<grid, c.block, 0, s>>>(a);
+            if (a.g5_in) launch_after(k_hop_r96<REP, PREC, 1>, early_start(a.g), grid, c.block, 0, s, a);
+            else launch_after(k_hop_r96<REP, PREC, 0>, early_start(a.g), grid, c.block, 0, s, a);
             st = hop_launched(ctx, a, grid, s, "hop kernel (96 registers)");
             return true;
         }
-        if (a.g5_in) k_hop<REP, PREC, 1><<<grid, c.block, 0, s>>>(a);
-        else k_hop<REP, PREC, 0><<<grid, c.block, 0, s>>>(a);
+        if (a.g5_in) launch_after(k_hop<REP, PREC, 1>, early_start(a.g), grid, c.block, 0, s, a);
+        else launch_after(k_hop<REP, PREC, 0>, early_start(a.g), grid, c.block, 0, s, a);
         st = hop_launched(ctx, a, grid, s, "hop kernel");
         return true;
     }
@@ -103,8 +103,8 @@ template <int REP, int PREC> struct PlainLaunch {
 template <int REP, int PREC> struct ClovLaunch {
     static bool run(hr_ctx *ctx, const HopArgs &a, int grid, int block, cudaStream_t s, hr_status &st)
     {
-        if (a.g5_in) k_hop_clov<REP, PREC, 1><<<grid, block, 0, s>>>(a);
-        else k_hop_clov<REP, PREC, 0><<<grid, block, 0, s>>>(a);
+        if (a.g5_in) launch_after(k_hop_clov<REP, PREC, 1>, early_start(a.g), grid, block, 0, s, a);
+        else launch_after(k_hop_clov<REP, PREC, 0>, early_start(a.g), grid, block, 0, s, a);
         st = hop_launched(ctx, a, grid, s, "hop kernel (clover epilogue)");
         return true;
     }

@@ -35,9 +35,9 @@ __device__ __forceinline__ void chunk_term(const HopArgs &a, const float *nrm, i
 {
     if constexpr (PREC == kF16) {
         const uint4 *sp = (const uint4 *)a.in;
-        const uint4 w0 = __ldg(sp + vec_index(jn, 0, 2));
-        const uint4 w1 = __ldg(sp + vec_index(jn, 1, 2));
-        const float sc = __ldg(nrm + jn);
+        const uint4 w0 = ld_field(sp + vec_index(jn, 0, 2));
+        const uint4 w1 = ld_field(sp + vec_index(jn, 1, 2));
+        const float sc = ld_field(nrm + jn);
         h16_compute<MU, FWD, FIRST, NEG>(w0, w1, sc, q, acc);
     } else {
         cpx<float> s[4][2];
@@ -60,7 +60,7 @@ __device__ __forceinline__ void chunk_body(const HopArgs &a)
 {
     constexpr int C = 1 << LC;
     constexpr bool NEG = G5IN != 0;
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const Geom &g = a.g;
     const int l = g.lrhs, lm = l - LC; // N / C = 2^lm threads per site
     const int nt = g.vh << lm;
@@ -125,8 +125,8 @@ template <int PREC>
 void launch_chunk(const HopArgs &a, int lc, int grid, int block, cudaStream_t s)
 {
     const bool g5 = a.g5_in != 0;
-    if (lc == 1) (g5 ? k_hop_chunk<PREC, 1, 1> : k_hop_chunk<PREC, 1, 0>)<<<grid, block, 0, s>>>(a);
-    else (g5 ? k_hop_chunk<PREC, 2, 1> : k_hop_chunk<PREC, 2, 0>)<<<grid, block, 0, s>>>(a);
+    if (lc == 1) launch_after(g5 ? k_hop_chunk<PREC, 1, 1> : k_hop_chunk<PREC, 1, 0>, early_start(a.g), grid, block, 0, s, a);
+    else launch_after(g5 ? k_hop_chunk<PREC, 2, 1> : k_hop_chunk<PREC, 2, 0>, early_start(a.g), grid, block, 0, s, a);
 }
 
 } // namespace

@@ -37,6 +37,14 @@ struct HopArgs {
     FinCond cond;          // host side: condition handle the finishing launch sets
 };
 
+// Waits for the launches before; nothing to do when gated off, or the solver
+// converged (a reducing launch then leaves no rows, and its finishing launch skips).
+__device__ __forceinline__ bool hop_skipped(const HopArgs &a)
+{
+    after_previous();
+    return (a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0);
+}
+
 // the grid of a hop kernel of one thread per item: a reducing launch is capped
 // so that its rows of partial sums fit the context's scratch
 inline int hop_grid(const HopArgs &a, long long n, int block)

@@ -35,9 +35,9 @@ __device__ __forceinline__ void h16_term(const HopArgs &a, const float *nrm, int
                                          cpx<float> (&acc)[4][2])
 {
     const uint4 *sp = (const uint4 *)a.in;
-    const uint4 w0 = __ldg(sp + vec_index(jn, 0, 2));
-    const uint4 w1 = __ldg(sp + vec_index(jn, 1, 2));
-    const float sc = __ldg(nrm + jn);
+    const uint4 w0 = ld_field(sp + vec_index(jn, 0, 2));
+    const uint4 w1 = ld_field(sp + vec_index(jn, 1, 2));
+    const float sc = ld_field(nrm + jn);
     float q[4];
     load_quat<kF16>(a.gauge, a.g.nblk_g, link_par, MU, site_link, q);
     h16_compute<MU, FWD, FIRST, NEG>(w0, w1, sc, q, acc);
@@ -56,7 +56,7 @@ template <int G5IN>
 __device__ __forceinline__ void h16_body(const HopArgs &a)
 {
     constexpr bool NEG = G5IN != 0;
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
     const int stride = gridDim.x * blockDim.x;
@@ -98,10 +98,10 @@ __device__ __forceinline__ void h16_fetch(const HopArgs &a, const float *nrm, in
     const int sl = FWD ? i : nb.bwd[MU];
     const int lp = FWD ? a.p : 1 - a.p;
     const uint4 *sp = (const uint4 *)a.in;
-    o.w0 = __ldg(sp + vec_index(jn, 0, 2));
-    o.w1 = __ldg(sp + vec_index(jn, 1, 2));
-    o.sc = __ldg(nrm + jn);
-    o.q = __ldg((const uint2 *)quat_addr<kF16>(a.gauge, a.g.nblk_g, lp, MU, sl, 0));
+    o.w0 = ld_field(sp + vec_index(jn, 0, 2));
+    o.w1 = ld_field(sp + vec_index(jn, 1, 2));
+    o.sc = ld_field(nrm + jn);
+    o.q = ld_field((const uint2 *)quat_addr<kF16>(a.gauge, a.g.nblk_g, lp, MU, sl, 0));
 }
 
 // direction K from buf[K % (D + 1)] after queueing the loads of direction K + D
@@ -121,7 +121,7 @@ template <int D, int G5IN>
 __device__ __forceinline__ void h16p_body(const HopArgs &a)
 {
     constexpr bool NEG = G5IN != 0;
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
     const int stride = gridDim.x * blockDim.x;
@@ -185,7 +185,7 @@ __device__ __forceinline__ void h16s_body(const HopArgs &a)
     using S = Stage<kRepFund, kF16>;
     constexpr bool NEG = G5IN != 0;
     extern __shared__ uint4 h16_stage_mem[];
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
     const int stride = gridDim.x * blockDim.x;
@@ -241,16 +241,16 @@ bool launch_hop_half(hr_ctx *ctx, const Geom &, int rep, int prec, const HopArgs
             attr_set = true;
         }
         const size_t sm = S::smem_bytes(c.block);
-        if (c.variant == kVarHalfStagedR64) (g5 ? k_hop_h16s_r64<1> : k_hop_h16s_r64<0>)<<<grid, c.block, sm, s>>>(a);
-        else (g5 ? k_hop_h16s<1> : k_hop_h16s<0>)<<<grid, c.block, sm, s>>>(a);
+        if (c.variant == kVarHalfStagedR64) launch_after(g5 ? k_hop_h16s_r64<1> : k_hop_h16s_r64<0>, early_start(a.g), grid, c.block, sm, s, a);
+        else launch_after(g5 ? k_hop_h16s<1> : k_hop_h16s<0>, early_start(a.g), grid, c.block, sm, s, a);
     } else if (c.variant == kVarHalfR64) {
-        (g5 ? k_hop_h16_r64<1> : k_hop_h16_r64<0>)<<<grid, c.block, 0, s>>>(a);
+        launch_after(g5 ? k_hop_h16_r64<1> : k_hop_h16_r64<0>, early_start(a.g), grid, c.block, 0, s, a);
     } else if (c.variant == kVarHalfPrefetch) {
-        (g5 ? k_hop_h16p_r80<1> : k_hop_h16p_r80<0>)<<<grid, c.block, 0, s>>>(a);
+        launch_after(g5 ? k_hop_h16p_r80<1> : k_hop_h16p_r80<0>, early_start(a.g), grid, c.block, 0, s, a);
     } else if (c.variant == kVarHalfPrefetch2) {
-        (g5 ? k_hop_h16p2_r96<1> : k_hop_h16p2_r96<0>)<<<grid, c.block, 0, s>>>(a);
+        launch_after(g5 ? k_hop_h16p2_r96<1> : k_hop_h16p2_r96<0>, early_start(a.g), grid, c.block, 0, s, a);
     } else {
-        (g5 ? k_hop_h16<1> : k_hop_h16<0>)<<<grid, c.block, 0, s>>>(a);
+        launch_after(g5 ? k_hop_h16<1> : k_hop_h16<0>, early_start(a.g), grid, c.block, 0, s, a);
     }
     st = hop_launched(ctx, a, grid, s, "binary16 hop kernel (half2 projection)");
     return true;

@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(256) k_hop_loop(HopArgs a)
     using S = Stage<REP, PREC>;
     constexpr int NC = S::NC;
     extern __shared__ uint4 stage_mem[];
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
     const int stride = gridDim.x * blockDim.x;
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(256) k_hop_sw(HopArgs a)
     using S = Stage<REP, PREC>;
     constexpr int NC = S::NC;
     extern __shared__ uint4 stage_mem[];
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
     const int stride = gridDim.x * blockDim.x;
@@ -328,7 +328,7 @@ template <int REP, int PREC> struct Launch {
             const size_t sm = Stage<REP, PREC>::smem_bytes(c.block);
             const int sm_max = (int)Stage<REP, PREC>::smem_bytes(256);
             if (c.variant == kVarLoop) {
-                k_hop_loop<REP, PREC, false><<<grid, c.block, 0, s>>>(a);
+                launch_after(k_hop_loop<REP, PREC, false>, early_start(a.g), grid, c.block, 0, s, a);
                 st = hop_launched(ctx, a, grid, s, "looped hop kernel");
                 return true;
             }
@@ -339,12 +339,12 @@ template <int REP, int PREC> struct Launch {
                                          sm_max);
                     attr_set = true;
                 }
-                k_hop_loop<REP, PREC, true><<<grid, c.block, sm, s>>>(a);
+                launch_after(k_hop_loop<REP, PREC, true>, early_start(a.g), grid, c.block, sm, s, a);
                 st = hop_launched(ctx, a, grid, s, "looped staged hop kernel");
                 return true;
             }
             if (c.variant == kVarSwitch) {
-                k_hop_sw<REP, PREC, false><<<grid, c.block, 0, s>>>(a);
+                launch_after(k_hop_sw<REP, PREC, false>, early_start(a.g), grid, c.block, 0, s, a);
                 st = hop_launched(ctx, a, grid, s, "switched hop kernel");
                 return true;
             }
@@ -355,7 +355,7 @@ template <int REP, int PREC> struct Launch {
                                          sm_max);
                     attr_set2 = true;
                 }
-                k_hop_sw<REP, PREC, true><<<grid, c.block, sm, s>>>(a);
+                launch_after(k_hop_sw<REP, PREC, true>, early_start(a.g), grid, c.block, sm, s, a);
                 st = hop_launched(ctx, a, grid, s, "switched staged hop kernel");
                 return true;
             }

@@ -59,9 +59,9 @@ __device__ __forceinline__ void p2_site(const HopArgs &a, const float *nrm, int 
     constexpr int F = NEG ? 2 : 0;
     if constexpr (PREC == kF16) {
         const uint4 *sp = (const uint4 *)a.in;
-        const uint4 w0 = __ldg(sp + vec_index(jn, 0, 2));
-        const uint4 w1 = __ldg(sp + vec_index(jn, 1, 2));
-        sc = __ldg(nrm + jn);
+        const uint4 w0 = ld_field(sp + vec_index(jn, 0, 2));
+        const uint4 w1 = ld_field(sp + vec_index(jn, 1, 2));
+        sc = ld_field(nrm + jn);
         const uint32_t u[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
         __half2 h0re, h0im, h1re, h1im;
         h2_project<(D::c0 + F) & 3>(as_h2(u[0]), as_h2(u[1]), as_h2(u[2 * D::pi0]), as_h2(u[2 * D::pi0 + 1]), h0re,
@@ -76,7 +76,7 @@ __device__ __forceinline__ void p2_site(const HopArgs &a, const float *nrm, int 
         const float4 *sp = (const float4 *)a.in;
         float4 s[4];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) s[v] = __ldg(sp + vec_index(jn, v, 4));
+        for (int v = 0; v < 4; ++v) s[v] = ld_field(sp + vec_index(jn, v, 4));
         sc = 1.f;
         f32_project<(D::c0 + F) & 3>(s[0], s[D::pi0], h.re[0], h.im[0]);
         f32_project<(D::c1 + F) & 3>(s[1], s[D::pi1], h.re[1], h.im[1]);
@@ -169,7 +169,7 @@ template <int PREC, int G5IN>
 __device__ __forceinline__ void p2_body(const HopArgs &a)
 {
     constexpr bool NEG = G5IN != 0;
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const K2 k = make_k2(a.unit, a.nil);
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
@@ -217,8 +217,8 @@ template <int PREC>
 void launch_p2(const HopArgs &a, HopChoice c, int grid, cudaStream_t s)
 {
     const bool g5 = a.g5_in != 0;
-    if (c.variant == kVarPairSitesR96) (g5 ? k_hop_p2_r96<PREC, 1> : k_hop_p2_r96<PREC, 0>)<<<grid, c.block, 0, s>>>(a);
-    else (g5 ? k_hop_p2<PREC, 1> : k_hop_p2<PREC, 0>)<<<grid, c.block, 0, s>>>(a);
+    if (c.variant == kVarPairSitesR96) launch_after(g5 ? k_hop_p2_r96<PREC, 1> : k_hop_p2_r96<PREC, 0>, early_start(a.g), grid, c.block, 0, s, a);
+    else launch_after(g5 ? k_hop_p2<PREC, 1> : k_hop_p2<PREC, 0>, early_start(a.g), grid, c.block, 0, s, a);
 }
 
 } // namespace

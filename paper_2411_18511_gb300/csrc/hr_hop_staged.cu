@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(256) k_hop_staged(HopArgs a)
     using S = Stage<REP, PREC>;
     constexpr int NC = S::NC;
     extern __shared__ uint4 stage_mem[];
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
     const int stride = gridDim.x * blockDim.x;
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(256) k_hop_pf(HopArgs a)
 {
     using T = typename PrecTraits<PREC>::T;
     constexpr int NC = RepTraits<REP>::NC;
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
     const int stride = gridDim.x * blockDim.x;
@@ -199,12 +199,12 @@ template <int REP, int PREC> struct Launch {
                                          (int)Stage<REP, PREC>::smem_bytes(256));
                     attr_set = true;
                 }
-                k_hop_staged<REP, PREC><<<grid, c.block, sm, s>>>(a);
+                launch_after(k_hop_staged<REP, PREC>, early_start(a.g), grid, c.block, sm, s, a);
                 st = hop_launched(ctx, a, grid, s, "staged hop kernel");
                 return true;
             }
             if (c.variant == kVarPrefetch) {
-                k_hop_pf<REP, PREC><<<grid, c.block, 0, s>>>(a);
+                launch_after(k_hop_pf<REP, PREC>, early_start(a.g), grid, c.block, 0, s, a);
                 st = hop_launched(ctx, a, grid, s, "prefetching hop kernel");
                 return true;
             }

@@ -62,7 +62,7 @@ __device__ __forceinline__ void hop_tile_body(const HopArgs &a)
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(tile_smem);
     const uint4 *stage = reinterpret_cast<const uint4 *>(tile_smem + S::kHead);
     __shared__ int s_landed;
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const Geom &g = a.g;
     const int l = g.lrhs;
     const int nv = g.vh << l;
@@ -178,11 +178,11 @@ template <int REP, int PREC> struct Launch {
             const long long ntiles = (nv + c.block - 1) / c.block;
             const int tgrid = hop_grid(a, ntiles, 1);
             if (c.variant == kVarTile) {
-                if (a.g5_in) k_hop_tile<REP, PREC, 1><<<tgrid, c.block, sm, s>>>(a);
-                else k_hop_tile<REP, PREC, 0><<<tgrid, c.block, sm, s>>>(a);
+                if (a.g5_in) launch_after(k_hop_tile<REP, PREC, 1>, early_start(a.g), tgrid, c.block, sm, s, a);
+                else launch_after(k_hop_tile<REP, PREC, 0>, early_start(a.g), tgrid, c.block, sm, s, a);
             } else {
-                if (a.g5_in) k_hop_tile_r96<REP, PREC, 1><<<tgrid, c.block, sm, s>>>(a);
-                else k_hop_tile_r96<REP, PREC, 0><<<tgrid, c.block, sm, s>>>(a);
+                if (a.g5_in) launch_after(k_hop_tile_r96<REP, PREC, 1>, early_start(a.g), tgrid, c.block, sm, s, a);
+                else launch_after(k_hop_tile_r96<REP, PREC, 0>, early_start(a.g), tgrid, c.block, sm, s, a);
             }
             st = hop_launched(ctx, a, tgrid, s, "tiled hop kernel");
             return true;

@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(128) k_hop_twist(HopArgs a)
 {
     using T = typename PrecTraits<PREC>::T;
     constexpr int NC = RepTraits<REP>::NC;
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
     const int stride = gridDim.x * blockDim.x;
@@ -166,10 +166,10 @@ __device__ __forceinline__ void x2t_term(const HopArgs &a, const K2 &k, int site
     const float4 *sp = (const float4 *)a.in;
     float4 w[8];
 #pragma unroll
-    for (int v = 0; v < 8; ++v) w[v] = __ldg(sp + vec_index(j_nb, v, 8));
+    for (int v = 0; v < 8; ++v) w[v] = ld_field(sp + vec_index(j_nb, v, 8));
     const float4 *qp = link_base<float4>(a.gauge, a.g.nblk_g, link_par, MU, 2);
-    const float4 qh = __ldg(qp + vec_index(site_link, 0, 2));
-    const float4 ql = __ldg(qp + vec_index(site_link, 1, 2));
+    const float4 qh = ld_field(qp + vec_index(site_link, 0, 2));
+    const float4 ql = ld_field(qp + vec_index(site_link, 1, 2));
     cdd2 sv[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
@@ -210,7 +210,7 @@ template <int G5IN, bool CLOV>
 __device__ __forceinline__ void x2t_body(const HopArgs &a)
 {
     constexpr bool NEG = G5IN != 0;
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const K2 k = make_k2(a.unit, a.nil);
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
@@ -242,13 +242,13 @@ template <int REP, int PREC> struct TwistLaunch {
     {
         if constexpr (REP == kRepFund && PREC == kF64) {
             const bool g5 = a.g5_in != 0, clov = a.clov_mode != kClovNone;
-            if (clov) (g5 ? k_hop_x2t<1, true> : k_hop_x2t<0, true>)<<<grid, kTwistBlock, 0, s>>>(a);
-            else (g5 ? k_hop_x2t<1, false> : k_hop_x2t<0, false>)<<<grid, kTwistBlock, 0, s>>>(a);
+            if (clov) launch_after(g5 ? k_hop_x2t<1, true> : k_hop_x2t<0, true>, early_start(a.g), grid, kTwistBlock, 0, s, a);
+            else launch_after(g5 ? k_hop_x2t<1, false> : k_hop_x2t<0, false>, early_start(a.g), grid, kTwistBlock, 0, s, a);
             st = hop_launched(ctx, a, grid, s, "paired hop kernel (twisted boundaries)");
             return true;
         }
-        if (a.clov_mode != kClovNone) k_hop_twist<REP, PREC, true><<<grid, kTwistBlock, 0, s>>>(a);
-        else k_hop_twist<REP, PREC, false><<<grid, kTwistBlock, 0, s>>>(a);
+        if (a.clov_mode != kClovNone) launch_after(k_hop_twist<REP, PREC, true>, early_start(a.g), grid, kTwistBlock, 0, s, a);
+        else launch_after(k_hop_twist<REP, PREC, false>, early_start(a.g), grid, kTwistBlock, 0, s, a);
         st = hop_launched(ctx, a, grid, s, "hop kernel (twisted boundaries)");
         return true;
     }

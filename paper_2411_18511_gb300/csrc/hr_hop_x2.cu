@@ -45,7 +45,7 @@ __device__ __forceinline__ void x2s_body(const HopArgs &a)
     static_assert(S::NSLOT == 10, "8 spinor + 2 link vectors per direction");
     constexpr bool NEG = G5IN != 0;
     extern __shared__ uint4 x2_stage_mem[];
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const K2 k = make_k2(a.unit, a.nil);
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
@@ -82,7 +82,7 @@ __device__ __forceinline__ void x2_body(const HopArgs &a)
 {
     using T = dd;
     constexpr bool NEG = G5IN != 0;
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const K2 k = make_k2(a.unit, a.nil);
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
@@ -223,7 +223,7 @@ __device__ __forceinline__ void f2_load_site(const HopArgs &a, int j, float2 (&s
         const float4 *p = (const float4 *)a.in;
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            const float4 w = __ldg(p + vec_index(j, v, 4));
+            const float4 w = ld_field(p + vec_index(j, v, 4));
             sv[2 * v] = make_float2(w.x, w.y);
             sv[2 * v + 1] = make_float2(w.z, w.w);
         }
@@ -232,12 +232,12 @@ __device__ __forceinline__ void f2_load_site(const HopArgs &a, int j, float2 (&s
         const uint4 *p = (const uint4 *)a.in;
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
-            const uint4 w = __ldg(p + vec_index(j, v, 2));
+            const uint4 w = ld_field(p + vec_index(j, v, 2));
             const uint32_t u[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
             for (int q = 0; q < 4; ++q) sv[4 * v + q] = __half22float2(*reinterpret_cast<const __half2 *>(&u[q]));
         }
-        sc = __ldg((const float *)((const char *)a.in + SpinorLayout<2, kF16>::data_bytes(a.g.nblk_s)) + j);
+        sc = ld_field((const float *)((const char *)a.in + SpinorLayout<2, kF16>::data_bytes(a.g.nblk_s)) + j);
     }
 }
 
@@ -269,7 +269,7 @@ template <int PREC, int G5IN>
 __device__ __forceinline__ void f2_body(const HopArgs &a)
 {
     constexpr bool NEG = G5IN != 0;
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const K2 k = make_k2(a.unit, a.nil);
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
@@ -348,7 +348,7 @@ __device__ __forceinline__ void f2s_body(const HopArgs &a)
     using S = Stage<kRepFund, PREC>;
     constexpr bool NEG = G5IN != 0;
     extern __shared__ uint4 f2_stage_mem[];
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const K2 k = make_k2(a.unit, a.nil);
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
@@ -546,7 +546,7 @@ __device__ __forceinline__ void x2a_link(const HopArgs &a, const K2 &k, int link
 {
     if constexpr (REP == kRepAdj) {
         const float4 *q = link_base<float4>(a.gauge, a.g.nblk_g, link_par, mu, 2) + vec_index(site_link, 0, 2);
-        quat_to_adj_x2(k, __ldg(q), __ldg(q + 32), R);
+        quat_to_adj_x2(k, ld_field(q), ld_field(q + 32), R);
     } else {
         load_mat<kF64>(a.gauge, a.g.nblk_g, link_par, mu, site_link, R);
     }
@@ -559,7 +559,7 @@ __device__ __forceinline__ void x2a_term(const HopArgs &a, const K2 &k, int site
     const float4 *sp = (const float4 *)a.in;
     float4 w[12];
 #pragma unroll
-    for (int v = 0; v < 12; ++v) w[v] = __ldg(sp + vec_index(j_nb, v, 12));
+    for (int v = 0; v < 12; ++v) w[v] = ld_field(sp + vec_index(j_nb, v, 12));
     dd R[3][3];
     x2a_link<REP>(a, k, link_par, MU, site_link, R);
     x2a_compute<MU, FWD, FIRST, NEG>(k, w, R, acc);
@@ -580,7 +580,7 @@ template <int REP, int G5IN>
 __device__ __forceinline__ void x2a_body(const HopArgs &a)
 {
     constexpr bool NEG = G5IN != 0;
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const K2 k = make_k2(a.unit, a.nil);
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
@@ -639,7 +639,7 @@ __device__ __forceinline__ void x2as_body(const HopArgs &a)
     static_assert(S::NSLOT == 14, "12 spinor + 2 link vectors per direction");
     constexpr bool NEG = G5IN != 0;
     extern __shared__ uint4 x2a_stage_mem[];
-    if ((a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0)) return;
+    if (hop_skipped(a)) return;
     const K2 k = make_k2(a.unit, a.nil);
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
@@ -693,10 +693,10 @@ template <int REP, int PREC> struct Launch {
             const size_t sm = S::smem_bytes(c.block);
             const bool g5 = a.g5_in != 0;
             switch (c.variant) {
-            case kVarPairedStaged: (g5 ? k_hop_x2s<1> : k_hop_x2s<0>)<<<grid, c.block, sm, s>>>(a); break;
-            case kVarPairedStagedR96: (g5 ? k_hop_x2s_r96<1> : k_hop_x2s_r96<0>)<<<grid, c.block, sm, s>>>(a); break;
-            case kVarPairedR96: (g5 ? k_hop_x2_r96<1> : k_hop_x2_r96<0>)<<<grid, c.block, 0, s>>>(a); break;
-            default: (g5 ? k_hop_x2<1> : k_hop_x2<0>)<<<grid, c.block, 0, s>>>(a); break;
+            case kVarPairedStaged: launch_after(g5 ? k_hop_x2s<1> : k_hop_x2s<0>, early_start(a.g), grid, c.block, sm, s, a); break;
+            case kVarPairedStagedR96: launch_after(g5 ? k_hop_x2s_r96<1> : k_hop_x2s_r96<0>, early_start(a.g), grid, c.block, sm, s, a); break;
+            case kVarPairedR96: launch_after(g5 ? k_hop_x2_r96<1> : k_hop_x2_r96<0>, early_start(a.g), grid, c.block, 0, s, a); break;
+            default: launch_after(g5 ? k_hop_x2<1> : k_hop_x2<0>, early_start(a.g), grid, c.block, 0, s, a); break;
             }
             st = hop_launched(ctx, a, grid, s, "paired hop kernel");
             return true;
@@ -706,7 +706,7 @@ template <int REP, int PREC> struct Launch {
             const bool g5 = a.g5_in != 0;
             if (c.variant == kVarPairedR96) {
                 // for the adjoint: the form with 168 registers
-                (g5 ? k_hop_x2a_big<REP, 1> : k_hop_x2a_big<REP, 0>)<<<grid, c.block, 0, s>>>(a);
+                launch_after(g5 ? k_hop_x2a_big<REP, 1> : k_hop_x2a_big<REP, 0>, early_start(a.g), grid, c.block, 0, s, a);
                 st = hop_launched(ctx, a, grid, s, "paired adjoint hop kernel (168 registers)");
                 return true;
             }
@@ -720,12 +720,12 @@ template <int REP, int PREC> struct Launch {
                                                  (int)S::smem_bytes(256));
                         attr_set = true;
                     }
-                    (g5 ? k_hop_x2as<1> : k_hop_x2as<0>)<<<grid, c.block, S::smem_bytes(c.block), s>>>(a);
+                    launch_after(g5 ? k_hop_x2as<1> : k_hop_x2as<0>, early_start(a.g), grid, c.block, S::smem_bytes(c.block), s, a);
                     st = hop_launched(ctx, a, grid, s, "paired adjoint hop kernel");
                     return true;
                 }
             }
-            (g5 ? k_hop_x2a<REP, 1> : k_hop_x2a<REP, 0>)<<<grid, c.block, 0, s>>>(a);
+            launch_after(g5 ? k_hop_x2a<REP, 1> : k_hop_x2a<REP, 0>, early_start(a.g), grid, c.block, 0, s, a);
             st = hop_launched(ctx, a, grid, s, "paired adjoint hop kernel");
             return true;
         } else if constexpr (REP == kRepFund) {
@@ -741,9 +741,9 @@ template <int REP, int PREC> struct Launch {
             }
             const bool g5 = a.g5_in != 0;
             if (c.variant == kVarPairedStaged)
-                (g5 ? k_hop_f2s<PREC, 1> : k_hop_f2s<PREC, 0>)<<<grid, c.block, S::smem_bytes(c.block), s>>>(a);
+                launch_after(g5 ? k_hop_f2s<PREC, 1> : k_hop_f2s<PREC, 0>, early_start(a.g), grid, c.block, S::smem_bytes(c.block), s, a);
             else
-                (g5 ? k_hop_f2<PREC, 1> : k_hop_f2<PREC, 0>)<<<grid, c.block, 0, s>>>(a);
+                launch_after(g5 ? k_hop_f2<PREC, 1> : k_hop_f2<PREC, 0>, early_start(a.g), grid, c.block, 0, s, a);
             st = hop_launched(ctx, a, grid, s, "paired hop kernel");
             return true;
         }
@@ -764,7 +764,7 @@ void launch_hop_clover_paired(hr_ctx *ctx, const HopArgs &a, int grid, int block
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_bytes(256));
         attr_set = true;
     }
-    (a.g5_in ? k_hop_x2s_clov<1> : k_hop_x2s_clov<0>)<<<grid, block, S::smem_bytes(block), s>>>(a);
+    launch_after(a.g5_in ? k_hop_x2s_clov<1> : k_hop_x2s_clov<0>, early_start(a.g), grid, block, S::smem_bytes(block), s, a);
     st = hop_launched(ctx, a, grid, s, "paired hop kernel (clover epilogue)");
 }
 

@@ -214,10 +214,10 @@ __device__ __forceinline__ void x2_term(const HopArgs &a, const K2 &k, int site_
     const float4 *sp = (const float4 *)a.in;
     float4 w[8];
 #pragma unroll
-    for (int v = 0; v < 8; ++v) w[v] = __ldg(sp + vec_index(j_nb, v, 8));
+    for (int v = 0; v < 8; ++v) w[v] = ld_field(sp + vec_index(j_nb, v, 8));
     const float4 *qp = link_base<float4>(a.gauge, a.g.nblk_g, link_par, MU, 2);
-    const float4 qh = __ldg(qp + vec_index(site_link, 0, 2));
-    const float4 ql = __ldg(qp + vec_index(site_link, 1, 2));
+    const float4 qh = ld_field(qp + vec_index(site_link, 0, 2));
+    const float4 ql = ld_field(qp + vec_index(site_link, 1, 2));
     x2_compute<MU, FWD, FIRST, NEG>(k, w, qh, ql, acc);
 }
 

@@ -306,6 +306,17 @@ __device__ __forceinline__ unsigned pack_range_flags(double v)
     return fabs(v) > 0x1p120 ? kPackAboveRange : 0u;
 }
 
+// ---------------------------------------------------------------- launch order
+// First statement of every kernel launched by launch_after (hr_host.h): waits until
+// the previous kernel of the stream has finished and its writes are visible.  (No
+// effect in a kernel launched the plain way.)  No kernel asks for an earlier start
+// of the next one: blocks that wait in the slots of an SM slowed large lattices by
+// 3 to 15 %.
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// a vector of a field or of links: a plain load, not ld.global.nc -- a kernel may
+// be resident while the one before it still writes them
+template <class V> __device__ __forceinline__ V ld_field(const V *p) { return *p; }
+
 // ---------------------------------------------------------------- layouts
 
 template <int PREC> struct PrecTraits;
@@ -439,21 +450,21 @@ __device__ __forceinline__ void load_spinor(const void *base, int nblk, int j, c
         const float4 *p = (const float4 *)base;
         float4 w[NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) w[v] = __ldg(p + vec_index(j, v, NV));
+        for (int v = 0; v < NV; ++v) w[v] = ld_field(p + vec_index(j, v, NV));
         f64_from_vecs<NC>(w, s);
     } else if constexpr (PREC == kF32) {
         const float4 *p = (const float4 *)base;
         float r[8 * NC];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) float4_to_floats(__ldg(p + vec_index(j, v, NV)), &r[4 * v]);
+        for (int v = 0; v < NV; ++v) float4_to_floats(ld_field(p + vec_index(j, v, NV)), &r[4 * v]);
         values_from_packed<NC>(r, 1.f, s);
     } else {
         const uint4 *p = (const uint4 *)base;
         const float *nrm = (const float *)((const char *)base + L::data_bytes(nblk));
-        const float sc = __ldg(nrm + j);
+        const float sc = ld_field(nrm + j);
         float r[8 * NC];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) halves_to_floats(__ldg(p + vec_index(j, v, NV)), &r[8 * v]);
+        for (int v = 0; v < NV; ++v) halves_to_floats(ld_field(p + vec_index(j, v, NV)), &r[8 * v]);
         values_from_packed<NC>(r, sc, s);
     }
 }
@@ -468,10 +479,10 @@ __device__ __forceinline__ void load_spinor_raw(const void *base, int nblk, int 
         using L = SpinorLayout<NC, PREC>;
         constexpr int NV = L::NVEC;
         const uint4 *p = (const uint4 *)base;
-        sc = __ldg((const float *)((const char *)base + L::data_bytes(nblk)) + j);
+        sc = ld_field((const float *)((const char *)base + L::data_bytes(nblk)) + j);
         float r[8 * NC];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) halves_to_floats(__ldg(p + vec_index(j, v, NV)), &r[8 * v]);
+        for (int v = 0; v < NV; ++v) halves_to_floats(ld_field(p + vec_index(j, v, NV)), &r[8 * v]);
         values_from_packed<NC>(r, 1.f, s);
     } else {
         sc = 1.f;
@@ -559,8 +570,8 @@ __device__ __forceinline__ void load_quat(const void *base, int nblk_g, int p, i
     if constexpr (PREC == kF64) {
         // (a0.h, a1.h, a2.h, a3.h) then (a0.l, a1.l, a2.l, a3.l)
         const float4 *q = link_base<float4>(base, nblk_g, p, mu, 2);
-        float4 hi = __ldg(q + vec_index(i, 0, 2));
-        float4 lo = __ldg(q + vec_index(i, 1, 2));
+        float4 hi = ld_field(q + vec_index(i, 0, 2));
+        float4 lo = ld_field(q + vec_index(i, 1, 2));
         if constexpr (std::is_same<T, dd>::value) {
             a[0] = dd(hi.x, lo.x); a[1] = dd(hi.y, lo.y); a[2] = dd(hi.z, lo.z); a[3] = dd(hi.w, lo.w);
         } else {
@@ -570,11 +581,11 @@ __device__ __forceinline__ void load_quat(const void *base, int nblk_g, int p, i
             a[3] = Real<T>::from_double(dd_to_double(dd(hi.w, lo.w)));
         }
     } else if constexpr (PREC == kF32) {
-        float4 w = __ldg(link_base<float4>(base, nblk_g, p, mu, 1) + i);
+        float4 w = ld_field(link_base<float4>(base, nblk_g, p, mu, 1) + i);
         a[0] = Real<T>::from_float(w.x); a[1] = Real<T>::from_float(w.y);
         a[2] = Real<T>::from_float(w.z); a[3] = Real<T>::from_float(w.w);
     } else {
-        uint2 w = __ldg(link_base<uint2>(base, nblk_g, p, mu, 1) + i);
+        uint2 w = ld_field(link_base<uint2>(base, nblk_g, p, mu, 1) + i);
         float2 f0 = __half22float2(*reinterpret_cast<__half2 *>(&w.x));
         float2 f1 = __half22float2(*reinterpret_cast<__half2 *>(&w.y));
         a[0] = Real<T>::from_float(f0.x); a[1] = Real<T>::from_float(f0.y);
@@ -737,11 +748,11 @@ __device__ __forceinline__ void load_mat(const void *base, int nblk_g, int p, in
         const int idx = vec_index(i, e, 9);
         T v;
         if constexpr (PREC == kF64) {
-            float2 w = __ldg(link_base<float2>(base, nblk_g, p, mu, 9) + idx);
+            float2 w = ld_field(link_base<float2>(base, nblk_g, p, mu, 9) + idx);
             if constexpr (std::is_same<T, dd>::value) v = dd(w.x, w.y);
             else v = Real<T>::from_double(dd_to_double(dd(w.x, w.y)));
         } else if constexpr (PREC == kF32) {
-            v = Real<T>::from_float(__ldg(link_base<float>(base, nblk_g, p, mu, 9) + idx));
+            v = Real<T>::from_float(ld_field(link_base<float>(base, nblk_g, p, mu, 9) + idx));
         } else {
             v = Real<T>::from_float(__half2float(link_base<__half>(base, nblk_g, p, mu, 9)[idx]));
         }
