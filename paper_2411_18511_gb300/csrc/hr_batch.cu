@@ -91,8 +91,10 @@ __global__ void __launch_bounds__(kFinThreads) k_batch_finish(BatchArgs B, int f
 // In the recurrence phase 3 updates x += alpha p, r -= alpha q with q in
 // registers and reduces |r|^2: a separate pass took 95 us for the 530 k sites of
 // twelve lattices (8^4 .. 24^4).
+// Registers: 96 and five blocks an SM without the late operands, 128 and four
+// with them (the compiler's own 134 leave three).
 template <int REP, int PHASE>
-__global__ void __launch_bounds__(kTile) k_batch_hop(BatchArgs B)
+__global__ void __launch_bounds__(kTile, REP != kRepFund ? 3 : PHASE & 1 ? 4 : 5) k_batch_hop(BatchArgs B)
 {
     using T = dd;
     after_previous();
