@@ -157,6 +157,23 @@ HR_HD inline fx fx_from_double(double x)
     const long long sg = (long long)u >> 63;
     return fx_split((long long)(t ^ (unsigned long long)sg) - sg);
 }
+// Digits of a double with |x| < 2, cut instead of split at the middle (|l| < 2^28):
+// 13 instead of 20 integer instructions
+HR_HD inline fx fx_from_unit(double x)
+{
+    const unsigned long long u = fx_dbits(x);
+    const unsigned long long m = ((u & 0xfffffffffffffULL) | 0x10000000000000ULL) << 4; // x 2^56 = m >> (1023 - e)
+    const int s = 1023 - ((int)(u >> 52) & 0x7ff), sg = (int)(u >> 32) >> 31;
+#ifdef __CUDA_ARCH__
+    unsigned long long th, tl;
+    asm("shr.u64 %0, %1, %2;" : "=l"(th) : "l"(m), "r"(s + 28)); // clamps at 64
+    asm("shr.u64 %0, %1, %2;" : "=l"(tl) : "l"(m), "r"(s));
+#else
+    const unsigned long long th = s + 28 > 63 ? 0 : m >> (s + 28), tl = s > 63 ? 0 : m >> s;
+#endif
+    const int h = (int)(unsigned)th, l = (int)((unsigned)tl & 0xfffffffu);
+    return {(h ^ sg) - sg, (l ^ sg) - sg};
+}
 // Digits of x / 2^(E - 1022) for |x| < 2^(E - 1022), E the biased exponent of the
 // largest number of a block
 HR_HD inline fx fx_from_double(double x, int E)
@@ -260,6 +277,13 @@ HR_HD inline bool fxq_near_unit(const fxq &q)
     }
     return n > 0.99f && n < 1.01f;
 }
+// the same test in 32-bit integers, for |components| < 2
+HR_HD inline bool fxq_near_unit_int(const fxq &q)
+{
+    int n = -(1 << 26);
+    for (int k = 0; k < 4; ++k) n += (q.c[k].h >> 15) * (q.c[k].h >> 15);
+    return n > -(1 << 26) / 100 && n < (1 << 26) / 100;
+}
 // the vector part of a b into s[0..2]
 HR_HD inline void fxq_mac_vec(fxa (&s)[3], const fxq &a, const fxq &b)
 {
@@ -275,6 +299,14 @@ HR_HD inline void fxq_mac_scalar(fxa &s, const fxq &a, const fxq &b)
     fx_mac(s, fx_neg(a.c[1]), b.c[1]);
     fx_mac(s, fx_neg(a.c[2]), b.c[2]);
     fx_mac(s, fx_neg(a.c[3]), b.c[3]);
+}
+// s += u x v
+HR_HD inline void fx_mac_cross(fxa (&s)[3], const fx (&u)[3], const fx (&v)[3])
+{
+    const fx n0 = fx_neg(v[0]), n1 = fx_neg(v[1]), n2 = fx_neg(v[2]);
+    fx_mac(s[0], u[1], v[2]); fx_mac(s[0], u[2], n1);
+    fx_mac(s[1], u[2], v[0]); fx_mac(s[1], u[0], n2);
+    fx_mac(s[2], u[0], v[1]); fx_mac(s[2], u[1], n0);
 }
 // s += k q or q k, k = (0, k1, k2, k3) a pure vector
 HR_HD inline void fxq_mac_pure_l(fxa (&s)[4], const fx (&k)[3], const fxq &q)

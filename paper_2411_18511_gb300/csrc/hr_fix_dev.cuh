@@ -55,6 +55,17 @@ template <bool VEC> __device__ __forceinline__ fxq load_fxq(const double *q, siz
     return r;
 }
 
+// the same with the cheaper conversion and test (low digits up to 2^28)
+template <bool VEC> __device__ __forceinline__ fxq load_fxq_unit(const double *q, size_t link, bool &ok)
+{
+    double c[4];
+    load_link4<VEC>(q, link, c);
+    const unsigned m = max(max(fx_abs_high(c[0]), fx_abs_high(c[1])), max(fx_abs_high(c[2]), fx_abs_high(c[3])));
+    const fxq r = {{fx_from_unit(c[0]), fx_from_unit(c[1]), fx_from_unit(c[2]), fx_from_unit(c[3])}};
+    ok = ok && m < kFxHigh2 && fxq_near_unit_int(r);
+    return r;
+}
+
 // the 16 reals of a packed FP64 spinor as digits, [2 (2 spin + colour) + (0 re, 1 im)],
 // in units of 2^(E - kFxPairBias); E = biased exponent of the largest |hi|.  false: out
 // of range (a nonzero spinor below 2^-105, Inf or NaN)

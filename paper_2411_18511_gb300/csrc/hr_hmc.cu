@@ -102,11 +102,143 @@ __device__ __noinline__ void gauge_force_native(const Geom &g, const double *q, 
     f[2] += s * W.z;
 }
 
-// F[mu][x][a] += coeff * beta/2 * vec(U_mu(x) V_mu(x))_a, one thread per link
-// (mu = blockIdx.y), staples in two-digit fixed point (hr_fix.cuh): 12 quaternion
-// products of 16 terms, bound by the integer pipes instead of the FP64 pipe.
-// 32^4: 2.03 ms in native FP64 (with 64-bit coordinate divisions), 0.90 ms here;
-// error against long double 1.7e-16 before, 0.7e-16 now.
+// F[mu][x][a] += coeff * beta/2 * vec(U_mu(x) V_mu(x))_a from plaquettes, in two
+// launches, both in two-digit fixed point (hr_fix.cuh).
+//
+// With P_mn(x) = U_m(x) U_n(x+m) U_m(x+n)^+ U_n(x)^+ the upper staple of a link
+// gives vec P_mn(x), and the lower one, with y = x - n, the rotated vector
+// -vec(U_n(y)^+ P_mn(y) U_n(y)).  The four links of a plaquette thus share one
+// vector: k_plaq_vec computes the six of a site (2.75 quaternion products each),
+// k_plaq_force rotates twelve (15 products of numbers each) and adds them up,
+// where one thread per link forms 13 quaternion products and converts 19 links.
+// A vector is stored as its three digit pairs, 24 bytes, so it needs no conversion.
+//
+// Both are bound by the integer pipes.  The vectors of the whole lattice would be
+// 144 bytes a site from HBM and unbounded scratch, so slabs of time slices that
+// fit the context's scratch (64 MiB, half of L2) go through both launches in turn.
+static_assert(kPlaqSiteBytes == 6 * (sizeof(int4) + sizeof(int2)), "six vectors a site");
+// below this many sites one thread per plane and per link, more of them in flight
+constexpr int kPlaqSplitSites = 1 << 17;
+constexpr int kPlaqBad = (int)0x80000000; // leading digit of a vector outside the fixed-point range
+
+// plane index of mu < nu: (01) (02) (03) (12) (13) (23)
+__device__ __forceinline__ int plane_of(int mu, int nu)
+{
+    const int a = min(mu, nu), b = max(mu, nu);
+    return a == 0 ? b - 1 : a + b;
+}
+
+// one thread per site and group of `per` planes: vec P of the n sites from slice `first` on
+template <bool VEC>
+__global__ void __launch_bounds__(128) k_plaq_vec(Geom g, const double *__restrict__ q, int first, int n, int per,
+                                                  int4 *__restrict__ pa, int2 *__restrict__ pb)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int V = 2 * g.vh, slice = g.d[1] * g.d[2] * g.d[3];
+    int t = first * slice + i;
+    if (t < 0) t += V;
+    const LexSite x = lex_site(g, t);
+#pragma unroll 1
+    for (int p = blockIdx.y * per; p < (blockIdx.y + 1) * per; ++p) {
+        const int mu = p < 3 ? 0 : p < 5 ? 1 : 2, nu = p < 3 ? p + 1 : p < 5 ? p - 1 : 3;
+        int up_mu, up_nu, unused;
+        lex_steps(g, x, mu, up_mu, unused);
+        lex_steps(g, x, nu, up_nu, unused);
+        const size_t bm = (size_t)mu * V + t, bn = (size_t)nu * V + t;
+        bool ok = true;
+        fxq a = load_fxq_unit<VEC>(q, bm, ok), b = load_fxq_unit<VEC>(q, bn + up_mu, ok);
+        const fxq A = fxq_mul(a, b);
+        a = load_fxq_unit<VEC>(q, bn, ok);
+        b = load_fxq_unit<VEC>(q, bm + up_nu, ok);
+        const fxq B = fxq_conj(fxq_mul(a, b));
+        fxa w[3] = {};
+        fxq_mac_vec(w, A, B);
+        const fx v0 = fx_of(w[0]), v1 = fx_of(w[1]), v2 = fx_of(w[2]);
+        pa[(size_t)p * n + i] = make_int4(ok ? v0.h : kPlaqBad, v0.l, v1.h, v1.l);
+        pb[(size_t)p * n + i] = make_int2(v2.h, v2.l);
+    }
+}
+
+// The force on the links of the sites t0 .. t0 + m - 1 from the n vectors a plane
+// that start at slice `first`; NMU = 4: one thread per site, 1: one per link
+// (mu = blockIdx.y).  With u the quaternion U_n(y), t = u x v:
+//   vec(U^+ v U) / |U|^2 = v + 2 (u0 t + u x t) / |U|^2,
+// and 1 / |U|^2 = 1 - d, d = |U|^2 - 1, so that links off unit length by up to
+// 2^-29 give the staple's value.  The others take native FP64.
+template <bool VEC, int NMU>
+__global__ void __launch_bounds__(128) k_plaq_force(Geom g, double s, const double *__restrict__ q,
+                                                    double *__restrict__ F, int t0, int m, int first, int n,
+                                                    const int4 *__restrict__ pa, const int2 *__restrict__ pb)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m) return;
+    const int V = 2 * g.vh, slice = g.d[1] * g.d[2] * g.d[3];
+    const int t = t0 + i, own = t - first * slice;
+    const LexSite x = lex_site(g, t);
+    fxa acc[NMU][3] = {};
+    bool ok = true;
+#pragma unroll 1
+    for (int nu = 0; nu < 4; ++nu) {
+        if (NMU == 1 && nu == (int)blockIdx.y) continue;
+        int unused, down;
+        lex_steps(g, x, nu, unused, down);
+        const fxq U = load_fxq_unit<VEC>(q, (size_t)nu * V + t + down, ok);
+        fxa nn = {-(1LL << 56), 0};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) fx_mac(nn, U.c[k], U.c[k]);
+        const long long d = fx_round(nn);
+        ok = ok && d < (1 << 27) && d > -(1 << 27);
+        const fx u[3] = {U.c[1], U.c[2], U.c[3]};
+        fx w[4]; // 2 u (1 - d)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            w[k] = {2 * U.c[k].h, 2 * (U.c[k].l - (int)(((long long)U.c[k].h * (int)d) >> 28))};
+        const fx wv[3] = {w[1], w[2], w[3]};
+        // y's vectors: the slab's first slice is the one before its first site's, unless it is the whole lattice
+        const int low = nu == 0 && x.x0 > first ? own - slice : own + down;
+#pragma unroll
+        for (int k = 0; k < NMU; ++k) {
+            const int mu = NMU == 1 ? (int)blockIdx.y : k;
+            if (mu == nu) continue;
+            const size_t p = (size_t)plane_of(mu, nu) * n;
+            const int4 oa = pa[p + own], ya = pa[p + low];
+            const int2 ob = pb[p + own], yb = pb[p + low];
+            ok = ok && oa.x != kPlaqBad && ya.x != kPlaqBad;
+            const fx v[3] = {{ya.x, ya.y}, {ya.z, ya.w}, {yb.x, yb.y}};
+            fxa tc[3] = {};
+            fx_mac_cross(tc, u, v);
+            // + (P(x) - rotated P(y)) for mu < nu, - for mu > nu
+            const int sg = mu < nu ? 1 : -1;
+            const fx o[3] = {{oa.x, oa.y}, {oa.z, oa.w}, {ob.x, ob.y}};
+            fx tn[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const fx tt = fx_of(tc[a]), df = fx_sub(o[a], v[a]);
+                tn[a] = {-sg * tt.h, -sg * tt.l};
+                acc[k][a].a += fx_units64({sg * df.h, sg * df.l});
+                fx_mac(acc[k][a], w[0], tn[a]);
+            }
+            fx_mac_cross(acc[k], wv, tn);
+        }
+    }
+    const double c = s * 0x1p-56;
+#pragma unroll
+    for (int k = 0; k < NMU; ++k) {
+        const int mu = NMU == 1 ? (int)blockIdx.y : k;
+        double *f = F + ((size_t)mu * V + t) * 3;
+        if (!ok) {
+            gauge_force_native(g, q, mu, t, s, f);
+            continue;
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) f[a] += c * (double)fx_round(acc[k][a]);
+    }
+}
+
+// Slices too large for the scratch (more than 230 k sites each): one thread per link,
+// F[mu][x][a] += coeff * beta/2 * vec(U_mu(x) V_mu(x))_a, staples in two-digit fixed
+// point, 12 quaternion products of 16 terms.
 template <bool VEC>
 __global__ void __launch_bounds__(128) k_gauge_force(Geom g, double s, const double *__restrict__ q,
                                                      double *__restrict__ F)
@@ -317,12 +449,35 @@ hr_status check_md(hr_ctx *ctx, hr_lattice lat)
     return validate_lattice(ctx, lat, 1);
 }
 
+template <bool VEC>
+void launch_gauge_force(hr_ctx *ctx, const Geom &g, double c, const double *q, double *F, cudaStream_t s)
+{
+    const int V = 2 * g.vh, T = g.d[0], slice = V / T;
+    const int slots = (int)std::min<long long>(T, (long long)(kPlaqBytes / kPlaqSiteBytes) / slice);
+    if (slots < 2) {
+        k_gauge_force<VEC><<<dim3((unsigned)((V + 127) / 128), 4), 128, 0, s>>>(g, c, q, F);
+        return;
+    }
+    // the whole lattice, or slabs of about equal numbers of slices, each with the slice before it
+    const int nslab = slots == T ? 1 : (T + slots - 2) / (slots - 1);
+    const bool small = V <= kPlaqSplitSites;
+    for (int k = 0; k < nslab; ++k) {
+        const int a = (int)((long long)T * k / nslab), b = (int)((long long)T * (k + 1) / nslab);
+        const int first = nslab == 1 ? 0 : a - 1, n = (b - first) * slice, m = (b - a) * slice;
+        int4 *pa = (int4 *)ctx->d_plaq;
+        int2 *pb = (int2 *)(pa + 6LL * n);
+        const unsigned nb = (unsigned)((n + 127) / 128), mb = (unsigned)((m + 127) / 128);
+        k_plaq_vec<VEC><<<dim3(nb, small ? 6 : 1), 128, 0, s>>>(g, q, first, n, small ? 1 : 6, pa, pb);
+        if (small) k_plaq_force<VEC, 1><<<dim3(mb, 4), 128, 0, s>>>(g, c, q, F, a * slice, m, first, n, pa, pb);
+        else k_plaq_force<VEC, 4><<<mb, 128, 0, s>>>(g, c, q, F, a * slice, m, first, n, pa, pb);
+    }
+}
+
 hr_status gauge_force(hr_ctx *ctx, const Geom &g, double beta, const double *q, double coeff, double *F, cudaStream_t s)
 {
-    const dim3 grid((unsigned)((2LL * g.vh + 127) / 128), 4);
     const double c = coeff * 0.5 * beta;
-    if (((uintptr_t)q & 15u) == 0) k_gauge_force<true><<<grid, 128, 0, s>>>(g, c, q, F);
-    else k_gauge_force<false><<<grid, 128, 0, s>>>(g, c, q, F);
+    if (((uintptr_t)q & 15u) == 0) launch_gauge_force<true>(ctx, g, c, q, F, s);
+    else launch_gauge_force<false>(ctx, g, c, q, F, s);
     return check_launch(ctx, "gauge force");
 }
 

@@ -23,6 +23,7 @@ constexpr int kMaxRhs = 32;
 constexpr int kMaxPartials = kMaxBlocks * kMaxRhs; // partial sums of one reducing launch
 constexpr int kFinBlocks = 64;       // blocks of a finishing launch, at most
 constexpr int kNumCounters = 64;
+constexpr size_t kPlaqBytes = 64u << 20, kPlaqSiteBytes = 144; // scratch of the gauge force
 constexpr int kScalDoubles = 64 * kMaxRhs;
 
 // launch shape of the hop kernel chosen by the autotuner
@@ -39,6 +40,7 @@ struct hr_ctx {
     std::string err;
     double *d_partials = nullptr;  // kMaxPartials, then kFinBlocks * kMaxRhs sums of a finishing launch's blocks
     unsigned *d_counters = nullptr;
+    void *d_plaq = nullptr;        // kPlaqBytes: plaquette vectors of the gauge force
     double *d_scal = nullptr;      // kScalDoubles
     double *h_scal = nullptr;      // pinned mirror
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
