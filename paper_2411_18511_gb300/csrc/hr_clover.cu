@@ -1341,7 +1341,7 @@ size_t hr_clover_force_workspace_bytes(hr_lattice lat)
     if (hr_gauge_packed_bytes(lat, HR_FUND, HR_F64) == 0) return 0;
     const Geom g = make_geom(lat, 1);
     const size_t half = spinor_half_bytes(g, HR_FUND, kF64);
-    return k_field_bytes(g) + 5 * half;
+    return k_field_bytes(g) + 3 * half;
 }
 
 hr_status hr_clover_insertion_force(hr_ctx *ctx, hr_lattice lat, double c_sw, const double *gauge, const double *lam,
@@ -1385,44 +1385,38 @@ hr_status hr_clover_fermion_force(hr_ctx *ctx, hr_lattice lat, hr_clover_kind ki
     const size_t half = spinor_half_bytes(g, HR_FUND, kF64);
     char *w = (char *)work;
     double *K = (double *)w;
-    char *a = w + k_field_bytes(g);  // full field (Y | W)
-    char *b = a + 2 * half;          // full field (X | Z)
-    char *t_odd = b + 2 * half;
+    char *a = w + k_field_bytes(g); // full field (Y | W)
+    char *z = a + 2 * half;         // odd half field Z
     const void *ainv_odd = clover_half(clover, g, HR_FUND, kF64, true, 1);
-    // Y = Mhat X, or the given Y
-    if (Y) {
-        cudaError_t ce = cudaMemcpyAsync(a, Y, half, cudaMemcpyDeviceToDevice, s);
-        if (ce != cudaSuccess) return set_error(ctx, HR_ERR_CUDA, "copy: %s", cudaGetErrorString(ce));
-    } else {
-        st = apply_eo_op(ctx, g, m0, HR_FUND, kF64, HR_OP_SCHUR, gauge_packed, X, a, t_odd, nullptr, kFinNone,
-                         nullptr, nullptr, s, nullptr, clover);
-        if (st) return st;
-    }
-    // Z = A_oo^-1 H_oe X,  W = A_oo^-1 g5 H_oe g5 Y  (A commutes with g5)
-    for (int k = 0; k < 2; ++k) {
+    // dst = A_oo^-1 [g5] H_oe [g5] src (A commutes with g5)
+    auto hop_oe = [&](const void *src, void *dst, int g5) {
         HopLaunch L{};
         L.p = 1;
         L.gauge = gauge_packed;
-        L.in = k == 0 ? X : (const void *)a;
-        L.out = k == 0 ? b + half : a + half;
+        L.in = src;
+        L.out = dst;
         L.beta = 1.0;
-        L.g5_in = L.g5_out = k;
+        L.g5_in = L.g5_out = g5;
         L.clov = ainv_odd;
         L.clov_mode = kClovOut;
-        st = launch_hop(ctx, g, HR_FUND, kF64, L, s);
-        if (st) return st;
-    }
-    cudaError_t e = cudaMemcpyAsync(b, X, half, cudaMemcpyDeviceToDevice, s);
-    if (e != cudaSuccess) return set_error(ctx, HR_ERR_CUDA, "copy: %s", cudaGetErrorString(e));
-    // the hops: 1/2 dRe<a, H b>
-    st = hr_force(ctx, lat, gauge_packed, a, b, 0.5 * coeff, force, stream);
+        return launch_hop(ctx, g, HR_FUND, kF64, L, s);
+    };
+    // Z = A_oo^-1 H_oe X, and Y = Mhat X, whose first hop is Z, unless Y is given
+    const void *y = Y ? Y : a;
+    st = Y ? hop_oe(X, z, 0)
+           : apply_eo_op(ctx, g, m0, HR_FUND, kF64, HR_OP_SCHUR, gauge_packed, X, a, z, nullptr, kFinNone, nullptr,
+                         nullptr, s, nullptr, clover);
+    // W = A_oo^-1 g5 H_oe g5 Y
+    if (!st) st = hop_oe(y, a + half, 1);
+    // the hops: 1/2 dRe<(Y, W), H (X, Z)>
+    if (!st) st = link_deriv(ctx, lat, gauge_packed, y, a + half, X, z, 0.5 * coeff, force, 0, s);
     if (st) return st;
     // the site term: c_sw df[Lam]
     KFieldArgs A;
     A.g = g;
-    A.X = b;
-    A.Y = a;
-    A.Z = b + half;
+    A.X = X;
+    A.Y = y;
+    A.Z = z;
     A.W = a + half;
     // the exponential form's det A_oo is a constant (C is traceless): no det force
     A.ainv = (with_det && kind == HR_CLOVER_SW) ? ainv_odd : nullptr;

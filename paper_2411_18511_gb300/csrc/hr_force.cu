@@ -315,23 +315,26 @@ template <int MODE> __global__ void __launch_bounds__(128, 3) k_link_deriv_fx(Fo
     }
 }
 
-hr_status launch(hr_ctx *ctx, hr_lattice lat, const void *gauge, const void *af, const void *bf, double beta,
-                 double *out, int mode, hr_stream stream)
+} // namespace
+
+namespace hr {
+
+hr_status link_deriv(hr_ctx *ctx, hr_lattice lat, const void *gauge, const void *a_even, const void *a_odd,
+                     const void *b_even, const void *b_odd, double beta, double *out, int mode, cudaStream_t s)
 {
     if (!ctx) return HR_ERR_INVALID_ARG;
     hr_status st = validate_lattice(ctx, lat, 1);
     if (st) return st;
     if (mode == 0 && !gauge) return set_error(ctx, HR_ERR_INVALID_ARG, "null pointer");
-    st = check_buffers(ctx, {af, bf}, {out}, {gauge});
+    st = check_buffers(ctx, {a_even, a_odd, b_even, b_odd}, {out}, {gauge});
     if (st) return st;
     ForceArgs A;
     A.g = make_geom(lat, 1);
-    size_t half = spinor_half_bytes(A.g, HR_FUND, kF64);
     A.gauge = gauge;
-    A.a[0] = af;
-    A.a[1] = (const char *)af + half;
-    A.b[0] = bf;
-    A.b[1] = (const char *)bf + half;
+    A.a[0] = a_even;
+    A.a[1] = a_odd;
+    A.b[0] = b_even;
+    A.b[1] = b_odd;
     A.beta = beta;
     A.out = out;
     A.mode = mode;
@@ -341,10 +344,29 @@ hr_status launch(hr_ctx *ctx, hr_lattice lat, const void *gauge, const void *af,
     }
     int bs = 128;
     int grid = (int)((2LL * A.g.vh + bs - 1) / bs);
-    if (A.g.twisted) k_link_deriv<<<grid, bs, 0, (cudaStream_t)stream>>>(A);
-    else if (mode == 0) k_link_deriv_fx<0><<<grid, bs, 0, (cudaStream_t)stream>>>(A);
-    else k_link_deriv_fx<1><<<grid, bs, 0, (cudaStream_t)stream>>>(A);
+    if (A.g.twisted) k_link_deriv<<<grid, bs, 0, s>>>(A);
+    else if (mode == 0) k_link_deriv_fx<0><<<grid, bs, 0, s>>>(A);
+    else k_link_deriv_fx<1><<<grid, bs, 0, s>>>(A);
     return check_launch(ctx, mode ? "link grad" : "force");
+}
+
+} // namespace hr
+
+namespace {
+
+// the same on full packed fields
+hr_status launch(hr_ctx *ctx, hr_lattice lat, const void *gauge, const void *af, const void *bf, double beta,
+                 double *out, int mode, hr_stream stream)
+{
+    if (!ctx) return HR_ERR_INVALID_ARG;
+    hr_status st = validate_lattice(ctx, lat, 1);
+    if (st) return st;
+    if (mode == 0 && !gauge) return set_error(ctx, HR_ERR_INVALID_ARG, "null pointer");
+    st = check_buffers(ctx, {af, bf}, {out}, {gauge});
+    if (st) return st;
+    const size_t half = spinor_half_bytes(make_geom(lat, 1), HR_FUND, kF64);
+    return link_deriv(ctx, lat, gauge, af, (const char *)af + half, bf, (const char *)bf + half, beta, out, mode,
+                      (cudaStream_t)stream);
 }
 
 // Link derivative of B(X, L) = Re<L, Mhat^+ Mhat X> at fixed even fields X, L
@@ -354,9 +376,11 @@ hr_status launch(hr_ctx *ctx, hr_lattice lat, const void *gauge, const void *af,
 //   Re<Y, dMhat Z> = -c dRe<(Y, H_eo^+ Y), H (Z, H_oe Z)>,
 // so each of the two terms is one application of the hop derivative (mode 0:
 // su(2) force, 1: quaternion gradient) to full fields a = (Mhat Y, H_eo^+ Mhat Y)
-// and b = (Z, H_oe Z) assembled in the work buffer: L = X needs one (doubled).
+// and b = (Z, H_oe Z): L = X needs one (doubled).  H_oe Z is the first hop of
+// Mhat Z, kept from there: three hops per term (hr_fermion_force at 32^4 818 us
+// with the fourth and a copy of Z).
 struct FermionWork {
-    char *a, *b, *t; // two full fields and an odd temporary
+    char *a, *b, *t; // two full fields and an odd half field
     static size_t bytes(const Geom &g)
     {
         const size_t half = spinor_half_bytes(g, HR_FUND, kF64);
@@ -386,34 +410,30 @@ hr_status fermion_deriv(hr_ctx *ctx, hr_lattice lat, double m0, hr_rep rep, cons
     cudaStream_t s = (cudaStream_t)stream;
     FermionWork w{(char *)work, (char *)work + 2 * half, (char *)work + 4 * half};
     const double c = 1.0 / (4.0 * (4.0 + m0));
-    // dst_odd = [g5] H_oe [g5] src_even
-    auto hop_oe = [&](const void *src, void *dst, int g5) {
+    // mz = Mhat Z, hz = H_oe Z
+    auto schur = [&](const void *Z, void *mz, void *hz) {
+        return apply_eo_op(ctx, g, m0, HR_FUND, kF64, HR_OP_SCHUR, gauge, Z, mz, hz, nullptr, kFinNone, nullptr, nullptr,
+                           s);
+    };
+    // out += coeff * (-c) * k * dRe<(my, H_eo^+ my), H (Z, hz)>, H_eo^+ my = g5 H_oe g5 my in w.a's odd half
+    auto term = [&](const void *my, const void *Z, const void *hz, double k) {
         HopLaunch H{};
         H.p = 1;
         H.gauge = gauge;
-        H.in = src;
-        H.out = dst;
+        H.in = my;
+        H.out = w.a + half;
         H.beta = 1.0;
-        H.g5_in = g5;
-        H.g5_out = g5;
-        return launch_hop(ctx, g, HR_FUND, kF64, H, s);
-    };
-    // out += coeff * (-c) * k * dRe<(Mhat Y, H_eo^+ Mhat Y), H (Z, H_oe Z)>
-    auto term = [&](const void *Y, const void *Z, double k) {
-        hr_status t = apply_eo_op(ctx, g, m0, HR_FUND, kF64, HR_OP_SCHUR, gauge, Y, w.a, w.t, nullptr, kFinNone,
-                                  nullptr, nullptr, s);
-        if (!t) t = hop_oe(w.a, w.a + half, 1);
-        if (!t) {
-            cudaError_t e = cudaMemcpyAsync(w.b, Z, half, cudaMemcpyDeviceToDevice, s);
-            if (e != cudaSuccess) t = set_error(ctx, HR_ERR_CUDA, "copy: %s", cudaGetErrorString(e));
-        }
-        if (!t) t = hop_oe(Z, w.b + half, 0);
-        if (!t) t = launch(ctx, lat, gauge, w.a, w.b, -c * k * coeff, out, mode, stream);
+        H.g5_in = H.g5_out = 1;
+        hr_status t = launch_hop(ctx, g, HR_FUND, kF64, H, s);
+        if (!t) t = link_deriv(ctx, lat, gauge, my, w.a + half, Z, hz, -c * k * coeff, out, mode, s);
         return t;
     };
-    if (!L || L == X) return term(X, X, 2.0);
-    st = term(L, X, 1.0);
-    if (!st) st = term(X, L, 1.0);
+    st = schur(X, w.b, w.b + half);
+    if (st) return st;
+    if (!L || L == X) return term(w.b, X, w.b + half, 2.0);
+    st = schur(L, w.a, w.t);
+    if (!st) st = term(w.a, X, w.b + half, 1.0);
+    if (!st) st = term(w.b, L, w.t, 1.0);
     return st;
 }
 

@@ -533,8 +533,8 @@ struct HmcWork {
     void *X;          // even half: (Mhat^+ Mhat)^-1 eta (Hasenbusch: at the heavy mass)
     void *X2, *eta2;  // Hasenbusch ratio term: eta2 = Mhat_H^+ phi, X2 = (Mhat^+ Mhat)^-1 eta2
     void *e1, *e2;    // even temporaries (g5 copies)
-    void *a, *b;      // full fields of the fermion force
-    void *t_odd;      // odd temporary of Mhat
+    void *a;          // full field of the fermion force
+    void *t_odd;      // odd temporary of Mhat, H_oe X of the fermion force
     void *cg;         // CG workspace
     size_t cg_bytes;
     void *clover;     // clover fermions: the packed FP64 clover field of the current links
@@ -565,7 +565,7 @@ size_t layout_hmc(hr_lattice lat, const hr_hmc_params &prm, char *w, HmcWork *hw
     void *gauge = take(gb);
     void *F = take(sizeof(double) * 12 * V);
     void *Fg = nested(prm) ? take(sizeof(double) * 12 * V) : nullptr;
-    void *X = take(half), *a = take(2 * half), *b = take(2 * half), *t = take(half);
+    void *X = take(half), *a = take(2 * half), *t = take(half);
     void *X2 = nullptr, *eta2 = nullptr, *e1 = nullptr, *e2 = nullptr;
     if (prm.hasenbusch) {
         X2 = take(half);
@@ -583,7 +583,7 @@ size_t layout_hmc(hr_lattice lat, const hr_hmc_params &prm, char *w, HmcWork *hw
         cf = take(cfb);
     }
     if (hw)
-        *hw = HmcWork{gauge, (double *)F, (double *)Fg, X, X2, eta2, e1, e2, a, b, t, cg, cgb, clover, clover_h, cf,
+        *hw = HmcWork{gauge, (double *)F, (double *)Fg, X, X2, eta2, e1, e2, a, t, cg, cgb, clover, clover_h, cf,
                       cfb};
     return off;
 }
@@ -699,30 +699,23 @@ struct Trajectory {
         return launch_hop(ctx, g, HR_FUND, kF64, L, s);
     }
 
-    // F += coeff dRe<a, H b>/dw with a = (u, H_eo^+ u), b = (v, H_oe v), H_eo^+ = g5 H_oe g5
-    hr_status pair_force(const void *u, const void *v, double coeff)
+    // F += coeff dRe<a, H b>/dw with a = (u, H_eo^+ u), b = (v, hv), H_eo^+ = g5 H_oe g5
+    hr_status pair_force(const void *u, const void *v, const void *hv, double coeff)
     {
-        char *a = (char *)w.a, *b = (char *)w.b;
-        hr_status st = copy(a, u);
-        if (!st) st = hop_oe(u, a + half, 1, 1);
-        if (!st) st = copy(b, v);
-        if (!st) st = hop_oe(v, b + half, 0, 0);
-        if (!st) st = hr_force(ctx, lat, w.gauge, a, b, coeff, w.F, (hr_stream)s);
+        char *a = (char *)w.a;
+        hr_status st = hop_oe(u, a + half, 1, 1);
+        if (!st) st = link_deriv(ctx, lat, w.gauge, u, a + half, v, hv, coeff, w.F, 0, s);
         return st;
     }
 
     // the force of Re<src, (Mhat^+ Mhat)^-1 src> at mass m0 with X its solution:
-    // 2c dRe<a, H b>/dw, a = (Mhat X, H_eo^+ Mhat X), b = (X, H_oe X), c = 1/(4 (4+m0))
+    // 2c dRe<a, H b>/dw, a = (Mhat X, H_eo^+ Mhat X), b = (X, H_oe X), c = 1/(4 (4+m0));
+    // H_oe X is the first hop of Mhat X
     hr_status solve_force(double m0, const void *X)
     {
         hr_status st = apply_eo_op(ctx, g, m0, HR_FUND, kF64, HR_OP_SCHUR, w.gauge, X, w.a, w.t_odd, nullptr,
                                    kFinNone, nullptr, nullptr, s);
-        if (st) return st;
-        char *a = (char *)w.a, *b = (char *)w.b; // Mhat X is a's even half already
-        st = hop_oe(a, a + half, 1, 1);
-        if (!st) st = copy(b, X);
-        if (!st) st = hop_oe(X, b + half, 0, 0);
-        if (!st) st = hr_force(ctx, lat, w.gauge, a, b, 2.0 / (4.0 * (4.0 + m0)), w.F, (hr_stream)s);
+        if (!st) st = pair_force(w.a, X, w.t_odd, 2.0 / (4.0 * (4.0 + m0)));
         return st;
     }
 
@@ -773,7 +766,8 @@ struct Trajectory {
                 if (!st) st = blas_gamma5(ctx, g, HR_FUND, w.e1, s);
                 if (!st) st = copy(w.e2, phi);
                 if (!st) st = blas_gamma5(ctx, g, HR_FUND, w.e2, s);
-                if (!st) st = pair_force(w.e1, w.e2, -2.0 / (4.0 * (4.0 + prm.m0_hasenbusch)));
+                if (!st) st = hop_oe(w.e2, w.t_odd, 0, 0);
+                if (!st) st = pair_force(w.e1, w.e2, w.t_odd, -2.0 / (4.0 * (4.0 + prm.m0_hasenbusch)));
             }
         }
         return st;

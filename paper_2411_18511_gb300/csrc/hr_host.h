@@ -180,6 +180,12 @@ hr_status apply_eo_op(hr_ctx *ctx, const Geom &g, double m0, int rep, int prec, 
                       const double *gate, const double *done, cudaStream_t s, const CgFuse *fuse = nullptr,
                       const void *clover = nullptr);
 
+// ---- link derivatives (hr_force.cu) ----
+// out += beta dRe<a, H b> for full fields given by their even and odd halves
+// (mode 0: su(2) force [4][V][3]; 1: quaternion gradient [4][V][4], no gauge field)
+hr_status link_deriv(hr_ctx *ctx, hr_lattice lat, const void *gauge, const void *a_even, const void *a_odd,
+                     const void *b_even, const void *b_odd, double beta, double *out, int mode, cudaStream_t s);
+
 // ---- clover site term (hr_clover.cu) ----
 // bytes of one of the four half-fields of a packed clover field (cp: kF64 / kF32)
 size_t clover_half_bytes(const Geom &g, int rep, int cp);
