@@ -3,7 +3,9 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
+#include "hr_cvt.cuh"
 #include "hr_host.h"
 
 using namespace hr;
@@ -94,6 +96,13 @@ size_t spinor_half_bytes(const Geom &g, int rep, int prec)
     return SpinorLayout<3, kF16>::bytes(g.nblk_s);
 }
 
+// the bytes of a half that the 32-site blocks' lanes cover
+static size_t packed_lane_bytes(const Geom &g, int rep, int prec)
+{
+    const size_t per = (size_t)8 * rep_nc(rep) * (prec == kF64 ? 8 : prec == kF32 ? 4 : 2) + (prec == kF16 ? 4 : 0);
+    return (size_t)g.nblk_s * 32 * per;
+}
+
 size_t gauge_bytes(const Geom &g, int rep, int prec)
 {
     size_t b;
@@ -116,33 +125,105 @@ __device__ __forceinline__ bool boundary_link(const Geom &g, int mu, const int (
     return ((g.bc >> mu) & 1) && x[mu] == g.d[mu] - 1;
 }
 
-// one thread per link (mu, lex site).  canon (adjoint): store the representative
-// of +-q with the sign bit of q0 clear, then set it on boundary links; the
-// fundamental stores -q on boundary links.
-template <int PREC>
-__global__ void k_gauge_pack_quat(Geom g, int canon, const double *__restrict__ can, void *packed, unsigned *status)
+// a double split on its way into a packed layout
+struct PairVal {
+    float h, l;
+};
+// x as a pair, by the FP64 pipe when it is out of the integer split's range;
+// range flags into bad
+struct PairFlags {
+    PairVal v;
+    unsigned bad;
+};
+__device__ __noinline__ PairFlags split_native(double x)
 {
-    long long V = 2LL * g.vh;
-    long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 4 * V) return;
-    int mu = (int)(t / V);
-    long long x = t - (long long)mu * V;
-    int x3 = (int)(x % g.d[3]);
-    long long r = x / g.d[3];
-    int x2 = (int)(r % g.d[2]);
-    r /= g.d[2];
-    int x1 = (int)(r % g.d[1]);
-    int x0 = (int)(r / g.d[1]);
-    int p = (x0 + x1 + x2 + x3) & 1;
-    int i = (int)(x >> 1);
-    double a[4] = {can[t * 4 + 0], can[t * 4 + 1], can[t * 4 + 2], can[t * 4 + 3]};
-    const unsigned bad = pack_range_flags(a[0]) | pack_range_flags(a[1]) | pack_range_flags(a[2]) | pack_range_flags(a[3]);
-    if (bad) atomicOr(status, bad);
+    const dd d = dd_from_double(x);
+    return {{d.h, d.l}, pack_range_flags(x)};
+}
+__device__ __forceinline__ PairVal split_val(double x, unsigned &bad)
+{
+    PairVal v;
+    if (!cvt_split(x, v.h, v.l)) {
+        const PairFlags f = split_native(x);
+        v = f.v;
+        bad |= f.bad;
+    }
+    return v;
+}
+__device__ __noinline__ double join_native(float h, float l) { return (double)h + (double)l; }
+__device__ __forceinline__ double join_val(dd v)
+{
+    double x;
+    if (!cvt_join(v.h, v.l, x)) x = join_native(v.h, v.l);
+    return x;
+}
+__device__ __forceinline__ double join_val(float v)
+{
+    double x;
+    if (!cvt_widen(v, x)) x = join_native(v, 0.f);
+    return x;
+}
+
+// 16 bytes of a canonical field (VEC: it is 16-byte aligned)
+template <bool VEC> __device__ __forceinline__ double2 load_pair(const double *p)
+{
+    if constexpr (VEC) return *(const double2 *)p;
+    else return make_double2(p[0], p[1]);
+}
+template <bool VEC> __device__ __forceinline__ void store_pair(double *p, double2 v)
+{
+    if constexpr (VEC) {
+        *(double2 *)p = v;
+    } else {
+        p[0] = v.x;
+        p[1] = v.y;
+    }
+}
+
+} // namespace
+
+namespace hr {
+template <> struct Real<PairVal> {
+    __device__ static dd to_dd(PairVal x) { return dd(x.h, x.l); }
+    __device__ static float to_float(PairVal x) { return x.h; }
+};
+} // namespace hr
+
+namespace {
+
+// one thread per link (mu = blockIdx.y, lex site).  canon (adjoint): store the
+// representative of +-q with the sign bit of q0 clear, then set it on boundary
+// links; the fundamental stores -q on boundary links.  The threads beyond the
+// sites zero the lanes that pad a parity's last block of 32.
+template <int PREC, bool VEC>
+__global__ void __launch_bounds__(256) k_gauge_pack_quat(Geom g, int canon, const double *__restrict__ can,
+                                                         void *packed, unsigned *status)
+{
+    const unsigned V = 2u * (unsigned)g.vh, pad = (unsigned)g.nblk_g * 32u - (unsigned)g.vh;
+    const unsigned x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int mu = blockIdx.y;
+    if (x >= V + 2u * pad) return;
+    if (x >= V) {
+        const unsigned k = x - V;
+        const PairVal z[4] = {};
+        store_quat<PREC>(packed, g.nblk_g, k >= pad ? 1 : 0, mu, g.vh + (int)(k >= pad ? k - pad : k), z);
+        return;
+    }
+    const int i = (int)(x >> 1), row = fdiv(i, g.div_h3), r1 = fdiv(row, g.div_d2);
+    const int x3 = (int)(x - (unsigned)row * (unsigned)g.d[3]), x2 = row - r1 * g.d[2];
+    const int x0 = fdiv(r1, g.div_d1), x1 = r1 - x0 * g.d[1];
+    const int p = (x0 + x1 + x2 + x3) & 1;
+    const double *src = can + ((size_t)mu * V + x) * 4;
+    const double2 q01 = load_pair<VEC>(src), q23 = load_pair<VEC>(src + 2);
+    double a[4] = {q01.x, q01.y, q23.x, q23.y};
     const int xc[4] = {x0, x1, x2, x3};
     const bool neg = (canon && sign_bit(a[0])) != boundary_link(g, mu, xc);
-    if (neg)
-        for (int k = 0; k < 4; ++k) a[k] = -a[k];
-    store_quat<PREC>(packed, g.nblk_g, p, mu, i, a);
+    PairVal v[4];
+    unsigned bad = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = split_val(neg ? -a[k] : a[k], bad);
+    if (bad) atomicOr(status, bad);
+    store_quat<PREC>(packed, g.nblk_g, p, mu, i, v);
 }
 
 template <int PREC>
@@ -175,65 +256,85 @@ __global__ void k_gauge_pack_mat(Geom g, const double *__restrict__ can, void *p
     }
 }
 
-// canonical double[nrhs][V][4][NC][2] -> packed virtual sites of parity p.
-// One thread per (rhs, even-odd site).
-template <int NC, int PREC>
-__global__ void k_spinor_pack(Geom g, int p, const double *__restrict__ can, void *packed, unsigned *status)
+// canonical double[nrhs][V][4][NC][2] <-> packed virtual sites, blockIdx.y-th of
+// the parities from p0 on (packed halves `half` bytes apart).  A warp moves 32
+// virtual sites: the packed side in 16-byte vectors of consecutive lanes, the
+// canonical side in whole sites of CH 16-byte chunks (consecutive lanes, consecutive
+// chunks), through a transposition in shared memory whose rows of CH + 1 chunks
+// are free of bank conflicts.  Both are then bound by HBM; a thread that read or
+// wrote a whole site in 8-byte steps and converted on the FP64 pipe took 590 us to
+// unpack a 48^4 field.
+constexpr int kConvWarps = 4;
+
+template <int NC, int PREC, bool VEC>
+__global__ void __launch_bounds__(32 * kConvWarps) k_spinor_pack(Geom g, int p0, const double *__restrict__ can,
+                                                                 char *packed, size_t half, unsigned *status)
 {
-    using T = double; // the canonical side is FP64; the layout code converts
-    long long n = (long long)g.vh << g.lrhs;
-    long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    int r = (int)(t / g.vh);
-    int i = (int)(t - (long long)r * g.vh);
-    long long lex = eo_to_lex(g, i, p);
-    long long V = 2LL * g.vh;
-    const double *src = can + ((long long)r * V + lex) * (8 * NC);
-    cpx<T> s[4][NC];
-    unsigned bad = 0;
+    constexpr int CH = 4 * NC;
+    __shared__ double2 tile[kConvWarps][32][CH + 1];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nv = g.vh << g.lrhs;
+    const int j0 = (blockIdx.x * kConvWarps + w) * 32, j = j0 + lane, p = p0 + blockIdx.y;
+    if (j0 >= g.nblk_s * 32) return; // the whole warp
+    unsigned site = 0; // r V + lex
+    if (j < nv) site = (unsigned)(j & (g.nrhs - 1)) * (2u * g.vh) + (unsigned)eo_to_lex(g, j >> g.lrhs, p);
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int q = lane; q < 32 * CH; q += 32) {
+        const int k = q / CH, c = q - k * CH;
+        const unsigned s = __shfl_sync(0xffffffffu, site, k);
+        if (j0 + k < nv) tile[w][k][c] = load_pair<VEC>(can + ((size_t)s * CH + c) * 2);
+    }
+    __syncwarp();
+    cpx<PairVal> v[4][NC] = {}; // padding lanes hold zeros
+    if (j < nv) {
+        unsigned bad = 0;
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            s[a][c] = {(T)src[(a * NC + c) * 2], (T)src[(a * NC + c) * 2 + 1]};
-            bad |= pack_range_flags(s[a][c].re) | pack_range_flags(s[a][c].im);
-        }
-    if (bad) atomicOr(status, bad);
-    store_spinor<NC, PREC>(packed, g.nblk_s, (i << g.lrhs) + r, s);
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const double2 x = tile[w][lane][a * NC + c];
+                v[a][c] = {split_val(x.x, bad), split_val(x.y, bad)};
+            }
+        if (bad) atomicOr(status, bad);
+    }
+    store_spinor<NC, PREC>(packed + blockIdx.y * half, g.nblk_s, j, v);
 }
 
-template <int NC, int PREC>
-__global__ void k_spinor_unpack(Geom g, int p, const void *packed, double *__restrict__ can)
+template <int NC, int PREC, bool VEC>
+__global__ void __launch_bounds__(32 * kConvWarps) k_spinor_unpack(Geom g, int p0, const char *packed, size_t half,
+                                                                   double *__restrict__ can)
 {
-    using T = double; // the canonical side is FP64; the layout code converts
-    long long n = (long long)g.vh << g.lrhs;
-    long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    int r = (int)(t / g.vh);
-    int i = (int)(t - (long long)r * g.vh);
-    long long lex = eo_to_lex(g, i, p);
-    long long V = 2LL * g.vh;
-    double *dst = can + ((long long)r * V + lex) * (8 * NC);
-    cpx<T> s[4][NC];
-    load_spinor<NC, PREC>(packed, g.nblk_s, (i << g.lrhs) + r, s);
+    using T = typename PrecTraits<PREC>::T;
+    constexpr int CH = 4 * NC;
+    __shared__ double2 tile[kConvWarps][32][CH + 1];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nv = g.vh << g.lrhs;
+    const int j0 = (blockIdx.x * kConvWarps + w) * 32, j = j0 + lane, p = p0 + blockIdx.y;
+    if (j0 >= nv) return; // the whole warp
+    unsigned site = 0;
+    if (j < nv) {
+        site = (unsigned)(j & (g.nrhs - 1)) * (2u * g.vh) + (unsigned)eo_to_lex(g, j >> g.lrhs, p);
+        cpx<T> v[4][NC];
+        load_spinor<NC, PREC>(packed + blockIdx.y * half, g.nblk_s, j, v);
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            dst[(a * NC + c) * 2] = (double)s[a][c].re;
-            dst[(a * NC + c) * 2 + 1] = (double)s[a][c].im;
-        }
+            for (int c = 0; c < NC; ++c) tile[w][lane][a * NC + c] = make_double2(join_val(v[a][c].re), join_val(v[a][c].im));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = lane; q < 32 * CH; q += 32) {
+        const int k = q / CH, c = q - k * CH;
+        const unsigned s = __shfl_sync(0xffffffffu, site, k);
+        if (j0 + k < nv) store_pair<VEC>(can + ((size_t)s * CH + c) * 2, tile[w][k][c]);
+    }
 }
 
-template <int NC, int PREC>
-hr_status launch_spinor_pack(hr_ctx *ctx, const Geom &g, int p, const double *can, void *packed, bool unpack,
-                             cudaStream_t s)
+template <int NC, int PREC, bool VEC>
+hr_status launch_spinor_convert(hr_ctx *ctx, const Geom &g, int p0, int np, double *can, char *packed, size_t half,
+                                bool unpack, cudaStream_t s)
 {
-    long long n = (long long)g.vh << g.lrhs;
-    int bs = 256;
-    int grid = (int)((n + bs - 1) / bs);
-    if (unpack) k_spinor_unpack<NC, PREC><<<grid, bs, 0, s>>>(g, p, packed, (double *)can);
-    else k_spinor_pack<NC, PREC><<<grid, bs, 0, s>>>(g, p, can, packed, ctx->d_counters + C_PACK);
+    const dim3 grid((unsigned)((g.nblk_s + kConvWarps - 1) / kConvWarps), (unsigned)np);
+    if (unpack) k_spinor_unpack<NC, PREC, VEC><<<grid, 32 * kConvWarps, 0, s>>>(g, p0, packed, half, can);
+    else k_spinor_pack<NC, PREC, VEC><<<grid, 32 * kConvWarps, 0, s>>>(g, p0, can, packed, half, ctx->d_counters + C_PACK);
     return check_launch(ctx, unpack ? "spinor unpack" : "spinor pack");
 }
 
@@ -250,21 +351,27 @@ hr_status spinor_convert(hr_ctx *ctx, hr_lattice lat, int rep, int prec, int par
     Geom g = make_geom(lat, n_rhs);
     size_t half = spinor_half_bytes(g, rep, prec);
     int nc = rep_nc(rep);
-    for (int p = 0; p < 2; ++p) {
-        if (parity != HR_FULL && parity != p) continue;
-        char *dst = (char *)packed + ((parity == HR_FULL && p == 1) ? half : 0);
-        if (nc == 2) {
-            if (prec == kF64) st = launch_spinor_pack<2, kF64>(ctx, g, p, can, dst, unpack, s);
-            else if (prec == kF32) st = launch_spinor_pack<2, kF32>(ctx, g, p, can, dst, unpack, s);
-            else st = launch_spinor_pack<2, kF16>(ctx, g, p, can, dst, unpack, s);
-        } else {
-            if (prec == kF64) st = launch_spinor_pack<3, kF64>(ctx, g, p, can, dst, unpack, s);
-            else if (prec == kF32) st = launch_spinor_pack<3, kF32>(ctx, g, p, can, dst, unpack, s);
-            else st = launch_spinor_pack<3, kF16>(ctx, g, p, can, dst, unpack, s);
+    const int p0 = parity == HR_FULL ? 0 : parity, np = parity == HR_FULL ? 2 : 1;
+    // the packed bytes that no lane covers (binary16: the scales' rounding to 256)
+    const size_t used = packed_lane_bytes(g, rep, prec);
+    if (!unpack && used < half) {
+        for (int k = 0; k < np; ++k) {
+            cudaError_t e = cudaMemsetAsync((char *)packed + k * half + used, 0, half - used, s);
+            if (e != cudaSuccess) return set_error(ctx, HR_ERR_CUDA, "spinor pack: %s", cudaGetErrorString(e));
         }
-        if (st) return st;
     }
-    return HR_OK;
+    const bool vec = ((uintptr_t)can & 15u) == 0;
+    auto go = [&](auto nc_, auto prec_) {
+        constexpr int NC = decltype(nc_)::value, PREC = decltype(prec_)::value;
+        return vec ? launch_spinor_convert<NC, PREC, true>(ctx, g, p0, np, (double *)can, (char *)packed, half, unpack, s)
+                   : launch_spinor_convert<NC, PREC, false>(ctx, g, p0, np, (double *)can, (char *)packed, half, unpack, s);
+    };
+    auto by_prec = [&](auto nc_) {
+        if (prec == kF64) return go(nc_, std::integral_constant<int, kF64>());
+        if (prec == kF32) return go(nc_, std::integral_constant<int, kF32>());
+        return go(nc_, std::integral_constant<int, kF16>());
+    };
+    return nc == 2 ? by_prec(std::integral_constant<int, 2>()) : by_prec(std::integral_constant<int, 3>());
 }
 
 // packed FP64 gauge -> packed gauge of precision PD, one thread per (p, mu, site)
@@ -449,21 +556,26 @@ hr_status hr_gauge_pack(hr_ctx *ctx, hr_lattice lat, hr_rep rep, hr_prec prec, c
     if (st) return st;
     Geom g = make_geom(lat, 1);
     cudaStream_t s = (cudaStream_t)stream;
-    // zero the padding lanes so packed buffers are fully defined
-    cudaMemsetAsync(packed, 0, gauge_bytes(g, rep, prec), s);
-    long long n = 8LL * g.vh;
-    int bs = 256;
-    int grid = (int)((n + bs - 1) / bs);
     unsigned *status = ctx->d_counters + C_PACK;
     if (rep == HR_ADJ_MAT) {
+        // zero the padding lanes so packed buffers are fully defined
+        cudaMemsetAsync(packed, 0, gauge_bytes(g, rep, prec), s);
+        const int bs = 256, grid = (int)((8LL * g.vh + bs - 1) / bs);
         if (prec == kF64) k_gauge_pack_mat<kF64><<<grid, bs, 0, s>>>(g, canonical, packed, status);
         else if (prec == kF32) k_gauge_pack_mat<kF32><<<grid, bs, 0, s>>>(g, canonical, packed, status);
         else k_gauge_pack_mat<kF16><<<grid, bs, 0, s>>>(g, canonical, packed, status);
     } else {
         const int canon = rep == HR_ADJ ? 1 : 0;
-        if (prec == kF64) k_gauge_pack_quat<kF64><<<grid, bs, 0, s>>>(g, canon, canonical, packed, status);
-        else if (prec == kF32) k_gauge_pack_quat<kF32><<<grid, bs, 0, s>>>(g, canon, canonical, packed, status);
-        else k_gauge_pack_quat<kF16><<<grid, bs, 0, s>>>(g, canon, canonical, packed, status);
+        const dim3 grid((unsigned)((64LL * g.nblk_g + 255) / 256), 4);
+        const bool vec = ((uintptr_t)canonical & 15u) == 0;
+        auto go = [&](auto prec_) {
+            constexpr int PREC = decltype(prec_)::value;
+            if (vec) k_gauge_pack_quat<PREC, true><<<grid, 256, 0, s>>>(g, canon, canonical, packed, status);
+            else k_gauge_pack_quat<PREC, false><<<grid, 256, 0, s>>>(g, canon, canonical, packed, status);
+        };
+        if (prec == kF64) go(std::integral_constant<int, kF64>());
+        else if (prec == kF32) go(std::integral_constant<int, kF32>());
+        else go(std::integral_constant<int, kF16>());
     }
     return check_launch(ctx, "gauge pack");
 }
@@ -471,8 +583,6 @@ hr_status hr_gauge_pack(hr_ctx *ctx, hr_lattice lat, hr_rep rep, hr_prec prec, c
 hr_status hr_spinor_pack(hr_ctx *ctx, hr_lattice lat, hr_rep rep, hr_prec prec, hr_parity parity, int n_rhs,
                          const double *canonical, void *packed, hr_stream stream)
 {
-    if (ctx && packed && valid_rep(rep) && valid_prec(prec) && lattice_ok(lat, n_rhs) && parity >= 0 && parity <= 2)
-        cudaMemsetAsync(packed, 0, hr_spinor_packed_bytes(lat, rep, prec, parity, n_rhs), (cudaStream_t)stream);
     return spinor_convert(ctx, lat, rep, prec, parity, n_rhs, canonical, packed, false, (cudaStream_t)stream);
 }
 

@@ -593,27 +593,31 @@ __device__ __forceinline__ void load_quat(const void *base, int nblk_g, int p, i
     }
 }
 
-// store one quaternion link in the packed layout of PREC (from double: pack kernels)
-template <int PREC>
-__device__ __forceinline__ void store_quat(void *base, int nblk_g, int p, int mu, int i, const double (&a)[4])
+// store one quaternion link in the packed layout of PREC
+template <int PREC, class T>
+__device__ __forceinline__ void store_quat(void *base, int nblk_g, int p, int mu, int i, const T (&a)[4])
 {
     size_t slot = (size_t)(p * 4 + mu) * nblk_g + (i >> 5);
     int lane = i & 31;
     if constexpr (PREC == kF64) {
         dd d[4];
-        for (int k = 0; k < 4; ++k) d[k] = dd_from_double(a[k]);
+        for (int k = 0; k < 4; ++k) d[k] = Real<T>::to_dd(a[k]);
         float4 *q = (float4 *)base;
         q[(slot * 2 + 0) * 32 + lane] = make_float4(d[0].h, d[1].h, d[2].h, d[3].h);
         q[(slot * 2 + 1) * 32 + lane] = make_float4(d[0].l, d[1].l, d[2].l, d[3].l);
-    } else if constexpr (PREC == kF32) {
-        ((float4 *)base)[slot * 32 + lane] = make_float4((float)a[0], (float)a[1], (float)a[2], (float)a[3]);
     } else {
-        __half2 h0 = __floats2half2_rn((float)a[0], (float)a[1]);
-        __half2 h1 = __floats2half2_rn((float)a[2], (float)a[3]);
-        uint2 w;
-        w.x = *reinterpret_cast<uint32_t *>(&h0);
-        w.y = *reinterpret_cast<uint32_t *>(&h1);
-        ((uint2 *)base)[slot * 32 + lane] = w;
+        float f[4];
+        for (int k = 0; k < 4; ++k) f[k] = Real<T>::to_float(a[k]);
+        if constexpr (PREC == kF32) {
+            ((float4 *)base)[slot * 32 + lane] = make_float4(f[0], f[1], f[2], f[3]);
+        } else {
+            __half2 h0 = __floats2half2_rn(f[0], f[1]);
+            __half2 h1 = __floats2half2_rn(f[2], f[3]);
+            uint2 w;
+            w.x = *reinterpret_cast<uint32_t *>(&h0);
+            w.y = *reinterpret_cast<uint32_t *>(&h1);
+            ((uint2 *)base)[slot * 32 + lane] = w;
+        }
     }
 }
 
