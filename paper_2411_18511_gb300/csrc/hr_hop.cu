@@ -76,12 +76,20 @@ __global__ void __launch_bounds__(256) k_hop_clov(HopArgs a)
 
 // ---------------------------------------------------------------- launch
 
+// The shape of a configuration that was never tuned: the family that was fastest,
+// or within 5 % of it, from 4^4 to 24^4, at 64 threads a block (small blocks spread
+// a small lattice over more SMs and leave a shorter tail on a large one).  us per
+// hop of Mhat^+ Mhat at 8^4 / 16^4 / 24^4, the plain kernel (256 threads for FP64,
+// 128 else) against the choice:
+//   fundamental FP64 11.6 / 13.7 / 36.3 -> 6.0 / 11.8 / 33.5, FP32 3.1 / 4.5 / 8.5 ->
+//   2.1 / 3.7 / 7.9, binary16 3.3 / 5.6 / 8.0 -> 2.2 / 4.2 / 6.3; adjoint FP64 17.0 /
+//   18.7 / 75.0 -> 9.2 / 18.9 / 49.6, stored matrices 13.9 / 14.9 / 70.6 -> 7.5 / 13.9 /
+//   50.8.  The adjoint in FP32 and binary16 has the plain kernel only.
 inline HopChoice default_choice(int rep, int prec)
 {
-    HopChoice c;
-    c.variant = kVarSimple;
-    c.block = (prec == kF64) ? 256 : 128;
-    return c;
+    if (prec == kF64) return {kVarPaired, 64};
+    if (rep == HR_FUND) return {prec == kF32 ? kVarSimpleR96 : kVarHalfPrefetch, 64};
+    return {kVarSimple, 128};
 }
 
 template <int REP, int PREC> struct PlainLaunch {
