@@ -70,16 +70,18 @@ __global__ void __launch_bounds__(kFinThreads) k_finish(const double *partials, 
 {
     __shared__ double sums[kFinThreads];
     after_previous();
-    if ((gate && *gate == 0.0) || (done && *done != 0.0)) {
+    // everything the kernel reads is requested before the first value is used
+    const bool skip = (gate && *gate == 0.0) | (done && *done != 0.0);
+    const FinIn in = load_fin(scal, nrhs);
+    const int first = blockIdx.x * rows;
+    sum_partials(partials + (size_t)first * nrhs, min(rows, nparts - first), nrhs, sums, skip);
+    if (skip) {
         // the update may be due from an earlier iteration of the pass
         if (cond.set && blockIdx.x == 0 && threadIdx.x == 0)
             cudaGraphSetConditional(cond.handle,
                                     sc(scal, S_FLAGS, F_GATE) != 0.0 && sc(scal, S_FLAGS, F_DONE) == 0.0 ? 1u : 0u);
         return;
     }
-    const FinIn in = load_fin(scal, nrhs);
-    const int first = blockIdx.x * rows;
-    sum_partials(partials + (size_t)first * nrhs, min(rows, nparts - first), nrhs, sums);
     if (gridDim.x > 1) {
         __shared__ bool last;
         if (threadIdx.x < nrhs) {

@@ -938,8 +938,9 @@ __device__ __forceinline__ double warp_sum_strided(double v, int nrhs)
 // result depends on nparts, nrhs and blockDim only.  The FP64 pipe runs 1.7
 // additions a clock on this GPU, so it counts them: a tree in shared memory
 // halves its lanes at each step, a shuffle tree would add on all 32.
-// Ends with a block barrier.
-__device__ inline void sum_partials(const double *partials, int nparts, int nrhs, double *smem)
+// Ends with a block barrier; skip (uniform): nothing is summed, the flag being
+// looked at only once the first rows are on their way.
+__device__ inline void sum_partials(const double *partials, int nparts, int nrhs, double *smem, bool skip = false)
 {
     const int t = threadIdx.x, r = t & (nrhs - 1), step = blockDim.x / nrhs;
     constexpr int K = 8;
@@ -948,16 +949,25 @@ __device__ inline void sum_partials(const double *partials, int nparts, int nrhs
         double v[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) v[k] = b + k * step < nparts ? __ldcg(partials + (size_t)(b + k * step) * nrhs + r) : 0.0;
+        if (skip) return;
 #pragma unroll
         for (int k = 0; k < K; ++k)
             if (b + k * step < nparts) acc += v[k];
     }
+    if (skip) return;
     smem[t] = acc;
     __syncthreads();
-    for (int n = blockDim.x >> 1; n >= nrhs; n >>= 1) {
+    for (int n = blockDim.x >> 1; n >= 32; n >>= 1) {
         if (t < n) smem[t] += smem[t + n];
         __syncthreads();
     }
+    if (t < 32) {
+        for (int n = 16; n >= nrhs; n >>= 1) {
+            if (t < n) smem[t] += smem[t + n];
+            __syncwarp();
+        }
+    }
+    __syncthreads();
 }
 
 // The warp stage of a grid reduction in the accumulator's own arithmetic:
@@ -1077,13 +1087,14 @@ __device__ __forceinline__ FinIn load_fin(double *scal, int nrhs)
     return f;
 }
 
-// Scalar updates run by one block on the finished sums (threads 0..nrhs-1 hold
-// one right-hand side each); thread 0 then refreshes the flags.  Returns, in
-// every thread, whether a reliable update is due (the gate is open and the
-// solve goes on).
+// Scalar updates on the finished sums by the first warp of a block (lanes
+// 0..nrhs-1 hold one right-hand side each); thread 0 then refreshes the flags.
+// Returns, in that warp, whether a reliable update is due (the gate is open and
+// the solve goes on).
 __device__ inline bool finish_reduction(int mode, const double *sums, int nrhs, double *scal, const FinIn &f)
 {
     const int r = threadIdx.x;
+    if (r >= 32) return false;
     bool act = false, bad = false, open = false, open2 = false;
     if (r < nrhs) {
         const double v = sums[r];
@@ -1160,8 +1171,8 @@ __device__ inline bool finish_reduction(int mode, const double *sums, int nrhs, 
         }
         if (mode == kFinBeta || mode == kFinResidual || mode == kFinInit) sc(scal, S_ACTIVE, r) = act ? 1.0 : 0.0;
     }
-    const bool any_bad = __syncthreads_or(bad), any_act = __syncthreads_or(act);
-    const bool any_open = __syncthreads_or(open), any_open2 = __syncthreads_or(open2);
+    const bool any_bad = __any_sync(0xffffffffu, bad), any_act = __any_sync(0xffffffffu, act);
+    const bool any_open = __any_sync(0xffffffffu, open), any_open2 = __any_sync(0xffffffffu, open2);
     if (mode == kFinStore) return false;
     bool done = !any_act, gate = f.gate != 0.0;
     if (threadIdx.x == 0 && any_bad) sc(scal, S_FLAGS, F_NUMERIC) = 1.0;
