@@ -1321,7 +1321,9 @@ template <int NC> __global__ void __launch_bounds__(128) k_clover_logdet(Geom g,
 
 constexpr int kLogdetBlocks = 256;
 
-size_t k_field_bytes(const Geom &g) { return ((size_t)2 * g.vh * 18 * sizeof(double) + 255) & ~(size_t)255; }
+// the insertion field's share of a caller's workspace: 48 doubles a site as the
+// entry points have always asked for, of which the field fills 18
+size_t k_field_bytes(const Geom &g) { return ((size_t)2 * g.vh * 48 * sizeof(double) + 255) & ~(size_t)255; }
 
 hr_status leaf_force(hr_ctx *ctx, const Geom &g, const double *can, const double *K, double scale, double *F,
                      cudaStream_t s)
@@ -1341,7 +1343,7 @@ size_t hr_clover_force_workspace_bytes(hr_lattice lat)
     if (hr_gauge_packed_bytes(lat, HR_FUND, HR_F64) == 0) return 0;
     const Geom g = make_geom(lat, 1);
     const size_t half = spinor_half_bytes(g, HR_FUND, kF64);
-    return k_field_bytes(g) + 3 * half;
+    return k_field_bytes(g) + 5 * half;
 }
 
 hr_status hr_clover_insertion_force(hr_ctx *ctx, hr_lattice lat, double c_sw, const double *gauge, const double *lam,
