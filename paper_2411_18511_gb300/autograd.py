@@ -65,8 +65,8 @@ class _Lattice:
 
     # packed buffers: a full field is [even half | odd half]
     def full(self, psi=None) -> torch.Tensor:
-        if psi is None:
-            return torch.zeros(2 * self.half, dtype=torch.uint8, device=self.dev)
+        if psi is None:  # an operator's result: every site gets written
+            return fields.empty_bytes(2 * self.half, self.dev)
         return fields.pack_spinor(self.ctx, self.dims, hr.HR_FUND, hr.HR_F64, hr.HR_FULL, psi.detach().contiguous())
 
     def even(self, psi=None) -> torch.Tensor:
@@ -127,18 +127,17 @@ class DiracApply(torch.autograd.Function):
         lat = _Lattice(ctx.dims, q)
         gp = lat.full(g.contiguous())
         grad_q = grad_psi = None
-        if ctx.needs_input_grad[1]:
-            t = gp.clone()                      # D^+ g = g5 D g5 g
-            lat.gamma5(lat.ev(t))
-            lat.gamma5(lat.od(t))
-            out = lat.full()
-            lat.dirac(ctx.m0, t, out)
-            lat.gamma5(lat.ev(out))
-            lat.gamma5(lat.od(out))
-            grad_psi = lat.unpack_full(out)
         if ctx.needs_input_grad[0]:
             grad_q = torch.zeros_like(q)
             hr.hr_link_grad(lat.ctx, ctx.dims, gp, lat.full(psi), -0.5, grad_q)
+        if ctx.needs_input_grad[1]:
+            lat.gamma5(lat.ev(gp))              # D^+ g = g5 D g5 g, g in place
+            lat.gamma5(lat.od(gp))
+            out = lat.full()
+            lat.dirac(ctx.m0, gp, out)
+            lat.gamma5(lat.ev(out))
+            lat.gamma5(lat.od(out))
+            grad_psi = lat.unpack_full(out)
         return grad_q, grad_psi, None, None
 
 

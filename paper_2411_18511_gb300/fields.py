@@ -66,7 +66,9 @@ def unpack_spinor(ctx, dims, rep, prec, parity, packed, n_rhs: int = 1, stream=N
     """Packed -> canonical complex128 [V,4,nc] (or [n_rhs,...]); other-parity sites are zero."""
     V = volume(dims)
     shape = (V, 4, nc_of(rep)) if n_rhs == 1 else (n_rhs, V, 4, nc_of(rep))
-    out = torch.zeros(shape, dtype=torch.complex128, device=packed.device)
+    # a full field writes every site
+    make = torch.empty if parity == hr.HR_FULL else torch.zeros
+    out = make(shape, dtype=torch.complex128, device=packed.device)
     hr.hr_spinor_unpack(ctx, dims, rep, prec, parity, n_rhs, packed, torch.view_as_real(out), stream)
     return out
 

@@ -86,6 +86,15 @@ class Lattice(tuple):
         self.theta = theta
         return self
 
+    def c_struct(self) -> "hr_lattice":
+        """The ``hr_lattice`` that every call passes by value, filled once and
+        again whenever ``bc`` or ``theta`` was assigned."""
+        now = (self.bc, self.theta)
+        made = self.__dict__.get("_made")
+        if made is None or made[0] != now:
+            made = self._made = (now, _fill_lattice(self, self.bc, self.theta))
+        return made[1]
+
     def __repr__(self):
         tw = f", theta={self.theta}" if self.theta is not None else ""
         return f"Lattice({tuple(self)}, bc={self.bc}{tw})"
@@ -217,16 +226,21 @@ def library_path() -> str:
 
 # ------------------------------------------------------------------ helpers
 
-def lattice(dims) -> hr_lattice:
+def _fill_lattice(dims, bc, theta) -> hr_lattice:
     lat = hr_lattice()
     for k in range(4):
         lat.dims[k] = int(dims[k])
-    lat.bc = int(getattr(dims, "bc", 0))
-    theta = getattr(dims, "theta", None)
+    lat.bc = int(bc)
     if theta is not None:
         for k in range(4):
             lat.theta[k] = float(theta[k])
     return lat
+
+
+def lattice(dims) -> hr_lattice:
+    if type(dims) is Lattice:
+        return dims.c_struct()
+    return _fill_lattice(dims, getattr(dims, "bc", 0), getattr(dims, "theta", None))
 
 
 def _ptr(x):
@@ -240,7 +254,8 @@ def _ptr(x):
 def _stream(stream):
     if stream is None:
         import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        # the raw handle of torch.cuda.current_stream(), without the Stream object around it
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     if hasattr(stream, "cuda_stream"):
         return ctypes.c_void_p(stream.cuda_stream)
     return ctypes.c_void_p(int(stream))
