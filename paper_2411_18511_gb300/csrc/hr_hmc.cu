@@ -128,30 +128,48 @@ __device__ __forceinline__ int plane_of(int mu, int nu)
     return a == 0 ? b - 1 : a + b;
 }
 
-// one thread per site and group of `per` planes: vec P of the n sites from slice `first` on
-template <bool VEC>
-__global__ void __launch_bounds__(128) k_plaq_vec(Geom g, const double *__restrict__ q, int first, int n, int per,
+// Vec P of the n sites from slice `first` on.  PER = 6: one thread per site, its own
+// four links converted once and kept in shared memory (a conversion is some 90
+// instructions, 24 of them a site were half of the kernel); 1: one per plane (blockIdx.y).
+template <bool VEC, int PER>
+__global__ void __launch_bounds__(128) k_plaq_vec(Geom g, const double *__restrict__ q, int first, int n,
                                                   int4 *__restrict__ pa, int2 *__restrict__ pb)
 {
+    constexpr int OWN = PER == 6 ? 8 : 1;
+    __shared__ int4 own[OWN][128]; // this thread's slots: no other thread reads them
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int V = 2 * g.vh, slice = g.d[1] * g.d[2] * g.d[3];
     int t = first * slice + i;
     if (t < 0) t += V;
     const LexSite x = lex_site(g, t);
+    bool ok_own = true;
+    if constexpr (PER == 6) {
 #pragma unroll 1
-    for (int p = blockIdx.y * per; p < (blockIdx.y + 1) * per; ++p) {
+        for (int mu = 0; mu < 4; ++mu) {
+            const fxq u = load_fxq_unit<VEC>(q, (size_t)mu * V + t, ok_own);
+            own[2 * mu][threadIdx.x] = make_int4(u.c[0].h, u.c[0].l, u.c[1].h, u.c[1].l);
+            own[2 * mu + 1][threadIdx.x] = make_int4(u.c[2].h, u.c[2].l, u.c[3].h, u.c[3].l);
+        }
+    }
+    auto own_link = [&](int mu, bool &ok) -> fxq {
+        if constexpr (PER == 6) {
+            const int4 a = own[2 * mu][threadIdx.x], b = own[2 * mu + 1][threadIdx.x];
+            return {{{a.x, a.y}, {a.z, a.w}, {b.x, b.y}, {b.z, b.w}}};
+        } else {
+            return load_fxq_unit<VEC>(q, (size_t)mu * V + t, ok);
+        }
+    };
+    const int p0 = PER == 6 ? 0 : blockIdx.y;
+#pragma unroll 1
+    for (int p = p0; p < p0 + PER; ++p) {
         const int mu = p < 3 ? 0 : p < 5 ? 1 : 2, nu = p < 3 ? p + 1 : p < 5 ? p - 1 : 3;
         int up_mu, up_nu, unused;
         lex_steps(g, x, mu, up_mu, unused);
         lex_steps(g, x, nu, up_nu, unused);
-        const size_t bm = (size_t)mu * V + t, bn = (size_t)nu * V + t;
-        bool ok = true;
-        fxq a = load_fxq_unit<VEC>(q, bm, ok), b = load_fxq_unit<VEC>(q, bn + up_mu, ok);
-        const fxq A = fxq_mul(a, b);
-        a = load_fxq_unit<VEC>(q, bn, ok);
-        b = load_fxq_unit<VEC>(q, bm + up_nu, ok);
-        const fxq B = fxq_conj(fxq_mul(a, b));
+        bool ok = ok_own;
+        const fxq A = fxq_mul(own_link(mu, ok), load_fxq_unit<VEC>(q, (size_t)nu * V + t + up_mu, ok));
+        const fxq B = fxq_conj(fxq_mul(own_link(nu, ok), load_fxq_unit<VEC>(q, (size_t)mu * V + t + up_nu, ok)));
         fxa w[3] = {};
         fxq_mac_vec(w, A, B);
         const fx v0 = fx_of(w[0]), v1 = fx_of(w[1]), v2 = fx_of(w[2]);
@@ -467,7 +485,8 @@ void launch_gauge_force(hr_ctx *ctx, const Geom &g, double c, const double *q, d
         int4 *pa = (int4 *)ctx->d_plaq;
         int2 *pb = (int2 *)(pa + 6LL * n);
         const unsigned nb = (unsigned)((n + 127) / 128), mb = (unsigned)((m + 127) / 128);
-        k_plaq_vec<VEC><<<dim3(nb, small ? 6 : 1), 128, 0, s>>>(g, q, first, n, small ? 1 : 6, pa, pb);
+        if (small) k_plaq_vec<VEC, 1><<<dim3(nb, 6), 128, 0, s>>>(g, q, first, n, pa, pb);
+        else k_plaq_vec<VEC, 6><<<nb, 128, 0, s>>>(g, q, first, n, pa, pb);
         if (small) k_plaq_force<VEC, 1><<<dim3(mb, 4), 128, 0, s>>>(g, c, q, F, a * slice, m, first, n, pa, pb);
         else k_plaq_force<VEC, 4><<<mb, 128, 0, s>>>(g, c, q, F, a * slice, m, first, n, pa, pb);
     }
