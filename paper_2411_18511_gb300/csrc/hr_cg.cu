@@ -195,21 +195,28 @@ struct Solver {
     // |r|^2 -> beta), then for the mixed solver the reliable update, then
     // part_b (p = r + beta p).  Both parts skip when the solve is done or a
     // reliable update is due; the update ends with part_b.  `cond`: the last
-    // reduction also sets the condition of the IF node that follows.
-    hr_status part_a(FinCond cond = {0, 0})
+    // reduction also sets the condition of the IF node that follows; `leave`:
+    // who finishes it (kLeaveFew: finish_b, which is then part_b too).
+    hr_status part_a(FinCond cond = {0, 0}, int leave = kLeaveNone)
     {
         const double *done = flag_ptr(ctx, F_SKIP);
         if (!mixed()) {
             // q = A p with the x/r update and |r|^2 fused into the last hop
-            const CgFuse fz{x, p64, r64, kFinBeta, cond};
+            const CgFuse fz{x, p64, r64, kFinBeta, cond, leave};
             return apply_eo_op(ctx, g, m0, rep, kF64, HR_OP_NORMAL, gauge, p64, q64, t64, u64, kFinAlpha, nullptr,
                                done, s, &fz, clov64);
         }
         // p, r in the inner precision, x_lo in FP32: fused as above (the
         // last hop's epilogue updates x_lo and r from q in registers)
-        const CgFuse fz{x_lo, p_lo, r_lo, kFinBetaMixed, cond};
+        const CgFuse fz{x_lo, p_lo, r_lo, kFinBetaMixed, cond, leave};
         return apply_eo_op(ctx, g, m0, rep, o.inner_prec, HR_OP_NORMAL, gauge_lo, p_lo, q_lo, t_lo, u_lo, kFinAlpha,
                            nullptr, done, s, &fz, clov_lo);
+    }
+    hr_status finish_b(FinCond cond)
+    {
+        if (ctx->fin_rows == 0) return part_b(); // the hop finished its sum
+        return blas_p_fin(ctx, g, rep, mixed() ? o.inner_prec : kF64, mixed() ? p_lo : p64, mixed() ? r_lo : r64,
+                          mixed() ? kFinBetaMixed : kFinBeta, flag_ptr(ctx, F_SKIP), cond, s);
     }
 
     // x += x_lo, r = b - A x in FP64, restart the low-precision residual;
@@ -398,8 +405,8 @@ hr_status capture_while_graph(Solver &sv, int per_pass, cudaGraph_t *out)
                 return fail("gate condition");
             cond = FinCond{1, hgate};
         }
-        if ((st = sv.part_a(cond))) return fail("iteration");
-        if ((st = sv.part_b())) return fail("iteration");
+        if ((st = sv.part_a(cond, kLeaveFew))) return fail("iteration");
+        if ((st = sv.finish_b(cond))) return fail("iteration");
         if (update) {
             cudaStreamCaptureStatus cst;
             const cudaGraphNode_t *d = nullptr;

@@ -96,13 +96,13 @@ template <int REP, int PREC> struct PlainLaunch {
     static bool run(hr_ctx *ctx, const HopArgs &a, HopChoice c, int grid, cudaStream_t s, hr_status &st)
     {
         if (c.variant == kVarSimpleR96) {
-            if (a.g5_in) launch_after(k_hop_r96<REP, PREC, 1>, early_start(a.g), grid, c.block, 0, s, a);
-            else launch_after(k_hop_r96<REP, PREC, 0>, early_start(a.g), grid, c.block, 0, s, a);
+            if (a.g5_in) launch_after(k_hop_r96<REP, PREC, 1>, hop_early(a), grid, c.block, 0, s, a);
+            else launch_after(k_hop_r96<REP, PREC, 0>, hop_early(a), grid, c.block, 0, s, a);
             st = hop_launched(ctx, a, grid, s, "hop kernel (96 registers)");
             return true;
         }
-        if (a.g5_in) launch_after(k_hop<REP, PREC, 1>, early_start(a.g), grid, c.block, 0, s, a);
-        else launch_after(k_hop<REP, PREC, 0>, early_start(a.g), grid, c.block, 0, s, a);
+        if (a.g5_in) launch_after(k_hop<REP, PREC, 1>, hop_early(a), grid, c.block, 0, s, a);
+        else launch_after(k_hop<REP, PREC, 0>, hop_early(a), grid, c.block, 0, s, a);
         st = hop_launched(ctx, a, grid, s, "hop kernel");
         return true;
     }
@@ -111,8 +111,8 @@ template <int REP, int PREC> struct PlainLaunch {
 template <int REP, int PREC> struct ClovLaunch {
     static bool run(hr_ctx *ctx, const HopArgs &a, int grid, int block, cudaStream_t s, hr_status &st)
     {
-        if (a.g5_in) launch_after(k_hop_clov<REP, PREC, 1>, early_start(a.g), grid, block, 0, s, a);
-        else launch_after(k_hop_clov<REP, PREC, 0>, early_start(a.g), grid, block, 0, s, a);
+        if (a.g5_in) launch_after(k_hop_clov<REP, PREC, 1>, hop_early(a), grid, block, 0, s, a);
+        else launch_after(k_hop_clov<REP, PREC, 0>, hop_early(a), grid, block, 0, s, a);
         st = hop_launched(ctx, a, grid, s, "hop kernel (clover epilogue)");
         return true;
     }
@@ -210,6 +210,8 @@ HopArgs make_args(hr_ctx *ctx, const Geom &g, const HopLaunch &L)
     a.clov = L.clov;
     a.clov_mode = L.clov ? L.clov_mode : kClovNone;
     a.cond = L.cond;
+    a.leave = L.leave;
+    a.joined = L.joined;
     return a;
 }
 
@@ -277,6 +279,11 @@ bool hop_variant_available(int rep, int prec, int variant, int nrhs)
     return variant == kVarSimple || (variant >= kVarStaged && variant < kNumHopVariants && rep != HR_ADJ_MAT);
 }
 
+static hr_status stream_wait(hr_ctx *ctx, cudaStream_t s, cudaEvent_t e)
+{
+    return cudaStreamWaitEvent(s, e, 0) == cudaSuccess ? HR_OK : check_launch(ctx, "stream wait");
+}
+
 // Even-site operators from two hops each:
 //   Mhat    : t_o = H_oe in;        out = A in - c H_eo t_o
 //   Mhat^+  : t_o = H_oe g5 in;     out = A in - c g5 H_eo t_o
@@ -299,7 +306,8 @@ hr_status apply_eo_op(hr_ctx *ctx, const Geom &g, double m0, int rep, int prec, 
     L.gauge = gauge;
     L.gate = gate;
     L.done = done;
-    auto schur = [&](const void *src, void *dst, bool dag, int fin, const CgFuse *fz) -> hr_status {
+    // join: the second hop waits for the finishing launch beside the first one
+    auto schur = [&](const void *src, void *dst, bool dag, int fin, const CgFuse *fz, bool join = false) -> hr_status {
         HopLaunch h1 = L;
         h1.p = 1;
         h1.in = src;
@@ -316,6 +324,7 @@ hr_status apply_eo_op(hr_ctx *ctx, const Geom &g, double m0, int rep, int prec, 
         }
         hr_status e = launch_hop(ctx, g, rep, prec, h1, s);
         if (e) return e;
+        if (join && (e = stream_wait(ctx, s, ctx->ev_join))) return e;
         HopLaunch h2 = L;
         h2.p = 0;
         h2.in = work_odd;
@@ -326,6 +335,8 @@ hr_status apply_eo_op(hr_ctx *ctx, const Geom &g, double m0, int rep, int prec, 
         h2.g5_in = 0;
         h2.g5_out = dag ? 1 : 0;
         h2.fin = fin;
+        h2.leave = fin == kFinAlpha ? kLeaveAll : kLeaveNone;
+        h2.joined = join;
         if (clover) {
             h2.alpha = 1.0;
             h2.beta = -0.25;
@@ -338,6 +349,7 @@ hr_status apply_eo_op(hr_ctx *ctx, const Geom &g, double m0, int rep, int prec, 
             h2.cg_p = fz->p;
             h2.cg_r = fz->r;
             h2.cond = fz->cond;
+            h2.leave = fz->leave;
         }
         return launch_hop(ctx, g, rep, prec, h2, s);
     };
@@ -347,7 +359,14 @@ hr_status apply_eo_op(hr_ctx *ctx, const Geom &g, double m0, int rep, int prec, 
     case HR_OP_NORMAL:
         st = schur(in, work_even, false, fin_schur, nullptr);
         if (st) return st;
-        return schur(work_even, out, true, kFinNone, fuse);
+        if (fin_schur != kFinAlpha) return schur(work_even, out, true, kFinNone, fuse);
+        // alpha is first used by the last hop: its sum is finished beside the third
+        // (4 to 9 us an iteration off the recurrence's chain)
+        if (cudaEventRecord(ctx->ev_fork, s) != cudaSuccess) return check_launch(ctx, "fork");
+        if ((st = stream_wait(ctx, ctx->side, ctx->ev_fork))) return st;
+        if ((st = finish_sums(ctx, ctx->fin_rows, g.nrhs, fin_schur, gate, done, ctx->side))) return st;
+        if (cudaEventRecord(ctx->ev_join, ctx->side) != cudaSuccess) return check_launch(ctx, "join");
+        return schur(work_even, out, true, kFinNone, fuse, true);
     }
     return set_error(ctx, HR_ERR_INVALID_ARG, "bad op %d", op);
 }

@@ -125,8 +125,8 @@ template <int PREC>
 void launch_chunk(const HopArgs &a, int lc, int grid, int block, cudaStream_t s)
 {
     const bool g5 = a.g5_in != 0;
-    if (lc == 1) launch_after(g5 ? k_hop_chunk<PREC, 1, 1> : k_hop_chunk<PREC, 1, 0>, early_start(a.g), grid, block, 0, s, a);
-    else launch_after(g5 ? k_hop_chunk<PREC, 2, 1> : k_hop_chunk<PREC, 2, 0>, early_start(a.g), grid, block, 0, s, a);
+    if (lc == 1) launch_after(g5 ? k_hop_chunk<PREC, 1, 1> : k_hop_chunk<PREC, 1, 0>, hop_early(a), grid, block, 0, s, a);
+    else launch_after(g5 ? k_hop_chunk<PREC, 2, 1> : k_hop_chunk<PREC, 2, 0>, hop_early(a), grid, block, 0, s, a);
 }
 
 } // namespace

@@ -34,7 +34,9 @@ struct HopArgs {
                            // kernels' copies but never queue them
     const void *clov;      // clover half-field of the output parity (kClovAux / kClovOut), or nullptr
     int clov_mode;
-    FinCond cond;          // host side: condition handle the finishing launch sets
+    FinCond cond;          // host side: condition handle the finishing launch sets,
+    int leave;             // who finishes (LeaveRows),
+    int joined;            // the launch follows two others
 };
 
 // Waits for the launches before; nothing to do when gated off, or the solver
@@ -45,6 +47,7 @@ __device__ __forceinline__ bool hop_skipped(const HopArgs &a)
     return (a.gate && *a.gate == 0.0) || (a.done && *a.done != 0.0);
 }
 
+inline bool hop_early(const HopArgs &a) { return !a.joined && early_start(a.g); }
 // the grid of a hop kernel of one thread per item: a reducing launch is capped
 // so that its rows of partial sums fit the context's scratch
 inline int hop_grid(const HopArgs &a, long long n, int block)
@@ -55,8 +58,10 @@ inline int hop_grid(const HopArgs &a, long long n, int block)
 inline hr_status hop_launched(hr_ctx *ctx, const HopArgs &a, int grid, cudaStream_t s, const char *what)
 {
     hr_status st = check_launch(ctx, what);
-    if (!st && a.fin) st = finish_sums(ctx, grid, a.g.nrhs, a.fin, a.gate, a.done, s, a.cond);
-    return st;
+    if (st || !a.fin) return st;
+    const bool leave = a.leave == kLeaveAll || (a.leave == kLeaveFew && (long long)grid * a.g.nrhs <= kFoldSums);
+    ctx->fin_rows = leave ? grid : 0;
+    return leave ? HR_OK : finish_sums(ctx, grid, a.g.nrhs, a.fin, a.gate, a.done, s, a.cond);
 }
 
 

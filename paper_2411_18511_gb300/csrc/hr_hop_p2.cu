@@ -217,8 +217,8 @@ template <int PREC>
 void launch_p2(const HopArgs &a, HopChoice c, int grid, cudaStream_t s)
 {
     const bool g5 = a.g5_in != 0;
-    if (c.variant == kVarPairSitesR96) launch_after(g5 ? k_hop_p2_r96<PREC, 1> : k_hop_p2_r96<PREC, 0>, early_start(a.g), grid, c.block, 0, s, a);
-    else launch_after(g5 ? k_hop_p2<PREC, 1> : k_hop_p2<PREC, 0>, early_start(a.g), grid, c.block, 0, s, a);
+    if (c.variant == kVarPairSitesR96) launch_after(g5 ? k_hop_p2_r96<PREC, 1> : k_hop_p2_r96<PREC, 0>, hop_early(a), grid, c.block, 0, s, a);
+    else launch_after(g5 ? k_hop_p2<PREC, 1> : k_hop_p2<PREC, 0>, hop_early(a), grid, c.block, 0, s, a);
 }
 
 } // namespace

@@ -178,11 +178,11 @@ template <int REP, int PREC> struct Launch {
             const long long ntiles = (nv + c.block - 1) / c.block;
             const int tgrid = hop_grid(a, ntiles, 1);
             if (c.variant == kVarTile) {
-                if (a.g5_in) launch_after(k_hop_tile<REP, PREC, 1>, early_start(a.g), tgrid, c.block, sm, s, a);
-                else launch_after(k_hop_tile<REP, PREC, 0>, early_start(a.g), tgrid, c.block, sm, s, a);
+                if (a.g5_in) launch_after(k_hop_tile<REP, PREC, 1>, hop_early(a), tgrid, c.block, sm, s, a);
+                else launch_after(k_hop_tile<REP, PREC, 0>, hop_early(a), tgrid, c.block, sm, s, a);
             } else {
-                if (a.g5_in) launch_after(k_hop_tile_r96<REP, PREC, 1>, early_start(a.g), tgrid, c.block, sm, s, a);
-                else launch_after(k_hop_tile_r96<REP, PREC, 0>, early_start(a.g), tgrid, c.block, sm, s, a);
+                if (a.g5_in) launch_after(k_hop_tile_r96<REP, PREC, 1>, hop_early(a), tgrid, c.block, sm, s, a);
+                else launch_after(k_hop_tile_r96<REP, PREC, 0>, hop_early(a), tgrid, c.block, sm, s, a);
             }
             st = hop_launched(ctx, a, tgrid, s, "tiled hop kernel");
             return true;

@@ -44,6 +44,10 @@ struct hr_ctx {
     double *d_scal = nullptr;      // kScalDoubles
     double *h_scal = nullptr;      // pinned mirror
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    // a finishing launch beside the next hop: its stream, fork and join
+    cudaStream_t side = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    int fin_rows = 0; // rows that the last reducing hop left to its caller (HopLaunch::leave)
     std::map<std::string, hr::HopChoice> tuned; // autotuner: configuration key -> launch shape
     std::string tune_cache_path;                // JSON cache (HR_AUTOTUNE_CACHE), "" = none
     // instantiated CG iteration graphs, keyed by everything they bake in
@@ -88,7 +92,7 @@ inline int grid_for(long long n, int block, int cap)
 // device counters: blocks of a finishing launch, native-path requests
 // (C_PACK: the pack status word, kPack* flags of the values packed since the
 // last check, read and cleared by consume_pack_status)
-enum Counter { C_FIN = 0, C_PACK = 62, C_STATUS = 63 };
+enum Counter { C_FIN = 0, C_FOLD = 1, C_PACK = 62, C_STATUS = 63 };
 
 // clover site term in a hop epilogue (hr_clover.cuh): none, A(x) on the aux
 // term (out = alpha A aux + beta acc), or A(x) on the result (out = A (alpha aux + beta acc))
@@ -129,6 +133,12 @@ struct FinCond {
 hr_status finish_sums(hr_ctx *ctx, int nparts, int nrhs, int fin, const double *gate, const double *done,
                       cudaStream_t s, FinCond cond = {0, 0});
 
+// Who finishes a reducing hop's rows: the launch itself; the caller; the caller if
+// they are few enough for every block of the next kernel to add them (kFoldSums), else
+// the launch (fin_rows = 0 then)
+enum LeaveRows { kLeaveNone = 0, kLeaveAll = 1, kLeaveFew = 2 };
+constexpr int kFoldSums = 1024;
+
 // ---- hop launches (hr_hop.cu) ----
 struct HopLaunch {
     int p;                 // output parity
@@ -151,6 +161,8 @@ struct HopLaunch {
     const void *clov;
     int clov_mode;
     FinCond cond;
+    int leave;  // of a reducing launch: kLeaveNone, or the caller finishes the rows (ctx->fin_rows)
+    int joined; // the launch waits for another stream too: no early start
 };
 // a CG x/r update fused into the last hop of an operator (the operator's
 // precision; x in FP32 when the operator runs in binary16)
@@ -160,6 +172,7 @@ struct CgFuse {
     void *r;
     int fin; // kFinBeta or kFinBetaMixed
     FinCond cond;
+    int leave; // LeaveRows of that hop
 };
 hr_status launch_hop(hr_ctx *ctx, const Geom &g, int rep, int prec, const HopLaunch &L, cudaStream_t s);
 hr_status launch_hop_with(hr_ctx *ctx, const Geom &g, int rep, int prec, const HopLaunch &L, HopChoice c,
@@ -200,6 +213,9 @@ hr_status clover_apply_half(hr_ctx *ctx, const Geom &g, int rep, int prec, const
 // ---- BLAS launches (hr_blas.cu) ----
 hr_status blas_norm2(hr_ctx *ctx, const Geom &g, int rep, int prec, const void *v, int fin, cudaStream_t s);
 hr_status blas_p(hr_ctx *ctx, const Geom &g, int rep, int pp, int pr, void *p, const void *r, cudaStream_t s);
+// the same after finishing the last hop's few rows (ctx->fin_rows) with the update `fin`
+hr_status blas_p_fin(hr_ctx *ctx, const Geom &g, int rep, int prec, void *p, const void *r, int fin, const double *done,
+                     FinCond cond, cudaStream_t s);
 hr_status blas_convert(hr_ctx *ctx, const Geom &g, int rep, int psrc, int pdst, const void *src, void *dst,
                        const double *gate, cudaStream_t s);
 // r = b - ax (FP64) with |r|^2 -> fin; also writes r in precision plo to r_lo when given

@@ -1065,7 +1065,7 @@ __device__ __forceinline__ double &sc(double *scal, int slot, int r) { return sc
 // The scalars one right-hand side's update reads, loaded together (and, by the
 // finishing kernel, before the sums are there): one round trip instead of a chain.
 struct FinIn {
-    double active, rr, rrold, stop, rmax, rref, d2, tol2, cap, dmid, iters, gate, tier2;
+    double active, rr, rrold, stop, rmax, rref, d2, tol2, cap, dmid, iters, gate, tier2, numeric;
 };
 __device__ __forceinline__ FinIn load_fin(double *scal, int nrhs)
 {
@@ -1084,17 +1084,29 @@ __device__ __forceinline__ FinIn load_fin(double *scal, int nrhs)
     f.iters = sc(scal, S_FLAGS, F_ITERS);
     f.gate = sc(scal, S_FLAGS, F_GATE);
     f.tier2 = sc(scal, S_FLAGS, F_TIER2);
+    f.numeric = sc(scal, S_FLAGS, F_NUMERIC);
     return f;
 }
 
 // Scalar updates on the finished sums by the first warp of a block (lanes
 // 0..nrhs-1 hold one right-hand side each); thread 0 then refreshes the flags.
-// Returns, in that warp, whether a reliable update is due (the gate is open and
-// the solve goes on).
-__device__ inline bool finish_reduction(int mode, const double *sums, int nrhs, double *scal, const FinIn &f)
+// WRITE = false: only the outcome, nothing is stored (a kernel in which every
+// block needs it and one stores).
+struct FinOut {
+    bool update; // a reliable update is due (the gate is open and the solve goes on)
+    bool skip;   // the recurrence stops here: done, or an update is due
+    double beta; // of this lane's right-hand side (kFinBeta, kFinBetaMixed)
+};
+template <bool WRITE = true>
+__device__ inline FinOut finish_reduction(int mode, const double *sums, int nrhs, double *scal, const FinIn &f)
 {
     const int r = threadIdx.x;
-    if (r >= 32) return false;
+    FinOut out = {false, false, 0.0};
+    if (r >= 32) return out;
+    // a scalar of this right-hand side
+    auto put = [&](int slot, double x) {
+        if constexpr (WRITE) sc(scal, slot, r) = x;
+    };
     bool act = false, bad = false, open = false, open2 = false;
     if (r < nrhs) {
         const double v = sums[r];
@@ -1102,23 +1114,23 @@ __device__ inline bool finish_reduction(int mode, const double *sums, int nrhs, 
         bad = !isfinite(v) && mode != kFinStore;
         switch (mode) {
         case kFinStore:
-            sc(scal, S_OUT, r) = v;
+            put(S_OUT, v);
             break;
         case kFinAlpha:
-            sc(scal, S_PAP, r) = v;
-            sc(scal, S_ALPHA, r) = (act && v > 0.0) ? f.rr / v : 0.0;
+            put(S_PAP, v);
+            put(S_ALPHA, (act && v > 0.0) ? f.rr / v : 0.0);
             break;
         case kFinBeta:
         case kFinBetaMixed: {
-            sc(scal, S_RROLD, r) = f.rr;
+            put(S_RROLD, f.rr);
             if (act) {
-                sc(scal, S_BETA, r) = v / f.rr;
-                sc(scal, S_RR, r) = v;
+                out.beta = v / f.rr;
+                put(S_RR, v);
                 if (mode == kFinBeta) {
                     if (v <= f.stop) act = false;
                 } else {
                     const double rmax = fmax(f.rmax, v);
-                    sc(scal, S_RMAX, r) = rmax;
+                    put(S_RMAX, rmax);
                     const bool conv = v <= f.stop;
                     if (conv || v < f.d2 * rmax) {
                         open = true;
@@ -1127,57 +1139,56 @@ __device__ inline bool finish_reduction(int mode, const double *sums, int nrhs, 
                         open2 = f.dmid == 0.0 || conv || v < f.dmid * f.rref;
                     }
                 }
-            } else {
-                sc(scal, S_BETA, r) = 0.0;
             }
+            put(S_BETA, out.beta);
             break;
         }
         case kFinInit:
-            sc(scal, S_RR, r) = v;
-            sc(scal, S_RMAX, r) = v;
-            sc(scal, S_RROLD, r) = v;
-            sc(scal, S_RREF, r) = v;
+            put(S_RR, v);
+            put(S_RMAX, v);
+            put(S_RROLD, v);
+            put(S_RREF, v);
             act = v > f.stop;
             break;
         case kFinBB:
-            sc(scal, S_BB, r) = v;
-            sc(scal, S_STOP, r) = f.tol2 * v;
+            put(S_BB, v);
+            put(S_STOP, f.tol2 * v);
             break;
         case kFinResidual:
             if (act) {
-                sc(scal, S_BETA, r) = v / f.rrold;
-                sc(scal, S_RR, r) = v;
-                sc(scal, S_RMAX, r) = v;
+                put(S_BETA, v / f.rrold);
+                put(S_RR, v);
+                put(S_RMAX, v);
                 if (v <= f.stop) act = false;
             } else {
-                sc(scal, S_BETA, r) = 0.0;
+                put(S_BETA, 0.0);
             }
-            sc(scal, S_OUT, r) = v;
-            sc(scal, S_RREF, r) = v;
+            put(S_OUT, v);
+            put(S_RREF, v);
             break;
         case kFinMid:
             // r = r_ref - A_32 dx is accurate to FP32 relative to r_ref only: it
             // restarts the recurrence but stops no right-hand side
             if (act) {
-                sc(scal, S_BETA, r) = v / f.rrold;
-                sc(scal, S_RR, r) = v;
-                sc(scal, S_RMAX, r) = v;
+                put(S_BETA, v / f.rrold);
+                put(S_RR, v);
+                put(S_RMAX, v);
             } else {
-                sc(scal, S_BETA, r) = 0.0;
+                put(S_BETA, 0.0);
             }
             break;
         default:
             break;
         }
-        if (mode == kFinBeta || mode == kFinResidual || mode == kFinInit) sc(scal, S_ACTIVE, r) = act ? 1.0 : 0.0;
+        if (mode == kFinBeta || mode == kFinResidual || mode == kFinInit) put(S_ACTIVE, act ? 1.0 : 0.0);
     }
     const bool any_bad = __any_sync(0xffffffffu, bad), any_act = __any_sync(0xffffffffu, act);
     const bool any_open = __any_sync(0xffffffffu, open), any_open2 = __any_sync(0xffffffffu, open2);
-    if (mode == kFinStore) return false;
+    if (mode == kFinStore) return out;
     bool done = !any_act, gate = f.gate != 0.0;
-    if (threadIdx.x == 0 && any_bad) sc(scal, S_FLAGS, F_NUMERIC) = 1.0;
-    if (mode == kFinBB) return false;
-    done = done || any_bad || sc(scal, S_FLAGS, F_NUMERIC) != 0.0;
+    if (WRITE && threadIdx.x == 0 && any_bad) sc(scal, S_FLAGS, F_NUMERIC) = 1.0;
+    if (mode == kFinBB) return out;
+    done = done || any_bad || f.numeric != 0.0;
     if (mode == kFinBeta || mode == kFinBetaMixed) {
         // the iteration cap also stops the recurrence (work already queued skips)
         done = done || (f.cap > 0.0 && f.iters + 1.0 >= f.cap);
@@ -1193,7 +1204,7 @@ __device__ inline bool finish_reduction(int mode, const double *sums, int nrhs, 
     } else if (mode == kFinMid) {
         gate = false;
     }
-    if (threadIdx.x == 0) {
+    if (WRITE && threadIdx.x == 0) {
         double *fl = scal + S_FLAGS * kMaxRhsSlots;
         if (mode == kFinBeta || mode == kFinBetaMixed) fl[F_ITERS] = f.iters + 1.0;
         if (mode == kFinBetaMixed) fl[F_TIER1] = tier1 ? 1.0 : 0.0;
@@ -1210,7 +1221,9 @@ __device__ inline bool finish_reduction(int mode, const double *sums, int nrhs, 
         fl[F_DONE] = done ? 1.0 : 0.0;
         fl[F_SKIP] = done || gate ? 1.0 : 0.0;
     }
-    return gate && !done;
+    out.update = gate && !done;
+    out.skip = gate || done;
+    return out;
 }
 
 } // namespace hr
