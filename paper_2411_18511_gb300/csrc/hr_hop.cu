@@ -73,6 +73,13 @@ __global__ void __launch_bounds__(256) k_hop_clov(HopArgs a)
 {
     hop_body<REP, PREC, G5IN, true>(a);
 }
+// FP32 and binary16: given 96 registers the compiler keeps more loads in flight
+// than in the 64 to 88 it takes by itself
+template <int REP, int PREC, int G5IN>
+__global__ void __maxnreg__(96) k_hop_clov_r96(HopArgs a)
+{
+    hop_body<REP, PREC, G5IN, true>(a);
+}
 
 // ---------------------------------------------------------------- launch
 
@@ -111,8 +118,11 @@ template <int REP, int PREC> struct PlainLaunch {
 template <int REP, int PREC> struct ClovLaunch {
     static bool run(hr_ctx *ctx, const HopArgs &a, int grid, int block, cudaStream_t s, hr_status &st)
     {
-        if (a.g5_in) launch_after(k_hop_clov<REP, PREC, 1>, hop_early(a), grid, block, 0, s, a);
-        else launch_after(k_hop_clov<REP, PREC, 0>, hop_early(a), grid, block, 0, s, a);
+        if constexpr (PREC == kF64)
+            launch_after(a.g5_in ? k_hop_clov<REP, PREC, 1> : k_hop_clov<REP, PREC, 0>, hop_early(a), grid, block, 0, s, a);
+        else
+            launch_after(a.g5_in ? k_hop_clov_r96<REP, PREC, 1> : k_hop_clov_r96<REP, PREC, 0>, hop_early(a), grid, block,
+                         0, s, a);
         st = hop_launched(ctx, a, grid, s, "hop kernel (clover epilogue)");
         return true;
     }
@@ -131,7 +141,7 @@ hr_status dispatch(hr_ctx *ctx, const Geom &g, int rep, int prec, const HopArgs 
     if (a.clov_mode != kClovNone) {
         // the clover instantiations: paired staged for fundamental FP64, else unrolled
         const bool paired = rep == HR_FUND && prec == kF64;
-        const int block = paired ? 256 : 128;
+        const int block = paired ? 256 : prec == kF64 ? 128 : 64;
         const int grid = hop_grid(a, nv, block);
         hr_status st = HR_OK;
         if (paired) launch_hop_clover_paired(ctx, a, grid, block, s, st);
