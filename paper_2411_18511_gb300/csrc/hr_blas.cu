@@ -100,6 +100,11 @@ __global__ void __launch_bounds__(kFinThreads) k_finish(const double *partials, 
     if (cond.set && threadIdx.x == 0) cudaGraphSetConditional(cond.handle, out.update ? 1u : 0u);
 }
 
+// r + beta p, with the contraction fixed: the solve loops run k_p or k_p_fin and
+// agree bit for bit
+__device__ __forceinline__ float p_value(float r, float be, float p) { return __fmaf_rn(be, p, r); }
+__device__ __forceinline__ dd p_value(dd r, dd be, dd p) { return r + be * p; }
+
 // p = r + beta p
 template <int NC, int PP, int PR>
 __global__ void __launch_bounds__(kBS) k_p(Geom g, void *p, const void *r, const double *scal)
@@ -116,7 +121,7 @@ __global__ void __launch_bounds__(kBS) k_p(Geom g, void *p, const void *r, const
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int c = 0; c < NC; ++c) pv[a][c] = {rv[a][c].re + be * pv[a][c].re, rv[a][c].im + be * pv[a][c].im};
+            for (int c = 0; c < NC; ++c) pv[a][c] = {p_value(rv[a][c].re, be, pv[a][c].re), p_value(rv[a][c].im, be, pv[a][c].im)};
         store_spinor<NC, PP>(p, g.nblk_s, j, pv);
     }
 }
@@ -169,7 +174,7 @@ __global__ void __launch_bounds__(kBS) k_p_fin(Geom g, void *p, const void *r, c
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int c = 0; c < NC; ++c) pv[a][c] = {rv[a][c].re + be * pv[a][c].re, rv[a][c].im + be * pv[a][c].im};
+            for (int c = 0; c < NC; ++c) pv[a][c] = {p_value(rv[a][c].re, be, pv[a][c].re), p_value(rv[a][c].im, be, pv[a][c].im)};
         store_spinor<NC, P>(p, g.nblk_s, j, pv);
     }
 }
