@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(128) k_plaq_vec(Geom g, const double *__restri
 // and 1 / |U|^2 = 1 - d, d = |U|^2 - 1, so that links off unit length by up to
 // 2^-29 give the staple's value.  The others take native FP64.
 template <bool VEC, int NMU>
-__global__ void __launch_bounds__(128) k_plaq_force(Geom g, double s, const double *__restrict__ q,
+__global__ void __launch_bounds__(128, 5) k_plaq_force(Geom g, double s, const double *__restrict__ q,
                                                     double *__restrict__ F, int t0, int m, int first, int n,
                                                     const int4 *__restrict__ pa, const int2 *__restrict__ pb)
 {
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(128) k_plaq_force(Geom g, double s, const doub
     const int V = 2 * g.vh, slice = g.d[1] * g.d[2] * g.d[3];
     const int t = t0 + i, own = t - first * slice;
     const LexSite x = lex_site(g, t);
-    fxa acc[NMU][3] = {};
+    long long sum[NMU][3] = {}; // units 2^-56, rounded once per neighbour
     bool ok = true;
 #pragma unroll 1
     for (int nu = 0; nu < 4; ++nu) {
@@ -230,14 +230,17 @@ __global__ void __launch_bounds__(128) k_plaq_force(Geom g, double s, const doub
             const int sg = mu < nu ? 1 : -1;
             const fx o[3] = {{oa.x, oa.y}, {oa.z, oa.w}, {ob.x, ob.y}};
             fx tn[3];
+            fxa acc[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 const fx tt = fx_of(tc[a]), df = fx_sub(o[a], v[a]);
                 tn[a] = {-sg * tt.h, -sg * tt.l};
-                acc[k][a].a += fx_units64({sg * df.h, sg * df.l});
-                fx_mac(acc[k][a], w[0], tn[a]);
+                acc[a] = {fx_units64({sg * df.h, sg * df.l}), 0};
+                fx_mac(acc[a], w[0], tn[a]);
             }
-            fx_mac_cross(acc[k], wv, tn);
+            fx_mac_cross(acc, wv, tn);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) sum[k][a] += fx_round(acc[a]);
         }
     }
     const double c = s * 0x1p-56;
@@ -250,7 +253,7 @@ __global__ void __launch_bounds__(128) k_plaq_force(Geom g, double s, const doub
             continue;
         }
 #pragma unroll
-        for (int a = 0; a < 3; ++a) f[a] += c * (double)fx_round(acc[k][a]);
+        for (int a = 0; a < 3; ++a) f[a] += c * (double)sum[k][a];
     }
 }
 
@@ -470,19 +473,17 @@ hr_status check_md(hr_ctx *ctx, hr_lattice lat)
 template <bool VEC>
 void launch_gauge_force(hr_ctx *ctx, const Geom &g, double c, const double *q, double *F, cudaStream_t s)
 {
-    const int V = 2 * g.vh, T = g.d[0], slice = V / T;
-    const int slots = (int)std::min<long long>(T, (long long)(kPlaqBytes / kPlaqSiteBytes) / slice);
-    if (slots < 2) {
+    const int V = 2 * g.vh, slice = V / g.d[0];
+    const Slabs slabs = make_slabs(g, kPlaqSiteBytes);
+    if (slabs.n == 0) {
         k_gauge_force<VEC><<<dim3((unsigned)((V + 127) / 128), 4), 128, 0, s>>>(g, c, q, F);
         return;
     }
-    // the whole lattice, or slabs of about equal numbers of slices, each with the slice before it
-    const int nslab = slots == T ? 1 : (T + slots - 2) / (slots - 1);
     const bool small = V <= kPlaqSplitSites;
-    for (int k = 0; k < nslab; ++k) {
-        const int a = (int)((long long)T * k / nslab), b = (int)((long long)T * (k + 1) / nslab);
-        const int first = nslab == 1 ? 0 : a - 1, n = (b - first) * slice, m = (b - a) * slice;
-        int4 *pa = (int4 *)ctx->d_plaq;
+    for (int k = 0; k < slabs.n; ++k) {
+        const int a = slabs.lo(k), b = slabs.hi(k), first = slabs.n == 1 ? 0 : a - 1; // with the slice before it
+        const int n = (b - first) * slice, m = (b - a) * slice;
+        int4 *pa = (int4 *)ctx->d_slab;
         int2 *pb = (int2 *)(pa + 6LL * n);
         const unsigned nb = (unsigned)((n + 127) / 128), mb = (unsigned)((m + 127) / 128);
         if (small) k_plaq_vec<VEC, 1><<<dim3(nb, 6), 128, 0, s>>>(g, q, first, n, pa, pb);

@@ -23,7 +23,9 @@ constexpr int kMaxRhs = 32;
 constexpr int kMaxPartials = kMaxBlocks * kMaxRhs; // partial sums of one reducing launch
 constexpr int kFinBlocks = 64;       // blocks of a finishing launch, at most
 constexpr int kNumCounters = 64;
-constexpr size_t kPlaqBytes = 64u << 20, kPlaqSiteBytes = 144; // scratch of the gauge force
+// scratch of the forces, filled slab by slab: vectors of the gauge force, digits
+// of the link derivatives (bytes a site)
+constexpr size_t kSlabBytes = 64u << 20, kPlaqSiteBytes = 144, kDigitSiteBytes = 264;
 constexpr int kScalDoubles = 64 * kMaxRhs;
 
 // launch shape of the hop kernel chosen by the autotuner
@@ -40,7 +42,7 @@ struct hr_ctx {
     std::string err;
     double *d_partials = nullptr;  // kMaxPartials, then kFinBlocks * kMaxRhs sums of a finishing launch's blocks
     unsigned *d_counters = nullptr;
-    void *d_plaq = nullptr;        // kPlaqBytes: plaquette vectors of the gauge force
+    void *d_slab = nullptr;        // kSlabBytes: scratch of the forces
     double *d_scal = nullptr;      // kScalDoubles
     double *h_scal = nullptr;      // pinned mirror
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -192,6 +194,22 @@ hr_status apply_eo_op(hr_ctx *ctx, const Geom &g, double m0, int rep, int prec, 
                       const void *in, void *out, void *work_odd, void *work_even, int fin_schur,
                       const double *gate, const double *done, cudaStream_t s, const CgFuse *fuse = nullptr,
                       const void *clover = nullptr);
+
+// Slabs of time slices whose data (bytes a site) fit the context's scratch, each with
+// one neighbouring slice: `slots` slices fit; 0 slabs: not even two do.  Slab k of n
+// holds slices [lo, hi); n == 1 is the whole lattice, without a neighbour.
+struct Slabs {
+    int n, T;
+    int lo(int k) const { return (int)((long long)T * k / n); }
+    int hi(int k) const { return lo(k + 1); }
+};
+inline Slabs make_slabs(const Geom &g, size_t site_bytes)
+{
+    const long long slice = (long long)g.d[1] * g.d[2] * g.d[3], fit = (long long)(kSlabBytes / site_bytes) / slice;
+    const int T = g.d[0];
+    if (fit >= T) return {1, T};
+    return {fit < 2 ? 0 : (int)((T + fit - 2) / (fit - 1)), T};
+}
 
 // ---- link derivatives (hr_force.cu) ----
 // out += beta dRe<a, H b> for full fields given by their even and odd halves
