@@ -210,22 +210,69 @@ template <bool DAG> __device__ __forceinline__ void mac_links(fxa (&g)[4], const
     }
 }
 
-// Measured: hr_fermion_force at 32^4 (four hops and this kernel) 4.39 ms with the
-// native kernel, of it 3.97 ms in the kernel (bound by the FP64 pipe: about 700
-// conversions and 1400 operations a site), 0.905 ms with this one; error
-// against a 64-bit evaluation 7.2e-15 with both (the hops').  The kernel alone:
-// 0.479 ms at the compiler's 216 registers, 0.399 at 168, 0.438 at 128 (spills).
+// The fields as digits, 16 pairs and an exponent a site: each is read at five sites of
+// the link kernel, and converting it there took more than half of its instructions.
+// Slices above 127 k sites do not fit the scratch twice and are converted there.
+// Field f, vector v of slab site k at d[(8 f + v) n + k], its exponent at e[f n + k].
+struct Digits {
+    const int4 *d;
+    const int *e;
+    int n;
+};
+constexpr int kDigitBad = -1; // exponent of a site outside the fixed-point range
+
+__global__ void __launch_bounds__(128) k_field_digits(ForceArgs A, int t0, int n, int4 *d, int *e)
+{
+    const Geom &g = A.g;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, f = blockIdx.y;
+    if (k >= n) return;
+    int t = t0 + k;
+    if (t >= 2 * g.vh) t -= 2 * g.vh;
+    const LexSite x = lex_site(g, t);
+    const int p = (x.x0 + x.x1 + x.x2 + x.x3) & 1;
+    fx v[16];
+    int E;
+    const bool ok = load_fx(f ? A.b[p] : A.a[p], t >> 1, v, E);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) d[(size_t)(8 * f + j) * n + k] = make_int4(v[2 * j].h, v[2 * j].l, v[2 * j + 1].h, v[2 * j + 1].l);
+    e[(size_t)f * n + k] = ok ? E : kDigitBad;
+}
+__device__ __forceinline__ bool load_digits(const Digits &D, int f, int k, fx (&v)[16], int &E)
+{
+    const int4 *p = D.d + (size_t)(8 * f) * D.n + k;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int4 w = __ldg(p + (size_t)j * D.n);
+        v[2 * j] = {w.x, w.y};
+        v[2 * j + 1] = {w.z, w.w};
+    }
+    E = __ldg(D.e + (size_t)f * D.n + k);
+    const bool ok = E != kDigitBad;
+    if (!ok) E = 127;
+    return ok;
+}
+
+// Measured: hr_fermion_force at 32^4 4.39 ms with the native kernel, of it 3.97 ms
+// in the kernel (bound by the FP64 pipe: about 700 conversions and 1400
+// operations a site); error against a 64-bit evaluation 7.2e-15 with both (the
+// hops').  This kernel, converting (DIG = false): 0.413 ms at 168 registers, 0.479
+// at 216, 0.438 at 128 (spills).  With the digits (96 registers): 0.30 ms and 0.09
+// for k_field_digits (which HBM bounds) at 32^4, 22 + 5 against 34 us at 16^4, 36 + 7
+// against 48 us at 20 x 14 x 18 x 22; the whole force at 32^4 0.71 ms.
 // One thread per site in lexicographic order (so that a warp's outputs are
 // contiguous), a run-time loop over the four directions around one copy of the
 // conversion and product code: unrolled, the kernel would not fit the
 // instruction cache.  Ranges: |h| <= 2^27 per component, 2^28 projected, 8 terms
 // of 2^56 per sum.  Each of the two terms of a link is brought to 56 bits below
 // its own largest component and the two are aligned before they are added.
-template <int MODE> __global__ void __launch_bounds__(128, 3) k_link_deriv_fx(ForceArgs A)
+// DIG: the m sites from t0 on with both fields' digits of a slab (`wrap`: of the whole
+// lattice, else of these slices and the next one); else all sites, converting.
+template <int MODE, bool DIG>
+__global__ void __launch_bounds__(128, DIG ? 5 : 3) k_link_deriv_fx(ForceArgs A, Digits D, int t0, int m, bool wrap)
 {
     const Geom &g = A.g;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 2 * g.vh) return;
+    const int own = blockIdx.x * blockDim.x + threadIdx.x, t = t0 + own;
+    if (own >= m) return;
     const int i = t >> 1;
     const int row = fdiv(i, g.div_h3);
     const int r1 = fdiv(row, g.div_d2);
@@ -233,28 +280,49 @@ template <int MODE> __global__ void __launch_bounds__(128, 3) k_link_deriv_fx(Fo
     const int x3 = t - row * g.d[3];
     const int p = (x0 + x1 + x2 + x3) & 1;
     const long long V = 2LL * g.vh;
-    fx ax[16], bx[16];
-    int ea, eb;
-    const bool ok_a = load_fx(A.a[p], i, ax, ea), ok_b = load_fx(A.b[p], i, bx, eb);
+    // own fields: DIG reads them again for each direction (L1), which leaves registers
+    // for five blocks an SM instead of three; a conversion is kept
+    fx ax[DIG ? 1 : 16], bx[DIG ? 1 : 16];
+    int ea = 0, eb = 0;
+    auto load = [&](int f, int par, int idx, int slot, fx(&v)[16], int &E) -> bool {
+        if constexpr (DIG) return load_digits(D, f, slot, v, E);
+        else return load_fx(f ? A.b[par] : A.a[par], idx, v, E);
+    };
+    bool ok_own = true;
+    if constexpr (!DIG) {
+        ok_own = load(0, p, i, own, ax, ea);
+        ok_own = load(1, p, i, own, bx, eb) && ok_own;
+    }
 #pragma unroll 1
     for (int mu = 0; mu < 4; ++mu) {
         const int xm = mu == 0 ? x0 : mu == 1 ? x1 : mu == 2 ? x2 : x3;
         const bool edge = xm == g.d[mu] - 1;
         const int stride = mu == 3 ? 1 : g.d[3] * (mu == 2 ? 1 : g.d[2] * (mu == 1 ? 1 : g.d[1]));
         const int tf = edge ? t - (g.d[mu] - 1) * stride : t + stride, ifw = tf >> 1;
+        const int slot = mu == 0 && !wrap ? own + stride : own + (tf - t);
         const double sg = (MODE == 1 && edge && ((g.bc >> mu) & 1)) ? -A.beta : A.beta;
         fxa g1[4] = {}, g2[4] = {};
         int eaf, ebf;
-        bool ok = ok_a && ok_b;
+        bool ok = ok_own;
         {
             fx s[16], h[8], hb[8];
-            ok = load_fx(A.a[1 - p], ifw, s, eaf) && ok;
+            ok = load(0, 1 - p, ifw, slot, s, eaf) && ok;
             project_fx(mu, false, s, h);  // (1 + g) a(x + mu)
-            project_fx(mu, false, bx, hb);
+            if constexpr (DIG) {
+                ok = load(1, p, i, own, s, eb) && ok;
+                project_fx(mu, false, s, hb);
+            } else {
+                project_fx(mu, false, bx, hb);
+            }
             mac_links<true>(g2, hb, h);
-            ok = load_fx(A.b[1 - p], ifw, s, ebf) && ok;
+            ok = load(1, 1 - p, ifw, slot, s, ebf) && ok;
             project_fx(mu, true, s, hb);
-            project_fx(mu, true, ax, h);  // (1 - g) a(x)
+            if constexpr (DIG) {
+                ok = load(0, p, i, own, s, ea) && ok;
+                project_fx(mu, true, s, h); // (1 - g) a(x)
+            } else {
+                project_fx(mu, true, ax, h);
+            }
             mac_links<false>(g1, hb, h);
         }
         fx u[4];
@@ -342,11 +410,27 @@ hr_status link_deriv(hr_ctx *ctx, hr_lattice lat, const void *gauge, const void 
         A.tc[k] = std::cos(lat.theta[k]);
         A.ts[k] = std::sin(lat.theta[k]);
     }
-    int bs = 128;
-    int grid = (int)((2LL * A.g.vh + bs - 1) / bs);
-    if (A.g.twisted) k_link_deriv<<<grid, bs, 0, s>>>(A);
-    else if (mode == 0) k_link_deriv_fx<0><<<grid, bs, 0, s>>>(A);
-    else k_link_deriv_fx<1><<<grid, bs, 0, s>>>(A);
+    const int bs = 128, V = 2 * A.g.vh;
+    auto blocks = [&](int n) { return (unsigned)((n + bs - 1) / bs); };
+    if (A.g.twisted) {
+        k_link_deriv<<<blocks(V), bs, 0, s>>>(A);
+        return check_launch(ctx, mode ? "link grad" : "force");
+    }
+    const Slabs slabs = make_slabs(A.g, kDigitSiteBytes);
+    if (slabs.n == 0) {
+        if (mode == 0) k_link_deriv_fx<0, false><<<blocks(V), bs, 0, s>>>(A, Digits{}, 0, V, true);
+        else k_link_deriv_fx<1, false><<<blocks(V), bs, 0, s>>>(A, Digits{}, 0, V, true);
+    }
+    const int slice = V / A.g.d[0];
+    for (int k = 0; k < slabs.n; ++k) {
+        const bool whole = slabs.n == 1;
+        const int t0 = slabs.lo(k) * slice, m = (slabs.hi(k) - slabs.lo(k)) * slice, n = whole ? m : m + slice;
+        int4 *d = (int4 *)ctx->d_slab;
+        int *e = (int *)(d + 16LL * n);
+        k_field_digits<<<dim3(blocks(n), 2), bs, 0, s>>>(A, t0, n, d, e);
+        if (mode == 0) k_link_deriv_fx<0, true><<<blocks(m), bs, 0, s>>>(A, Digits{d, e, n}, t0, m, whole);
+        else k_link_deriv_fx<1, true><<<blocks(m), bs, 0, s>>>(A, Digits{d, e, n}, t0, m, whole);
+    }
     return check_launch(ctx, mode ? "link grad" : "force");
 }
 
