@@ -366,7 +366,7 @@ hr_status hr_solve_full_clover(hr_ctx *ctx, hr_lattice lat, hr_rep rep, const hr
  * S_det = -2 sum_{x odd} log det A(x).  Forces are dS/dw_a under
  * U_mu(x) -> exp(i w.s/2) U_mu(x), [4][V][3] doubles, accumulated (+=), as
  * hr_force.  The derivative of C(x) runs through the 8 leaves of each plane
- * that hold a link (one thread per link, native FP64). */
+ * that hold a link (one thread per link, 64-bit accuracy). */
 
 /* Work bytes of hr_clover_insertion_force and hr_clover_fermion_force. */
 size_t hr_clover_force_workspace_bytes(hr_lattice lat);

@@ -25,6 +25,7 @@
 #include "hr_eigh.cuh"
 #include "hr_fix_dev.cuh"
 #include "hr_host.h"
+#include "hr_plaq.cuh"
 
 using namespace hr;
 
@@ -369,7 +370,9 @@ template <int NC, int CP> __global__ void __launch_bounds__(64) k_clover_build(B
 // the native code inside this kernel would hold it at 255 registers).
 // Measured: the clover solve of 24^4 (build, FP32-inner CG to 1e-10, links and
 // source in, solution out) 9.75 ms with the native build, 3.36 ms of it the
-// build, 7.03 ms with this one; solution error against 64 bits unchanged.
+// build, 7.03 ms with this one and 0.61 ms of it the build; leaves from the
+// plaquettes' vectors took another 0.33 ms off that build (5.80 -> 5.47 ms for
+// the solve by then); solution error against 64 bits unchanged.
 
 struct FxMat {
     fx m[3][3];
@@ -447,6 +450,59 @@ template <int CP> __device__ __forceinline__ void store_block(void *half, int i,
     }
 }
 
+// The same from the plaquettes' vectors of a slab that starts at slice `first`: the
+// leaf at x of the plaquette below in mu is its vector transported by U_mu(x - mu),
+// below in nu by U_nu(x - nu), and below in both by the one and then the other,
+//   sum = P(x) + T_mu P(x - mu) + T_nu [P(x - nu) + T_mu P(x - mu - nu)].
+// low: the transports by the four links below x.  One conversion and three
+// transports of 15 products where the leaves take 16 conversions and 11
+// quaternion products.
+struct LowLinks {
+    int4 (*w)[64]; // [4 mu + k][thread]
+    __device__ void put(int mu, const Transport &T)
+    {
+        w[4 * mu + 0][threadIdx.x] = make_int4(T.u[0].h, T.u[0].l, T.u[1].h, T.u[1].l);
+        w[4 * mu + 1][threadIdx.x] = make_int4(T.u[2].h, T.u[2].l, T.w[0].h, T.w[0].l);
+        w[4 * mu + 2][threadIdx.x] = make_int4(T.w[1].h, T.w[1].l, T.w[2].h, T.w[2].l);
+        w[4 * mu + 3][threadIdx.x] = make_int4(T.w[3].h, T.w[3].l, 0, 0);
+    }
+    __device__ Transport get(int mu) const
+    {
+        const int4 a = w[4 * mu][threadIdx.x], b = w[4 * mu + 1][threadIdx.x], c = w[4 * mu + 2][threadIdx.x],
+                   e = w[4 * mu + 3][threadIdx.x];
+        return {{{a.x, a.y}, {a.z, a.w}, {b.x, b.y}}, {{b.z, b.w}, {c.x, c.y}, {c.z, c.w}, {e.x, e.y}}};
+    }
+};
+template <bool VEC>
+__device__ __forceinline__ void leaf_sum_slab(const Geom &g, const double *can, const LexSite &x, const PlaqVecs &P,
+                                              int first, const LowLinks &low, int mu, int nu, long long (&f)[3], bool &ok)
+{
+    const int slice = g.d[1] * g.d[2] * g.d[3], own = x.t - first * slice, plane = plane_of(mu, nu);
+    int unused, dm, dn;
+    lex_steps(g, x, mu, unused, dm);
+    lex_steps(g, x, nu, unused, dn);
+    // (the slab's first slice is the one before its first site's, unless it is the whole lattice; nu > 0)
+    const int sm = mu == 0 && x.x0 > first ? -slice : dm;
+    fx v[3];
+    ok = load_plaq(P, plane, own, v) && ok;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) f[k] = fx_units64(v[k]);
+    ok = load_plaq(P, plane, own + sm, v) && ok;
+    const Transport Tm = low.get(mu);
+    transport_add(Tm, v, f);
+    long long h[3];
+    ok = load_plaq(P, plane, own + dn, v) && ok;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) h[k] = fx_units64(v[k]);
+    ok = load_plaq(P, plane, own + sm + dn, v) && ok;
+    const Transport Tw = make_transport(load_fxq<VEC>(can, (size_t)mu * 2 * g.vh + (x.t + dm + dn), ok), ok);
+    transport_add(Tw, v, h);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] = fx_split(h[k]);
+    const Transport Tn = low.get(nu);
+    transport_add(Tn, v, f);
+}
+
 struct BuildFx {
     fx kappa;    // c_sw / a
     fx am;       // a = am 2^ka, am in [1, 2)
@@ -454,21 +510,39 @@ struct BuildFx {
     double inva; // 1 / a
 };
 
-template <int CP, bool EXP, bool VEC> __global__ void __launch_bounds__(64, 6) k_clover_build_fx(BuildArgs B, BuildFx X)
+// The m sites from t0 on; SLAB: with the plaquettes' vectors of the slab from slice
+// `first` on, else (slices too large for the scratch) from the 16 links of each plane.
+template <int CP, bool EXP, bool VEC, bool SLAB>
+__global__ void __launch_bounds__(64, 6) k_clover_build_fx(BuildArgs B, BuildFx X, PlaqVecs P, int t0, int m, int first)
 {
     const Geom &g = B.g;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 2 * g.vh) return;
+    __shared__ int4 low_words[SLAB ? 16 : 1][64]; // this thread's slots: no other thread reads them
+    const int t = t0 + blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= t0 + m) return;
     const LexSite x = lex_site(g, t);
     const int p = (x.x0 + x.x1 + x.x2 + x.x3) & 1, i = t >> 1;
     bool ok = true;
+    LowLinks low = {low_words};
+    if constexpr (SLAB) {
+#pragma unroll 1
+        for (int mu = 0; mu < 4; ++mu) {
+            int unused, dm;
+            lex_steps(g, x, mu, unused, dm);
+            low.put(mu, make_transport(load_fxq<VEC>(B.can, (size_t)mu * 2 * g.vh + (t + dm), ok), ok));
+        }
+    }
     FxMat N[2];
 #pragma unroll 1
     for (int l = 0; l < 3; ++l) {
         long long e[3], f[3];
-        leaf_sum<VEC>(g, B.can, x, 0, l + 1, e, ok);
         // B_1 = F_23, B_2 = F_31 = -F_13, B_3 = F_12
-        leaf_sum<VEC>(g, B.can, x, l == 0 ? 2 : 1, l == 2 ? 2 : 3, f, ok);
+        if constexpr (SLAB) {
+            leaf_sum_slab<VEC>(g, B.can, x, P, first, low, 0, l + 1, e, ok);
+            leaf_sum_slab<VEC>(g, B.can, x, P, first, low, l == 0 ? 2 : 1, l == 2 ? 2 : 3, f, ok);
+        } else {
+            leaf_sum<VEC>(g, B.can, x, 0, l + 1, e, ok);
+            leaf_sum<VEC>(g, B.can, x, l == 0 ? 2 : 1, l == 2 ? 2 : 3, f, ok);
+        }
         fx row[2][3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -619,8 +693,23 @@ template <int CP, bool EXP, bool VEC> __global__ void __launch_bounds__(64, 6) k
     if (!ok) atomicOr(B.bad, kBuildOutside);
 }
 
+template <int CP, bool EXP, bool VEC>
+void launch_build_slabs(const BuildArgs &B, const BuildFx &X, const Slabs &slabs, void *scratch, cudaStream_t s)
+{
+    const Geom &g = B.g;
+    const int slice = g.d[1] * g.d[2] * g.d[3];
+    for (int k = 0; k < slabs.n; ++k) {
+        const int a = slabs.lo(k), b = slabs.hi(k), first = slabs.n == 1 ? 0 : a - 1; // with the slice before it
+        const int n = (b - first) * slice, m = (b - a) * slice;
+        int4 *pa = (int4 *)scratch;
+        int2 *pb = (int2 *)(pa + 6LL * n);
+        launch_plaq_vec<VEC>(g, B.can, first, n, pa, pb, s);
+        k_clover_build_fx<CP, EXP, VEC, true>
+            <<<(unsigned)((m + 63) / 64), 64, 0, s>>>(B, X, PlaqVecs{pa, pb, n}, a * slice, m, first);
+    }
+}
 template <int CP>
-void launch_build_fx(const BuildArgs &B, double a, cudaStream_t s)
+void launch_build_fx(hr_ctx *ctx, const BuildArgs &B, double a, cudaStream_t s)
 {
     BuildFx X;
     int k;
@@ -629,12 +718,21 @@ void launch_build_fx(const BuildArgs &B, double a, cudaStream_t s)
     X.am = fx_from_double(am);
     X.ka = std::ldexp(1.f, k - 1);
     X.inva = 1.0 / a;
-    const int bs = 64, grid = (int)((2LL * B.g.vh + bs - 1) / bs);
     const bool vec = ((uintptr_t)B.can & 15u) == 0, ex = B.kind == HR_CLOVER_EXP;
-    if (ex && vec) k_clover_build_fx<CP, true, true><<<grid, bs, 0, s>>>(B, X);
-    else if (ex) k_clover_build_fx<CP, true, false><<<grid, bs, 0, s>>>(B, X);
-    else if (vec) k_clover_build_fx<CP, false, true><<<grid, bs, 0, s>>>(B, X);
-    else k_clover_build_fx<CP, false, false><<<grid, bs, 0, s>>>(B, X);
+    const Slabs slabs = make_slabs(B.g, kPlaqSiteBytes);
+    if (slabs.n == 0) {
+        const int V = 2 * B.g.vh;
+        (ex ? k_clover_build_fx<CP, true, false, false> : k_clover_build_fx<CP, false, false, false>)
+            <<<(unsigned)((V + 63) / 64), 64, 0, s>>>(B, X, PlaqVecs{}, 0, V, 0);
+    } else if (ex && vec) {
+        launch_build_slabs<CP, true, true>(B, X, slabs, ctx->d_slab, s);
+    } else if (ex) {
+        launch_build_slabs<CP, true, false>(B, X, slabs, ctx->d_slab, s);
+    } else if (vec) {
+        launch_build_slabs<CP, false, true>(B, X, slabs, ctx->d_slab, s);
+    } else {
+        launch_build_slabs<CP, false, false>(B, X, slabs, ctx->d_slab, s);
+    }
 }
 
 // FP64 -> FP32 field, one thread per FP32 vector
@@ -763,11 +861,11 @@ hr_status hr_clover_build(hr_ctx *ctx, hr_lattice lat, hr_rep rep, hr_prec prec,
         cudaError_t e = cudaMemsetAsync(B.bad, 0, sizeof(unsigned), s);
         if (e != cudaSuccess) return set_error(ctx, HR_ERR_CUDA, "status reset: %s", cudaGetErrorString(e));
         if (prec == kF64) {
-            if (fixed) launch_build_fx<kF64>(B, a, s);
+            if (fixed) launch_build_fx<kF64>(ctx, B, a, s);
             else if (three) k_clover_build<3, kF64><<<grid, bs, 0, s>>>(B);
             else k_clover_build<2, kF64><<<grid, bs, 0, s>>>(B);
         } else {
-            if (fixed) launch_build_fx<kF32>(B, a, s);
+            if (fixed) launch_build_fx<kF32>(ctx, B, a, s);
             else if (three) k_clover_build<3, kF32><<<grid, bs, 0, s>>>(B);
             else k_clover_build<2, kF32><<<grid, bs, 0, s>>>(B);
         }
@@ -1177,9 +1275,10 @@ __device__ __noinline__ void leaf_force_native(const Geom &g, const double *can,
 // plaquette, where the 2 x 2 complex matrices of hr_clover_leaf.cuh take 700.
 // The kappa of a plaquette are read in units of their largest component, and
 // the running sum of the B follows the largest unit met so far.  20 x 14 x 18 x 22:
-// 4.99 ms in native FP64, 0.286 ms here (128 registers: 0.298); the whole
-// clover force (hops, link derivatives, kappa, this) 5.77 -> 0.48 ms, error
-// against 64 bits unchanged (7.8e-15, the hops').
+// 4.99 ms in native FP64, 0.252 ms here (0.286 with conversions of 20 instead of 13
+// instructions a number; 128 registers: 0.298); the whole clover force (hops, link
+// derivatives, kappa, this) 5.77 -> 0.42 ms, error against 64 bits unchanged
+// (7.8e-15, the hops').
 template <bool VEC>
 __global__ void __launch_bounds__(128, 3) k_clover_leaf_force(Geom g, const double *__restrict__ can,
                                                               const double *__restrict__ K, double scale,

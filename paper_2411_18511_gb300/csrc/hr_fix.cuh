@@ -268,17 +268,8 @@ HR_HD inline fxq fxq_add(fxq a, fxq b)
 {
     return {{fx_add(a.c[0], b.c[0]), fx_add(a.c[1], b.c[1]), fx_add(a.c[2], b.c[2]), fx_add(a.c[3], b.c[3])}};
 }
+// for |components| < 2, in 32-bit integers
 HR_HD inline bool fxq_near_unit(const fxq &q)
-{
-    float n = 0.f;
-    for (int k = 0; k < 4; ++k) {
-        const float f = (float)q.c[k].h * 0x1p-28f;
-        n = fx_fma(f, f, n);
-    }
-    return n > 0.99f && n < 1.01f;
-}
-// the same test in 32-bit integers, for |components| < 2
-HR_HD inline bool fxq_near_unit_int(const fxq &q)
 {
     int n = -(1 << 26);
     for (int k = 0; k < 4; ++k) n += (q.c[k].h >> 15) * (q.c[k].h >> 15);

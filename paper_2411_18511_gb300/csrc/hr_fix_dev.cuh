@@ -31,7 +31,7 @@ __device__ __forceinline__ void lex_steps(const Geom &g, const LexSite &s, int m
     up = x == d - 1 ? -(d - 1) * st : st;
     down = x == 0 ? (d - 1) * st : -st;
 }
-// a canonical link as digits; ok stays true only for links of unit length to 1 %
+// a canonical link as digits (low ones up to 2^28); ok stays true only for links of unit length to 1 %
 // (VEC: the field is 16-byte aligned)
 template <bool VEC> __device__ __forceinline__ void load_link4(const double *q, size_t link, double (&c)[4])
 {
@@ -50,19 +50,8 @@ template <bool VEC> __device__ __forceinline__ fxq load_fxq(const double *q, siz
     double c[4];
     load_link4<VEC>(q, link, c);
     const unsigned m = max(max(fx_abs_high(c[0]), fx_abs_high(c[1])), max(fx_abs_high(c[2]), fx_abs_high(c[3])));
-    const fxq r = {{fx_from_double(c[0]), fx_from_double(c[1]), fx_from_double(c[2]), fx_from_double(c[3])}};
-    ok = ok && m < kFxHigh2 && fxq_near_unit(r);
-    return r;
-}
-
-// the same with the cheaper conversion and test (low digits up to 2^28)
-template <bool VEC> __device__ __forceinline__ fxq load_fxq_unit(const double *q, size_t link, bool &ok)
-{
-    double c[4];
-    load_link4<VEC>(q, link, c);
-    const unsigned m = max(max(fx_abs_high(c[0]), fx_abs_high(c[1])), max(fx_abs_high(c[2]), fx_abs_high(c[3])));
     const fxq r = {{fx_from_unit(c[0]), fx_from_unit(c[1]), fx_from_unit(c[2]), fx_from_unit(c[3])}};
-    ok = ok && m < kFxHigh2 && fxq_near_unit_int(r);
+    ok = ok && m < kFxHigh2 && fxq_near_unit(r);
     return r;
 }
 

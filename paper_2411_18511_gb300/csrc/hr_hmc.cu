@@ -30,6 +30,7 @@
 
 #include "hr_fix_dev.cuh"
 #include "hr_host.h"
+#include "hr_plaq.cuh"
 
 using namespace hr;
 
@@ -116,67 +117,8 @@ __device__ __noinline__ void gauge_force_native(const Geom &g, const double *q, 
 // Both are bound by the integer pipes.  The vectors of the whole lattice would be
 // 144 bytes a site from HBM and unbounded scratch, so slabs of time slices that
 // fit the context's scratch (64 MiB, half of L2) go through both launches in turn.
-static_assert(kPlaqSiteBytes == 6 * (sizeof(int4) + sizeof(int2)), "six vectors a site");
-// below this many sites one thread per plane and per link, more of them in flight
+// below this many sites one thread per link instead of per site, more of them in flight
 constexpr int kPlaqSplitSites = 1 << 17;
-constexpr int kPlaqBad = (int)0x80000000; // leading digit of a vector outside the fixed-point range
-
-// plane index of mu < nu: (01) (02) (03) (12) (13) (23)
-__device__ __forceinline__ int plane_of(int mu, int nu)
-{
-    const int a = min(mu, nu), b = max(mu, nu);
-    return a == 0 ? b - 1 : a + b;
-}
-
-// Vec P of the n sites from slice `first` on.  PER = 6: one thread per site, its own
-// four links converted once and kept in shared memory (a conversion is some 90
-// instructions, 24 of them a site were half of the kernel); 1: one per plane (blockIdx.y).
-template <bool VEC, int PER>
-__global__ void __launch_bounds__(128) k_plaq_vec(Geom g, const double *__restrict__ q, int first, int n,
-                                                  int4 *__restrict__ pa, int2 *__restrict__ pb)
-{
-    constexpr int OWN = PER == 6 ? 8 : 1;
-    __shared__ int4 own[OWN][128]; // this thread's slots: no other thread reads them
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int V = 2 * g.vh, slice = g.d[1] * g.d[2] * g.d[3];
-    int t = first * slice + i;
-    if (t < 0) t += V;
-    const LexSite x = lex_site(g, t);
-    bool ok_own = true;
-    if constexpr (PER == 6) {
-#pragma unroll 1
-        for (int mu = 0; mu < 4; ++mu) {
-            const fxq u = load_fxq_unit<VEC>(q, (size_t)mu * V + t, ok_own);
-            own[2 * mu][threadIdx.x] = make_int4(u.c[0].h, u.c[0].l, u.c[1].h, u.c[1].l);
-            own[2 * mu + 1][threadIdx.x] = make_int4(u.c[2].h, u.c[2].l, u.c[3].h, u.c[3].l);
-        }
-    }
-    auto own_link = [&](int mu, bool &ok) -> fxq {
-        if constexpr (PER == 6) {
-            const int4 a = own[2 * mu][threadIdx.x], b = own[2 * mu + 1][threadIdx.x];
-            return {{{a.x, a.y}, {a.z, a.w}, {b.x, b.y}, {b.z, b.w}}};
-        } else {
-            return load_fxq_unit<VEC>(q, (size_t)mu * V + t, ok);
-        }
-    };
-    const int p0 = PER == 6 ? 0 : blockIdx.y;
-#pragma unroll 1
-    for (int p = p0; p < p0 + PER; ++p) {
-        const int mu = p < 3 ? 0 : p < 5 ? 1 : 2, nu = p < 3 ? p + 1 : p < 5 ? p - 1 : 3;
-        int up_mu, up_nu, unused;
-        lex_steps(g, x, mu, up_mu, unused);
-        lex_steps(g, x, nu, up_nu, unused);
-        bool ok = ok_own;
-        const fxq A = fxq_mul(own_link(mu, ok), load_fxq_unit<VEC>(q, (size_t)nu * V + t + up_mu, ok));
-        const fxq B = fxq_conj(fxq_mul(own_link(nu, ok), load_fxq_unit<VEC>(q, (size_t)mu * V + t + up_nu, ok)));
-        fxa w[3] = {};
-        fxq_mac_vec(w, A, B);
-        const fx v0 = fx_of(w[0]), v1 = fx_of(w[1]), v2 = fx_of(w[2]);
-        pa[(size_t)p * n + i] = make_int4(ok ? v0.h : kPlaqBad, v0.l, v1.h, v1.l);
-        pb[(size_t)p * n + i] = make_int2(v2.h, v2.l);
-    }
-}
 
 // The force on the links of the sites t0 .. t0 + m - 1 from the n vectors a plane
 // that start at slice `first`; NMU = 4: one thread per site, 1: one per link
@@ -201,7 +143,7 @@ __global__ void __launch_bounds__(128, 5) k_plaq_force(Geom g, double s, const d
         if (NMU == 1 && nu == (int)blockIdx.y) continue;
         int unused, down;
         lex_steps(g, x, nu, unused, down);
-        const fxq U = load_fxq_unit<VEC>(q, (size_t)nu * V + t + down, ok);
+        const fxq U = load_fxq<VEC>(q, (size_t)nu * V + t + down, ok);
         fxa nn = {-(1LL << 56), 0};
 #pragma unroll
         for (int k = 0; k < 4; ++k) fx_mac(nn, U.c[k], U.c[k]);
@@ -485,9 +427,8 @@ void launch_gauge_force(hr_ctx *ctx, const Geom &g, double c, const double *q, d
         const int n = (b - first) * slice, m = (b - a) * slice;
         int4 *pa = (int4 *)ctx->d_slab;
         int2 *pb = (int2 *)(pa + 6LL * n);
-        const unsigned nb = (unsigned)((n + 127) / 128), mb = (unsigned)((m + 127) / 128);
-        if (small) k_plaq_vec<VEC, 1><<<dim3(nb, 6), 128, 0, s>>>(g, q, first, n, pa, pb);
-        else k_plaq_vec<VEC, 6><<<nb, 128, 0, s>>>(g, q, first, n, pa, pb);
+        const unsigned mb = (unsigned)((m + 127) / 128);
+        launch_plaq_vec<VEC>(g, q, first, n, pa, pb, s);
         if (small) k_plaq_force<VEC, 1><<<dim3(mb, 4), 128, 0, s>>>(g, c, q, F, a * slice, m, first, n, pa, pb);
         else k_plaq_force<VEC, 4><<<mb, 128, 0, s>>>(g, c, q, F, a * slice, m, first, n, pa, pb);
     }

@@ -1,0 +1,139 @@
+// hr_plaq.cuh -- the vector parts of the plaquettes, vec P_mn(x) with
+// P_mn(x) = U_m(x) U_n(x+m) U_m(x+n)^+ U_n(x)^+, in two-digit fixed point (hr_fix.cuh),
+// and their transport by one link: shared by the gauge force (hr_hmc.cu) and the
+// clover build (hr_clover.cu), which need each at several sites.
+#pragma once
+
+#include "hr_fix_dev.cuh"
+#include "hr_host.h"
+
+namespace hr {
+
+static_assert(kPlaqSiteBytes == 6 * (sizeof(int4) + sizeof(int2)), "six vectors a site");
+constexpr int kPlaqBad = (int)0x80000000; // leading digit of a vector outside the fixed-point range
+
+// plane index of mu < nu: (01) (02) (03) (12) (13) (23)
+__device__ __forceinline__ int plane_of(int mu, int nu)
+{
+    const int a = min(mu, nu), b = max(mu, nu);
+    return a == 0 ? b - 1 : a + b;
+}
+
+// Vec P of the n sites from slice `first` on.  PER = 6: one thread per site, its own
+// four links converted once and kept in shared memory (a conversion is some 90
+// instructions, 24 of them a site were half of the kernel); 1: one per plane (blockIdx.y).
+template <bool VEC, int PER>
+__global__ void __launch_bounds__(128) k_plaq_vec(Geom g, const double *__restrict__ q, int first, int n,
+                                                  int4 *__restrict__ pa, int2 *__restrict__ pb)
+{
+    constexpr int OWN = PER == 6 ? 8 : 1;
+    __shared__ int4 own[OWN][128]; // this thread's slots: no other thread reads them
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int V = 2 * g.vh, slice = g.d[1] * g.d[2] * g.d[3];
+    int t = first * slice + i;
+    if (t < 0) t += V;
+    const LexSite x = lex_site(g, t);
+    bool ok_own = true;
+    if constexpr (PER == 6) {
+#pragma unroll 1
+        for (int mu = 0; mu < 4; ++mu) {
+            const fxq u = load_fxq<VEC>(q, (size_t)mu * V + t, ok_own);
+            own[2 * mu][threadIdx.x] = make_int4(u.c[0].h, u.c[0].l, u.c[1].h, u.c[1].l);
+            own[2 * mu + 1][threadIdx.x] = make_int4(u.c[2].h, u.c[2].l, u.c[3].h, u.c[3].l);
+        }
+    }
+    auto own_link = [&](int mu, bool &ok) -> fxq {
+        if constexpr (PER == 6) {
+            const int4 a = own[2 * mu][threadIdx.x], b = own[2 * mu + 1][threadIdx.x];
+            return {{{a.x, a.y}, {a.z, a.w}, {b.x, b.y}, {b.z, b.w}}};
+        } else {
+            return load_fxq<VEC>(q, (size_t)mu * V + t, ok);
+        }
+    };
+    const int p0 = PER == 6 ? 0 : blockIdx.y;
+#pragma unroll 1
+    for (int p = p0; p < p0 + PER; ++p) {
+        const int mu = p < 3 ? 0 : p < 5 ? 1 : 2, nu = p < 3 ? p + 1 : p < 5 ? p - 1 : 3;
+        int up_mu, up_nu, unused;
+        lex_steps(g, x, mu, up_mu, unused);
+        lex_steps(g, x, nu, up_nu, unused);
+        bool ok = ok_own;
+        const fxq A = fxq_mul(own_link(mu, ok), load_fxq<VEC>(q, (size_t)nu * V + t + up_mu, ok));
+        const fxq B = fxq_conj(fxq_mul(own_link(nu, ok), load_fxq<VEC>(q, (size_t)mu * V + t + up_nu, ok)));
+        fxa w[3] = {};
+        fxq_mac_vec(w, A, B);
+        const fx v0 = fx_of(w[0]), v1 = fx_of(w[1]), v2 = fx_of(w[2]);
+        pa[(size_t)p * n + i] = make_int4(ok ? v0.h : kPlaqBad, v0.l, v1.h, v1.l);
+        pb[(size_t)p * n + i] = make_int2(v2.h, v2.l);
+    }
+}
+
+// Up to this many sites k_plaq_vec runs one thread per plane, six times as many in
+// flight: 16^4 15.7 us against 18.1 with one thread per site.
+constexpr int kPlaqVecSplit = 1 << 17;
+template <bool VEC>
+inline void launch_plaq_vec(const Geom &g, const double *q, int first, int n, int4 *pa, int2 *pb, cudaStream_t s)
+{
+    const unsigned nb = (unsigned)((n + 127) / 128);
+    if (n <= kPlaqVecSplit) k_plaq_vec<VEC, 1><<<dim3(nb, 6), 128, 0, s>>>(g, q, first, n, pa, pb);
+    else k_plaq_vec<VEC, 6><<<nb, 128, 0, s>>>(g, q, first, n, pa, pb);
+}
+
+// the n vectors a plane of a slab
+struct PlaqVecs {
+    const int4 *a;
+    const int2 *b;
+    int n;
+};
+__device__ __forceinline__ bool load_plaq(const PlaqVecs &P, int plane, int slot, fx (&v)[3])
+{
+    const int4 a = __ldg(P.a + (size_t)plane * P.n + slot);
+    const int2 b = __ldg(P.b + (size_t)plane * P.n + slot);
+    v[0] = {a.x, a.y};
+    v[1] = {a.z, a.w};
+    v[2] = {b.x, b.y};
+    return a.x != kPlaqBad;
+}
+
+// A link that transports vectors: with u its vector part, t = u x v and d = |U|^2 - 1,
+//   vec(U^+ v U) / |U|^2 = v + 2 (u0 t + u x t) (1 - d)
+// to first order in d, which ok bounds by 2^-29.
+struct Transport {
+    fx u[3];
+    fx w[4]; // 2 U (1 - d)
+};
+__device__ __forceinline__ Transport make_transport(const fxq &U, bool &ok)
+{
+    fxa nn = {-(1LL << 56), 0};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) fx_mac(nn, U.c[k], U.c[k]);
+    const long long d = fx_round(nn);
+    ok = ok && d < (1 << 27) && d > -(1 << 27);
+    Transport r;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        r.w[k] = {2 * U.c[k].h, 2 * (U.c[k].l - (int)(((long long)U.c[k].h * (int)d) >> 28))};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) r.u[k] = U.c[k + 1];
+    return r;
+}
+// sum += the transported v, in units of 2^-56 (|v| < 4)
+__device__ __forceinline__ void transport_add(const Transport &T, const fx (&v)[3], long long (&sum)[3])
+{
+    fxa tc[3] = {}, acc[3];
+    fx_mac_cross(tc, T.u, v);
+    fx t[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        t[a] = fx_of(tc[a]);
+        acc[a] = {fx_units64(v[a]), 0};
+        fx_mac(acc[a], T.w[0], t[a]);
+    }
+    const fx wv[3] = {T.w[1], T.w[2], T.w[3]};
+    fx_mac_cross(acc, wv, t);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) sum[a] += fx_round(acc[a]);
+}
+
+} // namespace hr
