@@ -51,7 +51,7 @@ __device__ __forceinline__ void hop_body(const HopArgs &a)
 // The unrolled kernel: registers as the compiler likes (about 100 for
 // double-float, two 256-thread blocks per SM) ...
 template <int REP, int PREC, int G5IN>
-__global__ void __launch_bounds__(256) k_hop(HopArgs a)
+__global__ void __launch_bounds__(256, REP != kRepAdj || PREC != kF64 ? 2 : 1) k_hop(HopArgs a)
 {
     hop_body<REP, PREC, G5IN>(a);
 }
@@ -83,19 +83,27 @@ __global__ void __maxnreg__(96) k_hop_clov_r96(HopArgs a)
 
 // ---------------------------------------------------------------- launch
 
-// The shape of a configuration that was never tuned: the family that was fastest,
-// or within 5 % of it, from 4^4 to 24^4, at 64 threads a block (small blocks spread
-// a small lattice over more SMs and leave a shorter tail on a large one).  us per
-// hop of Mhat^+ Mhat at 8^4 / 16^4 / 24^4, the plain kernel (256 threads for FP64,
-// 128 else) against the choice:
-//   fundamental FP64 11.6 / 13.7 / 36.3 -> 6.0 / 11.8 / 33.5, FP32 3.1 / 4.5 / 8.5 ->
-//   2.1 / 3.7 / 7.9, binary16 3.3 / 5.6 / 8.0 -> 2.2 / 4.2 / 6.3; adjoint FP64 17.0 /
-//   18.7 / 75.0 -> 9.2 / 18.9 / 49.6, stored matrices 13.9 / 14.9 / 70.6 -> 7.5 / 13.9 /
-//   50.8.  The adjoint in FP32 and binary16 has the plain kernel only.
-inline HopChoice default_choice(int rep, int prec)
+// The shape of a configuration that was never tuned, by precision, representation
+// and virtual sites: the family that is fastest over the range, or within 5 % of it,
+// in small blocks for small lattices (they spread over more SMs) and larger ones
+// where the blocks' staged or shared operands pay.  us per hop of Mhat^+ Mhat, against
+// the plain kernel at 256 (FP64) or 128 threads and against one other choice:
+//   fundamental FP64   8^4 11.6 -> 5.2 (13@64 5.7), 16^4 13.7 -> 8.0 (13@192 10.9),
+//                      24^4 36.3 -> 31.4 (11@64 33.8), 32^4 83.5 (11@64 101.3, 13@192 85.3)
+//   adjoint FP64       8^4 17.0 -> 6.2 (12@192 9.1), 24^4 75.0 -> 44.5 (10@64 49.6),
+//                      32^4 124.3 (12@128 133.8); stored matrices 24^4 70.6 -> 43.5 (10@64 51.2)
+//   fundamental FP32   8^4 3.1 -> 2.1, 16^4 4.5 -> 3.7, 24^4 8.5 -> 7.9
+//   binary16           8^4 2.2 (7@64 2.3), 16^4 2.93 -> 2.84, 24^4 7.5 -> 7.1, 32^4 21.4 -> 20.3
+// The adjoint in FP32 and binary16 has the plain kernel only.
+inline HopChoice default_choice(const Geom &g, int rep, int prec)
 {
-    if (prec == kF64) return {kVarPaired, 64};
-    if (rep == HR_FUND) return {prec == kF32 ? kVarSimpleR96 : kVarHalfPrefetch, 64};
+    const long long nv = (long long)g.vh << g.lrhs;
+    const bool small = nv <= 1 << 16;
+    if (prec == kF64 && rep == HR_FUND)
+        return small ? HopChoice{kVarPairedStaged, 64} : HopChoice{kVarPairedStagedR96, nv <= 1 << 18 ? 192 : 256};
+    if (prec == kF64) return {kVarPairedR96, small ? 128 : 192};
+    // (the half2 kernels round the projection to binary16: only the tuner picks them)
+    if (rep == HR_FUND && (prec == kF32 || nv > 1 << 14)) return {kVarSimpleR96, 64};
     return {kVarSimple, 128};
 }
 
@@ -240,7 +248,7 @@ HopChoice hop_choice(hr_ctx *ctx, const Geom &g, int rep, int prec)
 {
     auto it = ctx->tuned.find(tune_key(g, rep, prec));
     if (it != ctx->tuned.end()) return it->second;
-    return default_choice(rep, prec);
+    return default_choice(g, rep, prec);
 }
 
 std::string tune_key_fin(const Geom &g, int rep, int prec) { return tune_key(g, rep, prec) + ":fin"; }

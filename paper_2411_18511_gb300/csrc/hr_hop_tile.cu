@@ -143,7 +143,7 @@ __device__ __forceinline__ void hop_tile_body(const HopArgs &a)
 }
 
 template <int REP, int PREC, int G5IN>
-__global__ void __launch_bounds__(256) k_hop_tile(HopArgs a)
+__global__ void __launch_bounds__(256, REP == kRepFund || PREC != kF64 ? 2 : 1) k_hop_tile(HopArgs a)
 {
     hop_tile_body<REP, PREC, G5IN>(a);
 }

@@ -110,8 +110,11 @@ __device__ __forceinline__ void twisted_dir(const HopArgs &a, int i, int rr, con
     twisted_term<MU, false, REP, PREC, false>(a, nb.bwd[MU], 1 - a.p, s, sc, g5, tw && x[MU] == 0, c, -sn, acc);
 }
 
+// (blocks an SM: without a bound the compiler takes up to 140 registers in FP32)
 template <int REP, int PREC, bool CLOV>
-__global__ void __launch_bounds__(128) k_hop_twist(HopArgs a)
+__global__ void
+__launch_bounds__(kTwistBlock, PREC == kF64 ? (REP == kRepFund ? 4 : CLOV ? 2 : 3) : CLOV && REP != kRepFund ? 4 : 5)
+    k_hop_twist(HopArgs a)
 {
     using T = typename PrecTraits<PREC>::T;
     constexpr int NC = RepTraits<REP>::NC;
