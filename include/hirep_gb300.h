@@ -40,9 +40,13 @@
  *   the caller) and the stream.  No hot call allocates memory.  Work buffers
  *   are passed in, sized by hr_workspace_bytes.  Calls are asynchronous on
  *   the given stream unless stated otherwise.
- * - A context's device scratch (reduction partials, solver scalars) is shared
- *   by the calls made with it: calls on one context must not overlap in time
- *   (use one stream per context, or one context per stream).
+ * - A context's device scratch (reduction partials, solver scalars, 64 MiB for
+ *   the forces and the clover build) is shared by the calls made with it: calls
+ *   on one context must not overlap in time (use one stream per context, or one
+ *   context per stream).  Exempt, as they use none of it or wait for one another
+ *   on the device: packing, operators, hr_gauge_force, hr_link_update,
+ *   hr_mom_update, hr_force and hr_link_grad may be queued on any streams, by any
+ *   threads and into CUDA graphs (where the forces take kernels without scratch).
  * - Errors: every call returns hr_status; argument errors are detected on the
  *   host before anything is launched; hr_last_error() gives a message.
  */

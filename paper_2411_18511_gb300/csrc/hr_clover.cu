@@ -720,18 +720,19 @@ void launch_build_fx(hr_ctx *ctx, const BuildArgs &B, double a, cudaStream_t s)
     X.inva = 1.0 / a;
     const bool vec = ((uintptr_t)B.can & 15u) == 0, ex = B.kind == HR_CLOVER_EXP;
     const Slabs slabs = make_slabs(B.g, kPlaqSiteBytes);
-    if (slabs.n == 0) {
+    const SlabLease slab(ctx, s, slabs.n > 0);
+    if (!slab.mem) {
         const int V = 2 * B.g.vh;
         (ex ? k_clover_build_fx<CP, true, false, false> : k_clover_build_fx<CP, false, false, false>)
             <<<(unsigned)((V + 63) / 64), 64, 0, s>>>(B, X, PlaqVecs{}, 0, V, 0);
     } else if (ex && vec) {
-        launch_build_slabs<CP, true, true>(B, X, slabs, ctx->d_slab, s);
+        launch_build_slabs<CP, true, true>(B, X, slabs, slab.mem, s);
     } else if (ex) {
-        launch_build_slabs<CP, true, false>(B, X, slabs, ctx->d_slab, s);
+        launch_build_slabs<CP, true, false>(B, X, slabs, slab.mem, s);
     } else if (vec) {
-        launch_build_slabs<CP, false, true>(B, X, slabs, ctx->d_slab, s);
+        launch_build_slabs<CP, false, true>(B, X, slabs, slab.mem, s);
     } else {
-        launch_build_slabs<CP, false, false>(B, X, slabs, ctx->d_slab, s);
+        launch_build_slabs<CP, false, false>(B, X, slabs, slab.mem, s);
     }
 }
 

@@ -478,6 +478,7 @@ hr_status hr_ctx_create(hr_ctx **out, int device)
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_counters, sizeof(unsigned) * kNumCounters);
     if (e == cudaSuccess) e = cudaMemset(ctx->d_counters, 0, sizeof(unsigned) * kNumCounters);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_slab, kSlabBytes);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_slab, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_scal, sizeof(double) * kScalDoubles);
     if (e == cudaSuccess) e = cudaMemset(ctx->d_scal, 0, sizeof(double) * kScalDoubles);
     if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_scal, sizeof(double) * kScalDoubles);
@@ -510,6 +511,7 @@ hr_status hr_ctx_destroy(hr_ctx *ctx)
     if (ctx->d_partials) cudaFree(ctx->d_partials);
     if (ctx->d_counters) cudaFree(ctx->d_counters);
     if (ctx->d_slab) cudaFree(ctx->d_slab);
+    if (ctx->ev_slab) cudaEventDestroy(ctx->ev_slab);
     if (ctx->d_scal) cudaFree(ctx->d_scal);
     if (ctx->h_scal) cudaFreeHost(ctx->h_scal);
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);

@@ -212,7 +212,8 @@ template <bool DAG> __device__ __forceinline__ void mac_links(fxa (&g)[4], const
 
 // The fields as digits, 16 pairs and an exponent a site: each is read at five sites of
 // the link kernel, and converting it there took more than half of its instructions.
-// Slices above 127 k sites do not fit the scratch twice and are converted there.
+// Slices above 127 k sites do not fit the scratch twice and are converted there, as
+// are all while a graph is captured (SlabLease).
 // Field f, vector v of slab site k at d[(8 f + v) n + k], its exponent at e[f n + k].
 struct Digits {
     const int4 *d;
@@ -417,15 +418,17 @@ hr_status link_deriv(hr_ctx *ctx, hr_lattice lat, const void *gauge, const void 
         return check_launch(ctx, mode ? "link grad" : "force");
     }
     const Slabs slabs = make_slabs(A.g, kDigitSiteBytes);
-    if (slabs.n == 0) {
+    const SlabLease slab(ctx, s, slabs.n > 0);
+    if (!slab.mem) {
         if (mode == 0) k_link_deriv_fx<0, false><<<blocks(V), bs, 0, s>>>(A, Digits{}, 0, V, true);
         else k_link_deriv_fx<1, false><<<blocks(V), bs, 0, s>>>(A, Digits{}, 0, V, true);
+        return check_launch(ctx, mode ? "link grad" : "force");
     }
     const int slice = V / A.g.d[0];
     for (int k = 0; k < slabs.n; ++k) {
         const bool whole = slabs.n == 1;
         const int t0 = slabs.lo(k) * slice, m = (slabs.hi(k) - slabs.lo(k)) * slice, n = whole ? m : m + slice;
-        int4 *d = (int4 *)ctx->d_slab;
+        int4 *d = (int4 *)slab.mem;
         int *e = (int *)(d + 16LL * n);
         k_field_digits<<<dim3(blocks(n), 2), bs, 0, s>>>(A, t0, n, d, e);
         if (mode == 0) k_link_deriv_fx<0, true><<<blocks(m), bs, 0, s>>>(A, Digits{d, e, n}, t0, m, whole);

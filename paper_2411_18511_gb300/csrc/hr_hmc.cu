@@ -199,7 +199,8 @@ __global__ void __launch_bounds__(128, 5) k_plaq_force(Geom g, double s, const d
     }
 }
 
-// Slices too large for the scratch (more than 230 k sites each): one thread per link,
+// Slices too large for the scratch (more than 230 k sites each), and a stream that is
+// being captured (SlabLease): one thread per link,
 // F[mu][x][a] += coeff * beta/2 * vec(U_mu(x) V_mu(x))_a, staples in two-digit fixed
 // point, 12 quaternion products of 16 terms.
 template <bool VEC>
@@ -417,7 +418,8 @@ void launch_gauge_force(hr_ctx *ctx, const Geom &g, double c, const double *q, d
 {
     const int V = 2 * g.vh, slice = V / g.d[0];
     const Slabs slabs = make_slabs(g, kPlaqSiteBytes);
-    if (slabs.n == 0) {
+    const SlabLease slab(ctx, s, slabs.n > 0);
+    if (!slab.mem) {
         k_gauge_force<VEC><<<dim3((unsigned)((V + 127) / 128), 4), 128, 0, s>>>(g, c, q, F);
         return;
     }
@@ -425,7 +427,7 @@ void launch_gauge_force(hr_ctx *ctx, const Geom &g, double c, const double *q, d
     for (int k = 0; k < slabs.n; ++k) {
         const int a = slabs.lo(k), b = slabs.hi(k), first = slabs.n == 1 ? 0 : a - 1; // with the slice before it
         const int n = (b - first) * slice, m = (b - a) * slice;
-        int4 *pa = (int4 *)ctx->d_slab;
+        int4 *pa = (int4 *)slab.mem;
         int2 *pb = (int2 *)(pa + 6LL * n);
         const unsigned mb = (unsigned)((m + 127) / 128);
         launch_plaq_vec<VEC>(g, q, first, n, pa, pb, s);

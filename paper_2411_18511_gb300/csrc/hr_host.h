@@ -7,6 +7,7 @@
 #include <cstdint>
 #include <initializer_list>
 #include <map>
+#include <mutex>
 #include <string>
 #include <utility>
 #include <vector>
@@ -42,7 +43,9 @@ struct hr_ctx {
     std::string err;
     double *d_partials = nullptr;  // kMaxPartials, then kFinBlocks * kMaxRhs sums of a finishing launch's blocks
     unsigned *d_counters = nullptr;
-    void *d_slab = nullptr;        // kSlabBytes: scratch of the forces
+    void *d_slab = nullptr;        // kSlabBytes: scratch of the forces, used under a SlabLease only
+    cudaEvent_t ev_slab = nullptr; // the last lease's work
+    std::mutex slab_mutex;
     double *d_scal = nullptr;      // kScalDoubles
     double *h_scal = nullptr;      // pinned mirror
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -210,6 +213,42 @@ inline Slabs make_slabs(const Geom &g, size_t site_bytes)
     if (fit >= T) return {1, T};
     return {fit < 2 ? 0 : (int)((T + fit - 2) / (fit - 1)), T};
 }
+
+// The context's slab scratch for the launches of one call on stream s.  The calls that
+// use it (gauge force, link derivatives, clover build) touch no other scratch of
+// the context, and a caller may not even choose the context (autograd keeps one per
+// device and runs each backward on its forward's stream), so they must not depend on
+// one stream: a lease holds the mutex while the call queues its launches, waits on
+// the device for the lease before it, whatever its stream, and marks the end of its
+// own launches.  Event calls alone, about 2 us of host time a call.
+// mem == nullptr: not wanted, or s is being captured into a graph, which may be
+// replayed beside anything (and after the context is gone); the caller then takes
+// its kernels without scratch.
+struct SlabLease {
+    hr_ctx *ctx;
+    cudaStream_t s;
+    void *mem = nullptr;
+    std::unique_lock<std::mutex> lock;
+    SlabLease(hr_ctx *c, cudaStream_t stream, bool want) : ctx(c), s(stream)
+    {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        if (!want) return;
+        if (cudaStreamIsCapturing(s, &st) != cudaSuccess) { // (the launches will say why)
+            cudaGetLastError();
+            return;
+        }
+        if (st != cudaStreamCaptureStatusNone) return;
+        lock = std::unique_lock<std::mutex>(ctx->slab_mutex);
+        if (cudaStreamWaitEvent(s, ctx->ev_slab, 0) == cudaSuccess) mem = ctx->d_slab;
+        else cudaGetLastError();
+    }
+    ~SlabLease()
+    {
+        if (mem) cudaEventRecord(ctx->ev_slab, s);
+    }
+    SlabLease(const SlabLease &) = delete;
+    SlabLease &operator=(const SlabLease &) = delete;
+};
 
 // ---- link derivatives (hr_force.cu) ----
 // out += beta dRe<a, H b> for full fields given by their even and odd halves
