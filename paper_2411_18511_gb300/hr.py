@@ -86,13 +86,16 @@ class Lattice(tuple):
         self.theta = theta
         return self
 
-    def c_struct(self) -> "hr_lattice":
-        """The ``hr_lattice`` that every call passes by value, filled once and
-        again whenever ``bc`` or ``theta`` was assigned."""
-        now = (self.bc, self.theta)
+    def _c_struct(self) -> "hr_lattice":
+        """The ``hr_lattice`` that every call of this module passes by value: filled
+        once and again when the numbers in ``bc`` or ``theta`` are others (compared by
+        value: ``theta`` may be a list or an array that was changed in place).  Kept
+        from callers, who get one of their own from :func:`lattice`."""
+        theta = self.theta
+        now = (int(self.bc), None if theta is None else tuple(float(theta[k]) for k in range(4)))
         made = self.__dict__.get("_made")
         if made is None or made[0] != now:
-            made = self._made = (now, _fill_lattice(self, self.bc, self.theta))
+            made = self._made = (now, _fill_lattice(self, *now))
         return made[1]
 
     def __repr__(self):
@@ -238,9 +241,12 @@ def _fill_lattice(dims, bc, theta) -> hr_lattice:
 
 
 def lattice(dims) -> hr_lattice:
-    if type(dims) is Lattice:
-        return dims.c_struct()
+    """A new ``hr_lattice`` of extents or of a :class:`Lattice`."""
     return _fill_lattice(dims, getattr(dims, "bc", 0), getattr(dims, "theta", None))
+
+
+def _lat(dims) -> hr_lattice:
+    return dims._c_struct() if type(dims) is Lattice else lattice(dims)
 
 
 def _ptr(x):
@@ -336,22 +342,22 @@ def hr_m0_to_kappa(m0: float) -> float:
 
 
 def hr_gauge_packed_bytes(dims, rep: int, prec: int) -> int:
-    return int(lib().hr_gauge_packed_bytes(lattice(dims), rep, prec))
+    return int(lib().hr_gauge_packed_bytes(_lat(dims), rep, prec))
 
 
 def hr_spinor_packed_bytes(dims, rep: int, prec: int, parity: int, n_rhs: int = 1) -> int:
-    return int(lib().hr_spinor_packed_bytes(lattice(dims), rep, prec, parity, n_rhs))
+    return int(lib().hr_spinor_packed_bytes(_lat(dims), rep, prec, parity, n_rhs))
 
 
 def hr_dirac_workspace_bytes(dims, rep: int, prec: int, op: int, n_rhs: int = 1) -> int:
-    return int(lib().hr_dirac_workspace_bytes(lattice(dims), rep, prec, op, n_rhs))
+    return int(lib().hr_dirac_workspace_bytes(_lat(dims), rep, prec, op, n_rhs))
 
 
 def hr_gauge_pack(ctx: Context, dims, rep, prec, canonical, packed, stream=None):
     V = _vol(dims)
     _need(canonical, 4 * V * 4 * 8, "canonical gauge")
     _need(packed, hr_gauge_packed_bytes(dims, rep, prec), "packed gauge")
-    return ctx.check(lib().hr_gauge_pack(ctx.handle, lattice(dims), rep, prec, _ptr(canonical),
+    return ctx.check(lib().hr_gauge_pack(ctx.handle, _lat(dims), rep, prec, _ptr(canonical),
                                          _ptr(packed), _stream(stream)))
 
 
@@ -359,7 +365,7 @@ def hr_spinor_pack(ctx: Context, dims, rep, prec, parity, n_rhs, canonical, pack
     nc = 2 if rep == HR_FUND else 3
     _need(canonical, n_rhs * _vol(dims) * 4 * nc * 16, "canonical spinor")
     _need(packed, hr_spinor_packed_bytes(dims, rep, prec, parity, n_rhs), "packed spinor")
-    return ctx.check(lib().hr_spinor_pack(ctx.handle, lattice(dims), rep, prec, parity, n_rhs,
+    return ctx.check(lib().hr_spinor_pack(ctx.handle, _lat(dims), rep, prec, parity, n_rhs,
                                           _ptr(canonical), _ptr(packed), _stream(stream)))
 
 
@@ -367,7 +373,7 @@ def hr_spinor_unpack(ctx: Context, dims, rep, prec, parity, n_rhs, packed, canon
     nc = 2 if rep == HR_FUND else 3
     _need(canonical, n_rhs * _vol(dims) * 4 * nc * 16, "canonical spinor")
     _need(packed, hr_spinor_packed_bytes(dims, rep, prec, parity, n_rhs), "packed spinor")
-    return ctx.check(lib().hr_spinor_unpack(ctx.handle, lattice(dims), rep, prec, parity, n_rhs,
+    return ctx.check(lib().hr_spinor_unpack(ctx.handle, _lat(dims), rep, prec, parity, n_rhs,
                                             _ptr(packed), _ptr(canonical), _stream(stream)))
 
 
@@ -375,7 +381,7 @@ def hr_dirac_apply(ctx: Context, dims, m0, rep, prec, gauge, inp, out, stream=No
     full = hr_spinor_packed_bytes(dims, rep, prec, HR_FULL, 1)
     _need(inp, full, "in")
     _need(out, full, "out")
-    return ctx.check(lib().hr_dirac_apply(ctx.handle, lattice(dims), float(m0), rep, prec,
+    return ctx.check(lib().hr_dirac_apply(ctx.handle, _lat(dims), float(m0), rep, prec,
                                           _ptr(gauge), _ptr(inp), _ptr(out), _stream(stream)))
 
 
@@ -385,7 +391,7 @@ def hr_dirac_eo(ctx: Context, dims, m0, rep, prec, out_parity, op, n_rhs, gauge,
     _need(inp, half, "in")
     _need(out, half, "out")
     wb = 0 if work is None else work.numel() * work.element_size()
-    return ctx.check(lib().hr_dirac_eo(ctx.handle, lattice(dims), float(m0), rep, prec, out_parity,
+    return ctx.check(lib().hr_dirac_eo(ctx.handle, _lat(dims), float(m0), rep, prec, out_parity,
                                        op, n_rhs, _ptr(gauge), _ptr(inp), _ptr(out), _ptr(work),
                                        wb, _stream(stream)))
 
@@ -395,7 +401,7 @@ def hr_solver_default_opts() -> hr_solver_opts:
 
 
 def hr_cg_workspace_bytes(dims, rep: int, opts: hr_solver_opts) -> int:
-    return int(lib().hr_cg_workspace_bytes(lattice(dims), rep, ctypes.byref(opts)))
+    return int(lib().hr_cg_workspace_bytes(_lat(dims), rep, ctypes.byref(opts)))
 
 
 def hr_cg_solve(ctx: Context, dims, m0, rep, opts: hr_solver_opts, gauge, b, x, work, stream=None,
@@ -406,7 +412,7 @@ def hr_cg_solve(ctx: Context, dims, m0, rep, opts: hr_solver_opts, gauge, b, x, 
     _need(x, half, "x")
     info = hr_solve_info()
     wb = 0 if work is None else work.numel() * work.element_size()
-    rc = lib().hr_cg_solve(ctx.handle, lattice(dims), float(m0), rep, ctypes.byref(opts),
+    rc = lib().hr_cg_solve(ctx.handle, _lat(dims), float(m0), rep, ctypes.byref(opts),
                            _ptr(gauge), _ptr(b), _ptr(x), ctypes.byref(info), _ptr(work), wb,
                            _stream(stream))
     if raise_on_error and rc not in (HR_OK, HR_ERR_NOT_CONVERGED):
@@ -415,7 +421,7 @@ def hr_cg_solve(ctx: Context, dims, m0, rep, opts: hr_solver_opts, gauge, b, x, 
 
 
 def hr_solve_full_workspace_bytes(dims, rep, opts: hr_solver_opts, system: int) -> int:
-    return int(lib().hr_solve_full_workspace_bytes(lattice(dims), rep, ctypes.byref(opts), system))
+    return int(lib().hr_solve_full_workspace_bytes(_lat(dims), rep, ctypes.byref(opts), system))
 
 
 def hr_solve_full(ctx: Context, dims, m0, rep, opts: hr_solver_opts, system, gauge, b, x, work, stream=None,
@@ -427,7 +433,7 @@ def hr_solve_full(ctx: Context, dims, m0, rep, opts: hr_solver_opts, system, gau
     _need(x, full, "x")
     info = hr_solve_info()
     wb = 0 if work is None else work.numel() * work.element_size()
-    rc = lib().hr_solve_full(ctx.handle, lattice(dims), float(m0), rep, ctypes.byref(opts), int(system),
+    rc = lib().hr_solve_full(ctx.handle, _lat(dims), float(m0), rep, ctypes.byref(opts), int(system),
                              _ptr(gauge), _ptr(b), _ptr(x), ctypes.byref(info), _ptr(work), wb,
                              _stream(stream))
     if raise_on_error and rc not in (HR_OK, HR_ERR_NOT_CONVERGED):
@@ -438,19 +444,19 @@ def hr_solve_full(ctx: Context, dims, m0, rep, opts: hr_solver_opts, system, gau
 # ---- clover and exponential-clover site terms
 
 def hr_clover_packed_bytes(dims, rep: int, prec: int) -> int:
-    return int(lib().hr_clover_packed_bytes(lattice(dims), rep, prec))
+    return int(lib().hr_clover_packed_bytes(_lat(dims), rep, prec))
 
 
 def hr_clover_build(ctx: Context, dims, rep, prec, kind, m0, c_sw, canonical, clover, stream=None):
     """Packed clover field (A and A^-1 on both parities) from the canonical gauge."""
     _need(canonical, 4 * _vol(dims) * 4 * 8, "canonical gauge")
     _need(clover, hr_clover_packed_bytes(dims, rep, prec), "clover")
-    return ctx.check(lib().hr_clover_build(ctx.handle, lattice(dims), rep, prec, int(kind), float(m0), float(c_sw),
+    return ctx.check(lib().hr_clover_build(ctx.handle, _lat(dims), rep, prec, int(kind), float(m0), float(c_sw),
                                            _ptr(canonical), _ptr(clover), _stream(stream)))
 
 
 def hr_clover_force_workspace_bytes(dims) -> int:
-    return int(lib().hr_clover_force_workspace_bytes(lattice(dims)))
+    return int(lib().hr_clover_force_workspace_bytes(_lat(dims)))
 
 
 def hr_clover_insertion_force(ctx: Context, dims, c_sw, gauge, lam, coeff, force, work, stream=None):
@@ -459,7 +465,7 @@ def hr_clover_insertion_force(ctx: Context, dims, c_sw, gauge, lam, coeff, force
     _need(gauge, 4 * V * 4 * 8, "gauge")
     _need(lam, V * 64 * 16, "lam")
     _need(force, 4 * V * 3 * 8, "force")
-    return ctx.check(lib().hr_clover_insertion_force(ctx.handle, lattice(dims), float(c_sw), _ptr(gauge), _ptr(lam),
+    return ctx.check(lib().hr_clover_insertion_force(ctx.handle, _lat(dims), float(c_sw), _ptr(gauge), _ptr(lam),
                                                      float(coeff), _ptr(force), _ptr(work), _nbytes(work),
                                                      _stream(stream)))
 
@@ -470,7 +476,7 @@ def hr_clover_fermion_force(ctx: Context, dims, m0, c_sw, gauge, gauge_packed, c
     _need(gauge, 4 * V * 4 * 8, "gauge")
     _need(force, 4 * V * 3 * 8, "force")
     _need(X, hr_spinor_packed_bytes(dims, HR_FUND, HR_F64, HR_EVEN, 1), "X")
-    return ctx.check(lib().hr_clover_fermion_force(ctx.handle, lattice(dims), int(kind), float(m0), float(c_sw),
+    return ctx.check(lib().hr_clover_fermion_force(ctx.handle, _lat(dims), int(kind), float(m0), float(c_sw),
                                                    _ptr(gauge),
                                                    _ptr(gauge_packed), _ptr(clover), _ptr(X), _ptr(Y),
                                                    int(bool(with_det)),
@@ -480,7 +486,7 @@ def hr_clover_fermion_force(ctx: Context, dims, m0, c_sw, gauge, gauge_packed, c
 
 def hr_clover_logdet(ctx: Context, dims, rep, clover, parity, stream=None) -> float:
     out = ctypes.c_double(0.0)
-    ctx.check(lib().hr_clover_logdet(ctx.handle, lattice(dims), rep, _ptr(clover), parity, ctypes.byref(out),
+    ctx.check(lib().hr_clover_logdet(ctx.handle, _lat(dims), rep, _ptr(clover), parity, ctypes.byref(out),
                                      _stream(stream)))
     return out.value
 
@@ -489,7 +495,7 @@ def hr_clover_apply(ctx: Context, dims, rep, prec, parity, inverse, n_rhs, clove
     half = hr_spinor_packed_bytes(dims, rep, prec, parity, n_rhs)
     _need(inp, half, "in")
     _need(out, half, "out")
-    return ctx.check(lib().hr_clover_apply(ctx.handle, lattice(dims), rep, prec, parity, int(bool(inverse)), n_rhs,
+    return ctx.check(lib().hr_clover_apply(ctx.handle, _lat(dims), rep, prec, parity, int(bool(inverse)), n_rhs,
                                            _ptr(clover), _ptr(inp), _ptr(out), _stream(stream)))
 
 
@@ -497,7 +503,7 @@ def hr_dirac_apply_clover(ctx: Context, dims, rep, prec, gauge, clover, inp, out
     full = hr_spinor_packed_bytes(dims, rep, prec, HR_FULL, 1)
     _need(inp, full, "in")
     _need(out, full, "out")
-    return ctx.check(lib().hr_dirac_apply_clover(ctx.handle, lattice(dims), rep, prec, _ptr(gauge), _ptr(clover),
+    return ctx.check(lib().hr_dirac_apply_clover(ctx.handle, _lat(dims), rep, prec, _ptr(gauge), _ptr(clover),
                                                  _ptr(inp), _ptr(out), _stream(stream)))
 
 
@@ -507,13 +513,13 @@ def hr_dirac_eo_clover(ctx: Context, dims, rep, prec, out_parity, op, n_rhs, gau
     _need(inp, half, "in")
     _need(out, half, "out")
     wb = 0 if work is None else work.numel() * work.element_size()
-    return ctx.check(lib().hr_dirac_eo_clover(ctx.handle, lattice(dims), rep, prec, out_parity, op, n_rhs,
+    return ctx.check(lib().hr_dirac_eo_clover(ctx.handle, _lat(dims), rep, prec, out_parity, op, n_rhs,
                                               _ptr(gauge), _ptr(clover), _ptr(inp), _ptr(out), _ptr(work), wb,
                                               _stream(stream)))
 
 
 def hr_cg_clover_workspace_bytes(dims, rep: int, opts: hr_solver_opts) -> int:
-    return int(lib().hr_cg_clover_workspace_bytes(lattice(dims), rep, ctypes.byref(opts)))
+    return int(lib().hr_cg_clover_workspace_bytes(_lat(dims), rep, ctypes.byref(opts)))
 
 
 def hr_cg_solve_clover(ctx: Context, dims, rep, opts: hr_solver_opts, gauge, clover, b, x, work, stream=None,
@@ -524,7 +530,7 @@ def hr_cg_solve_clover(ctx: Context, dims, rep, opts: hr_solver_opts, gauge, clo
     _need(x, half, "x")
     info = hr_solve_info()
     wb = 0 if work is None else work.numel() * work.element_size()
-    rc = lib().hr_cg_solve_clover(ctx.handle, lattice(dims), rep, ctypes.byref(opts), _ptr(gauge), _ptr(clover),
+    rc = lib().hr_cg_solve_clover(ctx.handle, _lat(dims), rep, ctypes.byref(opts), _ptr(gauge), _ptr(clover),
                                   _ptr(b), _ptr(x), ctypes.byref(info), _ptr(work), wb, _stream(stream))
     if raise_on_error and rc not in (HR_OK, HR_ERR_NOT_CONVERGED):
         ctx.check(rc)
@@ -532,7 +538,7 @@ def hr_cg_solve_clover(ctx: Context, dims, rep, opts: hr_solver_opts, gauge, clo
 
 
 def hr_solve_full_clover_workspace_bytes(dims, rep, opts: hr_solver_opts, system: int) -> int:
-    return int(lib().hr_solve_full_clover_workspace_bytes(lattice(dims), rep, ctypes.byref(opts), system))
+    return int(lib().hr_solve_full_clover_workspace_bytes(_lat(dims), rep, ctypes.byref(opts), system))
 
 
 def hr_solve_full_clover(ctx: Context, dims, rep, opts: hr_solver_opts, system, gauge, clover, b, x, work,
@@ -543,7 +549,7 @@ def hr_solve_full_clover(ctx: Context, dims, rep, opts: hr_solver_opts, system, 
     _need(x, full, "x")
     info = hr_solve_info()
     wb = 0 if work is None else work.numel() * work.element_size()
-    rc = lib().hr_solve_full_clover(ctx.handle, lattice(dims), rep, ctypes.byref(opts), int(system), _ptr(gauge),
+    rc = lib().hr_solve_full_clover(ctx.handle, _lat(dims), rep, ctypes.byref(opts), int(system), _ptr(gauge),
                                     _ptr(clover), _ptr(b), _ptr(x), ctypes.byref(info), _ptr(work), wb,
                                     _stream(stream))
     if raise_on_error and rc not in (HR_OK, HR_ERR_NOT_CONVERGED):
@@ -560,14 +566,14 @@ def _links(dims):
 def hr_gauge_force(ctx: Context, dims, beta, gauge, coeff, force, stream=None):
     _need(gauge, _links(dims) * 4 * 8, "gauge")
     _need(force, _links(dims) * 3 * 8, "force")
-    return ctx.check(lib().hr_gauge_force(ctx.handle, lattice(dims), float(beta), _ptr(gauge), float(coeff),
+    return ctx.check(lib().hr_gauge_force(ctx.handle, _lat(dims), float(beta), _ptr(gauge), float(coeff),
                                           _ptr(force), _stream(stream)))
 
 
 def hr_gauge_action(ctx: Context, dims, beta, gauge, stream=None) -> float:
     _need(gauge, _links(dims) * 4 * 8, "gauge")
     out = ctypes.c_double(0.0)
-    ctx.check(lib().hr_gauge_action(ctx.handle, lattice(dims), float(beta), _ptr(gauge), ctypes.byref(out),
+    ctx.check(lib().hr_gauge_action(ctx.handle, _lat(dims), float(beta), _ptr(gauge), ctypes.byref(out),
                                     _stream(stream)))
     return out.value
 
@@ -575,21 +581,21 @@ def hr_gauge_action(ctx: Context, dims, beta, gauge, stream=None) -> float:
 def hr_link_update(ctx: Context, dims, eps, mom, gauge, stream=None):
     _need(mom, _links(dims) * 3 * 8, "mom")
     _need(gauge, _links(dims) * 4 * 8, "gauge")
-    return ctx.check(lib().hr_link_update(ctx.handle, lattice(dims), float(eps), _ptr(mom), _ptr(gauge),
+    return ctx.check(lib().hr_link_update(ctx.handle, _lat(dims), float(eps), _ptr(mom), _ptr(gauge),
                                           _stream(stream)))
 
 
 def hr_mom_update(ctx: Context, dims, eps, force, mom, stream=None):
     _need(force, _links(dims) * 3 * 8, "force")
     _need(mom, _links(dims) * 3 * 8, "mom")
-    return ctx.check(lib().hr_mom_update(ctx.handle, lattice(dims), float(eps), _ptr(force), _ptr(mom),
+    return ctx.check(lib().hr_mom_update(ctx.handle, _lat(dims), float(eps), _ptr(force), _ptr(mom),
                                          _stream(stream)))
 
 
 def hr_kinetic_energy(ctx: Context, dims, mom, stream=None) -> float:
     _need(mom, _links(dims) * 3 * 8, "mom")
     out = ctypes.c_double(0.0)
-    ctx.check(lib().hr_kinetic_energy(ctx.handle, lattice(dims), _ptr(mom), ctypes.byref(out), _stream(stream)))
+    ctx.check(lib().hr_kinetic_energy(ctx.handle, _lat(dims), _ptr(mom), ctypes.byref(out), _stream(stream)))
     return out.value
 
 
@@ -604,7 +610,7 @@ def hr_hmc_params_default(beta: float, m0: float = 0.0, fermions: bool = True, n
 
 
 def hr_hmc_workspace_bytes(dims, prm: hr_hmc_params) -> int:
-    return int(lib().hr_hmc_workspace_bytes(lattice(dims), ctypes.byref(prm)))
+    return int(lib().hr_hmc_workspace_bytes(_lat(dims), ctypes.byref(prm)))
 
 
 def hr_hmc_trajectory(ctx: Context, dims, prm: hr_hmc_params, gauge, mom, eta, work, stream=None, phi=None):
@@ -619,31 +625,31 @@ def hr_hmc_trajectory(ctx: Context, dims, prm: hr_hmc_params, gauge, mom, eta, w
         _need(phi, half, "phi")
     info = hr_hmc_info()
     wb = 0 if work is None else work.numel() * work.element_size()
-    ctx.check(lib().hr_hmc_trajectory(ctx.handle, lattice(dims), ctypes.byref(prm), _ptr(gauge), _ptr(mom),
+    ctx.check(lib().hr_hmc_trajectory(ctx.handle, _lat(dims), ctypes.byref(prm), _ptr(gauge), _ptr(mom),
                                       _ptr(eta), _ptr(phi), ctypes.byref(info), _ptr(work), wb, _stream(stream)))
     return info
 
 
 def hr_force(ctx: Context, dims, gauge, a_full, b_full, beta, force, stream=None):
     _need(force, 4 * _vol(dims) * 3 * 8, "force")
-    return ctx.check(lib().hr_force(ctx.handle, lattice(dims), _ptr(gauge), _ptr(a_full),
+    return ctx.check(lib().hr_force(ctx.handle, _lat(dims), _ptr(gauge), _ptr(a_full),
                                     _ptr(b_full), float(beta), _ptr(force), _stream(stream)))
 
 
 def hr_link_grad(ctx: Context, dims, a_full, b_full, beta, grad, stream=None):
     _need(grad, 4 * _vol(dims) * 4 * 8, "grad")
-    return ctx.check(lib().hr_link_grad(ctx.handle, lattice(dims), _ptr(a_full), _ptr(b_full),
+    return ctx.check(lib().hr_link_grad(ctx.handle, _lat(dims), _ptr(a_full), _ptr(b_full),
                                         float(beta), _ptr(grad), _stream(stream)))
 
 
 def hr_fermion_force_workspace_bytes(dims) -> int:
-    return int(lib().hr_fermion_force_workspace_bytes(lattice(dims)))
+    return int(lib().hr_fermion_force_workspace_bytes(_lat(dims)))
 
 
 def hr_fermion_force(ctx: Context, dims, m0, rep, gauge, X, L, coeff, force, work, stream=None):
     """force += coeff d/dw Re<L, Mhat^+ Mhat X> (L = None: L = X)."""
     _need(force, 4 * _vol(dims) * 3 * 8, "force")
-    return ctx.check(lib().hr_fermion_force(ctx.handle, lattice(dims), float(m0), rep, _ptr(gauge), _ptr(X),
+    return ctx.check(lib().hr_fermion_force(ctx.handle, _lat(dims), float(m0), rep, _ptr(gauge), _ptr(X),
                                             _ptr(L), float(coeff), _ptr(force), _ptr(work), _nbytes(work),
                                             _stream(stream)))
 
@@ -651,7 +657,7 @@ def hr_fermion_force(ctx: Context, dims, m0, rep, gauge, X, L, coeff, force, wor
 def hr_fermion_link_grad(ctx: Context, dims, m0, rep, gauge, X, L, coeff, grad, work, stream=None):
     """grad += coeff d/dq Re<L, Mhat^+ Mhat X> (L = None: L = X)."""
     _need(grad, 4 * _vol(dims) * 4 * 8, "grad")
-    return ctx.check(lib().hr_fermion_link_grad(ctx.handle, lattice(dims), float(m0), rep, _ptr(gauge), _ptr(X),
+    return ctx.check(lib().hr_fermion_link_grad(ctx.handle, _lat(dims), float(m0), rep, _ptr(gauge), _ptr(X),
                                                 _ptr(L), float(coeff), _ptr(grad), _ptr(work), _nbytes(work),
                                                 _stream(stream)))
 
@@ -659,7 +665,7 @@ def hr_fermion_link_grad(ctx: Context, dims, m0, rep, gauge, X, L, coeff, grad, 
 def hr_dot(ctx: Context, dims, rep, a, b, stream=None) -> complex:
     """<a, b> = sum conj(a) b over packed FP64 fields of one parity."""
     re, im = ctypes.c_double(0.0), ctypes.c_double(0.0)
-    ctx.check(lib().hr_dot(ctx.handle, lattice(dims), rep, _ptr(a), _ptr(b), ctypes.byref(re), ctypes.byref(im),
+    ctx.check(lib().hr_dot(ctx.handle, _lat(dims), rep, _ptr(a), _ptr(b), ctypes.byref(re), ctypes.byref(im),
                            _stream(stream)))
     return complex(re.value, im.value)
 
@@ -672,35 +678,35 @@ def hr_fp32_fma_rate(ctx: Context, stream=None):
 
 
 def hr_dd_face_bytes(local_dims, rep, prec) -> int:
-    return int(lib().hr_dd_face_bytes(lattice(local_dims), rep, prec))
+    return int(lib().hr_dd_face_bytes(_lat(local_dims), rep, prec))
 
 
 def hr_dd_pack_faces(ctx: Context, local_dims, rep, prec, in_parity, gauge, inp, to_lower, to_upper, stream=None):
-    return ctx.check(lib().hr_dd_pack_faces(ctx.handle, lattice(local_dims), rep, prec, in_parity, _ptr(gauge),
+    return ctx.check(lib().hr_dd_pack_faces(ctx.handle, _lat(local_dims), rep, prec, in_parity, _ptr(gauge),
                                             _ptr(inp), _ptr(to_lower), _ptr(to_upper), _stream(stream)))
 
 
 def hr_dd_hop_boundary(ctx: Context, local_dims, rep, prec, out_parity, gauge, inp, from_lower, from_upper, out,
                        stream=None):
-    return ctx.check(lib().hr_dd_hop_boundary(ctx.handle, lattice(local_dims), rep, prec, out_parity, _ptr(gauge),
+    return ctx.check(lib().hr_dd_hop_boundary(ctx.handle, _lat(local_dims), rep, prec, out_parity, _ptr(gauge),
                                               _ptr(inp), _ptr(from_lower), _ptr(from_upper), _ptr(out),
                                               _stream(stream)))
 
 
 def hr_norm2(ctx: Context, dims, rep, v, stream=None) -> float:
     out = ctypes.c_double(0.0)
-    ctx.check(lib().hr_norm2(ctx.handle, lattice(dims), rep, _ptr(v), ctypes.byref(out),
+    ctx.check(lib().hr_norm2(ctx.handle, _lat(dims), rep, _ptr(v), ctypes.byref(out),
                              _stream(stream)))
     return out.value
 
 
 def hr_axpy(ctx: Context, dims, rep, a, x, y, stream=None):
-    return ctx.check(lib().hr_axpy(ctx.handle, lattice(dims), rep, float(a), _ptr(x), _ptr(y),
+    return ctx.check(lib().hr_axpy(ctx.handle, _lat(dims), rep, float(a), _ptr(x), _ptr(y),
                                    _stream(stream)))
 
 
 def hr_gamma5(ctx: Context, dims, rep, v, stream=None):
-    return ctx.check(lib().hr_gamma5(ctx.handle, lattice(dims), rep, _ptr(v), _stream(stream)))
+    return ctx.check(lib().hr_gamma5(ctx.handle, _lat(dims), rep, _ptr(v), _stream(stream)))
 
 
 def _vol(dims) -> int:
@@ -716,7 +722,7 @@ def hr_norm2_noalloc(dims, rep, n_rhs, v, result, stream=None) -> int:
     library's status code; raises ValueError only when ``result`` is not a
     contiguous CUDA tensor of at least n_rhs doubles."""
     _need(result, 8 * int(n_rhs), "result")
-    return int(lib().hr_norm2_noalloc(lattice(dims), rep, int(n_rhs), _ptr(v), _ptr(result),
+    return int(lib().hr_norm2_noalloc(_lat(dims), rep, int(n_rhs), _ptr(v), _ptr(result),
                                       _stream(stream)))
 
 
@@ -726,14 +732,14 @@ def hr_autotune_hop(ctx: Context, dims, rep, prec, out_parity, n_rhs, gauge, inp
     _need(inp, half, "in")
     _need(out, half, "out")
     res = hr_tune_result()
-    ctx.check(lib().hr_autotune_hop(ctx.handle, lattice(dims), rep, prec, out_parity, n_rhs, _ptr(gauge),
+    ctx.check(lib().hr_autotune_hop(ctx.handle, _lat(dims), rep, prec, out_parity, n_rhs, _ptr(gauge),
                                     _ptr(inp), _ptr(out), int(reps), ctypes.byref(res), _stream(stream)))
     return res
 
 
 def hr_tune_lookup(ctx: Context, dims, rep, prec, n_rhs=1):
     v, b = ctypes.c_int(-1), ctypes.c_int(-1)
-    ctx.check(lib().hr_tune_lookup(ctx.handle, lattice(dims), rep, prec, n_rhs, ctypes.byref(v),
+    ctx.check(lib().hr_tune_lookup(ctx.handle, _lat(dims), rep, prec, n_rhs, ctypes.byref(v),
                                    ctypes.byref(b)))
     return v.value, b.value
 
@@ -741,7 +747,7 @@ def hr_tune_lookup(ctx: Context, dims, rep, prec, n_rhs=1):
 def _lattice_array(dims_list):
     arr = (hr_lattice * len(dims_list))()
     for k, d in enumerate(dims_list):
-        arr[k] = lattice(d)
+        arr[k] = _lat(d)
     return arr
 
 
