@@ -115,11 +115,11 @@ HR_HD inline fx fx_split(long long t)
 HR_HD inline long long fx_units64(fx v) { return (long long)v.h * (1LL << 28) + v.l; }
 HR_HD inline fx fx_of(fxa s) { return fx_split(fx_round(s)); }
 
-// t 2^-56 as a double: the exponent field moves, no FP64 product
-HR_HD inline double fx_to_double(long long t)
+// t 2^-(56 + k) as a double, k <= 900: the exponent field moves, no FP64 product
+HR_HD inline double fx_to_double(long long t, int k = 0)
 {
     const double d = (double)t;
-    return t ? fx_double(fx_dbits(d) - (56ULL << 52)) : 0.0;
+    return t ? fx_double(fx_dbits(d) - ((unsigned long long)(unsigned)(56 + k) << 52)) : 0.0;
 }
 // t 2^-56 (|t| < 2^59) as a normalised float pair, to 2^-49 of the value: three
 // 22-bit pieces made floats through the mantissa field, then two Fast2Sums

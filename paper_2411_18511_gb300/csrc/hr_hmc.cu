@@ -295,9 +295,15 @@ __device__ __forceinline__ fx fx_fma_const(long long c, fx x, fx y)
 // neither |p| nor a division is needed.  The links come in with unit length, so
 // the renormalisation is 1 - d / 2 with d = |U|^2 - 1 (next term 3 d^2 / 8).
 // All of it in fixed point but the three products eps p / 2 and the conversion
-// of the result.  Steps with z > 1, and links with |d| > 2^-30, take native FP64.
-// 32^4: 0.78 ms in native FP64 (sin, cos, two square roots, two divisions), 0.156 ms
-// here (4.7 TB/s); error against long double 1.2e-16 before, 0.5e-16 now.
+// of the result.  Scalars (cos, U_0) are digits in units of 1, vectors (w, the link's)
+// in units of 2^-k, the largest of their six components below 1 and at least 1/2:
+// a link near the identity, or a short step from it, keeps 56 bits of its small
+// vector part.  A product of two vectors is then 2^-k (a vector) or 2^-2k (a
+// scalar) of its digits.  Steps with z > 1, links with |d| > 2^-30 and vectors
+// below 2^-900 take native FP64.
+// 32^4: 0.78 ms in native FP64 (sin, cos, two square roots, two divisions), 0.163 ms
+// here (4.5 TB/s; 0.158 with the vectors in units of 1).
+constexpr unsigned kLinkVecMin = (1023u - 900u) << 20; // high word of 2^-900
 template <bool VEC>
 __global__ void __launch_bounds__(128) k_link_update(long long n_links, double eps, const double *p, double *q)
 {
@@ -308,12 +314,14 @@ __global__ void __launch_bounds__(128) k_link_update(long long n_links, double e
     double c[4];
     load_link4<VEC>(q, (size_t)t, c);
     const unsigned mw = max(max(fx_abs_high(w0), fx_abs_high(w1)), fx_abs_high(w2));
-    const unsigned mq = max(max(fx_abs_high(c[0]), fx_abs_high(c[1])), max(fx_abs_high(c[2]), fx_abs_high(c[3])));
-    const fx w[3] = {fx_from_double(w0), fx_from_double(w1), fx_from_double(w2)};
+    const unsigned mu = max(max(fx_abs_high(c[1]), fx_abs_high(c[2])), fx_abs_high(c[3]));
+    const unsigned mq = max(fx_abs_high(c[0]), mu), mv = max(mw, mu);
+    const int E = min(max((int)(mv >> 20), 122), 1022), k = 1022 - E, k1 = min(k, 63), k2 = min(2 * k, 63);
+    const fx w[3] = {fx_from_double(w0, E), fx_from_double(w1, E), fx_from_double(w2, E)};
     fxa za = {0, 0};
 #pragma unroll
     for (int a = 0; a < 3; ++a) fx_mac(za, w[a], w[a]);
-    const long long zu = fx_round(za);
+    const long long zu = fx_round(za) >> k2;
     const fx z = fx_neg(fx_split(zu));
     fx cs = fx_split(fx_units(1.0 / 6402373705728000.0)), sn = fx_split(fx_units(1.0 / 121645100408832000.0));
     // 1 - z/2 (1 - z/12 (...)) summed from z^9: coefficients 1 / (2k)! and 1 / (2k+1)!, signs in z
@@ -322,45 +330,52 @@ __global__ void __launch_bounds__(128) k_link_update(long long n_links, double e
     constexpr double fs[9] = {1.0 / 355687428096000.0, 1.0 / 1307674368000.0, 1.0 / 6227020800.0, 1.0 / 39916800.0,
                               1.0 / 362880.0, 1.0 / 5040.0, 1.0 / 120.0, 1.0 / 6.0, 1.0};
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        cs = fx_fma_const(fx_units(fc[k]), z, cs);
-        sn = fx_fma_const(fx_units(fs[k]), z, sn);
+    for (int j = 0; j < 9; ++j) {
+        cs = fx_fma_const(fx_units(fc[j]), z, cs);
+        sn = fx_fma_const(fx_units(fs[j]), z, sn);
     }
-    fxq E;
-    E.c[0] = cs;
+    // E Q, E = (cs, e): scalar cs q0 - e.v, vector cs v + q0 e - e x v
+    const fx q0 = fx_from_double(c[0]);
+    const fx v[3] = {fx_from_double(c[1], E), fx_from_double(c[2], E), fx_from_double(c[3], E)};
+    fx e[3];
+    fxa s0 = {0, 0}, dot = {0, 0}, cross[3] = {}, vec[3] = {};
 #pragma unroll
-    for (int a = 0; a < 3; ++a) E.c[a + 1] = fx_fma_const(0, sn, w[a]);
-    const fxq Q = {{fx_from_double(c[0]), fx_from_double(c[1]), fx_from_double(c[2]), fx_from_double(c[3])}};
-    fxa ua[4] = {};
-    fxa v[3] = {};
-    fxq_mac_scalar(ua[0], E, Q);
-    fxq_mac_vec(v, E, Q);
-    long long u[4] = {fx_round(ua[0]), fx_round(v[0]), fx_round(v[1]), fx_round(v[2])};
+    for (int a = 0; a < 3; ++a) {
+        e[a] = fx_fma_const(0, sn, w[a]);
+        fx_mac(dot, e[a], v[a]);
+        fx_mac(vec[a], cs, v[a]);
+        fx_mac(vec[a], q0, e[a]);
+    }
+    fx_mac(s0, cs, q0);
+    fx_mac_cross(cross, v, e);
+    long long u[4] = {fx_round(s0) - (fx_round(dot) >> k2)};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) u[a + 1] = fx_round(vec[a]) + (fx_round(cross[a]) >> k1);
     fx d[4];
-    fxa n = {-(1LL << 56), 0};
+    fxa n0 = {-(1LL << 56), 0}, nv = {0, 0};
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        d[k] = fx_split(u[k]);
-        fx_mac(n, d[k], d[k]);
+    for (int a = 0; a < 4; ++a) {
+        d[a] = fx_split(u[a]);
+        fx_mac(a ? nv : n0, d[a], d[a]);
     }
-    const long long dn = fx_round(n); // |U|^2 - 1
+    const long long dn = fx_round(n0) + (fx_round(nv) >> k2); // |U|^2 - 1
     double *qq = q + t * 4;
-    if (mw >= kFxHigh1 || mq >= kFxHigh2 || zu > (1LL << 56) || dn > (1 << 26) || dn < -(1 << 26)) {
+    if (mw >= kFxHigh1 || mq >= kFxHigh2 || mv < kLinkVecMin || zu > (1LL << 56) || dn > (1 << 26) || dn < -(1 << 26)) {
         link_update_native(eps, pp, qq);
         return;
     }
     const int hd = (int)dn; // u (1 - d / 2): u d / 2 from the leading digit of u
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const long long r = u[k] - (((long long)d[k].h * hd + (1LL << 28)) >> 29);
-        c[k] = fx_to_double(r);
+    for (int a = 0; a < 4; ++a) {
+        const long long r = u[a] - (((long long)d[a].h * hd + (1LL << 28)) >> 29);
+        c[a] = fx_to_double(r, a ? k : 0);
     }
     if constexpr (VEC) {
         ((double2 *)qq)[0] = make_double2(c[0], c[1]);
         ((double2 *)qq)[1] = make_double2(c[2], c[3]);
     } else {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) qq[k] = c[k];
+        for (int a = 0; a < 4; ++a) qq[a] = c[a];
     }
 }
 
