@@ -45,14 +45,21 @@ template <bool VEC> __device__ __forceinline__ void load_link4(const double *q, 
         for (int k = 0; k < 4; ++k) c[k] = p[k];
     }
 }
-template <bool VEC> __device__ __forceinline__ fxq load_fxq(const double *q, size_t link, bool &ok)
+// (top: raised to the high word of the largest vector component)
+template <bool VEC> __device__ __forceinline__ fxq load_fxq(const double *q, size_t link, bool &ok, unsigned &top)
 {
     double c[4];
     load_link4<VEC>(q, link, c);
-    const unsigned m = max(max(fx_abs_high(c[0]), fx_abs_high(c[1])), max(fx_abs_high(c[2]), fx_abs_high(c[3])));
+    const unsigned v = max(max(fx_abs_high(c[1]), fx_abs_high(c[2])), fx_abs_high(c[3])), m = max(v, fx_abs_high(c[0]));
     const fxq r = {{fx_from_unit(c[0]), fx_from_unit(c[1]), fx_from_unit(c[2]), fx_from_unit(c[3])}};
     ok = ok && m < kFxHigh2 && fxq_near_unit(r);
+    top = max(top, v);
     return r;
+}
+template <bool VEC> __device__ __forceinline__ fxq load_fxq(const double *q, size_t link, bool &ok)
+{
+    unsigned top = 0;
+    return load_fxq<VEC>(q, link, ok, top);
 }
 
 // the 16 reals of a packed FP64 spinor as digits, [2 (2 spin + colour) + (0 re, 1 im)],

@@ -112,7 +112,8 @@ __device__ __noinline__ void gauge_force_native(const Geom &g, const double *q, 
 // vector: k_plaq_vec computes the six of a site (2.75 quaternion products each),
 // k_plaq_force rotates twelve (15 products of numbers each) and adds them up,
 // where one thread per link forms 13 quaternion products and converts 19 links.
-// A vector is stored as its three digit pairs, 24 bytes, so it needs no conversion.
+// A vector is stored as its three digit pairs, 24 bytes, so it needs no conversion
+// (plaquettes of links near the identity: three doubles, hr_plaq.cuh).
 //
 // Both are bound by the integer pipes.  The vectors of the whole lattice would be
 // 144 bytes a site from HBM and unbounded scratch, so slabs of time slices that
@@ -120,12 +121,50 @@ __device__ __noinline__ void gauge_force_native(const Geom &g, const double *q, 
 // below this many sites one thread per link instead of per site, more of them in flight
 constexpr int kPlaqSplitSites = 1 << 17;
 
+// One link from the same vectors in native FP64, where some of them are doubles:
+// every term then carries 2^-53 of itself.  false: a link or a plaquette is out of range.
+// 32^4, all links near the identity: 1.49 to 1.64 ms for the whole force (2.03 with
+// every staple in native FP64, 0.485 for links away from it).
+__device__ __noinline__ bool plaq_force_native(const Geom &g, const double *q, int mu, int t, double s, int first, int n,
+                                               const int4 *pa, const int2 *pb, double *f)
+{
+    const int V = 2 * g.vh, slice = g.d[1] * g.d[2] * g.d[3], own = t - first * slice;
+    const LexSite x = lex_site(g, t);
+    double sum[3] = {0.0, 0.0, 0.0};
+#pragma unroll 1
+    for (int nu = 0; nu < 4; ++nu) {
+        if (nu == mu) continue;
+        int unused, down;
+        lex_steps(g, x, nu, unused, down);
+        const size_t p = (size_t)plane_of(mu, nu) * n;
+        const int low = nu == 0 && x.x0 > first ? own - slice : own + down;
+        const int4 oa = pa[p + own], ya = pa[p + low];
+        const int2 ob = pb[p + own], yb = pb[p + low];
+        if (oa.x == kPlaqBad || ya.x == kPlaqBad) return false;
+        const PlaqVec o = plaq_doubles(oa, ob), v = plaq_doubles(ya, yb);
+        const double *u = q + 4 * ((size_t)nu * V + t + down);
+        const double u0 = u[0], u1 = u[1], u2 = u[2], u3 = u[3];
+        const double d = (u0 * u0 - 1.0) + (u1 * u1 + u2 * u2 + u3 * u3);
+        if (!(fabs(d) < 0x1p-29)) return false;
+        const double w = 2.0 * (1.0 - d), t0 = u2 * v.v[2] - u3 * v.v[1], t1 = u3 * v.v[0] - u1 * v.v[2],
+                     t2 = u1 * v.v[1] - u2 * v.v[0];
+        const double sg = mu < nu ? 1.0 : -1.0;
+        sum[0] += sg * ((o.v[0] - v.v[0]) - w * (u0 * t0 + (u2 * t2 - u3 * t1)));
+        sum[1] += sg * ((o.v[1] - v.v[1]) - w * (u0 * t1 + (u3 * t0 - u1 * t2)));
+        sum[2] += sg * ((o.v[2] - v.v[2]) - w * (u0 * t2 + (u1 * t1 - u2 * t0)));
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) f[a] += s * sum[a];
+    return true;
+}
+
 // The force on the links of the sites t0 .. t0 + m - 1 from the n vectors a plane
 // that start at slice `first`; NMU = 4: one thread per site, 1: one per link
 // (mu = blockIdx.y).  With u the quaternion U_n(y), t = u x v:
 //   vec(U^+ v U) / |U|^2 = v + 2 (u0 t + u x t) / |U|^2,
 // and 1 / |U|^2 = 1 - d, d = |U|^2 - 1, so that links off unit length by up to
-// 2^-29 give the staple's value.  The others take native FP64.
+// 2^-29 give the staple's value.  The others, and sites with a plaquette of links near
+// the identity, take native FP64.
 template <bool VEC, int NMU>
 __global__ void __launch_bounds__(128, 5) k_plaq_force(Geom g, double s, const double *__restrict__ q,
                                                     double *__restrict__ F, int t0, int m, int first, int n,
@@ -139,7 +178,7 @@ __global__ void __launch_bounds__(128, 5) k_plaq_force(Geom g, double s, const d
     long long sum[NMU][3] = {}; // units 2^-56, rounded once per neighbour
     bool ok = true;
 #pragma unroll 1
-    for (int nu = 0; nu < 4; ++nu) {
+    for (int nu = 0; nu < 4 && ok; ++nu) {
         if (NMU == 1 && nu == (int)blockIdx.y) continue;
         int unused, down;
         lex_steps(g, x, nu, unused, down);
@@ -164,7 +203,7 @@ __global__ void __launch_bounds__(128, 5) k_plaq_force(Geom g, double s, const d
             const size_t p = (size_t)plane_of(mu, nu) * n;
             const int4 oa = pa[p + own], ya = pa[p + low];
             const int2 ob = pb[p + own], yb = pb[p + low];
-            ok = ok && oa.x != kPlaqBad && ya.x != kPlaqBad;
+            ok = ok && !plaq_marked(oa.x) && !plaq_marked(ya.x);
             const fx v[3] = {{ya.x, ya.y}, {ya.z, ya.w}, {yb.x, yb.y}};
             fxa tc[3] = {};
             fx_mac_cross(tc, u, v);
@@ -191,7 +230,7 @@ __global__ void __launch_bounds__(128, 5) k_plaq_force(Geom g, double s, const d
         const int mu = NMU == 1 ? (int)blockIdx.y : k;
         double *f = F + ((size_t)mu * V + t) * 3;
         if (!ok) {
-            gauge_force_native(g, q, mu, t, s, f);
+            if (!plaq_force_native(g, q, mu, t, s, first, n, pa, pb, f)) gauge_force_native(g, q, mu, t, s, f);
             continue;
         }
 #pragma unroll
@@ -214,7 +253,8 @@ __global__ void __launch_bounds__(128) k_gauge_force(Geom g, double s, const dou
     int up_mu, unused;
     lex_steps(g, x, mu, up_mu, unused);
     bool ok = true;
-    const fxq U = load_fxq<VEC>(q, (size_t)mu * V + t, ok);
+    unsigned top = 0;
+    const fxq U = load_fxq<VEC>(q, (size_t)mu * V + t, ok, top);
     fxq S = {};
 #pragma unroll 1
     for (int k = 1; k < 4; ++k) {
@@ -223,19 +263,19 @@ __global__ void __launch_bounds__(128) k_gauge_force(Geom g, double s, const dou
         lex_steps(g, x, nu, up, down);
         const size_t bm = (size_t)mu * V + t, bn = (size_t)nu * V + t;
         // U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+ = U_nu(x+mu) [U_nu(x) U_mu(x+nu)]^+
-        fxq a = load_fxq<VEC>(q, bn, ok), b = load_fxq<VEC>(q, bm + up, ok);
+        fxq a = load_fxq<VEC>(q, bn, ok, top), b = load_fxq<VEC>(q, bm + up, ok, top);
         b = fxq_conj(fxq_mul(a, b));
-        a = load_fxq<VEC>(q, bn + up_mu, ok);
+        a = load_fxq<VEC>(q, bn + up_mu, ok, top);
         S = fxq_add(S, fxq_mul(a, b));
         // U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu) = [U_mu(x-nu) U_nu(x+mu-nu)]^+ U_nu(x-nu)
-        a = load_fxq<VEC>(q, bm + down, ok);
-        b = load_fxq<VEC>(q, bn + down + up_mu, ok);
+        a = load_fxq<VEC>(q, bm + down, ok, top);
+        b = load_fxq<VEC>(q, bn + down + up_mu, ok, top);
         b = fxq_conj(fxq_mul(a, b));
-        a = load_fxq<VEC>(q, bn + down, ok);
+        a = load_fxq<VEC>(q, bn + down, ok, top);
         S = fxq_add(S, fxq_mul(b, a));
     }
     double *f = F + ((size_t)mu * V + t) * 3;
-    if (!ok) {
+    if (!ok || top < kPlaqWeak) { // (near the identity: digits would hold less, hr_plaq.cuh)
         gauge_force_native(g, q, mu, t, s, f);
         return;
     }

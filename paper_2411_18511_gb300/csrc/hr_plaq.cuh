@@ -10,7 +10,53 @@
 namespace hr {
 
 static_assert(kPlaqSiteBytes == 6 * (sizeof(int4) + sizeof(int2)), "six vectors a site");
-constexpr int kPlaqBad = (int)0x80000000; // leading digit of a vector outside the fixed-point range
+
+// A vector in the scratch is three digit pairs (int4, int2) in units of 1.  Digits hold
+// an absolute 2^-56 and the products some 2^-56 more (1.3e-17 in root mean square),
+// native FP64 rounds at 2^-53 of the links' vector parts (1.3e-16 of them): the
+// same where the largest component of the four links is 1/8.  Links below that (near the
+// identity: cold starts, smooth fields) give the plaquette in native FP64, and the
+// scratch holds its three doubles, marked: the top two bits of a leading digit are equal
+// (|h| < 2^30), those of a double's high word are made to differ (it is below 2, so
+// the second is free).
+constexpr unsigned kPlaqWeak = (1023u - 3u) << 20; // high word of 1/8
+constexpr int kPlaqBad = 0x7fffffff;               // links outside the fixed-point range (marked too)
+__device__ __forceinline__ bool plaq_marked(int first) { return (first ^ (first << 1)) < 0; }
+
+struct PlaqVec {
+    double v[3];
+};
+__device__ __forceinline__ void store_marked(const PlaqVec &P, int4 &a, int2 &b)
+{
+    const int h = __double2hiint(P.v[0]);
+    a = make_int4((h & (int)0xbfffffff) | (int)(~(unsigned)h >> 1 & 0x40000000u), __double2loint(P.v[0]),
+                  __double2hiint(P.v[1]), __double2loint(P.v[1]));
+    b = make_int2(__double2hiint(P.v[2]), __double2loint(P.v[2]));
+}
+// the vector of either kind as doubles (kPlaqBad excepted)
+__device__ __forceinline__ PlaqVec plaq_doubles(int4 a, int2 b)
+{
+    if (plaq_marked(a.x))
+        return {{__hiloint2double(a.x & (int)0xbfffffff, a.y), __hiloint2double(a.z, a.w), __hiloint2double(b.x, b.y)}};
+    return {{fx_to_double(fx_units64({a.x, a.y})), fx_to_double(fx_units64({a.z, a.w})), fx_to_double(fx_units64({b.x, b.y}))}};
+}
+
+// vec of U_a U_b (U_c U_d)^+ in native FP64
+static __device__ __noinline__ PlaqVec plaq_vec_native(const double *q, size_t a, size_t b, size_t c, size_t d)
+{
+    auto mul = [&](size_t i, size_t j, double (&r)[4]) {
+        const double *x = q + 4 * i, *y = q + 4 * j;
+        r[0] = x[0] * y[0] - (x[1] * y[1] + x[2] * y[2] + x[3] * y[3]);
+        r[1] = x[0] * y[1] + y[0] * x[1] - (x[2] * y[3] - x[3] * y[2]);
+        r[2] = x[0] * y[2] + y[0] * x[2] - (x[3] * y[1] - x[1] * y[3]);
+        r[3] = x[0] * y[3] + y[0] * x[3] - (x[1] * y[2] - x[2] * y[1]);
+    };
+    double A[4], B[4];
+    mul(a, b, A);
+    mul(c, d, B);
+    return {{B[0] * A[1] - A[0] * B[1] + (A[2] * B[3] - A[3] * B[2]), B[0] * A[2] - A[0] * B[2] + (A[3] * B[1] - A[1] * B[3]),
+             B[0] * A[3] - A[0] * B[3] + (A[1] * B[2] - A[2] * B[1])}};
+}
 
 // plane index of mu < nu: (01) (02) (03) (12) (13) (23)
 __device__ __forceinline__ int plane_of(int mu, int nu)
@@ -28,6 +74,7 @@ __global__ void __launch_bounds__(128) k_plaq_vec(Geom g, const double *__restri
 {
     constexpr int OWN = PER == 6 ? 8 : 1;
     __shared__ int4 own[OWN][128]; // this thread's slots: no other thread reads them
+    __shared__ unsigned own_top[PER == 6 ? 4 : 1][128];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int V = 2 * g.vh, slice = g.d[1] * g.d[2] * g.d[3];
@@ -38,17 +85,20 @@ __global__ void __launch_bounds__(128) k_plaq_vec(Geom g, const double *__restri
     if constexpr (PER == 6) {
 #pragma unroll 1
         for (int mu = 0; mu < 4; ++mu) {
-            const fxq u = load_fxq<VEC>(q, (size_t)mu * V + t, ok_own);
+            unsigned top = 0;
+            const fxq u = load_fxq<VEC>(q, (size_t)mu * V + t, ok_own, top);
+            own_top[mu][threadIdx.x] = top;
             own[2 * mu][threadIdx.x] = make_int4(u.c[0].h, u.c[0].l, u.c[1].h, u.c[1].l);
             own[2 * mu + 1][threadIdx.x] = make_int4(u.c[2].h, u.c[2].l, u.c[3].h, u.c[3].l);
         }
     }
-    auto own_link = [&](int mu, bool &ok) -> fxq {
+    auto own_link = [&](int mu, bool &ok, unsigned &top) -> fxq {
         if constexpr (PER == 6) {
+            top = max(top, own_top[mu][threadIdx.x]);
             const int4 a = own[2 * mu][threadIdx.x], b = own[2 * mu + 1][threadIdx.x];
             return {{{a.x, a.y}, {a.z, a.w}, {b.x, b.y}, {b.z, b.w}}};
         } else {
-            return load_fxq<VEC>(q, (size_t)mu * V + t, ok);
+            return load_fxq<VEC>(q, (size_t)mu * V + t, ok, top);
         }
     };
     const int p0 = PER == 6 ? 0 : blockIdx.y;
@@ -59,13 +109,18 @@ __global__ void __launch_bounds__(128) k_plaq_vec(Geom g, const double *__restri
         lex_steps(g, x, mu, up_mu, unused);
         lex_steps(g, x, nu, up_nu, unused);
         bool ok = ok_own;
-        const fxq A = fxq_mul(own_link(mu, ok), load_fxq<VEC>(q, (size_t)nu * V + t + up_mu, ok));
-        const fxq B = fxq_conj(fxq_mul(own_link(nu, ok), load_fxq<VEC>(q, (size_t)mu * V + t + up_nu, ok)));
+        unsigned top = 0;
+        const size_t um = (size_t)mu * V + t, un = (size_t)nu * V + t;
+        const fxq A = fxq_mul(own_link(mu, ok, top), load_fxq<VEC>(q, un + up_mu, ok, top));
+        const fxq B = fxq_conj(fxq_mul(own_link(nu, ok, top), load_fxq<VEC>(q, um + up_nu, ok, top)));
         fxa w[3] = {};
         fxq_mac_vec(w, A, B);
         const fx v0 = fx_of(w[0]), v1 = fx_of(w[1]), v2 = fx_of(w[2]);
-        pa[(size_t)p * n + i] = make_int4(ok ? v0.h : kPlaqBad, v0.l, v1.h, v1.l);
-        pb[(size_t)p * n + i] = make_int2(v2.h, v2.l);
+        int4 a = make_int4(ok ? v0.h : kPlaqBad, v0.l, v1.h, v1.l);
+        int2 b = make_int2(v2.h, v2.l);
+        if (ok && top < kPlaqWeak) store_marked(plaq_vec_native(q, um, un + up_mu, un, um + up_nu), a, b);
+        pa[(size_t)p * n + i] = a;
+        pb[(size_t)p * n + i] = b;
     }
 }
 
@@ -93,7 +148,7 @@ __device__ __forceinline__ bool load_plaq(const PlaqVecs &P, int plane, int slot
     v[0] = {a.x, a.y};
     v[1] = {a.z, a.w};
     v[2] = {b.x, b.y};
-    return a.x != kPlaqBad;
+    return !plaq_marked(a.x);
 }
 
 // A link that transports vectors: with u its vector part, t = u x v and d = |U|^2 - 1,

@@ -1,5 +1,7 @@
-"""The link update near the identity (cold starts, smooth and perturbative fields,
-short steps): the links' small vector parts hold binary64's accuracy of themselves.
+"""Gauge force and link update of links near the identity (cold
+starts, smooth and perturbative fields, short steps): what they compute is as
+small as the links' vector parts and holds binary64's accuracy relative to
+those, in fields that are weak everywhere, in part, or on one link.
 
 Bounds: the native formulas make at most some 60 roundings of 2^-53 on terms as
 large as the largest vector component they read (a scalar part near 1 times a vector
@@ -9,9 +11,8 @@ part), and so does the reference in torch or NumPy binary64.
 import numpy as np
 import pytest
 
-import synth
 from oracle import hmc as ohmc
-from tests.test_gpu_gauge_force import links
+from tests.test_gpu_gauge_force import links, reference
 
 pytestmark = pytest.mark.gpu
 
@@ -48,6 +49,46 @@ def weak_links(dims, kind, seed):
         w.zero_()
         w[..., 0] = 1.0
     return w
+
+
+def neighbourhood(q, dims):
+    """Per link: the largest vector component among the links of its six plaquettes."""
+    n = q[..., 1:].abs().amax(-1).reshape(4, *dims)
+    out = []
+    for mu in range(4):
+        m = n[mu]
+        for nu in range(4):
+            if nu != mu:
+                ahead = torch.roll(n[nu], -1, mu)
+                for t in (n[nu], ahead, torch.roll(n[mu], -1, nu), torch.roll(n[nu], 1, nu), torch.roll(n[mu], 1, nu),
+                          torch.roll(ahead, 1, nu)):
+                    m = torch.maximum(m, t)
+        out.append(m)
+    return torch.stack(out).reshape(4, -1, 1)
+
+
+KINDS = [0.2, 0.05, 1e-3, 1e-6, 1e-13, "half", "one", "cold"]
+
+
+# one thread per link and per site, several slabs, slices too large for the scratch
+@pytest.mark.parametrize("dims", [(4, 2, 6, 10), (22, 18, 20, 18), (4, 60, 60, 64), (2, 64, 64, 64)])
+@pytest.mark.parametrize("kind", KINDS)
+def test_gauge_force(ctx, dims, kind):
+    q = weak_links(dims, kind, 41)
+    F = torch.zeros((4, q.shape[1], 3), dtype=torch.float64, device="cuda")
+    hr.hr_gauge_force(ctx, dims, 2.3, q, 1.0, F)
+    err = (F - reference(q, dims, 2.3)).abs()
+    assert bool((err <= 64 * 2.3 * ULP * neighbourhood(q, dims)).all())
+
+
+def test_gauge_force_unaligned(ctx):
+    dims = (18, 16, 20, 26)
+    q = weak_links(dims, "half", 42)
+    buf = torch.empty(q.numel() + 1, dtype=torch.float64, device="cuda")
+    buf[1:] = q.reshape(-1)
+    F = torch.full((4, q.shape[1], 3), 0.0, dtype=torch.float64, device="cuda")
+    hr.hr_gauge_force(ctx, dims, 2.3, buf[1:].reshape(q.shape), 1.0, F)
+    assert bool(((F - reference(q, dims, 2.3)).abs() <= 64 * 2.3 * ULP * neighbourhood(q, dims)).all())
 
 
 @pytest.mark.parametrize("eps", [0.3, 1e-3, 1e-12, 1e-18, 1e-200, 0.0])
