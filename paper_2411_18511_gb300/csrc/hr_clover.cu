@@ -18,6 +18,7 @@
 // (the argument is scaled below 1/2 in the 1-norm: truncation < 1e-19).
 // Storing the explicit inverse instead of LDL factors: the same n^2 reals, and
 // a matrix-vector product has no sequential dependency chain.
+#include <algorithm>
 #include <cmath>
 
 #include "hr_clover.cuh"
@@ -364,7 +365,14 @@ template <int NC, int CP> __global__ void __launch_bounds__(64) k_clover_build(B
 // exponential: the Taylor series of exp(+-X) to degree 18 (|X| <= 1: remainder
 // 8e-18) by Horner's rule on the four coefficients, three products a step
 // where a 4 x 4 complex matrix product has 256.  All of it in two-digit fixed
-// point (hr_fix.cuh).  A site with links off unit length, |N| too large, D near
+// point (hr_fix.cuh).
+// N is held as N' = 2^k N.  k = 0 on rough fields with c_sw / a of 1/16 or more.  Where
+// every plaquette of a site comes from links near the identity (doubles,
+// hr_plaq.cuh), a second pass takes them in units of the largest; a small c_sw / a
+// adds its power of two.  A's numbers off the diagonal are then as accurate as they
+// are small, and t, K, L, d, q, of second order and higher in N, are shifted back.
+// A site with links off unit length, |N| too large, k above 40, numbers of very
+// different size (a row of N below 2^-8 of the others: a pair holds 2^-49), D near
 // 0 or a factor out of range sets kBuildOutside, and the call, which reads its
 // status word in any case, builds the field again in native FP64 (a call to
 // the native code inside this kernel would hold it at 255 registers).
@@ -372,22 +380,25 @@ template <int NC, int CP> __global__ void __launch_bounds__(64) k_clover_build(B
 // source in, solution out) 9.75 ms with the native build, 3.36 ms of it the
 // build, 7.03 ms with this one and 0.61 ms of it the build; leaves from the
 // plaquettes' vectors took another 0.33 ms off that build (5.80 -> 5.47 ms for
-// the solve by then); solution error against 64 bits unchanged.
+// the solve by then); solution error against 64 bits unchanged.  The build alone at
+// 32^4: 10.1 ms native; 0.915 (exponential 1.29) on rough links, of it 0.04 for N's
+// own scale; 1.41 to 1.84 on links near the identity.
 
 struct FxMat {
     fx m[3][3];
 };
 
 // vector part of the sum of the four leaves of the (mu, nu) plane at x, in units of 2^-56
+// (top: raised to the largest vector component of the links)
 template <bool VEC>
 __device__ __forceinline__ void leaf_sum(const Geom &g, const double *can, const LexSite &x, int mu, int nu,
-                                         long long (&f)[3], bool &ok)
+                                         long long (&f)[3], bool &ok, unsigned &top)
 {
     int um, dm, un, dn;
     lex_steps(g, x, mu, um, dm);
     lex_steps(g, x, nu, un, dn);
     const size_t V = 2 * (size_t)g.vh, bm = (size_t)mu * V + x.t, bn = (size_t)nu * V + x.t;
-    auto U = [&](size_t at) { return load_fxq<VEC>(can, at, ok); };
+    auto U = [&](size_t at) { return load_fxq<VEC>(can, at, ok, top); };
     fxa s[3] = {};
     const fxq a = U(bm), b = U(bn);
     // U_mu(x) U_nu(x+mu) [U_nu(x) U_mu(x+nu)]^+
@@ -411,20 +422,23 @@ __device__ __forceinline__ void leaf_sum(const Geom &g, const double *can, const
     for (int k = 0; k < 3; ++k) f[k] = fx_round(s[k]);
 }
 
-// the 16 reals of a block u + sum P_lk s_l (x) s_k (units of 2^-56), each times
-// the digits `sc` and 2^ksc, as pairs
-__device__ __forceinline__ void block_pairs(long long u, const FxMat &P, fx sc, float ksc, float2 (&out)[16])
+// the 16 reals of a block u + 2^-k sum P_lk s_l (x) s_k (units of 2^-56), each times
+// the digits `sc` and the power of two ksc, as pairs; k <= 100
+__device__ __forceinline__ void block_pairs(long long u, const FxMat &P, int k, fx sc, float ksc, float2 (&out)[16])
 {
-    auto pair = [&](long long t) {
+    const float koff = ksc * fx_float((unsigned)(127 - k) << 23);
+    auto pair_by = [&](long long t, float by) {
         fxa s = {0, 0};
         fx_mac(s, fx_split(t), sc);
         float2 v;
         fx_to_pair(fx_round(s), v.x, v.y);
-        return make_float2(v.x * ksc, v.y * ksc);
+        return make_float2(v.x * by, v.y * by);
     };
+    auto pair = [&](long long t) { return pair_by(t, koff); };
     auto T = [](fx v) { return fx_units64(v); };
     auto neg = [](float2 v) { return make_float2(-v.x, -v.y); };
-    const float2 dp = pair(u + T(P.m[2][2])), dm = pair(u - T(P.m[2][2]));
+    const long long d = T(P.m[2][2]) >> min(k, 63);
+    const float2 dp = pair_by(u + d, ksc), dm = pair_by(u - d, ksc);
     out[0] = dp; out[1] = dm; out[2] = dm; out[3] = dp;
     const float2 p31 = pair(T(P.m[2][0])), p32 = pair(T(P.m[2][1])), p13 = pair(T(P.m[0][2])), p23 = pair(T(P.m[1][2]));
     out[4] = p31; out[5] = neg(p32);                 // (0, 1)
@@ -475,7 +489,8 @@ struct LowLinks {
 };
 template <bool VEC>
 __device__ __forceinline__ void leaf_sum_slab(const Geom &g, const double *can, const LexSite &x, const PlaqVecs &P,
-                                              int first, const LowLinks &low, int mu, int nu, long long (&f)[3], bool &ok)
+                                              int first, const LowLinks &low, int mu, int nu, int E, long long (&f)[3],
+                                              PlaqKinds &kinds, bool &ok)
 {
     const int slice = g.d[1] * g.d[2] * g.d[3], own = x.t - first * slice, plane = plane_of(mu, nu);
     int unused, dm, dn;
@@ -484,17 +499,17 @@ __device__ __forceinline__ void leaf_sum_slab(const Geom &g, const double *can, 
     // (the slab's first slice is the one before its first site's, unless it is the whole lattice; nu > 0)
     const int sm = mu == 0 && x.x0 > first ? -slice : dm;
     fx v[3];
-    ok = load_plaq(P, plane, own, v) && ok;
+    load_plaq(P, plane, own, E, v, kinds);
 #pragma unroll
     for (int k = 0; k < 3; ++k) f[k] = fx_units64(v[k]);
-    ok = load_plaq(P, plane, own + sm, v) && ok;
+    load_plaq(P, plane, own + sm, E, v, kinds);
     const Transport Tm = low.get(mu);
     transport_add(Tm, v, f);
     long long h[3];
-    ok = load_plaq(P, plane, own + dn, v) && ok;
+    load_plaq(P, plane, own + dn, E, v, kinds);
 #pragma unroll
     for (int k = 0; k < 3; ++k) h[k] = fx_units64(v[k]);
-    ok = load_plaq(P, plane, own + sm + dn, v) && ok;
+    load_plaq(P, plane, own + sm + dn, E, v, kinds);
     const Transport Tw = make_transport(load_fxq<VEC>(can, (size_t)mu * 2 * g.vh + (x.t + dm + dn), ok), ok);
     transport_add(Tw, v, h);
 #pragma unroll
@@ -504,7 +519,8 @@ __device__ __forceinline__ void leaf_sum_slab(const Geom &g, const double *can, 
 }
 
 struct BuildFx {
-    fx kappa;    // c_sw / a
+    fx kappa;    // 2^kk c_sw / a
+    int kk;
     fx am;       // a = am 2^ka, am in [1, 2)
     float ka;    // 2^ka
     double inva; // 1 / a
@@ -519,6 +535,7 @@ __global__ void __launch_bounds__(64, 6) k_clover_build_fx(BuildArgs B, BuildFx 
     __shared__ int4 low_words[SLAB ? 16 : 1][64]; // this thread's slots: no other thread reads them
     const int t = t0 + blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= t0 + m) return;
+    const unsigned bad = *(volatile const unsigned *)B.bad; // looked at once the first links are on their way
     const LexSite x = lex_site(g, t);
     const int p = (x.x0 + x.x1 + x.x2 + x.x3) & 1, i = t >> 1;
     bool ok = true;
@@ -531,37 +548,70 @@ __global__ void __launch_bounds__(64, 6) k_clover_build_fx(BuildArgs B, BuildFx 
             low.put(mu, make_transport(load_fxq<VEC>(B.can, (size_t)mu * 2 * g.vh + (t + dm), ok), ok));
         }
     }
+    if (bad & kBuildOutside) return; // the field will be built in native FP64
     FxMat N[2];
+    int E = 1022; // vectors in units of 2^(E - 1022)
 #pragma unroll 1
-    for (int l = 0; l < 3; ++l) {
-        long long e[3], f[3];
-        // B_1 = F_23, B_2 = F_31 = -F_13, B_3 = F_12
-        if constexpr (SLAB) {
-            leaf_sum_slab<VEC>(g, B.can, x, P, first, low, 0, l + 1, e, ok);
-            leaf_sum_slab<VEC>(g, B.can, x, P, first, low, l == 0 ? 2 : 1, l == 2 ? 2 : 3, f, ok);
-        } else {
-            leaf_sum<VEC>(g, B.can, x, 0, l + 1, e, ok);
-            leaf_sum<VEC>(g, B.can, x, l == 0 ? 2 : 1, l == 2 ? 2 : 3, f, ok);
-        }
-        fx row[2][3];
+    for (;;) {
+        bool rough = false;
+        unsigned top = 0, least = 0xffffffffu; // over the rows from links near the identity
+#pragma unroll 1
+        for (int l = 0; l < 3; ++l) {
+            long long e[3], f[3] = {0, 0, 0};
+            PlaqKinds row;
+            // B_1 = F_23, B_2 = F_31 = -F_13, B_3 = F_12
+            const int mu = l == 0 ? 2 : 1, nu = l == 2 ? 2 : 3;
+            if constexpr (SLAB) {
+                // (one copy of the code for both: 32^4 945 -> 913 us, exponential 1440 -> 1293)
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const long long bk = l == 1 ? -f[k] : f[k];
-            fxa u = {0, 0}, d = {0, 0};
-            fx_mac(u, fx_split((e[k] + bk) >> 3), X.kappa);
-            fx_mac(d, fx_split((bk - e[k]) >> 3), X.kappa);
-            row[0][k] = fx_of(u);
-            row[1][k] = fx_of(d);
-        }
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
+                    for (int k = 0; k < 3; ++k) e[k] = f[k];
+                    leaf_sum_slab<VEC>(g, B.can, x, P, first, low, h ? mu : 0, h ? nu : l + 1, E, f, row, ok);
+                }
+            } else {
+                leaf_sum<VEC>(g, B.can, x, 0, l + 1, e, ok, row.top);
+                leaf_sum<VEC>(g, B.can, x, mu, nu, f, ok, row.top);
+            }
+            ok = ok && !row.bad;
+            rough = rough || row.rough;
+            if (!row.rough) {
+                top = max(top, row.top);
+                if (row.top) least = min(least, row.top);
+            }
+            fx r[2][3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                if (l == 0) N[b].m[0][k] = row[b][k];
-                else if (l == 1) N[b].m[1][k] = row[b][k];
-                else N[b].m[2][k] = row[b][k];
+                const long long bk = l == 1 ? -f[k] : f[k];
+                fxa u = {0, 0}, d = {0, 0};
+                fx_mac(u, fx_split((e[k] + bk) >> 3), X.kappa);
+                fx_mac(d, fx_split((bk - e[k]) >> 3), X.kappa);
+                r[0][k] = fx_of(u);
+                r[1][k] = fx_of(d);
             }
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    if (l == 0) N[b].m[0][k] = r[b][k];
+                    else if (l == 1) N[b].m[1][k] = r[b][k];
+                    else N[b].m[2][k] = r[b][k];
+                }
+        }
+        const bool units = !SLAB || rough; // digits in units of 1 are what there is
+        if (least != 0xffffffffu && least + (8u << 20) < (units ? kFxHigh1 : top)) ok = false;
+        if (!ok || units || top == 0 || E < 1022) break;
+        E = (int)(top >> 20) + 2; // below 1/4: a site sums eight of them
+        if (E >= 1022) {
+            E = 1022;
+            break;
+        }
+        if (E < 1022 - 40) {
+            ok = false;
+            break;
+        }
     }
+    const int ks = 1022 - E + X.kk, k1 = min(ks, 63), k2 = min(2 * ks, 63), k3 = min(3 * ks, 63), k4 = min(4 * ks, 63);
     const long long one = 1LL << 56;
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
@@ -579,8 +629,8 @@ __global__ void __launch_bounds__(64, 6) k_clover_build_fx(BuildArgs B, BuildFx 
                 fx_mac(s, fx_neg(n.m[r1][c2]), n.m[r2][c1]);
                 K.m[r][c] = fx_of(s);
             }
-        const long long tt = fx_round(ta);
-        if (tt > (EXP ? one / 3 : one)) ok = false;
+        const long long ts = fx_round(ta), tt = ts >> k2;
+        if (ts > one || (EXP && tt > one / 3)) ok = false;
         fx S[3][3]; // N N^T (symmetric)
 #pragma unroll
         for (int r = 0; r < 3; ++r)
@@ -604,10 +654,19 @@ __global__ void __launch_bounds__(64, 6) k_clover_build_fx(BuildArgs B, BuildFx 
 #pragma unroll
         for (int c = 0; c < 3; ++c) fx_mac(da, n.m[0][c], K.m[0][c]);
         const fx td = fx_split(tt);
-        const long long dt = fx_round(da);
-        fxa qa = {-4 * ka.a, -4 * ka.b};
+        const long long dt = fx_round(da) >> k3;
+        fxa qa = {-((4 * fx_round(ka)) >> k4), 0};
         fx_mac(qa, td, td);
         const long long qt = fx_round(qa);
+        if (ks) { // K and L in N's units
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    K.m[r][c] = fx_split(fx_units64(K.m[r][c]) >> k1);
+                    L.m[r][c] = fx_split(fx_units64(L.m[r][c]) >> k2);
+                }
+        }
         // coefficients of 1, X, X^2, X^3 of A / a and A^-1 a (clover: times D)
         FxMat P, Q;
         long long u, v;
@@ -685,9 +744,9 @@ __global__ void __launch_bounds__(64, 6) k_clover_build_fx(BuildArgs B, BuildFx 
             ks_inv = fx_float((unsigned)(127 + min(max(k, -60), 60)) << 23);
         }
         float2 out[16];
-        block_pairs(u, P, X.am, X.ka, out);
+        block_pairs(u, P, ks, X.am, X.ka, out);
         store_block<CP>(B.half[p], i, b, out);
-        block_pairs(v, Q, sc_inv, ks_inv, out);
+        block_pairs(v, Q, ks, sc_inv, ks_inv, out);
         store_block<CP>(B.half[2 + p], i, b, out);
     }
     if (!ok) atomicOr(B.bad, kBuildOutside);
@@ -714,7 +773,10 @@ void launch_build_fx(hr_ctx *ctx, const BuildArgs &B, double a, cudaStream_t s)
     BuildFx X;
     int k;
     const double am = 2.0 * std::frexp(a, &k); // [1, 2)
-    X.kappa = fx_from_double(B.csw / a);
+    int e;
+    std::frexp(B.csw / a, &e);
+    X.kk = std::max(0, -3 - e); // from 1/16 on as it is, smaller ones between 1/16 and 1/8
+    X.kappa = fx_from_double(std::ldexp(B.csw / a, X.kk));
     X.am = fx_from_double(am);
     X.ka = std::ldexp(1.f, k - 1);
     X.inva = 1.0 / a;
@@ -856,7 +918,8 @@ hr_status hr_clover_build(hr_ctx *ctx, hr_lattice lat, hr_rep rep, hr_prec prec,
     const bool three = rep_nc(rep) == 3;
     // fixed point: fundamental links, 0 < a and |c_sw / a| within the digits' range
     const double a = 4.0 + m0;
-    bool fixed = !three && a > 0x1p-20 && a < 0x1p20 && std::fabs(c_sw) < 2.0 * a;
+    bool fixed = !three && a > 0x1p-20 && a < 0x1p20 && std::fabs(c_sw) < 2.0 * a &&
+                 (c_sw == 0.0 || std::fabs(c_sw) > 0x1p-40 * a);
     unsigned bad = 0;
     for (;;) {
         cudaError_t e = cudaMemsetAsync(B.bad, 0, sizeof(unsigned), s);

@@ -141,14 +141,32 @@ struct PlaqVecs {
     const int2 *b;
     int n;
 };
-__device__ __forceinline__ bool load_plaq(const PlaqVecs &P, int plane, int slot, fx (&v)[3])
+// what the vectors of a sum were
+struct PlaqKinds {
+    bool bad = false;   // one is out of range
+    bool rough = false; // one is digits: links away from the identity
+    unsigned top = 0;   // high word of the largest number among the doubles
+};
+// A vector as digits, doubles in units of 2^(E - 1022) (E = 1022 beside vectors in digits)
+__device__ __forceinline__ void load_plaq(const PlaqVecs &P, int plane, int slot, int E, fx (&v)[3], PlaqKinds &kinds)
 {
     const int4 a = __ldg(P.a + (size_t)plane * P.n + slot);
     const int2 b = __ldg(P.b + (size_t)plane * P.n + slot);
     v[0] = {a.x, a.y};
     v[1] = {a.z, a.w};
     v[2] = {b.x, b.y};
-    return !plaq_marked(a.x);
+    if (!plaq_marked(a.x)) {
+        kinds.rough = true;
+    } else if (a.x == kPlaqBad) {
+        kinds.bad = true;
+    } else {
+        const PlaqVec d = plaq_doubles(a, b);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            kinds.top = max(kinds.top, fx_abs_high(d.v[k]));
+            v[k] = fx_from_double(d.v[k], E);
+        }
+    }
 }
 
 // A link that transports vectors: with u its vector part, t = u x v and d = |U|^2 - 1,
