@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(128, DIG ? 5 : 3) k_link_deriv_fx(ForceArgs A,
         const unsigned long long us2 = fx_used(g2[0]) | fx_used(g2[1]) | fx_used(g2[2]) | fx_used(g2[3]);
         const int s1 = fx_block_shift(us1), s2 = fx_block_shift(us2);
         const int e1 = us1 ? ea + ebf - 2 * kFxPairBias - s1 : -4096, e2 = us2 ? eaf + eb - 2 * kFxPairBias - s2 : -4096;
-        const int e = max(max(e1, e2), -900);
+        const int e = max(max(e1, e2), -500); // (two zero sums; any others are far above)
         const int d1 = min(e - e1, 63), d2 = min(e - e2, 63);
         long long G[4];
 #pragma unroll
