@@ -260,6 +260,9 @@ BatchPlan plan_batch(int n, const hr_lattice *lats, int rep)
     return P;
 }
 
+// (early starts whatever the size: a batch above launch_after's line of 2^20 sites does not
+// lose by them -- 24 iterations of 16 x 24^4, 2.7 M even sites, 52.90 ms with and 52.92
+// without, of 16 x 32^4, 8.4 M, 163.88 and 163.93)
 template <int REP>
 hr_status batch_launch_iteration(hr_ctx *ctx, const BatchArgs &B, int grid, cudaStream_t s)
 {

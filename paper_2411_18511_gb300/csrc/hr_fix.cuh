@@ -4,18 +4,24 @@
 // GB300 executes native FP64 at 1.7 lane operations per clock and SM and an
 // FP64 <-> FP32 conversion at 2.0 (measured; FP32 FMA 124, 32-bit integer
 // multiply-add 64, 32 x 32 + 64 bit multiply-add about 30), so the kernels that
-// must not lose a bit against binary64 -- link derivatives, staples, the clover
-// field strength -- were bound by the FP64 pipe at 3 to 5 % of the memory rate.
+// compute on canonical doubles -- link derivatives, staples, the clover field
+// strength -- were bound by the FP64 pipe at 3 to 5 % of the memory rate.
 // Double-float pairs (48 bits) would be fast enough but less accurate.  A
 // number here is
-//   v = h 2^-28 + l 2^-56,   h, l int,  |l| <= about 2^27,
-// in units of a power of two chosen per link or per spinor: 57 bits below the
-// largest component of the block.  A product of two numbers is three
-// 32 x 32 -> 64 bit multiply-adds (the l l' term, below 2^-58, is dropped)
-// into two 64-bit sums that need no normalisation and no rounding:
-//   a += h h' (units 2^-56),  b += h l' + l h' (units 2^-84).
-// That is about 0.1 clocks per SM and term against 0.59 for a DFMA, with a
-// smaller error: a sum is exact until its one rounding at 2^-57.
+//   v = h 2^-28 + l 2^-56,   h, l int,
+// in units of a power of two that the caller chooses: an absolute accuracy of
+// 2^-56 of that unit, better than binary64's for numbers near it and worse for
+// numbers below about 2^-3 of it.  Callers whose results can be that small (vector
+// parts of links near the identity, sums that cancel) take a smaller unit or native
+// FP64.  |l| <= 2^27 from the conversions that split at the middle (fx_split,
+// fx_from_double, fx_from_pair: a little more), < 2^28 with the sign of v from
+// fx_from_unit, which cuts.  A product of two numbers is three 32 x 32 -> 64 bit
+// multiply-adds into two 64-bit sums that need no normalisation and no rounding:
+//   a += h h' (units 2^-56),  b += h l' + l h' (units 2^-84);
+// the dropped l l' is below 2^-58 for split digits, below 2^-56 and of the
+// product's sign for cut ones (|q|^2 of a unit quaternion: off by at most 4.4 2^-56,
+// 1.3 2^-56 on average).  That is about 0.1 clocks per SM and term against 0.59
+// for a DFMA; a sum is otherwise exact until its one rounding at 2^-57.
 // Callers guarantee the ranges (stated per function); blocks outside them
 // (Inf, NaN, links far from unit length) take native FP64.
 #pragma once
