@@ -127,18 +127,18 @@ HR_HD inline double fx_to_double(long long t, int k = 0)
     const double d = (double)t;
     return t ? fx_double(fx_dbits(d) - ((unsigned long long)(unsigned)(56 + k) << 52)) : 0.0;
 }
-// t 2^-56 (|t| < 2^59) as a normalised float pair, to 2^-49 of the value: three
-// 22-bit pieces made floats through the mantissa field, then two Fast2Sums
+// t 2^-56 (|t| < 2^59) as a normalised float pair: three 22-bit pieces made floats
+// through the mantissa field, summed without loss until the low part is rounded, so
+// the pair carries 2^-49 of the value, as one split from a double does
 HR_HD inline void fx_to_pair(long long t, float &hi, float &lo)
 {
     const float f2 = fx_sub(fx_float(0x4b400000u + (unsigned)(int)(t >> 44)), 12582912.f);
     const float f1 = fx_sub(fx_float(0x4b000000u | ((unsigned)(t >> 22) & 0x3fffffu)), 8388608.f);
     const float f0 = fx_sub(fx_float(0x4b000000u | ((unsigned)t & 0x3fffffu)), 8388608.f);
     const float a = fx_mul(f2, 0x1p-12f), b = fx_mul(f1, 0x1p-34f), c = fx_mul(f0, 0x1p-56f);
-    const float s = fx_add(a, b);
-    const float w = fx_add(fx_sub(b, fx_sub(s, a)), c);
-    hi = fx_add(s, w);
-    lo = fx_sub(w, fx_sub(hi, s));
+    const float s = fx_add(a, b), e = fx_sub(b, fx_sub(s, a)); // a + b = s + e
+    hi = fx_add(s, fx_add(e, c));
+    lo = fx_add(fx_sub(e, fx_sub(hi, s)), c); // (one rounding, of the low part)
 }
 // 2^k as a double, -1022 <= k <= 1023
 HR_HD inline double fx_pow2(int k) { return fx_double((unsigned long long)(unsigned)(k + 1023) << 52); }
