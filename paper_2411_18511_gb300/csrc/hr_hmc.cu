@@ -182,18 +182,8 @@ __global__ void __launch_bounds__(128, 5) k_plaq_force(Geom g, double s, const d
         if (NMU == 1 && nu == (int)blockIdx.y) continue;
         int unused, down;
         lex_steps(g, x, nu, unused, down);
-        const fxq U = load_fxq<VEC>(q, (size_t)nu * V + t + down, ok);
-        fxa nn = {-(1LL << 56), 0};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) fx_mac(nn, U.c[k], U.c[k]);
-        const long long d = fx_round(nn);
-        ok = ok && d < (1 << 27) && d > -(1 << 27);
-        const fx u[3] = {U.c[1], U.c[2], U.c[3]};
-        fx w[4]; // 2 u (1 - d)
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            w[k] = {2 * U.c[k].h, 2 * (U.c[k].l - (int)(((long long)U.c[k].h * (int)d) >> 28))};
-        const fx wv[3] = {w[1], w[2], w[3]};
+        const Transport T = make_transport(load_fxq<VEC>(q, (size_t)nu * V + t + down, ok), ok);
+        const fx wv[3] = {T.w[1], T.w[2], T.w[3]};
         // y's vectors: the slab's first slice is the one before its first site's, unless it is the whole lattice
         const int low = nu == 0 && x.x0 > first ? own - slice : own + down;
 #pragma unroll
@@ -206,7 +196,7 @@ __global__ void __launch_bounds__(128, 5) k_plaq_force(Geom g, double s, const d
             ok = ok && !plaq_marked(oa.x) && !plaq_marked(ya.x);
             const fx v[3] = {{ya.x, ya.y}, {ya.z, ya.w}, {yb.x, yb.y}};
             fxa tc[3] = {};
-            fx_mac_cross(tc, u, v);
+            fx_mac_cross(tc, T.u, v);
             // + (P(x) - rotated P(y)) for mu < nu, - for mu > nu
             const int sg = mu < nu ? 1 : -1;
             const fx o[3] = {{oa.x, oa.y}, {oa.z, oa.w}, {ob.x, ob.y}};
@@ -217,7 +207,7 @@ __global__ void __launch_bounds__(128, 5) k_plaq_force(Geom g, double s, const d
                 const fx tt = fx_of(tc[a]), df = fx_sub(o[a], v[a]);
                 tn[a] = {-sg * tt.h, -sg * tt.l};
                 acc[a] = {fx_units64({sg * df.h, sg * df.l}), 0};
-                fx_mac(acc[a], w[0], tn[a]);
+                fx_mac(acc[a], T.w[0], tn[a]);
             }
             fx_mac_cross(acc, wv, tn);
 #pragma unroll

@@ -33,8 +33,6 @@ template <int REP, int PREC, int G5IN, bool CLOV = false>
 __device__ __forceinline__ void hop_body(const HopArgs &a)
 {
     using T = typename PrecTraits<PREC>::T;
-    // nothing to do (gated off, or the solver converged); a reducing launch
-    // leaves its counter clean because no block reaches the reduction
     if (hop_skipped(a)) return;
     const Geom &g = a.g;
     const int nv = g.vh << g.lrhs;
@@ -94,7 +92,10 @@ __global__ void __maxnreg__(96) k_hop_clov_r96(HopArgs a)
 //                      32^4 124.3 (12@128 133.8); stored matrices 24^4 70.6 -> 43.5 (10@64 51.2)
 //   fundamental FP32   8^4 3.1 -> 2.1, 16^4 4.5 -> 3.7, 24^4 8.5 -> 7.9
 //   binary16           8^4 2.2 (7@64 2.3), 16^4 2.93 -> 2.84, 24^4 7.5 -> 7.1, 32^4 21.4 -> 20.3
-// The adjoint in FP32 and binary16 has the plain kernel only.
+// The adjoint in FP32 and binary16 has the plain kernel only.  Measured with one
+// right-hand side; with several only the virtual sites count (16 of them on
+// 26 x 22 x 18 x 20, FP32 inner: 24.0 -> 23.5 ms for the solve against the plain
+// kernel), and the kernels that serve several at once (variants 20, 21) are the tuner's.
 inline HopChoice default_choice(const Geom &g, int rep, int prec)
 {
     const long long nv = (long long)g.vh << g.lrhs;
