@@ -541,19 +541,19 @@ __device__ __forceinline__ void x2a_compute(const K2 &k, const float4 (&w)[12], 
     x2a_rebuild<D, F, FIRST, 2>(k, r, acc);
 }
 
-template <int REP>
+template <int REP, bool NC>
 __device__ __forceinline__ void x2a_link(const HopArgs &a, const K2 &k, int link_par, int mu, int site_link,
                                          dd (&R)[3][3])
 {
     if constexpr (REP == kRepAdj) {
         const float4 *q = link_base<float4>(a.gauge, a.g.nblk_g, link_par, mu, 2) + vec_index(site_link, 0, 2);
-        quat_to_adj_x2(k, ld_field(q), ld_field(q + 32), R);
+        quat_to_adj_x2(k, ld_link<NC>(q), ld_link<NC>(q + 32), R);
     } else {
-        load_mat<kF64>(a.gauge, a.g.nblk_g, link_par, mu, site_link, R);
+        load_mat<kF64, NC>(a.gauge, a.g.nblk_g, link_par, mu, site_link, R);
     }
 }
 
-template <int MU, bool FWD, bool FIRST, bool NEG, int REP>
+template <int MU, bool FWD, bool FIRST, bool NEG, int REP, bool NC>
 __device__ __forceinline__ void x2a_term(const HopArgs &a, const K2 &k, int site_link, int link_par, int j_nb,
                                          dd2 (&acc)[4][3])
 {
@@ -562,7 +562,7 @@ __device__ __forceinline__ void x2a_term(const HopArgs &a, const K2 &k, int site
 #pragma unroll
     for (int v = 0; v < 12; ++v) w[v] = ld_field(sp + vec_index(j_nb, v, 12));
     dd R[3][3];
-    x2a_link<REP>(a, k, link_par, MU, site_link, R);
+    x2a_link<REP, NC>(a, k, link_par, MU, site_link, R);
     x2a_compute<MU, FWD, FIRST, NEG>(k, w, R, acc);
 }
 
@@ -577,7 +577,7 @@ __device__ __forceinline__ void x2a_epilogue(const HopArgs &a, int j, const dd2 
     hop_epilogue<kF64>(a, j, o, al, be, bu, red);
 }
 
-template <int REP, int G5IN>
+template <int REP, int G5IN, bool NC>
 __device__ __forceinline__ void x2a_body(const HopArgs &a)
 {
     constexpr bool NEG = G5IN != 0;
@@ -596,14 +596,14 @@ __device__ __forceinline__ void x2a_body(const HopArgs &a)
         SiteNb nb;
         site_neighbours(g, i, a.p, nb);
         dd2 acc[4][3];
-        x2a_term<0, true, true, NEG, REP>(a, k, i, a.p, (nb.fwd[0] << l) + rr, acc);
-        x2a_term<0, false, false, NEG, REP>(a, k, nb.bwd[0], 1 - a.p, (nb.bwd[0] << l) + rr, acc);
-        x2a_term<1, true, false, NEG, REP>(a, k, i, a.p, (nb.fwd[1] << l) + rr, acc);
-        x2a_term<1, false, false, NEG, REP>(a, k, nb.bwd[1], 1 - a.p, (nb.bwd[1] << l) + rr, acc);
-        x2a_term<2, true, false, NEG, REP>(a, k, i, a.p, (nb.fwd[2] << l) + rr, acc);
-        x2a_term<2, false, false, NEG, REP>(a, k, nb.bwd[2], 1 - a.p, (nb.bwd[2] << l) + rr, acc);
-        x2a_term<3, true, false, NEG, REP>(a, k, i, a.p, (nb.fwd[3] << l) + rr, acc);
-        x2a_term<3, false, false, NEG, REP>(a, k, nb.bwd[3], 1 - a.p, (nb.bwd[3] << l) + rr, acc);
+        x2a_term<0, true, true, NEG, REP, NC>(a, k, i, a.p, (nb.fwd[0] << l) + rr, acc);
+        x2a_term<0, false, false, NEG, REP, NC>(a, k, nb.bwd[0], 1 - a.p, (nb.bwd[0] << l) + rr, acc);
+        x2a_term<1, true, false, NEG, REP, NC>(a, k, i, a.p, (nb.fwd[1] << l) + rr, acc);
+        x2a_term<1, false, false, NEG, REP, NC>(a, k, nb.bwd[1], 1 - a.p, (nb.bwd[1] << l) + rr, acc);
+        x2a_term<2, true, false, NEG, REP, NC>(a, k, i, a.p, (nb.fwd[2] << l) + rr, acc);
+        x2a_term<2, false, false, NEG, REP, NC>(a, k, nb.bwd[2], 1 - a.p, (nb.bwd[2] << l) + rr, acc);
+        x2a_term<3, true, false, NEG, REP, NC>(a, k, i, a.p, (nb.fwd[3] << l) + rr, acc);
+        x2a_term<3, false, false, NEG, REP, NC>(a, k, nb.bwd[3], 1 - a.p, (nb.bwd[3] << l) + rr, acc);
         x2a_epilogue(a, j, acc, al, be, bu, red);
     }
     if (a.fin) block_partials(red, g.nrhs, a.partials);
@@ -672,11 +672,14 @@ __device__ __forceinline__ void x2as_body(const HopArgs &a)
     if (a.fin) block_partials(red, g.nrhs, a.partials);
 }
 
-template <int REP, int G5IN> __global__ void __maxnreg__(128) k_hop_x2a(HopArgs a) { x2a_body<REP, G5IN>(a); }
+// NC: launches without an early start (more than kEarlySites virtual sites) read the
+// links with ld.global.nc, which saves spills and waits: tuned at 48^4, adjoint 592 -> 551
+// us, stored matrices 573 -> 559 (spinors too: 569 and 555)
+template <int REP, int G5IN, bool NC> __global__ void __maxnreg__(128) k_hop_x2a(HopArgs a) { x2a_body<REP, G5IN, NC>(a); }
 // the same with up to 168 registers: no spills (the 128-register form spills
 // about 100 bytes a thread for the quaternion links), 12 warps an SM at
 // blocks of 64, 128 or 192 threads
-template <int REP, int G5IN> __global__ void __maxnreg__(168) k_hop_x2a_big(HopArgs a) { x2a_body<REP, G5IN>(a); }
+template <int REP, int G5IN, bool NC> __global__ void __maxnreg__(168) k_hop_x2a_big(HopArgs a) { x2a_body<REP, G5IN, NC>(a); }
 template <int G5IN> __global__ void __launch_bounds__(256) k_hop_x2as(HopArgs a) { x2as_body<G5IN>(a); }
 
 template <int REP, int PREC> struct Launch {
@@ -704,10 +707,12 @@ template <int REP, int PREC> struct Launch {
         } else if constexpr (PREC == kF64) {
             // adjoint (quaternion or stored 3x3 links): (re, im) lanes
             if (c.variant != kVarPaired && c.variant != kVarPairedStaged && c.variant != kVarPairedR96) return false;
-            const bool g5 = a.g5_in != 0;
+            const bool g5 = a.g5_in != 0, nc = !hop_early(a);
             if (c.variant == kVarPairedR96) {
                 // for the adjoint: the form with 168 registers
-                launch_after(g5 ? k_hop_x2a_big<REP, 1> : k_hop_x2a_big<REP, 0>, hop_early(a), grid, c.block, 0, s, a);
+                launch_after(nc ? (g5 ? k_hop_x2a_big<REP, 1, true> : k_hop_x2a_big<REP, 0, true>)
+                                : (g5 ? k_hop_x2a_big<REP, 1, false> : k_hop_x2a_big<REP, 0, false>),
+                             !nc, grid, c.block, 0, s, a);
                 st = hop_launched(ctx, a, grid, s, "paired adjoint hop kernel (168 registers)");
                 return true;
             }
@@ -726,7 +731,9 @@ template <int REP, int PREC> struct Launch {
                     return true;
                 }
             }
-            launch_after(g5 ? k_hop_x2a<REP, 1> : k_hop_x2a<REP, 0>, hop_early(a), grid, c.block, 0, s, a);
+            launch_after(nc ? (g5 ? k_hop_x2a<REP, 1, true> : k_hop_x2a<REP, 0, true>)
+                            : (g5 ? k_hop_x2a<REP, 1, false> : k_hop_x2a<REP, 0, false>),
+                         !nc, grid, c.block, 0, s, a);
             st = hop_launched(ctx, a, grid, s, "paired adjoint hop kernel");
             return true;
         } else if constexpr (REP == kRepFund) {

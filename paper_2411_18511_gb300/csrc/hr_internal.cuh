@@ -316,6 +316,13 @@ __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.
 // a vector of a field or of links: a plain load, not ld.global.nc -- a kernel may
 // be resident while the one before it still writes them
 template <class V> __device__ __forceinline__ V ld_field(const V *p) { return *p; }
+// the same for links in a kernel that starts after the previous one (NC): as ld.global.nc
+// the compiler may place, and repeat, the load where it likes
+template <bool NC, class V> __device__ __forceinline__ V ld_link(const V *p)
+{
+    if constexpr (NC) return __ldg(p);
+    else return *p;
+}
 
 // ---------------------------------------------------------------- layouts
 
@@ -744,7 +751,7 @@ template <int PREC> struct GaugeMat {
     }
 };
 
-template <int PREC, class T>
+template <int PREC, bool NC = false, class T>
 __device__ __forceinline__ void load_mat(const void *base, int nblk_g, int p, int mu, int i, T (&R)[3][3])
 {
 #pragma unroll
@@ -752,11 +759,11 @@ __device__ __forceinline__ void load_mat(const void *base, int nblk_g, int p, in
         const int idx = vec_index(i, e, 9);
         T v;
         if constexpr (PREC == kF64) {
-            float2 w = ld_field(link_base<float2>(base, nblk_g, p, mu, 9) + idx);
+            float2 w = ld_link<NC>(link_base<float2>(base, nblk_g, p, mu, 9) + idx);
             if constexpr (std::is_same<T, dd>::value) v = dd(w.x, w.y);
             else v = Real<T>::from_double(dd_to_double(dd(w.x, w.y)));
         } else if constexpr (PREC == kF32) {
-            v = Real<T>::from_float(ld_field(link_base<float>(base, nblk_g, p, mu, 9) + idx));
+            v = Real<T>::from_float(ld_link<NC>(link_base<float>(base, nblk_g, p, mu, 9) + idx));
         } else {
             v = Real<T>::from_float(__half2float(link_base<__half>(base, nblk_g, p, mu, 9)[idx]));
         }
