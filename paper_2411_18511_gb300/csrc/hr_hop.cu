@@ -93,9 +93,8 @@ __global__ void __maxnreg__(96) k_hop_clov_r96(HopArgs a)
 //   fundamental FP32   8^4 3.1 -> 2.1, 16^4 4.5 -> 3.7, 24^4 8.5 -> 7.9
 //   binary16           8^4 2.2 (7@64 2.3), 16^4 2.93 -> 2.84, 24^4 7.5 -> 7.1, 32^4 21.4 -> 20.3
 // The adjoint in FP32 and binary16 has the plain kernel only.  Measured with one
-// right-hand side; with several only the virtual sites count (16 of them on
-// 26 x 22 x 18 x 20, FP32 inner: 24.0 -> 23.5 ms for the solve against the plain
-// kernel), and the kernels that serve several at once (variants 20, 21) are the tuner's.
+// right-hand side; with several only the virtual sites count, and the kernels that
+// serve several at once (variants 20, 21) are the tuner's to choose.
 inline HopChoice default_choice(const Geom &g, int rep, int prec)
 {
     const long long nv = (long long)g.vh << g.lrhs;
@@ -112,13 +111,13 @@ template <int REP, int PREC> struct PlainLaunch {
     static bool run(hr_ctx *ctx, const HopArgs &a, HopChoice c, int grid, cudaStream_t s, hr_status &st)
     {
         if (c.variant == kVarSimpleR96) {
-            if (a.g5_in) launch_after(k_hop_r96<REP, PREC, 1>, hop_early(a), grid, c.block, 0, s, a);
-            else launch_after(k_hop_r96<REP, PREC, 0>, hop_early(a), grid, c.block, 0, s, a);
+            if (a.g5_in) launch_reducible(ctx, k_hop_r96<REP, PREC, 1>, a, hop_early(a), grid, c.block, 0, s);
+            else launch_reducible(ctx, k_hop_r96<REP, PREC, 0>, a, hop_early(a), grid, c.block, 0, s);
             st = hop_launched(ctx, a, grid, s, "hop kernel (96 registers)");
             return true;
         }
-        if (a.g5_in) launch_after(k_hop<REP, PREC, 1>, hop_early(a), grid, c.block, 0, s, a);
-        else launch_after(k_hop<REP, PREC, 0>, hop_early(a), grid, c.block, 0, s, a);
+        if (a.g5_in) launch_reducible(ctx, k_hop<REP, PREC, 1>, a, hop_early(a), grid, c.block, 0, s);
+        else launch_reducible(ctx, k_hop<REP, PREC, 0>, a, hop_early(a), grid, c.block, 0, s);
         st = hop_launched(ctx, a, grid, s, "hop kernel");
         return true;
     }
@@ -128,10 +127,10 @@ template <int REP, int PREC> struct ClovLaunch {
     static bool run(hr_ctx *ctx, const HopArgs &a, int grid, int block, cudaStream_t s, hr_status &st)
     {
         if constexpr (PREC == kF64)
-            launch_after(a.g5_in ? k_hop_clov<REP, PREC, 1> : k_hop_clov<REP, PREC, 0>, hop_early(a), grid, block, 0, s, a);
+            launch_reducible(ctx, a.g5_in ? k_hop_clov<REP, PREC, 1> : k_hop_clov<REP, PREC, 0>, a, hop_early(a), grid, block, 0, s);
         else
-            launch_after(a.g5_in ? k_hop_clov_r96<REP, PREC, 1> : k_hop_clov_r96<REP, PREC, 0>, hop_early(a), grid, block,
-                         0, s, a);
+            launch_reducible(ctx, a.g5_in ? k_hop_clov_r96<REP, PREC, 1> : k_hop_clov_r96<REP, PREC, 0>, a, hop_early(a), grid, block,
+                         0, s);
         st = hop_launched(ctx, a, grid, s, "hop kernel (clover epilogue)");
         return true;
     }
@@ -200,7 +199,7 @@ bool is_pow2(double x)
     return m == 0.5;
 }
 
-HopArgs make_args(hr_ctx *ctx, const Geom &g, const HopLaunch &L)
+HopArgs make_args(hr_ctx *ctx, const Geom &g, int prec, const HopLaunch &L)
 {
     HopArgs a;
     a.g = g;
@@ -231,6 +230,7 @@ HopArgs make_args(hr_ctx *ctx, const Geom &g, const HopLaunch &L)
     a.cond = L.cond;
     a.leave = L.leave;
     a.joined = L.joined;
+    a.prec = prec;
     return a;
 }
 
@@ -264,13 +264,13 @@ HopChoice hop_choice_fin(hr_ctx *ctx, const Geom &g, int rep, int prec)
 hr_status launch_hop(hr_ctx *ctx, const Geom &g, int rep, int prec, const HopLaunch &L, cudaStream_t s)
 {
     const HopChoice c = L.fin != kFinNone ? hop_choice_fin(ctx, g, rep, prec) : hop_choice(ctx, g, rep, prec);
-    return dispatch(ctx, g, rep, prec, make_args(ctx, g, L), c, s);
+    return dispatch(ctx, g, rep, prec, make_args(ctx, g, prec, L), c, s);
 }
 
 hr_status launch_hop_with(hr_ctx *ctx, const Geom &g, int rep, int prec, const HopLaunch &L, HopChoice c,
                           cudaStream_t s)
 {
-    return dispatch(ctx, g, rep, prec, make_args(ctx, g, L), c, s);
+    return dispatch(ctx, g, rep, prec, make_args(ctx, g, prec, L), c, s);
 }
 
 bool hop_variant_available(int rep, int prec, int variant, int nrhs)

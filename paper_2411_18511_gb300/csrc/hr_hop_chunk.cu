@@ -122,11 +122,11 @@ template <int PREC, int LC, int G5IN> __global__ void __launch_bounds__(256) k_h
 }
 
 template <int PREC>
-void launch_chunk(const HopArgs &a, int lc, int grid, int block, cudaStream_t s)
+void launch_chunk(hr_ctx *ctx, const HopArgs &a, int lc, int &grid, int block, cudaStream_t s)
 {
     const bool g5 = a.g5_in != 0;
-    if (lc == 1) launch_after(g5 ? k_hop_chunk<PREC, 1, 1> : k_hop_chunk<PREC, 1, 0>, hop_early(a), grid, block, 0, s, a);
-    else launch_after(g5 ? k_hop_chunk<PREC, 2, 1> : k_hop_chunk<PREC, 2, 0>, hop_early(a), grid, block, 0, s, a);
+    if (lc == 1) launch_reducible(ctx, g5 ? k_hop_chunk<PREC, 1, 1> : k_hop_chunk<PREC, 1, 0>, a, hop_early(a), grid, block, 0, s, 2);
+    else launch_reducible(ctx, g5 ? k_hop_chunk<PREC, 2, 1> : k_hop_chunk<PREC, 2, 0>, a, hop_early(a), grid, block, 0, s, 4);
 }
 
 } // namespace
@@ -141,9 +141,9 @@ bool launch_hop_chunk(hr_ctx *ctx, const Geom &g, int rep, int prec, const HopAr
     // vals[] of the reduction holds blockDim x C doubles; whole warps
     if (c.block > 256 || c.block < 32 || (c.block & 31)) return false;
     const long long nt = (long long)g.vh << (g.lrhs - lc);
-    const int grid = hop_grid(a, nt, c.block);
-    if (prec == kF32) launch_chunk<kF32>(a, lc, grid, c.block, s);
-    else launch_chunk<kF16>(a, lc, grid, c.block, s);
+    int grid = hop_grid(a, nt, c.block);
+    if (prec == kF32) launch_chunk<kF32>(ctx, a, lc, grid, c.block, s);
+    else launch_chunk<kF16>(ctx, a, lc, grid, c.block, s);
     st = hop_launched(ctx, a, grid, s, "right-hand-side chunk hop kernel");
     return true;
 }

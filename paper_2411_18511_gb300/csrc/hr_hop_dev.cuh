@@ -4,6 +4,8 @@
 // and the epilogue out = alpha aux + beta [g5] H [g5] in with the fused |out|^2.
 #pragma once
 
+#include <algorithm>
+
 #include "hr_clover.cuh"
 #include "hr_host.h"
 
@@ -37,6 +39,7 @@ struct HopArgs {
     FinCond cond;          // host side: condition handle the finishing launch sets,
     int leave;             // who finishes (LeaveRows),
     int joined;            // the launch follows two others
+    int prec;              // of the fields
 };
 
 // Waits for the launches before; nothing to do when gated off, or the solver
@@ -53,6 +56,26 @@ inline bool hop_early(const HopArgs &a) { return !a.joined && early_start(a.g); 
 inline int hop_grid(const HopArgs &a, long long n, int block)
 {
     return grid_for(n, block, a.fin ? kMaxPartials / a.g.nrhs : (1 << 30));
+}
+// Launch a hop kernel; `grid` becomes the number of blocks that ran.  A reducing launch
+// that the scratch cuts (more blocks than kMaxPartials / n_rhs rows: many right-hand
+// sides) loops in any case, and in FP32 and binary16 it then runs the blocks that are
+// resident at once and no more: blocks at different turns of their loops share less
+// of L2, and fewer rows are to be added.  45 iterations, FP32 inner, tuned: 24^4 with 16
+// right-hand sides 34.7 -> 31.1 ms, 32^4 with 8 54.2 -> 50.1, 26 x 22 x 18 x 20 with 16
+// 21.1 -> 19.5; binary16 27.6 -> 26.1, 43.1 -> 41.1, 17.2 -> 16.9.  The FP64 kernels, bound
+// by the FP32 pipes, lose by it (24^4 with 16: 90.7 -> 97.6), and so may launches of
+// fewer turns (one right-hand side on 24^4, adjoint: 2.74 -> 2.89).
+template <class K>
+inline void launch_reducible(hr_ctx *ctx, K kernel, const HopArgs &a, bool early, int &grid, int block, size_t smem,
+                             cudaStream_t s, int sites = 1 /* of a thread and turn */)
+{
+    const long long rows = kMaxPartials / a.g.nrhs, nv = (long long)a.g.vh << a.g.lrhs;
+    int per = 0;
+    if (a.fin && a.prec != kF64 && nv > rows * block * sites &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, block, smem) == cudaSuccess && per > 0)
+        grid = std::min(grid, per * ctx->sm_count);
+    launch_after(kernel, early, grid, block, smem, s, a);
 }
 // after a hop kernel's launch: its error, and the finishing launch of a reducing one
 inline hr_status hop_launched(hr_ctx *ctx, const HopArgs &a, int grid, cudaStream_t s, const char *what)

@@ -241,16 +241,16 @@ bool launch_hop_half(hr_ctx *ctx, const Geom &, int rep, int prec, const HopArgs
             attr_set = true;
         }
         const size_t sm = S::smem_bytes(c.block);
-        if (c.variant == kVarHalfStagedR64) launch_after(g5 ? k_hop_h16s_r64<1> : k_hop_h16s_r64<0>, hop_early(a), grid, c.block, sm, s, a);
-        else launch_after(g5 ? k_hop_h16s<1> : k_hop_h16s<0>, hop_early(a), grid, c.block, sm, s, a);
+        if (c.variant == kVarHalfStagedR64) launch_reducible(ctx, g5 ? k_hop_h16s_r64<1> : k_hop_h16s_r64<0>, a, hop_early(a), grid, c.block, sm, s);
+        else launch_reducible(ctx, g5 ? k_hop_h16s<1> : k_hop_h16s<0>, a, hop_early(a), grid, c.block, sm, s);
     } else if (c.variant == kVarHalfR64) {
-        launch_after(g5 ? k_hop_h16_r64<1> : k_hop_h16_r64<0>, hop_early(a), grid, c.block, 0, s, a);
+        launch_reducible(ctx, g5 ? k_hop_h16_r64<1> : k_hop_h16_r64<0>, a, hop_early(a), grid, c.block, 0, s);
     } else if (c.variant == kVarHalfPrefetch) {
-        launch_after(g5 ? k_hop_h16p_r80<1> : k_hop_h16p_r80<0>, hop_early(a), grid, c.block, 0, s, a);
+        launch_reducible(ctx, g5 ? k_hop_h16p_r80<1> : k_hop_h16p_r80<0>, a, hop_early(a), grid, c.block, 0, s);
     } else if (c.variant == kVarHalfPrefetch2) {
-        launch_after(g5 ? k_hop_h16p2_r96<1> : k_hop_h16p2_r96<0>, hop_early(a), grid, c.block, 0, s, a);
+        launch_reducible(ctx, g5 ? k_hop_h16p2_r96<1> : k_hop_h16p2_r96<0>, a, hop_early(a), grid, c.block, 0, s);
     } else {
-        launch_after(g5 ? k_hop_h16<1> : k_hop_h16<0>, hop_early(a), grid, c.block, 0, s, a);
+        launch_reducible(ctx, g5 ? k_hop_h16<1> : k_hop_h16<0>, a, hop_early(a), grid, c.block, 0, s);
     }
     st = hop_launched(ctx, a, grid, s, "binary16 hop kernel (half2 projection)");
     return true;

@@ -328,7 +328,7 @@ template <int REP, int PREC> struct Launch {
             const size_t sm = Stage<REP, PREC>::smem_bytes(c.block);
             const int sm_max = (int)Stage<REP, PREC>::smem_bytes(256);
             if (c.variant == kVarLoop) {
-                launch_after(k_hop_loop<REP, PREC, false>, hop_early(a), grid, c.block, 0, s, a);
+                launch_reducible(ctx, k_hop_loop<REP, PREC, false>, a, hop_early(a), grid, c.block, 0, s);
                 st = hop_launched(ctx, a, grid, s, "looped hop kernel");
                 return true;
             }
@@ -339,12 +339,12 @@ template <int REP, int PREC> struct Launch {
                                          sm_max);
                     attr_set = true;
                 }
-                launch_after(k_hop_loop<REP, PREC, true>, hop_early(a), grid, c.block, sm, s, a);
+                launch_reducible(ctx, k_hop_loop<REP, PREC, true>, a, hop_early(a), grid, c.block, sm, s);
                 st = hop_launched(ctx, a, grid, s, "looped staged hop kernel");
                 return true;
             }
             if (c.variant == kVarSwitch) {
-                launch_after(k_hop_sw<REP, PREC, false>, hop_early(a), grid, c.block, 0, s, a);
+                launch_reducible(ctx, k_hop_sw<REP, PREC, false>, a, hop_early(a), grid, c.block, 0, s);
                 st = hop_launched(ctx, a, grid, s, "switched hop kernel");
                 return true;
             }
@@ -355,7 +355,7 @@ template <int REP, int PREC> struct Launch {
                                          sm_max);
                     attr_set2 = true;
                 }
-                launch_after(k_hop_sw<REP, PREC, true>, hop_early(a), grid, c.block, sm, s, a);
+                launch_reducible(ctx, k_hop_sw<REP, PREC, true>, a, hop_early(a), grid, c.block, sm, s);
                 st = hop_launched(ctx, a, grid, s, "switched staged hop kernel");
                 return true;
             }

@@ -214,11 +214,11 @@ template <int PREC, int G5IN> __global__ void __launch_bounds__(256) k_hop_p2(Ho
 template <int PREC, int G5IN> __global__ void __maxnreg__(96) k_hop_p2_r96(HopArgs a) { p2_body<PREC, G5IN>(a); }
 
 template <int PREC>
-void launch_p2(const HopArgs &a, HopChoice c, int grid, cudaStream_t s)
+void launch_p2(hr_ctx *ctx, const HopArgs &a, HopChoice c, int &grid, cudaStream_t s)
 {
     const bool g5 = a.g5_in != 0;
-    if (c.variant == kVarPairSitesR96) launch_after(g5 ? k_hop_p2_r96<PREC, 1> : k_hop_p2_r96<PREC, 0>, hop_early(a), grid, c.block, 0, s, a);
-    else launch_after(g5 ? k_hop_p2<PREC, 1> : k_hop_p2<PREC, 0>, hop_early(a), grid, c.block, 0, s, a);
+    if (c.variant == kVarPairSitesR96) launch_reducible(ctx, g5 ? k_hop_p2_r96<PREC, 1> : k_hop_p2_r96<PREC, 0>, a, hop_early(a), grid, c.block, 0, s, 2);
+    else launch_reducible(ctx, g5 ? k_hop_p2<PREC, 1> : k_hop_p2<PREC, 0>, a, hop_early(a), grid, c.block, 0, s, 2);
 }
 
 } // namespace
@@ -232,9 +232,9 @@ bool launch_hop_pair_sites(hr_ctx *ctx, const Geom &g, int rep, int prec, const 
     // one thread per pair of virtual sites
     const long long nv = (long long)g.vh << g.lrhs;
     const long long npairs = ((nv + 63) >> 6) << 5;
-    const int grid = hop_grid(a, npairs, c.block);
-    if (prec == kF32) launch_p2<kF32>(a, c, grid, s);
-    else launch_p2<kF16>(a, c, grid, s);
+    int grid = hop_grid(a, npairs, c.block);
+    if (prec == kF32) launch_p2<kF32>(ctx, a, c, grid, s);
+    else launch_p2<kF16>(ctx, a, c, grid, s);
     st = hop_launched(ctx, a, grid, s, "two-site hop kernel");
     return true;
 }

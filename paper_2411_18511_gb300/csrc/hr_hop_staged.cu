@@ -199,12 +199,12 @@ template <int REP, int PREC> struct Launch {
                                          (int)Stage<REP, PREC>::smem_bytes(256));
                     attr_set = true;
                 }
-                launch_after(k_hop_staged<REP, PREC>, hop_early(a), grid, c.block, sm, s, a);
+                launch_reducible(ctx, k_hop_staged<REP, PREC>, a, hop_early(a), grid, c.block, sm, s);
                 st = hop_launched(ctx, a, grid, s, "staged hop kernel");
                 return true;
             }
             if (c.variant == kVarPrefetch) {
-                launch_after(k_hop_pf<REP, PREC>, hop_early(a), grid, c.block, 0, s, a);
+                launch_reducible(ctx, k_hop_pf<REP, PREC>, a, hop_early(a), grid, c.block, 0, s);
                 st = hop_launched(ctx, a, grid, s, "prefetching hop kernel");
                 return true;
             }

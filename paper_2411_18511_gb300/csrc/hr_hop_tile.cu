@@ -176,13 +176,13 @@ template <int REP, int PREC> struct Launch {
             // one tile per block; a reducing launch loops over tiles within the partials' cap
             const long long nv = (long long)g.vh << g.lrhs;
             const long long ntiles = (nv + c.block - 1) / c.block;
-            const int tgrid = hop_grid(a, ntiles, 1);
+            int tgrid = hop_grid(a, ntiles, 1);
             if (c.variant == kVarTile) {
-                if (a.g5_in) launch_after(k_hop_tile<REP, PREC, 1>, hop_early(a), tgrid, c.block, sm, s, a);
-                else launch_after(k_hop_tile<REP, PREC, 0>, hop_early(a), tgrid, c.block, sm, s, a);
+                if (a.g5_in) launch_reducible(ctx, k_hop_tile<REP, PREC, 1>, a, hop_early(a), tgrid, c.block, sm, s);
+                else launch_reducible(ctx, k_hop_tile<REP, PREC, 0>, a, hop_early(a), tgrid, c.block, sm, s);
             } else {
-                if (a.g5_in) launch_after(k_hop_tile_r96<REP, PREC, 1>, hop_early(a), tgrid, c.block, sm, s, a);
-                else launch_after(k_hop_tile_r96<REP, PREC, 0>, hop_early(a), tgrid, c.block, sm, s, a);
+                if (a.g5_in) launch_reducible(ctx, k_hop_tile_r96<REP, PREC, 1>, a, hop_early(a), tgrid, c.block, sm, s);
+                else launch_reducible(ctx, k_hop_tile_r96<REP, PREC, 0>, a, hop_early(a), tgrid, c.block, sm, s);
             }
             st = hop_launched(ctx, a, tgrid, s, "tiled hop kernel");
             return true;

@@ -245,13 +245,13 @@ template <int REP, int PREC> struct TwistLaunch {
     {
         if constexpr (REP == kRepFund && PREC == kF64) {
             const bool g5 = a.g5_in != 0, clov = a.clov_mode != kClovNone;
-            if (clov) launch_after(g5 ? k_hop_x2t<1, true> : k_hop_x2t<0, true>, hop_early(a), grid, kTwistBlock, 0, s, a);
-            else launch_after(g5 ? k_hop_x2t<1, false> : k_hop_x2t<0, false>, hop_early(a), grid, kTwistBlock, 0, s, a);
+            if (clov) launch_reducible(ctx, g5 ? k_hop_x2t<1, true> : k_hop_x2t<0, true>, a, hop_early(a), grid, kTwistBlock, 0, s);
+            else launch_reducible(ctx, g5 ? k_hop_x2t<1, false> : k_hop_x2t<0, false>, a, hop_early(a), grid, kTwistBlock, 0, s);
             st = hop_launched(ctx, a, grid, s, "paired hop kernel (twisted boundaries)");
             return true;
         }
-        if (a.clov_mode != kClovNone) launch_after(k_hop_twist<REP, PREC, true>, hop_early(a), grid, kTwistBlock, 0, s, a);
-        else launch_after(k_hop_twist<REP, PREC, false>, hop_early(a), grid, kTwistBlock, 0, s, a);
+        if (a.clov_mode != kClovNone) launch_reducible(ctx, k_hop_twist<REP, PREC, true>, a, hop_early(a), grid, kTwistBlock, 0, s);
+        else launch_reducible(ctx, k_hop_twist<REP, PREC, false>, a, hop_early(a), grid, kTwistBlock, 0, s);
         st = hop_launched(ctx, a, grid, s, "hop kernel (twisted boundaries)");
         return true;
     }

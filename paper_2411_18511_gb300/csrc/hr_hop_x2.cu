@@ -697,10 +697,10 @@ template <int REP, int PREC> struct Launch {
             const size_t sm = S::smem_bytes(c.block);
             const bool g5 = a.g5_in != 0;
             switch (c.variant) {
-            case kVarPairedStaged: launch_after(g5 ? k_hop_x2s<1> : k_hop_x2s<0>, hop_early(a), grid, c.block, sm, s, a); break;
-            case kVarPairedStagedR96: launch_after(g5 ? k_hop_x2s_r96<1> : k_hop_x2s_r96<0>, hop_early(a), grid, c.block, sm, s, a); break;
-            case kVarPairedR96: launch_after(g5 ? k_hop_x2_r96<1> : k_hop_x2_r96<0>, hop_early(a), grid, c.block, 0, s, a); break;
-            default: launch_after(g5 ? k_hop_x2<1> : k_hop_x2<0>, hop_early(a), grid, c.block, 0, s, a); break;
+            case kVarPairedStaged: launch_reducible(ctx, g5 ? k_hop_x2s<1> : k_hop_x2s<0>, a, hop_early(a), grid, c.block, sm, s); break;
+            case kVarPairedStagedR96: launch_reducible(ctx, g5 ? k_hop_x2s_r96<1> : k_hop_x2s_r96<0>, a, hop_early(a), grid, c.block, sm, s); break;
+            case kVarPairedR96: launch_reducible(ctx, g5 ? k_hop_x2_r96<1> : k_hop_x2_r96<0>, a, hop_early(a), grid, c.block, 0, s); break;
+            default: launch_reducible(ctx, g5 ? k_hop_x2<1> : k_hop_x2<0>, a, hop_early(a), grid, c.block, 0, s); break;
             }
             st = hop_launched(ctx, a, grid, s, "paired hop kernel");
             return true;
@@ -710,9 +710,8 @@ template <int REP, int PREC> struct Launch {
             const bool g5 = a.g5_in != 0, nc = !hop_early(a);
             if (c.variant == kVarPairedR96) {
                 // for the adjoint: the form with 168 registers
-                launch_after(nc ? (g5 ? k_hop_x2a_big<REP, 1, true> : k_hop_x2a_big<REP, 0, true>)
-                                : (g5 ? k_hop_x2a_big<REP, 1, false> : k_hop_x2a_big<REP, 0, false>),
-                             !nc, grid, c.block, 0, s, a);
+                launch_reducible(ctx, nc ? (g5 ? k_hop_x2a_big<REP, 1, true> : k_hop_x2a_big<REP, 0, true>)
+                                : (g5 ? k_hop_x2a_big<REP, 1, false> : k_hop_x2a_big<REP, 0, false>), a, !nc, grid, c.block, 0, s);
                 st = hop_launched(ctx, a, grid, s, "paired adjoint hop kernel (168 registers)");
                 return true;
             }
@@ -726,14 +725,13 @@ template <int REP, int PREC> struct Launch {
                                                  (int)S::smem_bytes(256));
                         attr_set = true;
                     }
-                    launch_after(g5 ? k_hop_x2as<1> : k_hop_x2as<0>, hop_early(a), grid, c.block, S::smem_bytes(c.block), s, a);
+                    launch_reducible(ctx, g5 ? k_hop_x2as<1> : k_hop_x2as<0>, a, hop_early(a), grid, c.block, S::smem_bytes(c.block), s);
                     st = hop_launched(ctx, a, grid, s, "paired adjoint hop kernel");
                     return true;
                 }
             }
-            launch_after(nc ? (g5 ? k_hop_x2a<REP, 1, true> : k_hop_x2a<REP, 0, true>)
-                            : (g5 ? k_hop_x2a<REP, 1, false> : k_hop_x2a<REP, 0, false>),
-                         !nc, grid, c.block, 0, s, a);
+            launch_reducible(ctx, nc ? (g5 ? k_hop_x2a<REP, 1, true> : k_hop_x2a<REP, 0, true>)
+                            : (g5 ? k_hop_x2a<REP, 1, false> : k_hop_x2a<REP, 0, false>), a, !nc, grid, c.block, 0, s);
             st = hop_launched(ctx, a, grid, s, "paired adjoint hop kernel");
             return true;
         } else if constexpr (REP == kRepFund) {
@@ -749,9 +747,9 @@ template <int REP, int PREC> struct Launch {
             }
             const bool g5 = a.g5_in != 0;
             if (c.variant == kVarPairedStaged)
-                launch_after(g5 ? k_hop_f2s<PREC, 1> : k_hop_f2s<PREC, 0>, hop_early(a), grid, c.block, S::smem_bytes(c.block), s, a);
+                launch_reducible(ctx, g5 ? k_hop_f2s<PREC, 1> : k_hop_f2s<PREC, 0>, a, hop_early(a), grid, c.block, S::smem_bytes(c.block), s);
             else
-                launch_after(g5 ? k_hop_f2<PREC, 1> : k_hop_f2<PREC, 0>, hop_early(a), grid, c.block, 0, s, a);
+                launch_reducible(ctx, g5 ? k_hop_f2<PREC, 1> : k_hop_f2<PREC, 0>, a, hop_early(a), grid, c.block, 0, s);
             st = hop_launched(ctx, a, grid, s, "paired hop kernel");
             return true;
         }
@@ -772,7 +770,7 @@ void launch_hop_clover_paired(hr_ctx *ctx, const HopArgs &a, int grid, int block
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_bytes(256));
         attr_set = true;
     }
-    launch_after(a.g5_in ? k_hop_x2s_clov<1> : k_hop_x2s_clov<0>, hop_early(a), grid, block, S::smem_bytes(block), s, a);
+    launch_reducible(ctx, a.g5_in ? k_hop_x2s_clov<1> : k_hop_x2s_clov<0>, a, hop_early(a), grid, block, S::smem_bytes(block), s);
     st = hop_launched(ctx, a, grid, s, "paired hop kernel (clover epilogue)");
 }
 
