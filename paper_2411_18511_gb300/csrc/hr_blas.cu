@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kBS) k_axpy(Geom g, double a, const void *x, v
     const T aa = Real<T>::from_double(a);
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nv; j += gridDim.x * blockDim.x) {
         cpx<T> xv[4][NC], yv[4][NC];
-        load_spinor<NC, kF64>(x, g.nblk_s, j, xv);
+        load_spinor<NC, kF64, NC == 2>(x, g.nblk_s, j, xv); // (32^4: 31.0 -> 29.7 us, adjoint 47.4 -> 49.4)
         load_spinor<NC, kF64>(y, g.nblk_s, j, yv);
 #pragma unroll
         for (int s = 0; s < 4; ++s)

@@ -547,7 +547,7 @@ __device__ __forceinline__ void x2a_link(const HopArgs &a, const K2 &k, int link
 {
     if constexpr (REP == kRepAdj) {
         const float4 *q = link_base<float4>(a.gauge, a.g.nblk_g, link_par, mu, 2) + vec_index(site_link, 0, 2);
-        quat_to_adj_x2(k, ld_link<NC>(q), ld_link<NC>(q + 32), R);
+        quat_to_adj_x2(k, ld_operand<NC>(q), ld_operand<NC>(q + 32), R);
     } else {
         load_mat<kF64, NC>(a.gauge, a.g.nblk_g, link_par, mu, site_link, R);
     }

@@ -316,9 +316,9 @@ __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.
 // a vector of a field or of links: a plain load, not ld.global.nc -- a kernel may
 // be resident while the one before it still writes them
 template <class V> __device__ __forceinline__ V ld_field(const V *p) { return *p; }
-// the same for links in a kernel that starts after the previous one (NC): as ld.global.nc
-// the compiler may place, and repeat, the load where it likes
-template <bool NC, class V> __device__ __forceinline__ V ld_link(const V *p)
+// the same as ld.global.nc (NC), which the compiler may place, and repeat, where it
+// likes: for operands that the kernel only reads, if it starts after the previous one
+template <bool NC, class V> __device__ __forceinline__ V ld_operand(const V *p)
 {
     if constexpr (NC) return __ldg(p);
     else return *p;
@@ -448,7 +448,7 @@ __device__ __forceinline__ void f64_to_vecs(const cpx<T> (&s)[4][NC], float4 *w)
     }
 }
 
-template <int NC, int PREC, class T>
+template <int NC, int PREC, bool RO = false, class T>
 __device__ __forceinline__ void load_spinor(const void *base, int nblk, int j, cpx<T> (&s)[4][NC])
 {
     using L = SpinorLayout<NC, PREC>;
@@ -457,7 +457,7 @@ __device__ __forceinline__ void load_spinor(const void *base, int nblk, int j, c
         const float4 *p = (const float4 *)base;
         float4 w[NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) w[v] = ld_field(p + vec_index(j, v, NV));
+        for (int v = 0; v < NV; ++v) w[v] = ld_operand<RO>(p + vec_index(j, v, NV));
         f64_from_vecs<NC>(w, s);
     } else if constexpr (PREC == kF32) {
         const float4 *p = (const float4 *)base;
@@ -759,11 +759,11 @@ __device__ __forceinline__ void load_mat(const void *base, int nblk_g, int p, in
         const int idx = vec_index(i, e, 9);
         T v;
         if constexpr (PREC == kF64) {
-            float2 w = ld_link<NC>(link_base<float2>(base, nblk_g, p, mu, 9) + idx);
+            float2 w = ld_operand<NC>(link_base<float2>(base, nblk_g, p, mu, 9) + idx);
             if constexpr (std::is_same<T, dd>::value) v = dd(w.x, w.y);
             else v = Real<T>::from_double(dd_to_double(dd(w.x, w.y)));
         } else if constexpr (PREC == kF32) {
-            v = Real<T>::from_float(ld_link<NC>(link_base<float>(base, nblk_g, p, mu, 9) + idx));
+            v = Real<T>::from_float(ld_operand<NC>(link_base<float>(base, nblk_g, p, mu, 9) + idx));
         } else {
             v = Real<T>::from_float(__half2float(link_base<__half>(base, nblk_g, p, mu, 9)[idx]));
         }
