@@ -72,6 +72,8 @@ class Lattice(tuple):
     serves wherever extents do; every call of this module that takes ``dims``
     reads ``bc`` and ``theta`` from it."""
 
+    _given = None  # the twist angles that __new__ made, a tuple of floats
+
     def __new__(cls, dims, bc: int = 0, theta=None):
         self = super().__new__(cls, (int(d) for d in dims))
         if len(self) != 4:
@@ -83,7 +85,7 @@ class Lattice(tuple):
                 raise ValueError("four twist angles")
             if not any(theta):
                 theta = None
-        self.theta = theta
+        self.theta = self._given = theta
         return self
 
     def _c_struct(self) -> "hr_lattice":
@@ -92,10 +94,14 @@ class Lattice(tuple):
         value: ``theta`` may be a list or an array that was changed in place).  Kept
         from callers, who get one of their own from :func:`lattice`."""
         theta = self.theta
-        now = (int(self.bc), None if theta is None else tuple(float(theta[k]) for k in range(4)))
         made = self.__dict__.get("_made")
+        # floats of a tuple made by __new__ cannot change
+        if made is not None and theta is made[2] and theta is self._given and self.bc == made[0][0]:
+            return made[1]
+        now = (int(self.bc), None if theta is None else tuple(float(theta[k]) for k in range(4)))
         if made is None or made[0] != now:
-            made = self._made = (now, _fill_lattice(self, *now))
+            made = (now, _fill_lattice(self, *now))
+        self._made = made = (now, made[1], theta)
         return made[1]
 
     def __repr__(self):
