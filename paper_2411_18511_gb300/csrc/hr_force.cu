@@ -258,9 +258,9 @@ __device__ __forceinline__ bool load_digits(const Digits &D, int f, int k, fx (&
 // in the kernel (bound by the FP64 pipe: about 700 conversions and 1400
 // operations a site); error against a 64-bit evaluation 7.2e-15 with both (the
 // hops').  This kernel, converting (DIG = false): 0.413 ms at 168 registers, 0.479
-// at 216, 0.438 at 128 (spills).  With the digits (96 registers): 0.30 ms and 0.09
-// for k_field_digits (which HBM bounds) at 32^4, 22 + 5 against 34 us at 16^4, 36 + 7
-// against 48 us at 20 x 14 x 18 x 22; the whole force at 32^4 0.71 ms.
+// at 216, 0.438 at 128 (spills).  With the digits (96 registers): 0.31 ms and 0.09
+// for k_field_digits (load latency; its output stays in L2) at 32^4, 22 + 5 against 34 us
+// at 16^4, 36 + 7 against 48 us at 20 x 14 x 18 x 22; the whole force at 32^4 0.685 ms.
 // One thread per site in lexicographic order (so that a warp's outputs are
 // contiguous), a run-time loop over the four directions around one copy of the
 // conversion and product code: unrolled, the kernel would not fit the

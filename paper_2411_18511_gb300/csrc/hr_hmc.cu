@@ -332,7 +332,7 @@ __device__ __forceinline__ fx fx_fma_const(long long c, fx x, fx y)
 // scalar) of its digits.  Steps with z > 1, links with |d| > 2^-30 and vectors
 // below 2^-900 take native FP64.
 // 32^4: 0.78 ms in native FP64 (sin, cos, two square roots, two divisions), 0.163 ms
-// here (4.5 TB/s; 0.158 with the vectors in units of 1).
+// here (2.3 TB/s, bound by the integer pipes; 0.158 with the vectors in units of 1).
 constexpr unsigned kLinkVecMin = (1023u - 900u) << 20; // high word of 2^-900
 template <bool VEC>
 __global__ void __launch_bounds__(128) k_link_update(long long n_links, double eps, const double *p, double *q)
