@@ -1263,6 +1263,9 @@ __device__ __forceinline__ long long sigma_sigma(const fx *u, const fx *v, int l
 // Pi^b_lk = coef Re v^+ (s_l (x) s_k) u needs the real parts of 9 x 8 products
 // a block instead of the complex outer product u v^+; on odd sites the
 // determinant adds -8 (A^-1)_lk, the coefficient of s_l (x) s_k in A^-1.
+// One unit for a site's spinors is enough: a link's force sums the planes of four
+// corners of both parities and the hops' term of the same fields, whose native sums
+// round at the largest of them too, and the fields and A^-1 are pairs of 2^-49.
 __global__ void __launch_bounds__(128, 3) k_clover_kappa(KFieldArgs A)
 {
     const Geom &g = A.g;
@@ -1338,7 +1341,8 @@ __device__ __noinline__ void leaf_force_native(const Geom &g, const double *can,
 // the sum of the six B.  Fixed point (hr_fix.cuh): about 110 products a
 // plaquette, where the 2 x 2 complex matrices of hr_clover_leaf.cuh take 700.
 // The kappa of a plaquette are read in units of their largest component, and
-// the running sum of the B follows the largest unit met so far.  20 x 14 x 18 x 22:
+// the running sum of the B follows the largest unit met so far (native FP64 rounds
+// at that size as well: B is the sum of the rotated kappa).  20 x 14 x 18 x 22:
 // 4.99 ms in native FP64, 0.252 ms here (0.286 with conversions of 20 instead of 13
 // instructions a number; 128 registers: 0.298); the whole clover force (hops, link
 // derivatives, kappa, this) 5.77 -> 0.42 ms, error against 64 bits unchanged
