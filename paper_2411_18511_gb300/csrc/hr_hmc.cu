@@ -123,7 +123,7 @@ constexpr int kPlaqSplitSites = 1 << 17;
 
 // One link from the same vectors in native FP64, where some of them are doubles:
 // every term then carries 2^-53 of itself.  false: a link or a plaquette is out of range.
-// 32^4, all links near the identity: 1.49 to 1.64 ms for the whole force (2.03 with
+// 32^4, all links near the identity: 1.52 to 1.67 ms for the whole force (2.03 with
 // every staple in native FP64, 0.485 for links away from it).
 __device__ __noinline__ bool plaq_force_native(const Geom &g, const double *q, int mu, int t, double s, int first, int n,
                                                const int4 *pa, const int2 *pb, double *f)
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(128, 5) k_plaq_force(Geom g, double s, const d
     long long sum[NMU][3] = {}; // units 2^-56, rounded once per neighbour
     bool ok = true;
 #pragma unroll 1
-    for (int nu = 0; nu < 4 && ok; ++nu) {
+    for (int nu = 0; nu < 4; ++nu) {
         if (NMU == 1 && nu == (int)blockIdx.y) continue;
         int unused, down;
         lex_steps(g, x, nu, unused, down);
